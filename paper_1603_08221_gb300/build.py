@@ -11,6 +11,7 @@ SRC = os.path.join(HERE, "csrc", "lbm_mix.cu")
 SRCS = [SRC, os.path.join(HERE, "csrc", "lbm_adjoint.cu")]
 HDR = os.path.join(ROOT, "include", "lbm_mix.h")
 INTERNAL_HDR = os.path.join(HERE, "csrc", "lbm_internal.h")
+DEVICE_HDRS = [os.path.join(HERE, "csrc", n) for n in ("lbm_psi_table.cuh",)]
 LIB = os.path.join(HERE, "liblbm_mix.so")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-lineinfo",
@@ -27,7 +28,7 @@ def nvcc() -> str:
 def build(force: bool = False, verbose: bool = False) -> str:
     """Builds liblbm_mix.so unless it is newer than its sources: each
     translation unit is compiled in parallel, then linked."""
-    deps = SRCS + [HDR, INTERNAL_HDR]
+    deps = SRCS + [HDR, INTERNAL_HDR] + DEVICE_HDRS
     if (not force and os.path.exists(LIB)
             and os.path.getmtime(LIB) >= max(os.path.getmtime(s) for s in deps)):
         return LIB

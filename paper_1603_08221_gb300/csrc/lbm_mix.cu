@@ -43,6 +43,8 @@
 
 namespace {
 
+#include "lbm_psi_table.cuh"
+
 // ---------------------------------------------------------------- errors
 thread_local char g_err[512] = "";
 
@@ -85,22 +87,23 @@ struct Lat {
   float s[2];            // s_sigma = m_min / m_sigma
   float cw0[2];          // rest-equilibrium weights w_i alpha_si: rest (9 - 5s)/9,
   float cw1[2], cw5[2];  // axis s/9, diagonal s/36
-  // coefficients of the non-equilibrium energy moments on the deviations
-  // (rest, axis, diagonal): e: -2s, 3 - 2s, 6 - 2s; eps: 3s, 3s - 6, 3s - 3
-  float ke[2][3], kp[2][3];
-  // the same per-species constants as (species a, species b) pairs for the
-  // packed FP32x2 arithmetic
-  float2 s2, cw1_2, cw5_2, c_xl2, inv_c_xl2, ke2[3], kp2[3];
+  // the per-species constants as (species a, species b) pairs for the packed
+  // FP32x2 arithmetic; ke2, kp2: coefficients of the non-equilibrium energy
+  // moments on the deviations (rest, axis, diagonal: e: -2s, 3 - 2s, 6 - 2s;
+  // eps: 3s, 3s - 6, 3s - 3) times om_e / 36 and om_eps / 36, ku2: of
+  // rho u^2 (-3, 3) likewise
+  float2 s2, cw1_2, cw5_2, c_xl2, inv_c_xl2, ke2[3], kp2[3], ku2[2];
   float inv_c_lam;       // 1 / (3 mu sqrt(pi/6))
   float c_lam;           // 3 mu sqrt(pi/6): lambda = c_lam / (n sqrt(m_x))
   float c_xl[2];         // 3 mu_s sqrt(pi/(6 m_s)): x_s lambda_s = c_xl / n
   float inv_c_xl[2];
   float c_ts;            // sqrt(6/pi)
   float c_td;            // (3/2) sqrt(3 m0 m_a m_b / m_min)
-  float om_e, om_eps;    // 1/tau_e, 1/tau_eps
   float c_m0;
   float H;               // channel height = N
   double mh[2];          // m_sigma / m_min
+  float2 end_mass[2][2]; // N rho_s at the inlet, outlet ([end][species]) as a
+                         // sum of two floats
   double rho_in[2], rho_out[2];
   double C_in, C_out;    // light-species mole fraction at the ends
 };
@@ -126,10 +129,13 @@ __device__ __forceinline__ float e1_series(float x) {
 // x e^x E_1(x) for x >= 1: Hastings' rational approximation as tabulated in
 // Abramowitz & Stegun 5.1.56 (absolute error < 2e-8).
 __device__ __forceinline__ float xexe1_rational(float x) {
-  float num = (((x + 8.5733287401f) * x + 18.0590169730f) * x + 8.6347608925f) * x +
-              0.2677737343f;
-  float den = (((x + 9.5733223454f) * x + 25.6329561486f) * x + 21.0996530827f) * x +
-              3.9584969228f;
+  float num = x + 8.5733287401f, den = x + 9.5733223454f;
+  num = fmaf(num, x, 18.0590169730f);
+  num = fmaf(num, x, 8.6347608925f);
+  num = fmaf(num, x, 0.2677737343f);
+  den = fmaf(den, x, 25.6329561486f);
+  den = fmaf(den, x, 21.0996530827f);
+  den = fmaf(den, x, 3.9584969228f);
   return num / den;
 }
 
@@ -137,47 +143,44 @@ __device__ __forceinline__ float e1_dev(float x) {
   return x <= 1.0f ? e1_series(x) : expf(-x) * xexe1_rational(x) / x;
 }
 
-// psi(a) = 1 + (a - 1) e^{-a} - a^2 E_1(a)  (Eq. psi).
-//  a <= 1: with the series of E_1, psi(a) = Q(a) + a^2 ln a where
-//          Q(a) = 1 + (a - 1) e^{-a} + gamma a^2 - a^2 sum_k (-1)^{k+1} a^k/(k k!)
-//          is entire; its Taylor coefficients are 2, gamma - 3/2 and
-//          (-1)^m 2 / ((m - 2) m!) for m >= 3 (worked out from the two
-//          series); eleven terms leave < 4e-10 on [0, 1].
-//  1 < a < 15: psi = 1 + e^{-a} [(a - 1) - a (x e^x E_1)(a)] with the
-//          rational approximation above (no cancellation).
-//  a >= 15: 1 - psi < 2e^{-a}/a < 3e-8, below half an FP32 ulp of 1.
-__device__ __forceinline__ float psi_dev(float a) {
-  if (a <= 1.0f) {
-    if (!(a > 0.0f)) return 0.0f;
-    float q = -1.0f / 179625600.0f;
-    q = fmaf(q, a, 1.0f / 14515200.0f);
-    q = fmaf(q, a, -1.0f / 1270080.0f);
-    q = fmaf(q, a, 1.0f / 120960.0f);
-    q = fmaf(q, a, -1.0f / 12600.0f);
-    q = fmaf(q, a, 1.0f / 1440.0f);
-    q = fmaf(q, a, -1.0f / 180.0f);
-    q = fmaf(q, a, 1.0f / 24.0f);
-    q = fmaf(q, a, -1.0f / 3.0f);
-    q = fmaf(q, a, 0.5772156649f - 1.5f);
-    q = fmaf(q, a, 2.0f);
-    // __logf: absolute error ~2^-21 on ln a near a = 1, i.e. < 2e-7 in a^2 ln a
-    return fmaf(a * a, __logf(a), q * a);
-  }
-  if (a >= 16.0f) return 1.0f;  // 1 - psi(a) < 2 e^{-a}/a < 2^{-25}
-  float num = (((a + 8.5733287401f) * a + 18.0590169730f) * a + 8.6347608925f) * a +
-              0.2677737343f;
-  float den = (((a + 9.5733223454f) * a + 25.6329561486f) * a + 21.0996530827f) * a +
-              3.9584969228f;
-  return fmaf(__expf(-a), (a - 1.0f) - a * __fdividef(num, den), 1.0f);
+// psi(a) = 1 + (a - 1) e^{-a} - a^2 E_1(a)  (Eq. psi) and psi'(a), a >= 0,
+// from the cubics of lbm_psi_table.cuh: 12 instructions and one 16-byte load
+// that the lanes of a row share, against the 25 of a series for a <= 1 and a
+// rational form beyond, both evaluated.  At 57 % issue the FMA pipe was as
+// busy as the issue slots, and half of its work was psi.  Relative error below
+// 1.6e-7 (series and rational form: 1.9e-7).  T: the table, in shared memory
+// wherever a thread evaluates more than one value.
+__device__ __forceinline__ float psi_cubic(const float4* T, float am) {
+  const unsigned edge = __float_as_uint(fmaxf(am, 0x1p-22f)) & 0xfff80000u;
+  const float4 q = *reinterpret_cast<const float4*>(reinterpret_cast<const char*>(T) +
+                                                    ((edge >> 15) - (105u << 8)));
+  const float u = am - __uint_as_float(edge);
+  return fmaf(fmaf(fmaf(q.w, u, q.z), u, q.y), u, q.x);
+}
+__device__ __forceinline__ float psi_dev(const float4* T, float a) {
+  return __fmul_rn(psi_cubic(T, fminf(a, 16.0f)), fminf(a, 1.0f));
+}
+__device__ __forceinline__ float dpsi_dev(const float4* T, float a) {
+  return psi_cubic(T, fminf(a, 16.0f));
 }
 
-// psi'(a) = 2 e^{-a} - 2 a E_1(a).
-__device__ __forceinline__ float dpsi_dev(float a) {
-  if (a <= 1.0f) {
-    if (!(a > 0.0f)) return 2.0f;
-    return 2.0f * expf(-a) - 2.0f * a * e1_series(a);
-  }
-  return 2.0f * expf(-a) * (1.0f - xexe1_rational(a));
+// Copies psi's table to shared memory (the caller synchronises).
+__device__ __forceinline__ void load_psi_table(float4* dst, int tid, int threads) {
+  for (int k = tid; k < PSI_SEGMENTS; k += threads) dst[k] = kPsiTab[k];
+}
+
+// Reciprocal and reciprocal square root of the special-function unit (1 and
+// 2 ulp), without the scaling steps for subnormal arguments: densities,
+// masses and mean free paths are nowhere near them.
+__device__ __forceinline__ float rcp_fast(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float rsqrt_fast(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 
 // ------------------------------------------------- packed FP32x2 helpers
@@ -190,62 +193,6 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) {
   return __ffma2_rn(b, f2(-1.0f), a);  // exact: a - b with one rounding
-}
-
-// psi at two positive arguments at once.  The lanes of a warp sweep one row
-// (the same y) of 32 neighbouring columns, whose mean free paths differ
-// little, so with SKIP the two formulas of psi_dev are taken as warp-uniform
-// branches: the entire-part series when some lane has an argument <= 1, the
-// rational form when some lane has one in (1, 16).  Without SKIP both are
-// evaluated and selected (straight-line code that the compiler can
-// interleave with the loads of a memory-bound sweep).  At a >= 16,
-// 1 - psi(a) < 2 e^{-a}/a < 2^{-25} rounds away and psi = 1.
-template <bool SKIP>
-__device__ __forceinline__ float2 psi2(float2 a) {
-  const bool small = (a.x <= 1.0f) || (a.y <= 1.0f);
-  const bool mid = (a.x > 1.0f && a.x < 16.0f) || (a.y > 1.0f && a.y < 16.0f);
-  bool do_small = true, do_mid = true;
-  if (SKIP) {
-    const unsigned lanes = __activemask();
-    do_small = __any_sync(lanes, small);
-    do_mid = __any_sync(lanes, mid);
-  }
-  float2 ps = f2(0.0f), pl = f2(1.0f);
-  if (do_small) {
-    const float2 as = make_float2(fminf(a.x, 1.0f), fminf(a.y, 1.0f));
-    float2 q = f2(-1.0f / 179625600.0f);
-    q = fma2(q, as, f2(1.0f / 14515200.0f));
-    q = fma2(q, as, f2(-1.0f / 1270080.0f));
-    q = fma2(q, as, f2(1.0f / 120960.0f));
-    q = fma2(q, as, f2(-1.0f / 12600.0f));
-    q = fma2(q, as, f2(1.0f / 1440.0f));
-    q = fma2(q, as, f2(-1.0f / 180.0f));
-    q = fma2(q, as, f2(1.0f / 24.0f));
-    q = fma2(q, as, f2(-1.0f / 3.0f));
-    q = fma2(q, as, f2(0.5772156649f - 1.5f));
-    q = fma2(q, as, f2(2.0f));
-    const float2 lg = make_float2(__logf(as.x), __logf(as.y));
-    ps = fma2(mul2(as, as), lg, mul2(q, as));
-  }
-  if (do_mid) {
-    // the argument is clamped to [1, 16]: at 16 the formula gives 1 in FP32
-    // (1 - psi(16) < 2^-25), and larger arguments cannot overflow it
-    const float2 al = make_float2(fminf(fmaxf(a.x, 1.0f), 16.0f), fminf(fmaxf(a.y, 1.0f), 16.0f));
-    float2 num = add2(al, f2(8.5733287401f));
-    num = fma2(num, al, f2(18.0590169730f));
-    num = fma2(num, al, f2(8.6347608925f));
-    num = fma2(num, al, f2(0.2677737343f));
-    float2 den = add2(al, f2(9.5733223454f));
-    den = fma2(den, al, f2(25.6329561486f));
-    den = fma2(den, al, f2(21.0996530827f));
-    den = fma2(den, al, f2(3.9584969228f));
-    const float2 R = make_float2(__fdividef(num.x, den.x), __fdividef(num.y, den.y));
-    const float2 e = make_float2(__expf(-al.x), __expf(-al.y));
-    // 1 + e^{-a} [(a - 1) - a R]
-    pl = fma2(e, fma2(make_float2(-al.x, -al.y), R, add2(al, f2(-1.0f))), f2(1.0f));
-  }
-  // arguments are y / lambda > 0 (y >= 1/2)
-  return make_float2(a.x <= 1.0f ? ps.x : pl.x, a.y <= 1.0f ? ps.y : pl.y);
 }
 
 // ------------------------------------------------------------- storage
@@ -436,13 +383,15 @@ __device__ __forceinline__ void pull_node(const ST* __restrict__ f, const Lat& L
       // leaves column x + 1 as c_7
       const float q = 1.0f - r_bot;
       g[2] = ld(f, L, sp, 4, j, x);
-      g[5] = fmaf(r_bot, ld(f, L, sp, 7, j, x), q * fmaf(c5, dl, src(f, L, E, c5, sp, 8, j, xm)));
-      g[6] = fmaf(r_bot, ld(f, L, sp, 8, j, x), q * fmaf(c5, dr, src(f, L, E, c5, sp, 7, j, xp)));
+      g[5] = fmaf(r_bot, ld(f, L, sp, 7, j, x),
+                  __fmul_rn(q, fmaf(c5, dl, src(f, L, E, c5, sp, 8, j, xm))));
+      g[6] = fmaf(r_bot, ld(f, L, sp, 8, j, x),
+                  __fmul_rn(q, fmaf(c5, dr, src(f, L, E, c5, sp, 7, j, xp))));
     } else if (bot) {
       float o4 = ld(f, L, sp, 4, j, x), o7 = ld(f, L, sp, 7, j, x), o8 = ld(f, L, sp, 8, j, x);
       // the equilibrium parts t/6, t/6 and t - 2 t/6 sum to t exactly up
       // to one rounding, so the wall conserves mass without an FP32 bias
-      float t = r_bot * (o4 + o7 + o8), q = 1.0f - r_bot, t6 = t * (1.0f / 6.0f);
+      float t = __fmul_rn(r_bot, o4 + o7 + o8), q = 1.0f - r_bot, t6 = __fmul_rn(t, 1.0f / 6.0f);
       g[2] = fmaf(q, o4, fmaf(-2.0f, t6, t));
       g[5] = fmaf(q, o7, t6);
       g[6] = fmaf(q, o8, t6);
@@ -456,11 +405,13 @@ __device__ __forceinline__ void pull_node(const ST* __restrict__ f, const Lat& L
       // of c_5 from column x - 1
       const float q = 1.0f - r_top;
       g[4] = ld(f, L, sp, 2, j, x);
-      g[7] = fmaf(r_top, ld(f, L, sp, 5, j, x), q * fmaf(c5, dr, src(f, L, E, c5, sp, 6, j, xp)));
-      g[8] = fmaf(r_top, ld(f, L, sp, 6, j, x), q * fmaf(c5, dl, src(f, L, E, c5, sp, 5, j, xm)));
+      g[7] = fmaf(r_top, ld(f, L, sp, 5, j, x),
+                  __fmul_rn(q, fmaf(c5, dr, src(f, L, E, c5, sp, 6, j, xp))));
+      g[8] = fmaf(r_top, ld(f, L, sp, 6, j, x),
+                  __fmul_rn(q, fmaf(c5, dl, src(f, L, E, c5, sp, 5, j, xm))));
     } else if (top) {
       float o2 = ld(f, L, sp, 2, j, x), o5 = ld(f, L, sp, 5, j, x), o6 = ld(f, L, sp, 6, j, x);
-      float t = r_top * (o2 + o5 + o6), q = 1.0f - r_top, t6 = t * (1.0f / 6.0f);
+      float t = __fmul_rn(r_top, o2 + o5 + o6), q = 1.0f - r_top, t6 = __fmul_rn(t, 1.0f / 6.0f);
       g[4] = fmaf(q, o2, fmaf(-2.0f, t6, t));
       g[7] = fmaf(q, o5, t6);
       g[8] = fmaf(q, o6, t6);
@@ -493,12 +444,18 @@ __device__ __forceinline__ void pull_fast(const ST* __restrict__ p, const ST* __
 }
 
 // ---------------------------------------------------------------- moments
+// The node arithmetic is written with explicit fma, mul and add wherever a
+// product feeds a sum, so that every kernel that inlines it rounds alike:
+// the step kernel, the wall kernel and the tile kernel give the same bits.
 struct Macro {
   float sd[2];           // sum of deviations: rho_s - rhobar_s
-  float rho[2], jx[2], jy[2];
-  float ux, uy;
+  float rho[2];
   float n, inv_n, mx;
 };
+
+__device__ __forceinline__ float number_density(const Lat& L, float rho_a, float rho_b) {
+  return fmaf(rho_a, L.s[0], __fmul_rn(rho_b, L.s[1]));  // Eq. P
+}
 
 __device__ __forceinline__ void macro(const Lat& L, const ColRef& C, const float fs[2][9],
                                       Macro& m) {
@@ -507,16 +464,10 @@ __device__ __forceinline__ void macro(const Lat& L, const ColRef& C, const float
     const float* g = fs[sp];
     m.sd[sp] = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
     m.rho[sp] = C.rb[sp] + m.sd[sp];
-    m.jx[sp] = (g[1] - g[3]) + (g[5] - g[6]) + (g[8] - g[7]);
-    m.jy[sp] = (g[2] - g[4]) + (g[5] - g[7]) + (g[6] - g[8]);
   }
-  float rho = m.rho[0] + m.rho[1];
-  float inv_rho = __fdividef(1.0f, rho);
-  m.ux = (m.jx[0] + m.jx[1]) * inv_rho;
-  m.uy = (m.jy[0] + m.jy[1]) * inv_rho;
-  m.n = fmaf(m.rho[0], L.s[0], m.rho[1] * L.s[1]);  // number density (Eq. P)
-  m.inv_n = __fdividef(1.0f, m.n);
-  m.mx = rho * m.inv_n;  // m_x = rho / n
+  m.n = number_density(L, m.rho[0], m.rho[1]);
+  m.inv_n = rcp_fast(m.n);
+  m.mx = __fmul_rn(__fadd_rn(m.rho[0], m.rho[1]), m.inv_n);  // m_x = rho / n
 }
 
 // ------------------------------------------- packed per-node arithmetic
@@ -525,57 +476,81 @@ __device__ __forceinline__ void macro(const Lat& L, const ColRef& C, const float
 struct Macro2 {
   float2 sd;   // sum of deviations: rho_s - rhobar_s
   float2 rho;  // species densities
-  float2 jx, jy;
-  float ux, uy;
-  float n, inv_n, mx;
+  float n, inv_n, inv_rho, mx;
 };
 
-__device__ __forceinline__ void macro2(const Lat& L, const ColRef& C, const float2 g[9],
-                                       Macro2& m) {
-  m.sd = add2(add2(add2(add2(g[0], g[1]), add2(g[2], g[3])), add2(add2(g[4], g[5]), add2(g[6], g[7]))),
-              g[8]);
-  m.rho = add2(make_float2(C.rb[0], C.rb[1]), m.sd);
-  m.jx = add2(add2(sub2(g[1], g[3]), sub2(g[5], g[6])), sub2(g[8], g[7]));
-  m.jy = add2(add2(sub2(g[2], g[4]), sub2(g[5], g[7])), sub2(g[6], g[8]));
-  const float rho = m.rho.x + m.rho.y;
-  const float inv_rho = __fdividef(1.0f, rho);
-  m.ux = (m.jx.x + m.jx.y) * inv_rho;
-  m.uy = (m.jy.x + m.jy.y) * inv_rho;
-  m.n = fmaf(m.rho.x, L.s[0], m.rho.y * L.s[1]);  // number density (Eq. P)
-  m.inv_n = __fdividef(1.0f, m.n);
-  m.mx = rho * m.inv_n;  // m_x = rho / n
+// Density deviations of both species from the pulled populations.
+__device__ __forceinline__ float2 density_sum(const float2 g[9]) {
+  const float2 a14 = add2(add2(g[1], g[3]), add2(g[2], g[4]));
+  const float2 a58 = add2(add2(g[5], g[7]), add2(g[6], g[8]));
+  return add2(g[0], add2(a14, a58));
+}
+
+__device__ __forceinline__ void macro2(const Lat& L, float2 rb, const float2 g[9], Macro2& m) {
+  m.sd = density_sum(g);
+  m.rho = add2(rb, m.sd);
+  const float rho = __fadd_rn(m.rho.x, m.rho.y);
+  m.inv_rho = rcp_fast(rho);
+  m.n = number_density(L, m.rho.x, m.rho.y);
+  m.inv_n = rcp_fast(m.n);
+  m.mx = __fmul_rn(rho, m.inv_n);  // m_x = rho / n
+}
+
+// Sums and differences of opposite populations, from which the momenta, the
+// other moments and the collision are formed, and the mixture velocity.
+// Formed after the relaxation rates: carried across their evaluation they
+// would not fit the registers.
+struct Flow2 {
+  float2 s13, s24, s57, s68, d13, d24, d57, d68, dx, dy, jx, jy;
+  float ux, uy;
+};
+__device__ __forceinline__ void flow2(const float2 g[9], float inv_rho, Flow2& w) {
+  w.s13 = add2(g[1], g[3]);
+  w.s24 = add2(g[2], g[4]);
+  w.s57 = add2(g[5], g[7]);
+  w.s68 = add2(g[6], g[8]);
+  w.d13 = sub2(g[1], g[3]);
+  w.d24 = sub2(g[2], g[4]);
+  w.d57 = sub2(g[5], g[7]);
+  w.d68 = sub2(g[6], g[8]);
+  w.dx = sub2(w.d57, w.d68);  // diagonal momenta
+  w.dy = add2(w.d57, w.d68);
+  w.jx = add2(w.d13, w.dx);
+  w.jy = add2(w.d24, w.dy);
+  w.ux = __fmul_rn(__fadd_rn(w.jx.x, w.jx.y), inv_rho);
+  w.uy = __fmul_rn(__fadd_rn(w.jy.x, w.jy.y), inv_rho);
 }
 
 // 1/tau_s (Eq. taos) and 1/tau_d (Eq. EQFrsp with lambda_se = lambda_s
 // Psi(y; lambda_s), lambda_s = (mu_s/p_s) sqrt(pi k_B T/(2 m_s)), p_s = x_s p),
 // with the wall-confinement factor Psi(y) = (psi(y/lambda) + psi((H-y)/lambda))/2
-// of the effective mean free path; the six psi values come from three packed
-// evaluations.
-template <bool SKIP>
-__device__ __forceinline__ void rates2(const Lat& L, const Macro2& m, float y, float& om_s,
-                                       float& om_d) {
-  const float rs_mx = rsqrtf(m.mx);
-  const float lam = L.c_lam * m.inv_n * rs_mx;                // mixture mean free path
-  const float inv_lam = L.inv_c_lam * m.n * (m.mx * rs_mx);  // 1 / lambda
-  const float2 yy = make_float2(y, L.H - y);
+// of the effective mean free path.  T: psi's table in shared memory.
+__device__ __forceinline__ void rates2(const Lat& L, const float4* T, const Macro2& m, float y,
+                                       float& om_s, float& om_d) {
+  const float rs_mx = rsqrt_fast(m.mx);
+  const float lam = __fmul_rn(__fmul_rn(L.c_lam, m.inv_n), rs_mx);  // mixture mean free path
+  const float inv_lam = __fmul_rn(__fmul_rn(L.inv_c_lam, m.n), __fmul_rn(m.mx, rs_mx));
+  const float y2 = __fsub_rn(L.H, y);
   // 1 / lambda_s: n_s / c_xl with the partial pressure, n / c_xl with the
   // mixture pressure
   const float2 ns = mul2(m.rho, L.s2);
   const float2 inv_ls = mul2(L.lam_mix ? f2(m.n) : ns, L.inv_c_xl2);
-  const float2 pm = psi2<SKIP>(mul2(yy, f2(inv_lam)));
-  const float2 pa = psi2<SKIP>(mul2(yy, f2(inv_ls.x)));
-  const float2 pb = psi2<SKIP>(mul2(yy, f2(inv_ls.y)));
-  const float ts = lam * (0.5f * (pm.x + pm.y)) * L.c_ts * rs_mx;  // tau_s - 1/2
-  om_s = __fdividef(1.0f, 0.5f + ts);
+  auto confined = [&](float il) {  // 2 Psi
+    return __fadd_rn(psi_dev(T, __fmul_rn(y, il)), psi_dev(T, __fmul_rn(y2, il)));
+  };
+  const float pm = confined(inv_lam);
+  const float2 ps = make_float2(confined(inv_ls.x), confined(inv_ls.y));
+  // tau_s - 1/2 = lambda Psi c_ts / sqrt(m_x)
+  const float tsm = __fmul_rn(__fmul_rn(lam, __fmul_rn(0.5f, pm)), L.c_ts);
+  om_s = rcp_fast(fmaf(tsm, rs_mx, 0.5f));
   // x_s lambda_se = c_xl / n * Psi(y; lambda_s) (partial pressure), times
   // x_s = n_s / n with the mixture pressure
   const float2 xs = L.lam_mix ? mul2(ns, f2(m.inv_n)) : f2(1.0f);
-  const float2 xle = mul2(mul2(mul2(L.c_xl2, f2(0.5f * m.inv_n)), xs),
-                          make_float2(pa.x + pa.y, pb.x + pb.y));
-  const float br = rsqrtf(xle.x) + rsqrtf(xle.y);
+  const float2 xle = mul2(mul2(mul2(L.c_xl2, f2(__fmul_rn(0.5f, m.inv_n))), xs), ps);
+  const float br = __fadd_rn(rsqrt_fast(xle.x), rsqrt_fast(xle.y));
   // tau_d = 1/2 + c_td / (m_x br^2)  =>  1/tau_d = d / (d/2 + c_td), d = m_x br^2
-  const float d = m.mx * br * br;
-  om_d = __fdividef(d, fmaf(0.5f, d, L.c_td));
+  const float d = __fmul_rn(__fmul_rn(m.mx, br), br);
+  om_d = __fmul_rn(d, rcp_fast(fmaf(0.5f, d, L.c_td)));
 }
 
 // MRT collision of both species at once (Eqs. MR, S, feq) on the deviations g from
@@ -585,72 +560,79 @@ __device__ __forceinline__ void rates2(const Lat& L, const Macro2& m, float y, f
 // -u_x, u_y, -u_y, u_x^2 - u_y^2, u_x u_y).  The reference has m = m^eq(u=0),
 // so e - e^eq = sum_i (e_i + 4 - 2s) g_i - 3 rho u^2 and
 // eps - eps^eq = sum_i (eps_i - 4 + 3s) g_i + 3 rho u^2 need no large terms
-// (ke, kp hold those coefficients for the rest, axis and diagonal classes).
+// (ke, kp hold those coefficients for the rest, axis and diagonal classes,
+// times om_e / 36 and om_eps / 36, the classes' common factor in M^{-1}).
 // Returns the x components of the species momenta of Eq. rhou,
 // j_x - (j_x - rho_s u_x)/(2 tau_d).
-__device__ __forceinline__ float2 collide2(float2 g[9], const Lat& L, float2 rho, float ux,
-                                           float uy, float om_e, float om_eps, float om_d,
+__device__ __forceinline__ float2 collide2(float2 g[9], const Lat& L, const Macro2& m, float om_d,
                                            float om_q, float om_s) {
-  const float2 ru2 = mul2(f2(3.0f * (ux * ux + uy * uy)), rho);
-  const float2 a14 = add2(add2(g[1], g[2]), add2(g[3], g[4]));
-  const float2 a58 = add2(add2(g[5], g[6]), add2(g[7], g[8]));
-  const float2 ne =
-      fma2(L.ke2[0], g[0], fma2(L.ke2[1], a14, fma2(L.ke2[2], a58, make_float2(-ru2.x, -ru2.y))));
-  const float2 neps = fma2(L.kp2[0], g[0], fma2(L.kp2[1], a14, fma2(L.kp2[2], a58, ru2)));
-  const float2 d13 = sub2(g[1], g[3]), d24 = sub2(g[2], g[4]);
-  const float2 dx56 = add2(sub2(g[5], g[6]), sub2(g[8], g[7]));
-  const float2 dy56 = add2(sub2(g[5], g[7]), sub2(g[6], g[8]));
-  const float2 jx = add2(d13, dx56);
-  const float2 jy = add2(d24, dy56);
-  const float2 qx = fma2(f2(-2.0f), d13, dx56);
-  const float2 qy = fma2(f2(-2.0f), d24, dy56);
-  const float2 pxx = sub2(add2(g[1], g[3]), add2(g[2], g[4]));
-  const float2 pxy = sub2(add2(g[5], g[7]), add2(g[6], g[8]));
-  const float2 de = mul2(f2(om_e), ne);
-  const float2 deps = mul2(f2(om_eps), neps);
-  const float2 djx = mul2(f2(om_d), fma2(rho, f2(-ux), jx));
-  const float2 djy = mul2(f2(om_d), fma2(rho, f2(-uy), jy));
-  const float2 dqx = mul2(f2(om_q), fma2(rho, f2(ux), qx));
-  const float2 dqy = mul2(f2(om_q), fma2(rho, f2(uy), qy));
-  const float2 dpxx = mul2(f2(om_s), fma2(rho, f2(-(ux * ux - uy * uy)), pxx));
-  const float2 dpxy = mul2(f2(om_s), fma2(rho, f2(-(ux * uy)), pxy));
-  const float2 c0 = mul2(sub2(de, deps), f2(1.0f / 9.0f));
-  const float2 c14 = fma2(de, f2(1.0f / 36.0f), mul2(deps, f2(1.0f / 18.0f)));
-  const float2 c58 = fma2(de, f2(-1.0f / 18.0f), mul2(deps, f2(-1.0f / 36.0f)));
-  const float2 ax = mul2(sub2(dqx, djx), f2(1.0f / 6.0f));
-  const float2 ay = mul2(sub2(dqy, djy), f2(1.0f / 6.0f));
-  const float2 bx = fma2(djx, f2(-1.0f / 6.0f), mul2(dqx, f2(-1.0f / 12.0f)));
-  const float2 by = fma2(djy, f2(-1.0f / 6.0f), mul2(dqy, f2(-1.0f / 12.0f)));
-  const float2 pp = mul2(dpxx, f2(0.25f)), pq = mul2(dpxy, f2(0.25f));
+  Flow2 w;
+  flow2(g, m.inv_rho, w);
+  const float ux = w.ux, uy = w.uy, uy2 = __fmul_rn(uy, uy);
+  const float2 rho = m.rho;
+  const float2 ru2 = mul2(f2(fmaf(ux, ux, uy2)), rho);
+  const float2 a14 = add2(w.s13, w.s24), a58 = add2(w.s57, w.s68);
+  const float2 de = fma2(L.ke2[0], g[0],
+                         fma2(L.ke2[1], a14, fma2(L.ke2[2], a58, mul2(L.ku2[0], ru2))));
+  const float2 dp = fma2(L.kp2[0], g[0],
+                         fma2(L.kp2[1], a14, fma2(L.kp2[2], a58, mul2(L.ku2[1], ru2))));
+  const float2 qx = fma2(f2(-2.0f), w.d13, w.dx);
+  const float2 qy = fma2(f2(-2.0f), w.d24, w.dy);
+  const float2 pxx = sub2(w.s13, w.s24), pxy = sub2(w.s57, w.s68);
+  // relaxed moments over |M_k|^2: momenta om_d / 6, heat fluxes om_q / 12,
+  // stresses om_s / 4
+  const float2 od = f2(__fmul_rn(om_d, 1.0f / 6.0f)), oq = f2(__fmul_rn(om_q, 1.0f / 12.0f)),
+               os = f2(__fmul_rn(om_s, 0.25f));
+  const float2 Jx = mul2(od, fma2(rho, f2(-ux), w.jx));
+  const float2 Jy = mul2(od, fma2(rho, f2(-uy), w.jy));
+  const float2 Qx = mul2(oq, fma2(rho, f2(ux), qx));
+  const float2 Qy = mul2(oq, fma2(rho, f2(uy), qy));
+  const float2 pp = mul2(os, fma2(rho, f2(fmaf(-ux, ux, uy2)), pxx));
+  const float2 pq = mul2(os, fma2(rho, f2(__fmul_rn(-ux, uy)), pxy));
+  const float2 c14 = fma2(f2(2.0f), dp, de);  // axis class
+  const float2 c58 = fma2(f2(2.0f), de, dp);  // minus the diagonal class
+  const float2 ax = fma2(f2(-2.0f), Qx, Jx), ay = fma2(f2(-2.0f), Qy, Jy);
+  const float2 bx = add2(Jx, Qx), by = add2(Jy, Qy);
   const float2 u1 = sub2(c14, pp), u2 = add2(c14, pp);  // shared by opposite axis pairs
-  const float2 v5 = sub2(c58, pq), v6 = add2(c58, pq);  // and by opposite diagonal pairs
-  const float2 w5 = add2(bx, by), w6 = sub2(by, bx);
-  g[0] = add2(g[0], c0);
-  g[1] = add2(g[1], add2(u1, ax));
-  g[3] = add2(g[3], sub2(u1, ax));
-  g[2] = add2(g[2], add2(u2, ay));
-  g[4] = add2(g[4], sub2(u2, ay));
-  g[5] = add2(g[5], add2(v5, w5));
-  g[7] = add2(g[7], sub2(v5, w5));
-  g[6] = add2(g[6], add2(v6, w6));
-  g[8] = add2(g[8], sub2(v6, w6));
-  return fma2(f2(-0.5f), djx, jx);
+  const float2 v5 = add2(c58, pq), v6 = sub2(c58, pq);  // and by opposite diagonal pairs
+  const float2 w5 = add2(bx, by), w6 = sub2(bx, by);
+  g[0] = fma2(f2(4.0f), sub2(de, dp), g[0]);
+  g[1] = add2(g[1], sub2(u1, ax));
+  g[3] = add2(g[3], add2(u1, ax));
+  g[2] = add2(g[2], sub2(u2, ay));
+  g[4] = add2(g[4], add2(u2, ay));
+  g[5] = sub2(g[5], add2(v5, w5));
+  g[7] = sub2(g[7], sub2(v5, w5));
+  g[6] = sub2(g[6], sub2(v6, w6));
+  g[8] = sub2(g[8], add2(v6, w6));
+  return fma2(f2(-3.0f), Jx, w.jx);
 }
 
-// tau_q of Eq. taoq from the wall node's lambda and m_x (tau'_s(0) in its
-// last term, dx = 1) and the node's accommodation coefficient (Eq. A12).
-__device__ __forceinline__ float tau_q_wall(const Lat& L, const Macro& m, float alpha) {
+// (A1, A2) of Eq. A12 from a wall node's accommodation coefficient.
+__device__ __forceinline__ float2 slip_coefficients(float alpha) {
+  const float A1 = __fmul_rn((2.0f - alpha) / alpha, fmaf(-0.1817f, alpha, 1.0f));
+  return make_float2(A1, fmaf(__fmul_rn(0.5f, A1), A1, 1.0f / kPi));
+}
+
+// 1/tau_q of Eq. taoq from the wall node's n, 1/n and m_x (tau'_s(0) in its
+// last term, dx = 1) and A = (A1, A2) of its accommodation coefficient.  P,
+// D: the tables of psi and psi'.
+__device__ __forceinline__ float inv_tau_q(const Lat& L, const float4* P, const float4* D,
+                                           float n, float inv_n, float mx, float2 A) {
   const float vs = 0.72360125455f;  // varsigma = sqrt(pi/6)
-  float rs_mx = rsqrtf(m.mx);
-  float lam = L.c_lam * m.inv_n * rs_mx;
-  float g = L.c_ts * rs_mx;  // sqrt(6/(pi m_x))
-  float a = L.H / lam;
-  float tt = lam * 0.5f * psi_dev(a) * g;
-  float dtt = 0.5f * g * (2.0f - dpsi_dev(a));
-  float A1 = (2.0f - alpha) / alpha * (1.0f - 0.1817f * alpha);
-  float A2 = 1.0f / kPi + 0.5f * A1 * A1;
-  return 0.5f + (3.0f + 24.0f * vs * vs * tt * tt * A2) / (16.0f * tt) +
-         dtt * (12.0f + 30.0f * tt * vs * A1) / (16.0f * tt * tt);
+  const float rs_mx = rsqrt_fast(mx);
+  const float lam = __fmul_rn(__fmul_rn(L.c_lam, inv_n), rs_mx);
+  const float a = __fmul_rn(L.H, __fmul_rn(__fmul_rn(L.inv_c_lam, n), __fmul_rn(mx, rs_mx)));
+  const float g = __fmul_rn(L.c_ts, rs_mx);  // sqrt(6/(pi m_x))
+  const float tt = __fmul_rn(__fmul_rn(__fmul_rn(lam, 0.5f), psi_dev(P, a)), g);
+  const float dtt = __fmul_rn(__fmul_rn(0.5f, g), __fsub_rn(2.0f, dpsi_dev(D, a)));
+  const float tt2 = __fmul_rn(tt, tt);
+  // tau_q = 1/2 + p / (16 tt) + dtt q / (16 tt^2) over one denominator
+  const float p = fmaf(__fmul_rn(24.0f * vs * vs, tt2), A.y, 3.0f);
+  const float q = fmaf(__fmul_rn(30.0f * vs, tt), A.x, 12.0f);
+  const float num = fmaf(dtt, q, __fmul_rn(tt, p));
+  const float den = __fmul_rn(16.0f, tt2);
+  return den / fmaf(0.5f, den, num);
 }
 
 // r of Eq. R, r = 2 - 2/(1 + X), from the mixture molecular mass of the
@@ -660,6 +642,24 @@ __device__ __forceinline__ float tau_q_wall(const Lat& L, const Macro& m, float 
 // m_x/(6 m_s)) (m_min replaced by the species mass) or c_m sqrt(pi m_x^2/(6
 // m_s)) (second printed form, m_r = m_s/m_x).  With the BSR wall the
 // bounce-back fraction 1/(1 + X) of the same slip factor X.
+__device__ __forceinline__ float slip_cm(const Lat& L, float alpha) {
+  return __fmul_rn(L.c_m0, __fsub_rn(2.0f, alpha)) / alpha;
+}
+__device__ __forceinline__ float2 slip_r(const Lat& L, float rho_a, float rho_b, float cm) {
+  const float mx = __fadd_rn(rho_a, rho_b) / number_density(L, rho_a, rho_b);
+  const float q = sqrtf(__fmul_rn(kPi / 6.0f, mx));
+  float X0 = __fmul_rn(cm, q);
+  if (L.r_form == LBM_R_SECOND) X0 = __fmul_rn(X0, sqrtf(mx));
+  float r[2];
+#pragma unroll
+  for (int sp = 0; sp < 2; ++sp) {
+    // 1 + X with one rounding
+    const float den =
+        L.r_form == LBM_R_FIRST ? fmaf(cm, q, 1.0f) : fmaf(X0, L.rsqrt_mh[sp], 1.0f);
+    r[sp] = L.wall_mode == LBM_WALL_BSR ? 1.0f / den : __fsub_rn(2.0f, 2.0f / den);
+  }
+  return make_float2(r[0], r[1]);
+}
 template <typename ST>
 __device__ __forceinline__ float2 dbb_r(const Lat& L, const ColRef& C, const ST* __restrict__ f,
                                         int x, int j, float alpha) {
@@ -671,16 +671,45 @@ __device__ __forceinline__ float2 dbb_r(const Lat& L, const ColRef& C, const ST*
     for (int i = 0; i < 9; ++i) acc += ld(f, L, sp, i, j, x);
     rho[sp] = C.rb[sp] + acc;
   }
-  float mx = (rho[0] + rho[1]) / fmaf(rho[0], L.s[0], rho[1] * L.s[1]);
-  float cm = L.c_m0 * (2.0f - alpha) / alpha;
-  const float X0 = cm * sqrtf(kPi * mx / 6.0f) * (L.r_form == LBM_R_SECOND ? sqrtf(mx) : 1.0f);
-  float r[2];
-#pragma unroll
-  for (int sp = 0; sp < 2; ++sp) {
-    const float X = L.r_form == LBM_R_FIRST ? X0 : X0 * L.rsqrt_mh[sp];
-    r[sp] = L.wall_mode == LBM_WALL_BSR ? 1.0f / (1.0f + X) : 2.0f - 2.0f / (1.0f + X);
-  }
-  return make_float2(r[0], r[1]);
+  return slip_r(L, rho[0], rho[1], slip_cm(L, alpha));
+}
+
+// A sum of two floats, hi + lo with |lo| <= ulp(hi) / 2: 48 bits of the
+// slow FP64 pipe's work in a few FP32 operations.
+__device__ __forceinline__ float2 split_double(double v) {
+  const float hi = (float)v;
+  return make_float2(hi, (float)(v - (double)hi));
+}
+// a + b with its rounding error (Knuth's two-sum).
+__device__ __forceinline__ float2 two_sum(float a, float b) {
+  const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+  return make_float2(s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb)));
+}
+// The same for |a| >= |b| (Dekker).
+__device__ __forceinline__ float2 quick_two_sum(float a, float b) {
+  const float s = __fadd_rn(a, b);
+  return make_float2(s, __fsub_rn(b, __fsub_rn(s, a)));
+}
+
+// kappa = mass / (2 c1 - c2) of one species at one end (Eq. rho2; mass = N
+// rho_end) from the column sums c1, c2 of the two columns next to it, and the
+// ghost reference offset kappa (2 r1 - r2) - r0.  In float pairs: sixteen
+// dependent FP64 operations took 2400 cycles, this takes under 200, and its
+// error (2^-44) vanishes in the rounding of the results to FP32.
+__device__ __forceinline__ void end_factors(float2 mass, float2 c1, float2 c2, float r0, float r1,
+                                            float r2, float& kappa, float& offset) {
+  float2 D = two_sum(__fmul_rn(2.0f, c1.x), -c2.x);
+  D = quick_two_sum(D.x, __fadd_rn(D.y, fmaf(2.0f, c1.y, -c2.y)));
+  const float inv = rcp_fast(D.x);
+  const float q = __fmul_rn(mass.x, inv);
+  const float rest = __fadd_rn(fmaf(-q, D.x, mass.x), fmaf(-q, D.y, mass.y));
+  const float2 k = quick_two_sum(q, __fmul_rn(rest, inv));
+  const float2 R = two_sum(__fmul_rn(2.0f, r1), -r2);
+  const float p = __fmul_rn(k.x, R.x);
+  const float pl = __fadd_rn(fmaf(k.x, R.x, -p), fmaf(k.x, R.y, __fmul_rn(k.y, R.x)));
+  const float2 o = two_sum(p, -r0);
+  kappa = k.x;
+  offset = __fadd_rn(o.x, __fadd_rn(o.y, pl));
 }
 
 // Density-correction factors of Eq. rho2 for the ghost columns, from the
@@ -701,16 +730,12 @@ __device__ __forceinline__ Ends load_ends(const Lat& L, const double* __restrict
   for (int sp = 0; sp < 2; ++sp) {
     const double* c = cs + (size_t)sp * Nx;
     const float* r = refrho + sp * Nx;
-    if (x0 <= 1 && 1 < x0 + width) {
-      double k = L.N * L.rho_in[sp] / (2.0 * c[1] - c[2]);
-      E.kin[sp] = (float)k;
-      E.gin[sp] = (float)(k * (2.0 * (double)r[1] - (double)r[2]) - (double)r[0]);
-    }
-    if (x0 <= Nx - 2 && Nx - 2 < x0 + width) {
-      double k = L.N * L.rho_out[sp] / (2.0 * c[Nx - 2] - c[Nx - 3]);
-      E.kout[sp] = (float)k;
-      E.gout[sp] = (float)(k * (2.0 * (double)r[Nx - 2] - (double)r[Nx - 3]) - (double)r[Nx - 1]);
-    }
+    if (x0 <= 1 && 1 < x0 + width)
+      end_factors(L.end_mass[0][sp], split_double(c[1]), split_double(c[2]), r[0], r[1], r[2],
+                  E.kin[sp], E.gin[sp]);
+    if (x0 <= Nx - 2 && Nx - 2 < x0 + width)
+      end_factors(L.end_mass[1][sp], split_double(c[Nx - 2]), split_double(c[Nx - 3]), r[Nx - 1],
+                  r[Nx - 2], r[Nx - 3], E.kout[sp], E.gout[sp]);
   }
   return E;
 }
@@ -756,7 +781,7 @@ __device__ __forceinline__ void wall_task(const Lat& L, const ST* __restrict__ f
     pull_node(fin, L, E, C, x, jw, rr, rr, fs);
     Macro m;
     macro(L, C, fs, m);
-    v = 1.0f / tau_q_wall(L, m, al);
+    v = inv_tau_q(L, kPsiTab, kDpsiTab, m.n, m.inv_n, m.mx, slip_coefficients(al));
   }
 }
 
@@ -1074,9 +1099,11 @@ template <typename ST, bool DIAG, bool WK = (sizeof(ST) < 4)>
 __global__ void __launch_bounds__(TX* TY, 3) lbm_step_kernel(Lat L, StepArgs<ST> a) {
   __shared__ WallSmem wsm;
   __shared__ RedSmem rsm;
+  __shared__ float4 psi_tab[PSI_SEGMENTS];
   if (a.pdl_early) pdl_launch_dependents();
-  pdl_wait();
   const int tx = threadIdx.x, ty = threadIdx.y;
+  load_psi_table(psi_tab, ty * TX + tx, TX * TY);  // overlaps the kernel before this one
+  pdl_wait();
   const int x0 = blockIdx.x * TX, x = x0 + tx;
   const ColRef C = col_ref(L, a.refrho, x);
   const Ends E = load_ends(L, a.cs_in, a.refrho, blockIdx.x * TX, TX);
@@ -1089,7 +1116,10 @@ __global__ void __launch_bounds__(TX* TY, 3) lbm_step_kernel(Lat L, StepArgs<ST>
   // r and 1/tau_q of this column: from lbm_walls_kernel (WK, read where they
   // are used) or from the CTA's wall prologue
   const int xc = x < L.Nx ? x : L.Nx - 1;
-  if constexpr (!WK) wall_prologue<true>(L, a.fin, a.alpha, E, C, x, j_begin, j_end, wsm);
+  if constexpr (!WK)
+    wall_prologue<true>(L, a.fin, a.alpha, E, C, x, j_begin, j_end, wsm);
+  else
+    __syncthreads();  // psi's table
   auto wall_r = [&](int w) -> float2 {
     if constexpr (WK) return a.wall_r[w * L.Nx + xc];
     else return wsm.r[w][tx];
@@ -1130,14 +1160,11 @@ __global__ void __launch_bounds__(TX* TY, 3) lbm_step_kernel(Lat L, StepArgs<ST>
         for (int i = 0; i < 9; ++i) g[i] = make_float2(fs[0][i], fs[1][i]);
       }
       Macro2 m;
-      macro2(L, C, g, m);
+      macro2(L, make_float2(C.rb[0], C.rb[1]), g, m);
       float om_s, om_d;
-      // 16-bit storage halves the bytes and leaves the sweep bound by
-      // instruction issue: there skipping psi work pays, for FP32 it does not
-      rates2<(sizeof(ST) < 4)>(L, m, (float)j + 0.5f, om_s, om_d);
+      rates2(L, psi_tab, m, (float)j + 0.5f, om_s, om_d);
       const float om_q = wall_omq(j < half ? 0 : 1);
-      const float2 mxs =
-          collide2(g, L, m.rho, m.ux, m.uy, L.om_e, L.om_eps, om_d, om_q, om_s);
+      const float2 mxs = collide2(g, L, m, om_d, om_q, om_s);
       if (reduce) {
         acc[0].add(m.sd.x);
         acc[1].add(m.sd.y);
@@ -1177,11 +1204,16 @@ __global__ void __launch_bounds__(TX* TY)
                        const double* __restrict__ cs_in, const float* __restrict__ alpha,
                        int direct, double* __restrict__ out) {
   __shared__ WallSmem wsm;
+  __shared__ float4 psi_tab[PSI_SEGMENTS];
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int x = blockIdx.x * TX + tx;
+  load_psi_table(psi_tab, ty * TX + tx, TX * TY);
   const ColRef C = col_ref(L, refrho, x);
   const Ends E = load_ends(L, cs_in, refrho, blockIdx.x * TX, TX);
-  if (!direct) wall_prologue<false>(L, fin, alpha, E, C, x, 0, L.N, wsm);
+  if (!direct)
+    wall_prologue<false>(L, fin, alpha, E, C, x, 0, L.N, wsm);
+  else
+    __syncthreads();
   if (!interior(L, x)) return;
   const size_t plane = (size_t)L.N * L.Nx;
   for (int j = ty; j < L.N; j += TY) {
@@ -1198,18 +1230,20 @@ __global__ void __launch_bounds__(TX* TY)
 #pragma unroll
     for (int i = 0; i < 9; ++i) g[i] = make_float2(fs[0][i], fs[1][i]);
     Macro2 m;
-    macro2(L, C, g, m);
+    macro2(L, make_float2(C.rb[0], C.rb[1]), g, m);
     float om_s, om_d;
-    rates2<false>(L, m, (float)j + 0.5f, om_s, om_d);
+    rates2(L, psi_tab, m, (float)j + 0.5f, om_s, om_d);
+    Flow2 w;
+    flow2(g, m.inv_rho, w);
     // Eq. rhou: (2 tau_d - 1)/(2 tau_d) = 1 - om_d/2, 1/(2 tau_d) = om_d/2
     const float w1 = 1.0f - 0.5f * om_d, w2 = 0.5f * om_d;
     const size_t o = (size_t)j * L.Nx + x;
     const float rho_s[2] = {m.rho.x, m.rho.y}, sd[2] = {m.sd.x, m.sd.y};
-    const float jxs[2] = {m.jx.x, m.jx.y}, jys[2] = {m.jy.x, m.jy.y};
+    const float jxs[2] = {w.jx.x, w.jx.y}, jys[2] = {w.jy.x, w.jy.y};
 #pragma unroll
     for (int sp = 0; sp < 2; ++sp) {
-      float mx = fmaf(w1, jxs[sp], w2 * rho_s[sp] * m.ux);
-      float my = fmaf(w1, jys[sp], w2 * rho_s[sp] * m.uy);
+      float mx = fmaf(w1, jxs[sp], w2 * rho_s[sp] * w.ux);
+      float my = fmaf(w1, jys[sp], w2 * rho_s[sp] * w.uy);
       out[sp * plane + o] = (double)C.rb[sp] + (double)sd[sp];
       out[(2 + 2 * sp) * plane + o] = (double)(mx / rho_s[sp]);
       out[(3 + 2 * sp) * plane + o] = (double)(my / rho_s[sp]);
@@ -1388,7 +1422,7 @@ __global__ void lbm_special_kernel(const double* __restrict__ x, double* __restr
   if (k >= n) return;
   float v = (float)x[k];
   e1[k] = (double)e1_dev(v);
-  ps[k] = (double)psi_dev(v);
+  ps[k] = (double)psi_dev(kPsiTab, v);
 }
 
 }  // namespace
@@ -1518,23 +1552,20 @@ Lat derive(const lbm_mix_params* p, int Nx) {
     L.cw0[sp] = (float)((9.0 - 5.0 * (double)L.s[sp]) / 9.0);
     L.cw1[sp] = (float)((double)L.s[sp] / 9.0);
     L.cw5[sp] = (float)((double)L.s[sp] / 36.0);
-    const float sf = L.s[sp];
-    L.ke[sp][0] = -2.0f * sf;
-    L.ke[sp][1] = 3.0f - 2.0f * sf;
-    L.ke[sp][2] = 6.0f - 2.0f * sf;
-    L.kp[sp][0] = 3.0f * sf;
-    L.kp[sp][1] = 3.0f * sf - 6.0f;
-    L.kp[sp][2] = 3.0f * sf - 3.0f;
   }
   for (int sp = 0; sp < 2; ++sp) {
     float* s2 = &L.s2.x;
     s2[sp] = L.s[sp];
     (&L.cw1_2.x)[sp] = L.cw1[sp];
     (&L.cw5_2.x)[sp] = L.cw5[sp];
+    const double sd = (double)L.s[sp], we = 1.0 / (36.0 * p->tau_e),
+                 wp = 1.0 / (36.0 * p->tau_eps);
     for (int k = 0; k < 3; ++k) {
-      (&L.ke2[k].x)[sp] = L.ke[sp][k];
-      (&L.kp2[k].x)[sp] = L.kp[sp][k];
+      (&L.ke2[k].x)[sp] = (float)(we * (3.0 * k - 2.0 * sd));
+      (&L.kp2[k].x)[sp] = (float)(wp * (3.0 * sd - (k == 0 ? 0.0 : k == 1 ? 6.0 : 3.0)));
     }
+    (&L.ku2[0].x)[sp] = (float)(-3.0 * we);
+    (&L.ku2[1].x)[sp] = (float)(3.0 * wp);
     L.mh[sp] = mh[sp];
     L.rsqrt_mh[sp] = (float)(1.0 / sqrt(mh[sp]));
     double cxl = 3.0 * mu_s[sp] * sqrt(PI / (6.0 * mh[sp]));
@@ -1544,14 +1575,16 @@ Lat derive(const lbm_mix_params* p, int Nx) {
     (&L.inv_c_xl2.x)[sp] = L.inv_c_xl[sp];
     L.rho_in[sp] = p->theta * Ci[sp] * mh[sp];
     L.rho_out[sp] = Co[sp] * mh[sp];
+    for (int end = 0; end < 2; ++end) {
+      const double m = L.N * (end == 0 ? L.rho_in[sp] : L.rho_out[sp]);
+      L.end_mass[end][sp] = make_float2((float)m, (float)(m - (double)(float)m));
+    }
   }
   double clam = 3.0 * mu * sqrt(PI / 6.0);
   L.c_lam = (float)clam;
   L.inv_c_lam = (float)(1.0 / clam);
   L.c_ts = (float)sqrt(6.0 / PI);
   L.c_td = (float)(1.5 * sqrt(3.0 * (mh[0] + mh[1]) * mh[0] * mh[1] / 1.0));
-  L.om_e = (float)(1.0 / p->tau_e);
-  L.om_eps = (float)(1.0 / p->tau_eps);
   L.c_m0 = (float)p->c_m0;
   L.H = (float)p->N;
   return L;
