@@ -134,14 +134,17 @@ void lbm_mix_destroy(lbm_mix* h);
  * C_l_out, populations at equilibrium (Eq. feq).  Resets the step count. */
 int lbm_mix_init(lbm_mix* h);
 
-/* Advances nsteps >= 0 time steps (Eq. MRT), one fused collide-stream pass
- * per step on the handle's stream, asynchronously.  With 16-bit storage, and
- * with FP32 storage when the step's grid holds two or more waves of CTAs on
- * the device, a small kernel computes r (Eq. R) and tau_q (Eq. taoq) of
- * every column ahead of each pass; both are launched with programmatic
- * dependent launch.  The pass of every
- * diag_every-th step (counted from init) and of the last step of the call
- * also reduces the separation diagnostics of the new state in FP64 (one
+/* Advances nsteps >= 0 time steps (Eq. MRT) on the handle's stream,
+ * asynchronously.  FP32 channels of up to 200 000 nodes whose columns fit in
+ * shared memory take several steps per launch (tiles of whole columns with
+ * halos, see lbm_mix_set_rows_per_block); a call gives the same bits however
+ * its steps are split over calls.  All others take one fused collide-stream
+ * pass per step: with 16-bit storage, and with FP32 storage when the step's
+ * grid holds two or more waves of CTAs on the device, a small kernel computes
+ * r (Eq. R) and tau_q (Eq. taoq) of every column ahead of each pass.  All
+ * are launched with programmatic dependent launch.  Every
+ * diag_every-th step (counted from init) and the last step of the call
+ * also reduce the separation diagnostics of the new state in FP64 (one
  * history record each), so lbm_mix_separation after lbm_mix_step always
  * describes the current state.  After every reref_every-th step (counted
  * from init) the stored deviations are re-referenced (lbm_mix_rereference). */
@@ -250,10 +253,12 @@ int lbm_mix_get_post_state_f64(lbm_mix* h, double* f, long n);
 /* Lattice size and steps taken since init / set_post_state. */
 int lbm_mix_dims(const lbm_mix* h, int* N, int* N_x, long* steps);
 
-/* Kernel launches of one lbm_mix_step step under h's current schedule
- * (lbm_mix_set_rows_per_block): 2 when the wall kernel runs ahead of the
- * step kernel (16-bit storage; FP32 grids of two or more waves of CTAs),
- * else 1; re-referencing adds its own.  Returns the count, or LBM_EINVAL
+/* Kernel launches of an lbm_mix_step call of one step under h's current
+ * schedule (lbm_mix_set_rows_per_block): 2 when the wall kernel runs ahead of
+ * the step kernel (16-bit storage; FP32 grids of two or more waves of CTAs)
+ * and for channels that take several steps per launch (the steps and their
+ * records; longer calls need fewer per step), else 1; re-referencing adds its
+ * own.  Returns the count, or LBM_EINVAL
  * for a NULL handle. */
 int lbm_mix_launches_per_step(const lbm_mix* h);
 
@@ -316,17 +321,19 @@ int lbm_mix_step_noalloc(const lbm_mix_params* p, const float* d_in, float* d_ou
 
 /* Node-to-CTA schedule of h: rows of one strip handled by one CTA of the
  * step kernel, a multiple of 8 (capped at N rounded up to 8); 0 restores the
- * library default (96 rows).  Changes only the order
- * of the FP64 column reductions.  May allocate; not during stream capture.
+ * library default (96 rows; several steps per launch where the channel
+ * qualifies, see lbm_mix_step, which a row count turns off).  Changes only
+ * the order of the FP64 column reductions.  May allocate; not during stream capture.
  * Errors: LBM_EINVAL (bad handle, rows not a multiple of 8), LBM_ENOMEM,
  * LBM_ECUDA. */
 int lbm_mix_set_rows_per_block(lbm_mix* h, int rows);
 
 /* Picks the node-to-CTA schedule of h by timing real steps: for each of the
  * n candidate row counts (multiples of 8; candidates = NULL takes 64, 72,
- * 80, 88, 96, 112 and 128) it runs 2 untimed steps and `steps` steps timed
+ * 80, 88, 96, 112 and 128, and the default schedule before them where that
+ * takes several steps per launch) it runs 2 untimed steps and `steps` steps timed
  * with CUDA events on the handle's stream, then keeps the fastest (ties to
- * the earlier candidate) and writes it to *best_rows (NULL-safe).  Which
+ * the earlier candidate) and writes its row count to *best_rows (NULL-safe).  Which
  * count is fastest depends on how the grid's CTAs fill the device's waves,
  * so it differs between channel sizes and storage types.  The steps advance
  * the state (n * (steps + 2) of them, with their diagnostic records):

@@ -4,7 +4,8 @@
 // Wang, Xu & Guo (arXiv:1603.08221, Sec. 3) is ONE fused kernel launch
 // (lbm_step_kernel; on grids of two or more waves and with 16-bit storage,
 // lbm_walls_kernel computes the wall parameters r and tau_q of every column
-// ahead of it): pull-streaming from the previous post-collision buffer
+// ahead of it), and small FP32 channels take several steps per launch
+// (lbm_tile_kernel, lbm_tile.cuh): pull-streaming from the previous post-collision buffer
 // with the diffuse-bounce-back walls (Eqs. bot, bot2, R) and the
 // extrapolation-correction ends (Eqs. rho1, rho2) folded into the loads,
 // moments (Eq. rhou), effective relaxation times (Eqs. EQFrb, EQFrsp, psi,
@@ -462,7 +463,8 @@ __device__ __forceinline__ void macro(const Lat& L, const ColRef& C, const float
 #pragma unroll
   for (int sp = 0; sp < 2; ++sp) {
     const float* g = fs[sp];
-    m.sd[sp] = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
+    // the order of density_sum, so that every wall task gives the same bits
+    m.sd[sp] = g[0] + (((g[1] + g[3]) + (g[2] + g[4])) + ((g[5] + g[7]) + (g[6] + g[8])));
     m.rho[sp] = C.rb[sp] + m.sd[sp];
   }
   m.n = number_density(L, m.rho[0], m.rho[1]);
@@ -1194,6 +1196,8 @@ __global__ void __launch_bounds__(TX* TY, 3) lbm_step_kernel(Lat L, StepArgs<ST>
   column_epilogue<DIAG>(L, a, x, accd, rsm);
 }
 
+#include "lbm_tile.cuh"
+
 // ---------------------------------------------------------- moments kernel
 // Fields of the state obtained by streaming fin (direct = 0), or of fin
 // itself (direct = 1), FP64 [6][N][Nx]: rho_a, rho_b, u_a (x, y), u_b (x, y)
@@ -1465,6 +1469,13 @@ struct lbm_mix {
   // the next kernel's CTAs are then spread over the SMs the step frees;
   // 0.2197 instead of 0.2235 s for 5000 steps of a 1280 x 64 channel).
   bool pdl_early;
+  // Several steps per launch (lbm_tile_kernel): own columns per tile and
+  // most steps of a launch; tile_W = 0: the channel does not qualify.  A
+  // schedule the caller set (rows_set) takes the step kernel instead.
+  int tile_W, tile_k;
+  bool rows_set;
+  float2* hist;      // [hist_rows][4][Nx] column sums awaiting lbm_records_kernel
+  int hist_rows;
   int cur;           // buffer holding the latest post-collision state
   long steps;
   bool have_snap;
@@ -1771,6 +1782,154 @@ int launch_step(lbm_mix* h, bool diag) {
   return LBM_OK;
 }
 
+// ------------------------------------------------- several steps per launch
+// Estimated time of one step (us) of a channel cut into tiles of W columns
+// that take k steps per launch on `sms` SMs: a launch costs TILE_LAUNCH_US,
+// a step TILE_STEP_US plus TILE_NODE_US per node of the tile (fitted to 320 x
+// 16, 700 x 20, 1001 x 37, 2048 x 32 and 1280 x 64 at k = 1 ... 15; the
+// minimum over k is flat).
+constexpr double TILE_LAUNCH_US = 4.6, TILE_STEP_US = 1.15, TILE_NODE_US = 0.0020;
+double tile_cost(int N, int nup, int W, int k, int sms) {
+  const int tiles = (nup + W - 1) / W;
+  const double waves = (tiles + sms - 1) / sms;
+  double us = 0.0;
+  for (int t = 1; t <= k; ++t)
+    us += TILE_STEP_US + TILE_NODE_US * (W + 2 * (k - t)) * tile_stride(N);
+  return (TILE_LAUNCH_US + waves * us) / k;
+}
+
+// Tile width and steps per launch (odd, so that launches alternate the two
+// buffers as single steps do) of least estimated cost on `sms` SMs; W = 0
+// where no tile fits shared memory.
+void plan_tiles(const Lat& L, int sms, int* W_out, int* k_out, double* us_out) {
+  const int nup = L.x_periodic ? L.Nx : L.Nx - 2;
+  *W_out = 0;
+  *k_out = 0;
+  *us_out = INFINITY;
+  for (int k = 1; k <= TILE_KMAX; k += 2) {
+    if (tile_smem(L.N, 1 + 2 * k) > (size_t)TILE_SMEM_MAX) break;
+    for (int W = 1; W <= nup; ++W) {
+      if (tile_smem(L.N, W + 2 * k) > (size_t)TILE_SMEM_MAX) break;
+      const double us = tile_cost(L.N, nup, W, k, sms);
+      if (us < *us_out) {
+        *us_out = us;
+        *W_out = W;
+        *k_out = k;
+      }
+      if ((nup + W - 1) / W == 1) break;
+    }
+  }
+}
+
+// Largest channel that takes tiles, and the size of a handle's record rows.
+constexpr long TILE_MAX_NODES = 200000, HIST_BYTES = 2 << 20;
+
+bool uses_tiles(const lbm_mix* h) { return h->tile_W > 0 && !h->rows_set; }
+
+// Launches kernel<NI> for n channels with programmatic stream serialisation.
+template <typename B>
+int launch_batch(void (*kern)(B), const B& batch, dim3 grid, dim3 block, size_t smem,
+                 cudaStream_t st) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  CK(cudaLaunchKernelEx(&cfg, kern, batch));
+  return LBM_OK;
+}
+
+// One launch of k steps for the n <= NI channels hs, whose record rows used
+// so far are rows[]; last: step k ends the call.
+template <int NI>
+int launch_tiles(lbm_mix* const* hs, int n, int k, bool last, int* rows, cudaStream_t st) {
+  TileBatch<NI> B;
+  B.k = k;
+  int blocks = 0, nodes = 0;
+  size_t smem = 0;
+  for (int q = 0; q < NI; ++q) {
+    B.block0[q] = blocks;
+    if (q >= n) continue;
+    lbm_mix* h = hs[q];
+    const Lat& L = h->L;
+    TileInst& I = B.inst[q];
+    const int b = h->cur, de = h->p.diag_every;
+    I.L = L;
+    I.fin = (const float*)h->buf[b];
+    I.fout = (float*)h->buf[1 - b];
+    I.refrho = h->refrho;
+    I.alpha = h->alpha;
+    I.cs_in = h->cs[b];
+    I.cs_out = h->cs[1 - b];
+    I.hist = h->hist + (size_t)rows[q] * 4 * L.Nx;
+    I.W = h->tile_W;
+    I.diag_every = de;
+    I.diag_phase = (int)(h->steps % de);
+    I.last = last ? 1 : 0;
+    rows[q] += (int)((h->steps + k) / de - h->steps / de);
+    if (last && (h->steps + k) % de != 0) rows[q]++;
+    const int nup = L.x_periodic ? L.Nx : L.Nx - 2;
+    blocks += (nup + I.W - 1) / I.W;
+    const int own = I.W < nup ? I.W : nup, busy = (own + 2 * k - 2) * (L.N - 2);
+    nodes = busy > nodes ? busy : nodes;
+    const size_t sm = tile_smem(L.N, own + 2 * k);
+    smem = sm > smem ? sm : smem;
+  }
+  B.block0[NI] = blocks;
+  int threads = (nodes + 31) / 32 * 32;
+  threads = threads < 32 ? 32 : threads < TILE_INNER ? threads : TILE_INNER;
+  int s = launch_batch(lbm_tile_kernel<NI>, B, dim3(blocks),
+                       dim3(threads + TILE_WALL + TILE_TAUQ), smem, st);
+  if (s) return s;
+  for (int q = 0; q < n; ++q) {
+    hs[q]->cur = 1 - hs[q]->cur;
+    hs[q]->steps += k;
+  }
+  return LBM_OK;
+}
+
+// The records of rows[] column-sum rows of every channel; rows[] to zero.
+template <int NI>
+int launch_records(lbm_mix* const* hs, int n, int* rows, cudaStream_t st) {
+  RecBatch<NI> B;
+  int most = 0;
+  for (int q = 0; q < n; ++q) {
+    lbm_mix* h = hs[q];
+    B.inst[q] = RecInst{h->L,       h->hist,    h->refrho, h->diag, h->diag_count,
+                        h->counter, h->clprof, rows[q]};
+    most = rows[q] > most ? rows[q] : most;
+    rows[q] = 0;
+  }
+  if (most == 0) return LBM_OK;
+  return launch_batch(lbm_records_kernel<NI>, B, dim3(most, n), dim3(256), 0, st);
+}
+
+// nsteps steps of the n <= NI channels hs on stream st: launches of kmax
+// steps or fewer, the last one of a single step, so that the two buffers end
+// up holding the states of the last two steps.  end: the last step ends the
+// call and is recorded.
+template <int NI>
+int tile_steps(lbm_mix* const* hs, int n, int kmax, long nsteps, bool end, cudaStream_t st) {
+  int rows[NI] = {};
+  int s = LBM_OK;
+  for (long left = nsteps; left > 0;) {
+    int k = left - 1 < kmax ? (int)(left - 1) : kmax;
+    k -= 1 - (k & 1);  // odd
+    if (k < 1) k = 1;
+    bool full = false;
+    for (int q = 0; q < n; ++q) full |= rows[q] + k + 1 > hs[q]->hist_rows;
+    if (full && (s = launch_records<NI>(hs, n, rows, st))) return s;
+    if ((s = launch_tiles<NI>(hs, n, k, end && left == k, rows, st))) return s;
+    left -= k;
+  }
+  return launch_records<NI>(hs, n, rows, st);
+}
+
 int launch_moments(lbm_mix* h, double* d_out) {
   // The state of step n is the stream of buffer P_{n-1}; right after init or
   // an upload only the buffer itself exists.
@@ -1966,6 +2125,7 @@ void lbm_mix_destroy(lbm_mix* h) {
   cudaFree(h->wall_omq);
   cudaFree(h->colpart);
   cudaFree(h->strip_cnt);
+  cudaFree(h->hist);
   cudaFree(h->resid);
   cudaFree(h->mom);
   if (h->h_pinned) cudaFreeHost(h->h_pinned);
@@ -2031,6 +2191,19 @@ int lbm_mix_create(const lbm_mix_params* p, void* stream, lbm_mix** out) {
   ALLOC(h->colpart, sizeof(double) * 4 * (size_t)Nx * (size_t)h->R);
   ALLOC(h->strip_cnt, sizeof(unsigned) * (size_t)h->nblocks);
   ALLOC(h->resid, sizeof(double));
+  if (p->storage == LBM_FP32) {
+    double us = 0.0;
+    plan_tiles(h->L, h->nsm, &h->tile_W, &h->tile_k, &us);
+    if ((long)h->L.N * Nx > TILE_MAX_NODES) h->tile_W = 0;
+    if (h->tile_W > 0) {
+      const long fit = HIST_BYTES / (long)(sizeof(float2) * 4 * (size_t)Nx);
+      h->hist_rows = (int)(fit < TILE_KMAX + 1 ? TILE_KMAX + 1 : fit < 256 ? fit : 256);
+      ALLOC(h->hist, sizeof(float2) * 4 * (size_t)Nx * (size_t)h->hist_rows);
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(lbm_tile_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 TILE_SMEM_MAX);
+    }
+  }
 #undef ALLOC
   if (e == cudaSuccess) e = cudaMallocHost((void**)&h->h_pinned, sizeof(double) * 64);
   if (e != cudaSuccess) {
@@ -2104,6 +2277,16 @@ int lbm_mix_step(lbm_mix* h, long nsteps) {
   if (nsteps < 0) return set_err(LBM_EINVAL, "nsteps < 0");
   const long reref = h->p.reref_every >= 0 ? h->p.reref_every
                                            : (h->p.storage == LBM_FP32 ? 0 : 256);
+  if (uses_tiles(h)) {
+    for (long left = nsteps; left > 0;) {
+      long n = left;
+      if (reref > 0 && n > reref - h->steps % reref) n = reref - h->steps % reref;
+      if ((st = tile_steps<1>(&h, 1, h->tile_k, n, n == left, h->stream))) return st;
+      if (reref > 0 && h->steps % reref == 0 && (st = rereference(h))) return st;
+      left -= n;
+    }
+    return LBM_OK;
+  }
   // diagnostics on every diag_every-th step and on the last step of the call
   for (long t = 0; t < nsteps; ++t) {
     const bool diag = (t == nsteps - 1) || ((h->steps + 1) % h->p.diag_every == 0);
@@ -2154,14 +2337,17 @@ int lbm_mix_run_to_steady(lbm_mix* h, double tol, long max_steps, long check_eve
 int lbm_mix_set_rows_per_block(lbm_mix* h, int rows) {
   int st = check_handle(h);
   if (st) return st;
-  return set_rows_per_block(h, rows);
+  if ((st = set_rows_per_block(h, rows))) return st;
+  h->rows_set = rows > 0;
+  return LBM_OK;
 }
 
 int lbm_mix_tune_rows(lbm_mix* h, const int* candidates, int n, long steps, int* best_rows) {
   int st = check_handle(h);
   if (st) return st;
   static const int kDefault[] = {64, 72, 80, 88, 96, 112, 128};
-  if (!candidates) {
+  const bool own_list = !candidates;
+  if (own_list) {
     candidates = kDefault;
     n = (int)(sizeof kDefault / sizeof kDefault[0]);
   }
@@ -2175,9 +2361,14 @@ int lbm_mix_tune_rows(lbm_mix* h, const int* candidates, int n, long steps, int*
     return set_err(LBM_ECUDA, "cudaEventCreate failed");
   }
   int best = h->rows_per_block;
+  bool best_set = h->rows_set;
   float best_ms = INFINITY;
-  for (int k = 0; k < n && st == LBM_OK; ++k) {
-    if ((st = set_rows_per_block(h, candidates[k]))) break;
+  // the library's own list starts with its default where that is not a row
+  // count of the step kernel but lbm_tile_kernel
+  const int first = own_list && h->tile_W > 0 ? -1 : 0;
+  for (int k = first; k < n && st == LBM_OK; ++k) {
+    if ((st = set_rows_per_block(h, k < 0 ? 0 : candidates[k]))) break;
+    h->rows_set = k >= 0;
     // two untimed steps settle the new schedule (first-touch of its buffers)
     if ((st = lbm_mix_step(h, 2))) break;
     if (cudaEventRecord(e0, h->stream) != cudaSuccess ||
@@ -2191,12 +2382,14 @@ int lbm_mix_tune_rows(lbm_mix* h, const int* candidates, int n, long steps, int*
     if (ms < best_ms) {
       best_ms = ms;
       best = h->rows_per_block;
+      best_set = h->rows_set;
     }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (st) return st;
   if ((st = set_rows_per_block(h, best))) return st;
+  h->rows_set = best_set;
   if (best_rows) *best_rows = best;
   return LBM_OK;
 }
@@ -2358,7 +2551,7 @@ int lbm_mix_dims(const lbm_mix* h, int* N, int* N_x, long* steps) {
 int lbm_mix_launches_per_step(const lbm_mix* h) {
   int st = check_handle(h);
   if (st) return st;
-  return (h->elem < 4 || uses_wall_kernel(h)) ? 2 : 1;
+  return (h->elem < 4 || uses_tiles(h) || uses_wall_kernel(h)) ? 2 : 1;
 }
 
 int lbm_mix_sync(lbm_mix* h) {
@@ -2467,6 +2660,7 @@ struct SweepCapKey {
   const void* colpart;
   const void* refrho;
   long phase;
+  bool tiles;
 };
 
 struct lbm_sweep {
@@ -2483,12 +2677,12 @@ namespace {
 
 SweepCapKey cap_key(const lbm_mix* h) {
   return SweepCapKey{h->cur, h->rows_per_block, h->R, h->colpart, h->refrho,
-                     h->steps % h->p.diag_every};
+                     h->steps % h->p.diag_every, uses_tiles(h)};
 }
 
 bool same_key(const SweepCapKey& a, const SweepCapKey& b) {
   return a.cur == b.cur && a.rows == b.rows && a.R == b.R && a.colpart == b.colpart &&
-         a.refrho == b.refrho && a.phase == b.phase;
+         a.refrho == b.refrho && a.phase == b.phase && a.tiles == b.tiles;
 }
 
 // Instance i has a graph of K steps that is valid for its current state.
@@ -2556,10 +2750,11 @@ int capture_steps(lbm_sweep* s, int i, long K) {
 int apply_policy(lbm_sweep* s, int p) {
   for (int i = 0; i < s->n; ++i) {
     lbm_mix* h = s->h[i];
-    const int before = h->rows_per_block;
+    const SweepCapKey before = cap_key(h);
     int st = set_rows_per_block(h, policy_rows(h, p));
     if (st) return st;
-    if (h->rows_per_block != before) drop_graph(s, i);
+    h->rows_set = p > 0;
+    if (!same_key(before, cap_key(h))) drop_graph(s, i);
   }
   s->policy = p;
   return LBM_OK;
