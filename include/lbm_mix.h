@@ -321,8 +321,9 @@ int lbm_mix_step_noalloc(const lbm_mix_params* p, const float* d_in, float* d_ou
 
 /* Node-to-CTA schedule of h: rows of one strip handled by one CTA of the
  * step kernel, a multiple of 8 (capped at N rounded up to 8); 0 restores the
- * library default (96 rows; several steps per launch where the channel
- * qualifies, see lbm_mix_step, which a row count turns off).  Changes only
+ * library default (16 to 80 rows by the channel's size; several steps per
+ * launch where the channel qualifies, see lbm_mix_step, which a row count
+ * turns off).  Changes only
  * the order of the FP64 column reductions.  May allocate; not during stream capture.
  * Errors: LBM_EINVAL (bad handle, rows not a multiple of 8), LBM_ENOMEM,
  * LBM_ECUDA. */
@@ -355,8 +356,7 @@ int lbm_mix_tune_rows(lbm_mix* h, const int* candidates, int n, long steps, int*
  * ------------------------------------------------------------------- */
 typedef struct lbm_sweep lbm_sweep;
 
-/* Node-to-CTA schedules the autotuner tries: 0 library default (96 rows per
- * CTA), 1: 64, 2: 32, 3: 16 rows, 4: enough rows per CTA to give each
+/* Node-to-CTA schedules the autotuner tries: 0 library default, 1: 64, 2: 32, 3: 16 rows, 4: enough rows per CTA to give each
  * instance about two CTAs per SM. */
 #define LBM_SWEEP_NPOLICY 5
 

@@ -88,18 +88,20 @@ struct Lat {
   float s[2];            // s_sigma = m_min / m_sigma
   float cw0[2];          // rest-equilibrium weights w_i alpha_si: rest (9 - 5s)/9,
   float cw1[2], cw5[2];  // axis s/9, diagonal s/36
+  // coefficients of the non-equilibrium energy moments on the deviations
+  // (rest, axis, diagonal): e: -2s, 3 - 2s, 6 - 2s; eps: 3s, 3s - 6, 3s - 3
+  float ke[2][3], kp[2][3];
   // the per-species constants as (species a, species b) pairs for the packed
-  // FP32x2 arithmetic; ke2, kp2: coefficients of the non-equilibrium energy
-  // moments on the deviations (rest, axis, diagonal: e: -2s, 3 - 2s, 6 - 2s;
-  // eps: 3s, 3s - 6, 3s - 3) times om_e / 36 and om_eps / 36, ku2: of
-  // rho u^2 (-3, 3) likewise
-  float2 s2, cw1_2, cw5_2, c_xl2, inv_c_xl2, ke2[3], kp2[3], ku2[2];
+  // FP32x2 arithmetic; ce2, cp2: ke2 om_e / 36 and kp2 om_eps / 36, cu2: the
+  // coefficients of rho u^2 (-3, 3) likewise
+  float2 s2, cw1_2, cw5_2, c_xl2, inv_c_xl2, ke2[3], kp2[3], ce2[3], cp2[3], cu2[2];
   float inv_c_lam;       // 1 / (3 mu sqrt(pi/6))
   float c_lam;           // 3 mu sqrt(pi/6): lambda = c_lam / (n sqrt(m_x))
   float c_xl[2];         // 3 mu_s sqrt(pi/(6 m_s)): x_s lambda_s = c_xl / n
   float inv_c_xl[2];
   float c_ts;            // sqrt(6/pi)
   float c_td;            // (3/2) sqrt(3 m0 m_a m_b / m_min)
+  float om_e, om_eps;    // 1/tau_e, 1/tau_eps
   float c_m0;
   float H;               // channel height = N
   double mh[2];          // m_sigma / m_min
@@ -562,7 +564,7 @@ __device__ __forceinline__ void rates2(const Lat& L, const float4* T, const Macr
 // -u_x, u_y, -u_y, u_x^2 - u_y^2, u_x u_y).  The reference has m = m^eq(u=0),
 // so e - e^eq = sum_i (e_i + 4 - 2s) g_i - 3 rho u^2 and
 // eps - eps^eq = sum_i (eps_i - 4 + 3s) g_i + 3 rho u^2 need no large terms
-// (ke, kp hold those coefficients for the rest, axis and diagonal classes,
+// (ce2, cp2 hold those coefficients for the rest, axis and diagonal classes,
 // times om_e / 36 and om_eps / 36, the classes' common factor in M^{-1}).
 // Returns the x components of the species momenta of Eq. rhou,
 // j_x - (j_x - rho_s u_x)/(2 tau_d).
@@ -574,10 +576,10 @@ __device__ __forceinline__ float2 collide2(float2 g[9], const Lat& L, const Macr
   const float2 rho = m.rho;
   const float2 ru2 = mul2(f2(fmaf(ux, ux, uy2)), rho);
   const float2 a14 = add2(w.s13, w.s24), a58 = add2(w.s57, w.s68);
-  const float2 de = fma2(L.ke2[0], g[0],
-                         fma2(L.ke2[1], a14, fma2(L.ke2[2], a58, mul2(L.ku2[0], ru2))));
-  const float2 dp = fma2(L.kp2[0], g[0],
-                         fma2(L.kp2[1], a14, fma2(L.kp2[2], a58, mul2(L.ku2[1], ru2))));
+  const float2 de = fma2(L.ce2[0], g[0],
+                         fma2(L.ce2[1], a14, fma2(L.ce2[2], a58, mul2(L.cu2[0], ru2))));
+  const float2 dp = fma2(L.cp2[0], g[0],
+                         fma2(L.cp2[1], a14, fma2(L.cp2[2], a58, mul2(L.cu2[1], ru2))));
   const float2 qx = fma2(f2(-2.0f), w.d13, w.dx);
   const float2 qy = fma2(f2(-2.0f), w.d24, w.dy);
   const float2 pxx = sub2(w.s13, w.s24), pxy = sub2(w.s57, w.s68);
@@ -746,6 +748,16 @@ __device__ __forceinline__ bool interior(const Lat& L, int x) {
   return L.x_periodic ? (x < L.Nx) : (x >= 1 && x <= L.Nx - 2);
 }
 
+#include "lbm_node16.cuh"
+
+// The density-correction factors in the storage form's arithmetic.
+template <typename ST>
+__device__ __forceinline__ Ends ends_of(const Lat& L, const double* __restrict__ cs,
+                                        const float* __restrict__ refrho, int x0, int width) {
+  if constexpr (sizeof(ST) < 4) return n16::load_ends(L, cs, refrho, x0, width);
+  else return load_ends(L, cs, refrho, x0, width);
+}
+
 // Per-CTA wall data for the strip: r (both walls), 1/tau_q (both walls).
 struct WallSmem {
   float2 r[2][TX];  // (species a, species b) per wall and column
@@ -774,16 +786,25 @@ __device__ __forceinline__ void wall_task(const Lat& L, const ST* __restrict__ f
   if (!interior(L, x)) return;
   const int jw = wall == 0 ? 0 : L.N - 1;
   const float al = alpha[wall * L.Nx + x];
+  auto r_of = [&]() -> float2 {
+    if constexpr (sizeof(ST) < 4) return n16::dbb_r(L, C, fin, x, jw, al);
+    else return dbb_r(L, C, fin, x, jw, al);
+  };
   if (!tq) {
-    rv = dbb_r(L, C, fin, x, jw, al);
+    rv = r_of();
   } else {
     float fs[2][9];
-    const float2 rr = L.wall_mode == LBM_WALL_BSR ? dbb_r(L, C, fin, x, jw, al)
-                                                  : make_float2(0.0f, 0.0f);
+    const float2 rr = L.wall_mode == LBM_WALL_BSR ? r_of() : make_float2(0.0f, 0.0f);
     pull_node(fin, L, E, C, x, jw, rr, rr, fs);
-    Macro m;
-    macro(L, C, fs, m);
-    v = inv_tau_q(L, kPsiTab, kDpsiTab, m.n, m.inv_n, m.mx, slip_coefficients(al));
+    if constexpr (sizeof(ST) < 4) {
+      n16::Macro m;
+      n16::macro(L, C, fs, m);
+      v = 1.0f / n16::tau_q_wall(L, m, al);
+    } else {
+      Macro m;
+      macro(L, C, fs, m);
+      v = inv_tau_q(L, kPsiTab, kDpsiTab, m.n, m.inv_n, m.mx, slip_coefficients(al));
+    }
   }
 }
 
@@ -831,7 +852,7 @@ __global__ void __launch_bounds__(128) lbm_walls_kernel(Lat L, const ST* __restr
   const int wall = blockIdx.y & 1;
   const bool tq = blockIdx.y >= 2;
   const ColRef C = col_ref(L, refrho, x);
-  const Ends E = load_ends(L, cs_in, refrho, blockIdx.x * blockDim.x, blockDim.x);
+  const Ends E = ends_of<ST>(L, cs_in, refrho, blockIdx.x * blockDim.x, blockDim.x);
   float2 rv;
   float v;
   wall_task(L, fin, alpha, E, C, x, wall, tq, rv, v);
@@ -875,6 +896,23 @@ __device__ __forceinline__ unsigned lcg_next(unsigned& s) {
   s = s * 1664525u + 1013904223u;
   return s ^ (s >> 16);
 }
+
+// Rows of one sequence of the stochastic rounding: a thread's generator is
+// seeded anew every RNG_ROWS rows and takes nine numbers per row it visits
+// (every TY-th), so a node's random bits depend on its place and the step
+// alone, not on the rows per CTA.
+constexpr int RNG_ROWS = 96;
+static_assert(RNG_ROWS % TY == 0, "a thread's rows meet a seeding row");
+// Nine steps of lcg_next's congruence at once: s -> A9 s + C9.
+struct Lcg9 {
+  unsigned a = 1u, c = 0u;
+  constexpr Lcg9() {
+    for (int k = 0; k < 9; ++k) {
+      a *= 1664525u;
+      c = c * 1664525u + 1013904223u;
+    }
+  }
+};
 
 template <typename ST>
 struct StepArgs {
@@ -1101,14 +1139,15 @@ template <typename ST, bool DIAG, bool WK = (sizeof(ST) < 4)>
 __global__ void __launch_bounds__(TX* TY, 3) lbm_step_kernel(Lat L, StepArgs<ST> a) {
   __shared__ WallSmem wsm;
   __shared__ RedSmem rsm;
-  __shared__ float4 psi_tab[PSI_SEGMENTS];
+  constexpr bool FP32 = sizeof(ST) == 4;
+  __shared__ float4 psi_tab[FP32 ? PSI_SEGMENTS : 1];
   if (a.pdl_early) pdl_launch_dependents();
   const int tx = threadIdx.x, ty = threadIdx.y;
-  load_psi_table(psi_tab, ty * TX + tx, TX * TY);  // overlaps the kernel before this one
+  if (FP32) load_psi_table(psi_tab, ty * TX + tx, TX * TY);  // overlaps the kernel before
   pdl_wait();
   const int x0 = blockIdx.x * TX, x = x0 + tx;
   const ColRef C = col_ref(L, a.refrho, x);
-  const Ends E = load_ends(L, a.cs_in, a.refrho, blockIdx.x * TX, TX);
+  const Ends E = ends_of<ST>(L, a.cs_in, a.refrho, blockIdx.x * TX, TX);
   const int j_begin = blockIdx.y * a.rows_per_block;
   const int j_end = min(L.N, j_begin + a.rows_per_block);
   // the first row of each warp is on its way into L2 while the wall prologue
@@ -1120,7 +1159,7 @@ __global__ void __launch_bounds__(TX* TY, 3) lbm_step_kernel(Lat L, StepArgs<ST>
   const int xc = x < L.Nx ? x : L.Nx - 1;
   if constexpr (!WK)
     wall_prologue<true>(L, a.fin, a.alpha, E, C, x, j_begin, j_end, wsm);
-  else
+  else if (FP32)
     __syncthreads();  // psi's table
   auto wall_r = [&](int w) -> float2 {
     if constexpr (WK) return a.wall_r[w * L.Nx + xc];
@@ -1141,13 +1180,18 @@ __global__ void __launch_bounds__(TX* TY, 3) lbm_step_kernel(Lat L, StepArgs<ST>
   const int half = (L.N + 1) / 2;  // rows j < half (1-based 2J <= N+1) use the bottom tau_q
   KahanF acc[4];
   const bool reduce = DIAG || edge_strip;
-  // per-thread generator of the stochastic rounding (16-bit storage only)
-  unsigned rng = sizeof(ST) < 4
-                     ? hash32(a.seed ^ hash32((blockIdx.y * gridDim.x + blockIdx.x) * (TX * TY) +
-                                             ty * TX + tx))
-                     : 0u;
-  if (in) {
-    for (int j = j_begin + ty; j < j_end; j += TY) {
+  unsigned rng = 0u;  // generator of the stochastic rounding
+  // one run over the rows, with 16-bit storage one per sequence of random bits
+  for (int js = j_begin, je; in && js < j_end; js = je) {
+    je = j_end;
+    if (!FP32 && a.seed != 0u) {
+      constexpr Lcg9 jump;
+      const int block = js / RNG_ROWS;
+      je = min(j_end, (block + 1) * RNG_ROWS);
+      rng = hash32(a.seed ^ hash32((block * gridDim.x + blockIdx.x) * (TX * TY) + ty * TX + tx));
+      for (int r = (js - block * RNG_ROWS) / TY; r > 0; --r) rng = rng * jump.a + jump.c;
+    }
+    for (int j = js + ty; j < je; j += TY) {
       float2 g[9];
       const ST* p = a.fin + base + j * RS;
       // row start is 16-byte aligned (RS * sizeof(ST) is a multiple of 16);
@@ -1161,15 +1205,27 @@ __global__ void __launch_bounds__(TX* TY, 3) lbm_step_kernel(Lat L, StepArgs<ST>
 #pragma unroll
         for (int i = 0; i < 9; ++i) g[i] = make_float2(fs[0][i], fs[1][i]);
       }
-      Macro2 m;
-      macro2(L, make_float2(C.rb[0], C.rb[1]), g, m);
+      float2 sd, mxs;
       float om_s, om_d;
-      rates2(L, psi_tab, m, (float)j + 0.5f, om_s, om_d);
-      const float om_q = wall_omq(j < half ? 0 : 1);
-      const float2 mxs = collide2(g, L, m, om_d, om_q, om_s);
+      if constexpr (FP32) {
+        Macro2 m;
+        macro2(L, make_float2(C.rb[0], C.rb[1]), g, m);
+        rates2(L, psi_tab, m, (float)j + 0.5f, om_s, om_d);
+        const float om_q = wall_omq(j < half ? 0 : 1);
+        mxs = collide2(g, L, m, om_d, om_q, om_s);
+        sd = m.sd;
+      } else {
+        n16::Macro2 m;
+        n16::macro2(L, C, g, m);
+        // bound by instruction issue: skipping the unused form of psi pays
+        n16::rates2<true>(L, m, (float)j + 0.5f, om_s, om_d);
+        const float om_q = wall_omq(j < half ? 0 : 1);
+        mxs = n16::collide2(g, L, m.rho, m.ux, m.uy, L.om_e, L.om_eps, om_d, om_q, om_s);
+        sd = m.sd;
+      }
       if (reduce) {
-        acc[0].add(m.sd.x);
-        acc[1].add(m.sd.y);
+        acc[0].add(sd.x);
+        acc[1].add(sd.y);
         acc[2].add(mxs.x);
         acc[3].add(mxs.y);
       }
@@ -1563,20 +1619,29 @@ Lat derive(const lbm_mix_params* p, int Nx) {
     L.cw0[sp] = (float)((9.0 - 5.0 * (double)L.s[sp]) / 9.0);
     L.cw1[sp] = (float)((double)L.s[sp] / 9.0);
     L.cw5[sp] = (float)((double)L.s[sp] / 36.0);
+    const float sf = L.s[sp];
+    L.ke[sp][0] = -2.0f * sf;
+    L.ke[sp][1] = 3.0f - 2.0f * sf;
+    L.ke[sp][2] = 6.0f - 2.0f * sf;
+    L.kp[sp][0] = 3.0f * sf;
+    L.kp[sp][1] = 3.0f * sf - 6.0f;
+    L.kp[sp][2] = 3.0f * sf - 3.0f;
   }
   for (int sp = 0; sp < 2; ++sp) {
     float* s2 = &L.s2.x;
     s2[sp] = L.s[sp];
     (&L.cw1_2.x)[sp] = L.cw1[sp];
     (&L.cw5_2.x)[sp] = L.cw5[sp];
-    const double sd = (double)L.s[sp], we = 1.0 / (36.0 * p->tau_e),
-                 wp = 1.0 / (36.0 * p->tau_eps);
+    const double we = 1.0 / (36.0 * p->tau_e), wp = 1.0 / (36.0 * p->tau_eps);
+    const double sd = (double)L.s[sp];
     for (int k = 0; k < 3; ++k) {
-      (&L.ke2[k].x)[sp] = (float)(we * (3.0 * k - 2.0 * sd));
-      (&L.kp2[k].x)[sp] = (float)(wp * (3.0 * sd - (k == 0 ? 0.0 : k == 1 ? 6.0 : 3.0)));
+      (&L.ke2[k].x)[sp] = L.ke[sp][k];
+      (&L.kp2[k].x)[sp] = L.kp[sp][k];
+      (&L.ce2[k].x)[sp] = (float)(we * (3.0 * k - 2.0 * sd));
+      (&L.cp2[k].x)[sp] = (float)(wp * (3.0 * sd - (k == 0 ? 0.0 : k == 1 ? 6.0 : 3.0)));
     }
-    (&L.ku2[0].x)[sp] = (float)(-3.0 * we);
-    (&L.ku2[1].x)[sp] = (float)(3.0 * wp);
+    (&L.cu2[0].x)[sp] = (float)(-3.0 * we);
+    (&L.cu2[1].x)[sp] = (float)(3.0 * wp);
     L.mh[sp] = mh[sp];
     L.rsqrt_mh[sp] = (float)(1.0 / sqrt(mh[sp]));
     double cxl = 3.0 * mu_s[sp] * sqrt(PI / (6.0 * mh[sp]));
@@ -1596,6 +1661,8 @@ Lat derive(const lbm_mix_params* p, int Nx) {
   L.inv_c_lam = (float)(1.0 / clam);
   L.c_ts = (float)sqrt(6.0 / PI);
   L.c_td = (float)(1.5 * sqrt(3.0 * (mh[0] + mh[1]) * mh[0] * mh[1] / 1.0));
+  L.om_e = (float)(1.0 / p->tau_e);
+  L.om_eps = (float)(1.0 / p->tau_eps);
   L.c_m0 = (float)p->c_m0;
   L.H = (float)p->N;
   return L;
@@ -1612,13 +1679,24 @@ unsigned host_hash32(unsigned x) {
 }
 
 // Rows of one strip per CTA of the step kernel unless the caller sets a
-// schedule: measured on GB300 against 64 ... 512 rows, 96 is within 1 % of
-// the best on the 32768 x 512 and 16384 x 256 channels (128 rows: 2 % and
-// 11 % slower; 512: 30 % slower).
-constexpr int DEFAULT_ROWS = 96;
-int default_rows(int N) {
-  const int n8 = (N + TY - 1) / TY * TY;
-  return n8 < DEFAULT_ROWS ? n8 : DEFAULT_ROWS;
+// schedule: as many as leave WAVES waves of resident CTAs (3 per SM), a
+// multiple of TY within [16, 56] (FP32) or [16, 80] (16-bit).  A warp takes
+// its CTA's rows one after another, every TY-th, so on a channel of few strips
+// fewer rows per CTA shorten the step until the CTAs' own start-up counts.
+// Measured on GB300, us per step at 96 rows (the rule before) and at this
+// rule's count: FP32 5001 x 130 54.5 -> 34.6 (16 rows), 8000 x 128 67.7 ->
+// 43.9 (16), 16384 x 256 131 -> 117 (40), 32768 x 512 396.6 -> 384.6 (56);
+// BF16 67.8 -> 35.5, 72.6 -> 43.9, 131 -> 105, 313 -> 312 (80).
+constexpr int WAVES = 8;
+int default_rows(int N, int strips, int nsm, bool fp32) {
+  const int n8 = (N + TY - 1) / TY * TY, most = fp32 ? 56 : 80;
+  const long ctas = (long)WAVES * 3 * (nsm > 0 ? nsm : 1);
+  long rows = ((long)N * strips / ctas + TY - 1) / TY * TY;
+  rows = rows < 16 ? 16 : rows < most ? rows : most;
+  return (int)(rows < n8 ? rows : n8);
+}
+int default_rows(const lbm_mix* h) {
+  return default_rows(h->L.N, h->nblocks, h->nsm, h->p.storage == LBM_FP32);
 }
 
 // Calls f(type tag) with the storage element type of the handle.
@@ -1681,7 +1759,7 @@ int launch_residual(lbm_mix* h, long k) {
 // partials grow when a schedule needs more row blocks than allocated.
 int set_rows_per_block(lbm_mix* h, int rows) {
   const int nmax = (h->L.N + TY - 1) / TY * TY;
-  if (rows <= 0) rows = default_rows(h->L.N);
+  if (rows <= 0) rows = default_rows(h);
   if (rows % TY != 0) return set_err(LBM_EINVAL, "rows per block must be a multiple of %d", TY);
   if (rows > nmax) rows = nmax;
   const int R = (h->L.N + rows - 1) / rows;
@@ -1785,18 +1863,25 @@ int launch_step(lbm_mix* h, bool diag) {
 // ------------------------------------------------- several steps per launch
 // Estimated time of one step (us) of a channel cut into tiles of W columns
 // that take k steps per launch on `sms` SMs: a launch costs TILE_LAUNCH_US,
-// a step TILE_STEP_US plus TILE_NODE_US per node of the tile (fitted to 320 x
-// 16, 700 x 20, 1001 x 37, 2048 x 32 and 1280 x 64 at k = 1 ... 15; the
+// each wave of tiles TILE_LOAD_US to load and store, and each of its steps
+// TILE_STEP_US plus TILE_NODE_US per node of the tile.  Fitted to channels of
+// 16 to 128 rows and 5 000 to 600 000 nodes, k = 1 ... 15 (within 20 %; the
 // minimum over k is flat).
-constexpr double TILE_LAUNCH_US = 4.6, TILE_STEP_US = 1.15, TILE_NODE_US = 0.0020;
+constexpr double TILE_LAUNCH_US = 0.6, TILE_LOAD_US = 4.0, TILE_STEP_US = 1.0,
+                 TILE_NODE_US = 0.0025;
 double tile_cost(int N, int nup, int W, int k, int sms) {
   const int tiles = (nup + W - 1) / W;
   const double waves = (tiles + sms - 1) / sms;
-  double us = 0.0;
-  for (int t = 1; t <= k; ++t)
-    us += TILE_STEP_US + TILE_NODE_US * (W + 2 * (k - t)) * tile_stride(N);
-  return (TILE_LAUNCH_US + waves * us) / k;
+  // sum over t = 1 ... k of the W + 2 (k - t) columns of step t
+  const double nodes = (double)k * (W + k - 1) * tile_stride(N);
+  return (TILE_LAUNCH_US + waves * (TILE_LOAD_US + k * TILE_STEP_US + TILE_NODE_US * nodes)) / k;
 }
+// The same for the step kernel under its default schedule (measured from
+// 96 x 1600, 20.7 us, to 128 x 8000, 43.9 us): below about 600 000 nodes of
+// at most 64 rows the tiles win (64 x 6000: 17.0 against 23.6 us), with 128
+// rows only up to 1300 columns (13.2 against 18.3 us; 2560: 25.1 against
+// 23.9).
+double step_kernel_cost(int N, int Nx) { return 14.0 + 2.9e-5 * (double)N * Nx; }
 
 // Tile width and steps per launch (odd, so that launches alternate the two
 // buffers as single steps do) of least estimated cost on `sms` SMs; W = 0
@@ -1821,8 +1906,8 @@ void plan_tiles(const Lat& L, int sms, int* W_out, int* k_out, double* us_out) {
   }
 }
 
-// Largest channel that takes tiles, and the size of a handle's record rows.
-constexpr long TILE_MAX_NODES = 200000, HIST_BYTES = 2 << 20;
+// Size of a handle's record rows.
+constexpr long HIST_BYTES = 2 << 20;
 
 bool uses_tiles(const lbm_mix* h) { return h->tile_W > 0 && !h->rows_set; }
 
@@ -2182,10 +2267,8 @@ int lbm_mix_create(const lbm_mix_params* p, void* stream, lbm_mix** out) {
   ALLOC(h->clprof, sizeof(double) * (size_t)Nx);
   ALLOC(h->wall_r, sizeof(float2) * 2 * (size_t)Nx);
   ALLOC(h->wall_omq, sizeof(float) * 2 * (size_t)Nx);
-  // Row blocks: split each strip's rows over R CTAs of DEFAULT_ROWS rows so
-  // that the grid holds many waves of CTAs on the device's SMs and its last,
-  // partial wave is a small share of the launch.
-  h->rows_per_block = default_rows(h->L.N);
+  // Row blocks: each strip's rows are split over R CTAs (default_rows).
+  h->rows_per_block = default_rows(h);
   h->R = (h->L.N + h->rows_per_block - 1) / h->rows_per_block;
   h->R_alloc = h->R;
   ALLOC(h->colpart, sizeof(double) * 4 * (size_t)Nx * (size_t)h->R);
@@ -2194,7 +2277,7 @@ int lbm_mix_create(const lbm_mix_params* p, void* stream, lbm_mix** out) {
   if (p->storage == LBM_FP32) {
     double us = 0.0;
     plan_tiles(h->L, h->nsm, &h->tile_W, &h->tile_k, &us);
-    if ((long)h->L.N * Nx > TILE_MAX_NODES) h->tile_W = 0;
+    if (us > step_kernel_cost(h->L.N, Nx)) h->tile_W = 0;
     if (h->tile_W > 0) {
       const long fit = HIST_BYTES / (long)(sizeof(float2) * 4 * (size_t)Nx);
       h->hist_rows = (int)(fit < TILE_KMAX + 1 ? TILE_KMAX + 1 : fit < 256 ? fit : 256);
@@ -2694,7 +2777,7 @@ bool graph_valid(const lbm_sweep* s, int i, long K) {
 int policy_rows(const lbm_mix* h, int p) {
   const int N = h->L.N;
   switch (p) {
-    case 0: return 0;  // library default: row blocks of DEFAULT_ROWS rows
+    case 0: return 0;  // library default
     case 1: return 64;
     case 2: return 32;
     case 3: return 16;
