@@ -38,7 +38,9 @@
 #include <string.h>
 
 #include <mutex>
+#include <algorithm>
 #include <new>
+#include <type_traits>
 
 #include "../../include/lbm_mix.h"
 
@@ -76,37 +78,44 @@ constexpr int NREC = 8;         // doubles per diagnostic record
 constexpr int DIAG_CAP = 4096;  // diagnostic records kept
 constexpr float kPi = 3.14159265358979323846f;
 
-struct Lat {
-  int N, Nx, pitch;
+// What the FP32 node arithmetic and the tile kernel need; small, so that a
+// launch can carry one for each channel of a sweep.
+struct LatCore {
+  int N, Nx;
   unsigned SS;           // floats per strip: N * RS
   int x_periodic;
   int wall_mode;         // LBM_WALL_DBB or LBM_WALL_BSR
   int r_form;            // LBM_R_FIRST, LBM_R_SPECIES or LBM_R_SECOND (Eq. R)
   int lam_mix;           // lambda_s with the mixture (1) or partial (0) pressure
   float rsqrt_mh[2];     // 1 / sqrt(m_s / m_min)
-  int light;             // index of the light species
   float s[2];            // s_sigma = m_min / m_sigma
-  float cw0[2];          // rest-equilibrium weights w_i alpha_si: rest (9 - 5s)/9,
-  float cw1[2], cw5[2];  // axis s/9, diagonal s/36
-  // coefficients of the non-equilibrium energy moments on the deviations
-  // (rest, axis, diagonal): e: -2s, 3 - 2s, 6 - 2s; eps: 3s, 3s - 6, 3s - 3
-  float ke[2][3], kp[2][3];
-  // the per-species constants as (species a, species b) pairs for the packed
-  // FP32x2 arithmetic; ce2, cp2: ke2 om_e / 36 and kp2 om_eps / 36, cu2: the
-  // coefficients of rho u^2 (-3, 3) likewise
-  float2 s2, cw1_2, cw5_2, c_xl2, inv_c_xl2, ke2[3], kp2[3], ce2[3], cp2[3], cu2[2];
+  // per-species constants as (species a, species b) pairs for the packed
+  // FP32x2 arithmetic; ce2, cp2: coefficients of the non-equilibrium energy
+  // moments on the deviations (rest, axis, diagonal: e: -2s, 3 - 2s, 6 - 2s;
+  // eps: 3s, 3s - 6, 3s - 3) times om_e / 36 and om_eps / 36, cu2: of rho u^2
+  // (-3, 3) likewise
+  float2 s2, cw1_2, cw5_2, c_xl2, inv_c_xl2, ce2[3], cp2[3], cu2[2];
   float inv_c_lam;       // 1 / (3 mu sqrt(pi/6))
   float c_lam;           // 3 mu sqrt(pi/6): lambda = c_lam / (n sqrt(m_x))
-  float c_xl[2];         // 3 mu_s sqrt(pi/(6 m_s)): x_s lambda_s = c_xl / n
-  float inv_c_xl[2];
   float c_ts;            // sqrt(6/pi)
   float c_td;            // (3/2) sqrt(3 m0 m_a m_b / m_min)
-  float om_e, om_eps;    // 1/tau_e, 1/tau_eps
   float c_m0;
   float H;               // channel height = N
-  double mh[2];          // m_sigma / m_min
   float2 end_mass[2][2]; // N rho_s at the inlet, outlet ([end][species]) as a
                          // sum of two floats
+};
+
+struct Lat : LatCore {
+  int pitch;
+  int light;             // index of the light species
+  float cw0[2];          // rest-equilibrium weights w_i alpha_si: rest (9 - 5s)/9,
+  float cw1[2], cw5[2];  // axis s/9, diagonal s/36
+  float ke[2][3], kp[2][3];  // the coefficients behind ce2, cp2, unscaled
+  float2 ke2[3], kp2[3];     // the same in pairs
+  float c_xl[2];         // 3 mu_s sqrt(pi/(6 m_s)): x_s lambda_s = c_xl / n
+  float inv_c_xl[2];
+  float om_e, om_eps;    // 1/tau_e, 1/tau_eps
+  double mh[2];          // m_sigma / m_min
   double rho_in[2], rho_out[2];
   double C_in, C_out;    // light-species mole fraction at the ends
 };
@@ -285,10 +294,11 @@ __device__ __forceinline__ unsigned idx(const Lat& L, int sp, int i, int j, int 
 // stream-serialisation attribute may start while the kernel before it in the
 // stream is still running.  The kernels of the step sequence wait for their
 // predecessor's completion and memory (wait) before their first global
-// memory access.  The wall kernel lets its successor (the step) launch as
-// soon as all of its own CTAs run (launch_dependents); the step kernel does
-// so for the instances of a sweep only, and otherwise lets its successor
-// launch when it completes.  Launched without the attribute, both
+// memory access.  The wall kernel and the tile kernel let their successor
+// launch as soon as all of their own CTAs run (launch_dependents); the step
+// kernel lets it launch when it completes (the next kernel's CTAs are then
+// spread evenly over the SMs the step frees: 0.2197 against 0.2235 s for 5000
+// steps of a 1280 x 64 channel).  Launched without the attribute, both
 // instructions return at once.
 __device__ __forceinline__ void pdl_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -456,7 +466,7 @@ struct Macro {
   float n, inv_n, mx;
 };
 
-__device__ __forceinline__ float number_density(const Lat& L, float rho_a, float rho_b) {
+__device__ __forceinline__ float number_density(const LatCore& L, float rho_a, float rho_b) {
   return fmaf(rho_a, L.s[0], __fmul_rn(rho_b, L.s[1]));  // Eq. P
 }
 
@@ -490,7 +500,7 @@ __device__ __forceinline__ float2 density_sum(const float2 g[9]) {
   return add2(g[0], add2(a14, a58));
 }
 
-__device__ __forceinline__ void macro2(const Lat& L, float2 rb, const float2 g[9], Macro2& m) {
+__device__ __forceinline__ void macro2(const LatCore& L, float2 rb, const float2 g[9], Macro2& m) {
   m.sd = density_sum(g);
   m.rho = add2(rb, m.sd);
   const float rho = __fadd_rn(m.rho.x, m.rho.y);
@@ -529,7 +539,7 @@ __device__ __forceinline__ void flow2(const float2 g[9], float inv_rho, Flow2& w
 // Psi(y; lambda_s), lambda_s = (mu_s/p_s) sqrt(pi k_B T/(2 m_s)), p_s = x_s p),
 // with the wall-confinement factor Psi(y) = (psi(y/lambda) + psi((H-y)/lambda))/2
 // of the effective mean free path.  T: psi's table in shared memory.
-__device__ __forceinline__ void rates2(const Lat& L, const float4* T, const Macro2& m, float y,
+__device__ __forceinline__ void rates2(const LatCore& L, const float4* T, const Macro2& m, float y,
                                        float& om_s, float& om_d) {
   const float rs_mx = rsqrt_fast(m.mx);
   const float lam = __fmul_rn(__fmul_rn(L.c_lam, m.inv_n), rs_mx);  // mixture mean free path
@@ -568,7 +578,7 @@ __device__ __forceinline__ void rates2(const Lat& L, const float4* T, const Macr
 // times om_e / 36 and om_eps / 36, the classes' common factor in M^{-1}).
 // Returns the x components of the species momenta of Eq. rhou,
 // j_x - (j_x - rho_s u_x)/(2 tau_d).
-__device__ __forceinline__ float2 collide2(float2 g[9], const Lat& L, const Macro2& m, float om_d,
+__device__ __forceinline__ float2 collide2(float2 g[9], const LatCore& L, const Macro2& m, float om_d,
                                            float om_q, float om_s) {
   Flow2 w;
   flow2(g, m.inv_rho, w);
@@ -621,7 +631,7 @@ __device__ __forceinline__ float2 slip_coefficients(float alpha) {
 // 1/tau_q of Eq. taoq from the wall node's n, 1/n and m_x (tau'_s(0) in its
 // last term, dx = 1) and A = (A1, A2) of its accommodation coefficient.  P,
 // D: the tables of psi and psi'.
-__device__ __forceinline__ float inv_tau_q(const Lat& L, const float4* P, const float4* D,
+__device__ __forceinline__ float inv_tau_q(const LatCore& L, const float4* P, const float4* D,
                                            float n, float inv_n, float mx, float2 A) {
   const float vs = 0.72360125455f;  // varsigma = sqrt(pi/6)
   const float rs_mx = rsqrt_fast(mx);
@@ -646,10 +656,10 @@ __device__ __forceinline__ float inv_tau_q(const Lat& L, const float4* P, const 
 // m_x/(6 m_s)) (m_min replaced by the species mass) or c_m sqrt(pi m_x^2/(6
 // m_s)) (second printed form, m_r = m_s/m_x).  With the BSR wall the
 // bounce-back fraction 1/(1 + X) of the same slip factor X.
-__device__ __forceinline__ float slip_cm(const Lat& L, float alpha) {
+__device__ __forceinline__ float slip_cm(const LatCore& L, float alpha) {
   return __fmul_rn(L.c_m0, __fsub_rn(2.0f, alpha)) / alpha;
 }
-__device__ __forceinline__ float2 slip_r(const Lat& L, float rho_a, float rho_b, float cm) {
+__device__ __forceinline__ float2 slip_r(const LatCore& L, float rho_a, float rho_b, float cm) {
   const float mx = __fadd_rn(rho_a, rho_b) / number_density(L, rho_a, rho_b);
   const float q = sqrtf(__fmul_rn(kPi / 6.0f, mx));
   float X0 = __fmul_rn(cm, q);
@@ -744,7 +754,7 @@ __device__ __forceinline__ Ends load_ends(const Lat& L, const double* __restrict
   return E;
 }
 
-__device__ __forceinline__ bool interior(const Lat& L, int x) {
+__device__ __forceinline__ bool interior(const LatCore& L, int x) {
   return L.x_periodic ? (x < L.Nx) : (x >= 1 && x <= L.Nx - 2);
 }
 
@@ -877,6 +887,38 @@ struct KahanF {
   __device__ __forceinline__ double value() const { return (double)s - (double)c; }
 };
 
+// Sum of v(0) .. v(N - 1), the rows of a column, by eight neighbouring lanes
+// (sub = lane & 7, every lane of the warp here): each
+// takes every eighth row in order, compensated, then three error-free
+// additions.  Every lane of the eight gets the same (sum, error) pair.
+template <typename V>
+__device__ __forceinline__ float2 column_sum8(int N, int sub, V&& v) {
+  KahanF a;
+  for (int j = sub; j < N; j += 8) a.add(v(j));
+  float hi = a.s, lo = -a.c;
+#pragma unroll
+  for (int o = 1; o < 8; o <<= 1) {
+    const float h2 = __shfl_xor_sync(0xffffffffu, hi, o);
+    const float l2 = __shfl_xor_sync(0xffffffffu, lo, o);
+    const float2 s = two_sum(hi, h2);
+    lo = __fadd_rn(__fadd_rn(lo, l2), s.y);
+    hi = s.x;
+  }
+  return make_float2(hi, lo);
+}
+__device__ __forceinline__ double pair_value(float2 v) { return (double)v.x + (double)v.y; }
+
+// N ref + (sum of deviations) as a float pair whose low part is cut at 2^-48
+// of the high one, so that its FP64 value splits into the same pair again: a
+// launch that starts from the stored FP64 sums continues bit for bit.
+__device__ __forceinline__ float2 column_total(int N, float ref, float2 dev) {
+  const float n = (float)N, p = __fmul_rn(n, ref), pl = fmaf(n, ref, -p);
+  float2 s = two_sum(p, dev.x);
+  s = quick_two_sum(s.x, __fadd_rn(s.y, __fadd_rn(pl, dev.y)));
+  const float grid = __fmul_rn(s.x, 0x1p-24f);
+  return make_float2(s.x, __fsub_rn(__fadd_rn(s.y, grid), grid));
+}
+
 // ------------------------------------------------------------ step kernel
 // Random bits of the stochastic rounding: a 32-bit integer hash (the
 // "lowbias32" xorshift-multiply hash of C. Wellons) seeds one linear
@@ -936,9 +978,10 @@ struct StepArgs {
   // bottom then top), in place of the wall prologue (WK kernels only)
   const float2* __restrict__ wall_r;
   const float* __restrict__ wall_omq;
-  // 1: let the next kernel in the stream launch as soon as every CTA of
-  // this one runs; 0: when this one completes (see lbm_mix::pdl_early)
-  int pdl_early;
+  // [4][N] density deviations of columns 1, 2, Nx - 2, Nx - 3 (FP32 storage
+  // with pressure ends; null: their sums come from the row blocks like all
+  // others)
+  float2* __restrict__ end_sd;
 };
 
 struct RedSmem {
@@ -972,12 +1015,18 @@ __device__ __forceinline__ void warp_min(double& v, int& idx) {
 // the last CTA to finish reduces the partials in CTA order into one record.
 // DIAG = false: only the column sums (the next step's Eq. rho2 input) are
 // produced; DIAG = true: also C_l(x), the per-strip partials and the record.
+// g: the CTA's place in its channel's grid.
+struct GridPos {
+  int strip, block;     // strip and row block of this CTA
+  int strips, blocks;   // of the channel
+};
 template <bool DIAG, typename ST>
-__device__ __forceinline__ void column_epilogue(const Lat& L, const StepArgs<ST>& a, int x,
-                                                const double acc[4], RedSmem& rs) {
+__device__ __forceinline__ void column_epilogue(const Lat& L, const StepArgs<ST>& a,
+                                                const GridPos& gp, int x, const double acc[4],
+                                                RedSmem& rs) {
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int tid = ty * TX + tx;
-  const int R = gridDim.y;  // row blocks per strip
+  const int R = gp.blocks;  // row blocks per strip
 #pragma unroll
   for (int k = 0; k < 4; ++k) rs.col[k][ty][tx] = acc[k];
   __syncthreads();
@@ -997,13 +1046,13 @@ __device__ __forceinline__ void column_epilogue(const Lat& L, const StepArgs<ST>
       if (x < L.Nx) {
 #pragma unroll
         for (int k = 0; k < 4; ++k)
-          a.colpart[((size_t)blockIdx.y * 4 + k) * L.Nx + x] = c[k];
+          a.colpart[((size_t)gp.block * 4 + k) * L.Nx + x] = c[k];
       }
       __threadfence();  // the writers publish before the ticket is taken
     }
     __syncthreads();
     if (tid == 0) {
-      unsigned ticket = atomicAdd(a.strip_cnt + blockIdx.x, 1u);
+      unsigned ticket = atomicAdd(a.strip_cnt + gp.strip, 1u);
       rs.last_strip = (ticket == (unsigned)R - 1u);
     }
     __syncthreads();
@@ -1017,7 +1066,26 @@ __device__ __forceinline__ void column_epilogue(const Lat& L, const StepArgs<ST>
           for (int r = 0; r < R; ++r) v += __ldcg(a.colpart + ((size_t)r * 4 + k) * L.Nx + x);
         c[k] = v;
       }
-      if (tx == 0) a.strip_cnt[blockIdx.x] = 0u;
+      if (tx == 0) a.strip_cnt[gp.strip] = 0u;
+    }
+  }
+  if (sizeof(ST) == 4 && a.end_sd && ty == 0) {
+    // The columns behind the next step's density correction, in the order of
+    // column_sum8 over all rows: the populations of a run are then the same
+    // bits under every schedule, this kernel's and lbm_tile_kernel's.
+    const int x0 = x - tx;
+    for (int e = 0; e < 4; ++e) {
+      const int xe = e == 0 ? 1 : e == 1 ? 2 : e == 2 ? L.Nx - 2 : L.Nx - 3;
+      if (xe < x0 || xe >= x0 + TX) continue;  // warp-uniform
+#pragma unroll
+      for (int sp = 0; sp < 2; ++sp) {
+        const float2 v = column_sum8(L.N, tx & 7, [&](int r) {
+          const float2 d = __ldcg(a.end_sd + (size_t)e * L.N + r);
+          return sp ? d.y : d.x;
+        });
+        const double t = pair_value(column_total(L.N, a.refrho[sp * L.Nx + xe], v));
+        if (x == xe) c[sp] = t;
+      }
     }
   }
   if (!DIAG) {
@@ -1051,7 +1119,7 @@ __device__ __forceinline__ void column_epilogue(const Lat& L, const StepArgs<ST>
     double p_rb = warp_sum(in ? c[1] : 0.0);
     double p_n = warp_sum(in ? 1.0 : 0.0);
     if (tx == 0) {
-      double* p = a.partials + (size_t)blockIdx.x * NPART;
+      double* p = a.partials + (size_t)gp.strip * NPART;
       p[0] = vmin;
       p[1] = (double)imin;
       p[2] = p_dev;
@@ -1066,7 +1134,7 @@ __device__ __forceinline__ void column_epilogue(const Lat& L, const StepArgs<ST>
   __syncthreads();
   if (tid == 0) {
     unsigned ticket = atomicAdd(a.counter, 1u);
-    rs.last = (ticket == gridDim.x - 1);
+    rs.last = (ticket == (unsigned)gp.strips - 1u);
   }
   __syncthreads();
   if (!rs.last) return;
@@ -1077,7 +1145,7 @@ __device__ __forceinline__ void column_epilogue(const Lat& L, const StepArgs<ST>
   const int nt = TX * TY;
   double vmin = INFINITY, sm[6] = {0, 0, 0, 0, 0, 0};
   int imin = 0x7fffffff;
-  for (int b = tid; b < (int)gridDim.x; b += nt) {
+  for (int b = tid; b < gp.strips; b += nt) {
     const double* p = a.partials + (size_t)b * NPART;
     double v = __ldcg(p + 0);
     int i = (int)__ldcg(p + 1);
@@ -1135,25 +1203,25 @@ __device__ __forceinline__ void column_epilogue(const Lat& L, const StepArgs<ST>
 // WK: r and 1/tau_q of the columns come from lbm_walls_kernel, launched
 // ahead of the step (always with 16-bit storage), instead of the CTA's wall
 // prologue.
-template <typename ST, bool DIAG, bool WK = (sizeof(ST) < 4)>
-__global__ void __launch_bounds__(TX* TY, 3) lbm_step_kernel(Lat L, StepArgs<ST> a) {
+template <typename ST, bool WK>
+__device__ __forceinline__ void step_cta(const Lat& L, const StepArgs<ST>& a, const GridPos& gp,
+                                         bool diag) {
   __shared__ WallSmem wsm;
   __shared__ RedSmem rsm;
   constexpr bool FP32 = sizeof(ST) == 4;
   __shared__ float4 psi_tab[FP32 ? PSI_SEGMENTS : 1];
-  if (a.pdl_early) pdl_launch_dependents();
   const int tx = threadIdx.x, ty = threadIdx.y;
   if (FP32) load_psi_table(psi_tab, ty * TX + tx, TX * TY);  // overlaps the kernel before
   pdl_wait();
-  const int x0 = blockIdx.x * TX, x = x0 + tx;
+  const int x0 = gp.strip * TX, x = x0 + tx;
   const ColRef C = col_ref(L, a.refrho, x);
-  const Ends E = ends_of<ST>(L, a.cs_in, a.refrho, blockIdx.x * TX, TX);
-  const int j_begin = blockIdx.y * a.rows_per_block;
+  const Ends E = ends_of<ST>(L, a.cs_in, a.refrho, gp.strip * TX, TX);
+  const int j_begin = gp.block * a.rows_per_block;
   const int j_end = min(L.N, j_begin + a.rows_per_block);
   // the first row of each warp is on its way into L2 while the wall prologue
   // (if any) runs
   if (tx == 0 && j_begin + ty < j_end)
-    prefetch_row_l2(a.fin + (size_t)blockIdx.x * L.SS + (size_t)(j_begin + ty) * RS);
+    prefetch_row_l2(a.fin + (size_t)gp.strip * L.SS + (size_t)(j_begin + ty) * RS);
   // r and 1/tau_q of this column: from lbm_walls_kernel (WK, read where they
   // are used) or from the CTA's wall prologue
   const int xc = x < L.Nx ? x : L.Nx - 1;
@@ -1170,16 +1238,19 @@ __global__ void __launch_bounds__(TX* TY, 3) lbm_step_kernel(Lat L, StepArgs<ST>
     else return wsm.om_q[h][tx];
   };
   const bool in = interior(L, x);
-  // strips holding column 1 or N_x - 2 take the general pull (ghost columns)
-  const bool edge_strip = !L.x_periodic && (x0 <= 1 || x0 + TX > L.Nx - 2);
+  // strips holding one of the columns 1, 2, N_x - 3, N_x - 2 take the general
+  // pull (ghost columns) and reduce their column sums at every step
+  const bool edge_strip = !L.x_periodic && (x0 <= 2 || x0 + TX > L.Nx - 3);
+  const int end_l = x == 1 ? 0 : x == 2 ? 1 : -1;
+  const int end_r = x == L.Nx - 2 ? 2 : x == L.Nx - 3 ? 3 : -1;
   int xm = x - 1, xp = x + 1;
   if (xm < 0) xm += L.Nx;
   if (xp >= L.Nx) xp -= L.Nx;
-  const unsigned base = blockIdx.x * L.SS + 2 * tx;  // row 0, i = 0, species a of column x
+  const unsigned base = gp.strip * L.SS + 2 * tx;  // row 0, i = 0, species a of column x
   const int offl = (int)(idx(L, 0, 0, 0, xm) - base), offr = (int)(idx(L, 0, 0, 0, xp) - base);
   const int half = (L.N + 1) / 2;  // rows j < half (1-based 2J <= N+1) use the bottom tau_q
   KahanF acc[4];
-  const bool reduce = DIAG || edge_strip;
+  const bool reduce = diag || edge_strip;
   unsigned rng = 0u;  // generator of the stochastic rounding
   // one run over the rows, with 16-bit storage one per sequence of random bits
   for (int js = j_begin, je; in && js < j_end; js = je) {
@@ -1188,7 +1259,7 @@ __global__ void __launch_bounds__(TX* TY, 3) lbm_step_kernel(Lat L, StepArgs<ST>
       constexpr Lcg9 jump;
       const int block = js / RNG_ROWS;
       je = min(j_end, (block + 1) * RNG_ROWS);
-      rng = hash32(a.seed ^ hash32((block * gridDim.x + blockIdx.x) * (TX * TY) + ty * TX + tx));
+      rng = hash32(a.seed ^ hash32((block * gp.strips + gp.strip) * (TX * TY) + ty * TX + tx));
       for (int r = (js - block * RNG_ROWS) / TY; r > 0; --r) rng = rng * jump.a + jump.c;
     }
     for (int j = js + ty; j < je; j += TY) {
@@ -1223,6 +1294,10 @@ __global__ void __launch_bounds__(TX* TY, 3) lbm_step_kernel(Lat L, StepArgs<ST>
         mxs = n16::collide2(g, L, m.rho, m.ux, m.uy, L.om_e, L.om_eps, om_d, om_q, om_s);
         sd = m.sd;
       }
+      if (FP32 && edge_strip && a.end_sd) {
+        if (end_l >= 0) a.end_sd[end_l * L.N + j] = sd;
+        if (end_r >= 0) a.end_sd[end_r * L.N + j] = sd;
+      }
       if (reduce) {
         acc[0].add(sd.x);
         acc[1].add(sd.y);
@@ -1242,15 +1317,50 @@ __global__ void __launch_bounds__(TX* TY, 3) lbm_step_kernel(Lat L, StepArgs<ST>
   if (!reduce) return;  // CTA-uniform
   // column sum of rho_s = N rhobar_s + sum of deviations; the reference part
   // is added once per column (by the ty = 0 thread of the first row block)
-  const bool adds_ref = in && ty == 0 && blockIdx.y == 0;
+  const bool adds_ref = in && ty == 0 && gp.block == 0;
   double accd[4];
 #pragma unroll
   for (int sp = 0; sp < 2; ++sp)
     accd[sp] = (adds_ref ? (double)L.N * (double)C.rb[sp] : 0.0) + acc[sp].value();
   accd[2] = acc[2].value();
   accd[3] = acc[3].value();
-  column_epilogue<DIAG>(L, a, x, accd, rsm);
+  if (diag)
+    column_epilogue<true>(L, a, gp, x, accd, rsm);
+  else
+    column_epilogue<false>(L, a, gp, x, accd, rsm);
 }
+
+template <typename ST, bool DIAG, bool WK = (sizeof(ST) < 4)>
+__global__ void __launch_bounds__(TX* TY, 3) lbm_step_kernel(Lat L, StepArgs<ST> a) {
+  const GridPos gp{(int)blockIdx.x, (int)blockIdx.y, (int)gridDim.x, (int)gridDim.y};
+  step_cta<ST, WK>(L, a, gp, DIAG);
+}
+
+// One step of several channels (FP32 storage, wall prologue) as one launch:
+// the CTAs of channel q are [block0[q], block0[q + 1]), strips fastest, as in
+// the channel's own grid.  A sweep of 52 channels of 700 x 20 spent 147 us per
+// step on 52 launches from as many graphs, 2.8 us each.
+struct StepInst {
+  Lat L;
+  StepArgs<float> a;
+  int strips, blocks, diag;
+};
+template <int NI>
+struct StepBatch {
+  int block0[NI + 1];
+  StepInst inst[NI];
+};
+template <int NI>
+__global__ void __launch_bounds__(TX* TY, 3)
+    lbm_step_batch_kernel(const __grid_constant__ StepBatch<NI> B) {
+  int q = 0;
+  while ((int)blockIdx.x >= B.block0[q + 1]) ++q;
+  const StepInst& I = B.inst[q];
+  const int b = (int)blockIdx.x - B.block0[q];
+  const GridPos gp{b % I.strips, b / I.strips, I.strips, I.blocks};
+  step_cta<float, false>(I.L, I.a, gp, I.diag != 0);
+}
+
 
 #include "lbm_tile.cuh"
 
@@ -1446,10 +1556,25 @@ __global__ void lbm_volume_flow_kernel(const double* __restrict__ mom, int N, in
 }
 
 // Steady-state residual over the column sums: R = |c - c_old| / (K |c|),
-// then c_old = c.  One CTA.
-__global__ void lbm_residual_kernel(const double* __restrict__ c, double* __restrict__ c_old,
-                                    long n, double K, int have_old, double* __restrict__ R) {
+// then c_old = c.  One CTA per channel.
+struct ResidInst {
+  const double* c;
+  double* c_old;
+  long n;
+  int have_old;
+};
+template <int NI>
+struct ResidBatch {
+  ResidInst inst[NI];
+};
+template <int NI>
+__global__ void lbm_residual_kernel(const __grid_constant__ ResidBatch<NI> B, double K,
+                                    double* __restrict__ R) {
   __shared__ double s1[32], s2[32];
+  const double* __restrict__ c = B.inst[blockIdx.x].c;
+  double* __restrict__ c_old = B.inst[blockIdx.x].c_old;
+  const long n = B.inst[blockIdx.x].n;
+  const int have_old = B.inst[blockIdx.x].have_old;
   double d2 = 0.0, c2 = 0.0;
   for (long k = threadIdx.x; k < n; k += blockDim.x) {
     double v = c[k];
@@ -1472,7 +1597,7 @@ __global__ void lbm_residual_kernel(const double* __restrict__ c, double* __rest
     c2 = lane < nw ? s2[lane] : 0.0;
     d2 = warp_sum(d2);
     c2 = warp_sum(c2);
-    if (lane == 0) *R = have_old ? sqrt(d2) / (K * sqrt(c2)) : INFINITY;
+    if (lane == 0) R[blockIdx.x] = have_old ? sqrt(d2) / (K * sqrt(c2)) : INFINITY;
   }
 }
 
@@ -1512,19 +1637,16 @@ struct lbm_mix {
   double* clprof;
   float2* wall_r;      // [2][Nx] r per wall and column (lbm_walls_kernel)
   float* wall_omq;     // [2][Nx] 1/tau_q per half and column (lbm_walls_kernel)
+  float2* end_sd;      // [4][N] (FP32 storage with pressure ends, else null)
   double* colpart;     // [R][4][Nx]
+  double* colpart0;    // its place in the arena
+  void* arena;         // holds the arrays above and below but scratch and mom
   unsigned* strip_cnt; // [nblocks]
   int R, rows_per_block;
   int R_alloc;        // row blocks colpart has room for
   double* resid;
   double* mom;
   double* h_pinned;  // small pinned staging area
-  // The step kernel lets the next kernel launch as soon as all of its CTAs
-  // run (instances of a sweep, whose streams compete for the SMs: the sweep
-  // took 57.9 instead of 60.1 s), or only when it completes (lone handles:
-  // the next kernel's CTAs are then spread over the SMs the step frees;
-  // 0.2197 instead of 0.2235 s for 5000 steps of a 1280 x 64 channel).
-  bool pdl_early;
   // Several steps per launch (lbm_tile_kernel): own columns per tile and
   // most steps of a launch; tile_W = 0: the channel does not qualify.  A
   // schedule the caller set (rows_set) takes the step kernel instead.
@@ -1747,8 +1869,9 @@ int rereference(lbm_mix* h) {
 // Steady-state residual of the last k steps (Sec. 4 convergence check, over
 // the column sums of the latest DIAG step) into h->h_pinned[0], async.
 int launch_residual(lbm_mix* h, long k) {
-  lbm_residual_kernel<<<1, 1024, 0, h->stream>>>(h->cs[h->cur], h->cs_snap, 4L * h->L.Nx,
-                                                 (double)k, h->have_snap ? 1 : 0, h->resid);
+  ResidBatch<1> B;
+  B.inst[0] = ResidInst{h->cs[h->cur], h->cs_snap, 4L * h->L.Nx, h->have_snap ? 1 : 0};
+  lbm_residual_kernel<1><<<1, 1024, 0, h->stream>>>(B, (double)k, h->resid);
   CK(cudaGetLastError());
   h->have_snap = true;
   CK(cudaMemcpyAsync(h->h_pinned, h->resid, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
@@ -1767,7 +1890,7 @@ int set_rows_per_block(lbm_mix* h, int rows) {
     double* cp = nullptr;
     CK(cudaStreamSynchronize(h->stream));
     CK(cudaMalloc((void**)&cp, sizeof(double) * 4 * (size_t)h->L.Nx * (size_t)R));
-    cudaFree(h->colpart);
+    if (h->colpart != h->colpart0) cudaFree(h->colpart);
     h->colpart = cp;
     h->R_alloc = R;
   }
@@ -1795,32 +1918,39 @@ bool uses_wall_kernel(const lbm_mix* h) {
   return ctas >= WALL_KERNEL_WAVES * 3L * (long)(h->nsm > 0 ? h->nsm : 1);
 }
 
-int launch_step(lbm_mix* h, bool diag) {
+// Arguments of h's next step.
+template <typename ST>
+StepArgs<ST> step_args(const lbm_mix* h) {
   const int b = h->cur;
+  StepArgs<ST> a;
+  a.fin = (const ST*)h->buf[b];
+  a.fout = (ST*)h->buf[1 - b];
+  a.refrho = h->refrho;
+  a.cs_in = h->cs[b];
+  a.cs_out = h->cs[1 - b];
+  a.alpha = h->alpha;
+  a.partials = h->partials;
+  a.counter = h->counter;
+  a.diag = h->diag;
+  a.diag_count = h->diag_count;
+  a.clprof = h->clprof;
+  a.colpart = h->colpart;
+  a.strip_cnt = h->strip_cnt;
+  a.rows_per_block = h->rows_per_block;
+  // stochastic rounding of 16-bit stores: a fresh seed every step (never 0)
+  a.seed = (sizeof(ST) < 4 && h->p.rounding == LBM_ROUND_STOCHASTIC)
+               ? (host_hash32((unsigned)(h->steps + 1)) | 1u)
+               : 0u;
+  a.wall_r = h->wall_r;
+  a.wall_omq = h->wall_omq;
+  a.end_sd = h->end_sd;
+  return a;
+}
+
+int launch_step(lbm_mix* h, bool diag) {
   int st = with_storage(h, [&](auto tag) -> int {
     using ST = decltype(tag);
-    StepArgs<ST> a;
-    a.fin = (const ST*)h->buf[b];
-    a.fout = (ST*)h->buf[1 - b];
-    a.refrho = h->refrho;
-    a.cs_in = h->cs[b];
-    a.cs_out = h->cs[1 - b];
-    a.alpha = h->alpha;
-    a.partials = h->partials;
-    a.counter = h->counter;
-    a.diag = h->diag;
-    a.diag_count = h->diag_count;
-    a.clprof = h->clprof;
-    a.colpart = h->colpart;
-    a.strip_cnt = h->strip_cnt;
-    a.rows_per_block = h->rows_per_block;
-    // stochastic rounding of 16-bit stores: a fresh seed every step (never 0)
-    a.seed = (sizeof(ST) < 4 && h->p.rounding == LBM_ROUND_STOCHASTIC)
-                 ? (host_hash32((unsigned)(h->steps + 1)) | 1u)
-                 : 0u;
-    a.wall_r = h->wall_r;
-    a.wall_omq = h->wall_omq;
-    a.pdl_early = h->pdl_early ? 1 : 0;
+    const StepArgs<ST> a = step_args<ST>(h);
     // Both kernels are launched with programmatic stream serialisation, so
     // that each one's launch and CTA ramp overlap the end of the kernel
     // before it (see pdl_wait).
@@ -1855,7 +1985,7 @@ int launch_step(lbm_mix* h, bool diag) {
     return LBM_OK;
   });
   if (st) return st;
-  h->cur = 1 - b;
+  h->cur = 1 - h->cur;
   h->steps++;
   return LBM_OK;
 }
@@ -1929,10 +2059,11 @@ int launch_batch(void (*kern)(B), const B& batch, dim3 grid, dim3 block, size_t 
   return LBM_OK;
 }
 
-// One launch of k steps for the n <= NI channels hs, whose record rows used
-// so far are rows[]; last: step k ends the call.
+// One launch of k steps for the n <= NI channels hs in tiles of W[] columns,
+// whose record rows used so far are rows[]; last: step k ends the call.
 template <int NI>
-int launch_tiles(lbm_mix* const* hs, int n, int k, bool last, int* rows, cudaStream_t st) {
+int launch_tiles(lbm_mix* const* hs, const int* W, int n, int k, bool last, int* rows,
+                 cudaStream_t st) {
   TileBatch<NI> B;
   B.k = k;
   int blocks = 0, nodes = 0;
@@ -1952,7 +2083,7 @@ int launch_tiles(lbm_mix* const* hs, int n, int k, bool last, int* rows, cudaStr
     I.cs_in = h->cs[b];
     I.cs_out = h->cs[1 - b];
     I.hist = h->hist + (size_t)rows[q] * 4 * L.Nx;
-    I.W = h->tile_W;
+    I.W = W[q];
     I.diag_every = de;
     I.diag_phase = (int)(h->steps % de);
     I.last = last ? 1 : 0;
@@ -1985,8 +2116,10 @@ int launch_records(lbm_mix* const* hs, int n, int* rows, cudaStream_t st) {
   int most = 0;
   for (int q = 0; q < n; ++q) {
     lbm_mix* h = hs[q];
-    B.inst[q] = RecInst{h->L,       h->hist,    h->refrho, h->diag, h->diag_count,
-                        h->counter, h->clprof, rows[q]};
+    const Lat& L = h->L;
+    B.inst[q] = RecInst{L.N,     L.Nx,    L.x_periodic, L.light, {L.s[0], L.s[1]}, L.C_in,
+                        L.C_out, h->hist, h->refrho,    h->diag, h->diag_count,    h->counter,
+                        h->clprof, rows[q]};
     most = rows[q] > most ? rows[q] : most;
     rows[q] = 0;
   }
@@ -1999,7 +2132,8 @@ int launch_records(lbm_mix* const* hs, int n, int* rows, cudaStream_t st) {
 // up holding the states of the last two steps.  end: the last step ends the
 // call and is recorded.
 template <int NI>
-int tile_steps(lbm_mix* const* hs, int n, int kmax, long nsteps, bool end, cudaStream_t st) {
+int tile_steps(lbm_mix* const* hs, const int* W, int n, int kmax, long nsteps, bool end,
+               cudaStream_t st) {
   int rows[NI] = {};
   int s = LBM_OK;
   for (long left = nsteps; left > 0;) {
@@ -2009,7 +2143,7 @@ int tile_steps(lbm_mix* const* hs, int n, int kmax, long nsteps, bool end, cudaS
     bool full = false;
     for (int q = 0; q < n; ++q) full |= rows[q] + k + 1 > hs[q]->hist_rows;
     if (full && (s = launch_records<NI>(hs, n, rows, st))) return s;
-    if ((s = launch_tiles<NI>(hs, n, k, end && left == k, rows, st))) return s;
+    if ((s = launch_tiles<NI>(hs, W, n, k, end && left == k, rows, st))) return s;
     left -= k;
   }
   return launch_records<NI>(hs, n, rows, st);
@@ -2191,27 +2325,9 @@ void lbm_mix_destroy(lbm_mix* h) {
   cudaGetDevice(&prev);
   cudaSetDevice(h->device);
   if (h->stream) cudaStreamSynchronize(h->stream);
-  cudaFree(h->buf[0]);
-  cudaFree(h->buf[1]);
-  cudaFree(h->refrho);
-  cudaFree(h->refrho_alt);
-  cudaFree(h->cs_tmp);
+  cudaFree(h->arena);
+  if (h->colpart != h->colpart0) cudaFree(h->colpart);
   cudaFree(h->scratch);
-  cudaFree(h->cs[0]);
-  cudaFree(h->cs[1]);
-  cudaFree(h->cs_snap);
-  cudaFree(h->alpha);
-  cudaFree(h->partials);
-  cudaFree(h->counter);
-  cudaFree(h->diag);
-  cudaFree(h->diag_count);
-  cudaFree(h->clprof);
-  cudaFree(h->wall_r);
-  cudaFree(h->wall_omq);
-  cudaFree(h->colpart);
-  cudaFree(h->strip_cnt);
-  cudaFree(h->hist);
-  cudaFree(h->resid);
   cudaFree(h->mom);
   if (h->h_pinned) cudaFreeHost(h->h_pinned);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
@@ -2249,31 +2365,10 @@ int lbm_mix_create(const lbm_mix_params* p, void* stream, lbm_mix** out) {
   const size_t fbytes = h->elem * 18 * (size_t)h->L.N * h->L.pitch;
   const size_t cbytes = sizeof(double) * 4 * (size_t)Nx;
   cudaError_t e = cudaSuccess;
-#define ALLOC(ptr, bytes) \
-  if (e == cudaSuccess) e = cudaMalloc((void**)&(ptr), (bytes))
-  ALLOC(h->buf[0], fbytes);
-  ALLOC(h->buf[1], fbytes);
-  ALLOC(h->refrho, sizeof(float) * 2 * (size_t)Nx);
-  ALLOC(h->refrho_alt, sizeof(float) * 2 * (size_t)Nx);
-  ALLOC(h->cs_tmp, cbytes);
-  ALLOC(h->cs[0], cbytes);
-  ALLOC(h->cs[1], cbytes);
-  ALLOC(h->cs_snap, cbytes);
-  ALLOC(h->alpha, sizeof(float) * 2 * (size_t)Nx);
-  ALLOC(h->partials, sizeof(double) * NPART * (size_t)h->nblocks);
-  ALLOC(h->counter, sizeof(unsigned));
-  ALLOC(h->diag, sizeof(double) * DIAG_CAP * NREC);
-  ALLOC(h->diag_count, sizeof(unsigned long long));
-  ALLOC(h->clprof, sizeof(double) * (size_t)Nx);
-  ALLOC(h->wall_r, sizeof(float2) * 2 * (size_t)Nx);
-  ALLOC(h->wall_omq, sizeof(float) * 2 * (size_t)Nx);
   // Row blocks: each strip's rows are split over R CTAs (default_rows).
   h->rows_per_block = default_rows(h);
   h->R = (h->L.N + h->rows_per_block - 1) / h->rows_per_block;
   h->R_alloc = h->R;
-  ALLOC(h->colpart, sizeof(double) * 4 * (size_t)Nx * (size_t)h->R);
-  ALLOC(h->strip_cnt, sizeof(unsigned) * (size_t)h->nblocks);
-  ALLOC(h->resid, sizeof(double));
   if (p->storage == LBM_FP32) {
     double us = 0.0;
     plan_tiles(h->L, h->nsm, &h->tile_W, &h->tile_k, &us);
@@ -2281,13 +2376,50 @@ int lbm_mix_create(const lbm_mix_params* p, void* stream, lbm_mix** out) {
     if (h->tile_W > 0) {
       const long fit = HIST_BYTES / (long)(sizeof(float2) * 4 * (size_t)Nx);
       h->hist_rows = (int)(fit < TILE_KMAX + 1 ? TILE_KMAX + 1 : fit < 256 ? fit : 256);
-      ALLOC(h->hist, sizeof(float2) * 4 * (size_t)Nx * (size_t)h->hist_rows);
-      if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(lbm_tile_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 TILE_SMEM_MAX);
+      e = cudaFuncSetAttribute(lbm_tile_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               TILE_SMEM_MAX);
     }
   }
-#undef ALLOC
+  // One allocation holds every array of the handle (twenty calls took most of
+  // lbm_mix_create); the row-block partials can grow and may move out of it.
+  // Arrays that start at zero come first.
+  size_t zeroed = 0, total = 0;
+  auto carve = [&](char* base, size_t bytes, auto** ptr) {
+    if (base) *ptr = (std::remove_reference_t<decltype(*ptr)>)(base + total);
+    total += (bytes + 255) / 256 * 256;
+  };
+  auto layout = [&](char* base) {
+    total = 0;
+    carve(base, fbytes, &h->buf[0]);
+    carve(base, fbytes, &h->buf[1]);
+    carve(base, sizeof(unsigned), &h->counter);
+    carve(base, sizeof(unsigned) * (size_t)h->nblocks, &h->strip_cnt);
+    carve(base, cbytes, &h->cs[0]);
+    carve(base, cbytes, &h->cs[1]);
+    carve(base, sizeof(unsigned long long), &h->diag_count);
+    carve(base, sizeof(double) * DIAG_CAP * NREC, &h->diag);
+    zeroed = total;
+    carve(base, sizeof(float) * 2 * (size_t)Nx, &h->refrho);
+    carve(base, sizeof(float) * 2 * (size_t)Nx, &h->refrho_alt);
+    carve(base, sizeof(float) * 2 * (size_t)Nx, &h->alpha);
+    carve(base, cbytes, &h->cs_tmp);
+    carve(base, cbytes, &h->cs_snap);
+    carve(base, sizeof(double) * NPART * (size_t)h->nblocks, &h->partials);
+    carve(base, sizeof(double) * (size_t)Nx, &h->clprof);
+    carve(base, sizeof(float2) * 2 * (size_t)Nx, &h->wall_r);
+    carve(base, sizeof(float) * 2 * (size_t)Nx, &h->wall_omq);
+    if (p->storage == LBM_FP32 && !p->x_periodic)
+      carve(base, sizeof(float2) * 4 * (size_t)h->L.N, &h->end_sd);
+    carve(base, sizeof(double) * 4 * (size_t)Nx * (size_t)h->R, &h->colpart0);
+    carve(base, sizeof(double), &h->resid);
+    if (h->tile_W > 0) carve(base, sizeof(float2) * 4 * (size_t)Nx * h->hist_rows, &h->hist);
+  };
+  layout(nullptr);
+  if (e == cudaSuccess) e = cudaMalloc((void**)&h->arena, total);
+  if (e == cudaSuccess) {
+    layout((char*)h->arena);
+    h->colpart = h->colpart0;
+  }
   if (e == cudaSuccess) e = cudaMallocHost((void**)&h->h_pinned, sizeof(double) * 64);
   if (e != cudaSuccess) {
     int code = (e == cudaErrorMemoryAllocation) ? LBM_ENOMEM : LBM_ECUDA;
@@ -2296,14 +2428,8 @@ int lbm_mix_create(const lbm_mix_params* p, void* stream, lbm_mix** out) {
     lbm_mix_destroy(h);
     return code;
   }
-  // zero everything so that padding and ghost columns hold defined values
-  e = cudaMemsetAsync(h->buf[0], 0, fbytes, h->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(h->buf[1], 0, fbytes, h->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(h->counter, 0, sizeof(unsigned), h->stream);
-  if (e == cudaSuccess)
-    e = cudaMemsetAsync(h->strip_cnt, 0, sizeof(unsigned) * (size_t)h->nblocks, h->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(h->cs[0], 0, cbytes, h->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(h->cs[1], 0, cbytes, h->stream);
+  // zero, so that padding and ghost columns hold defined values
+  e = cudaMemsetAsync(h->arena, 0, zeroed, h->stream);
   if (e == cudaSuccess) {
     float* a = (float*)malloc(sizeof(float) * 4 * Nx);
     if (!a) e = cudaErrorMemoryAllocation;
@@ -2330,10 +2456,6 @@ int lbm_mix_create(const lbm_mix_params* p, void* stream, lbm_mix** out) {
   }
   if (e != cudaSuccess) {
     set_err(LBM_ECUDA, "initialisation failed: %s", cudaGetErrorString(e));
-    lbm_mix_destroy(h);
-    return LBM_ECUDA;
-  }
-  if (reset_diag(h) != LBM_OK) {
     lbm_mix_destroy(h);
     return LBM_ECUDA;
   }
@@ -2364,7 +2486,7 @@ int lbm_mix_step(lbm_mix* h, long nsteps) {
     for (long left = nsteps; left > 0;) {
       long n = left;
       if (reref > 0 && n > reref - h->steps % reref) n = reref - h->steps % reref;
-      if ((st = tile_steps<1>(&h, 1, h->tile_k, n, n == left, h->stream))) return st;
+      if ((st = tile_steps<1>(&h, &h->tile_W, 1, h->tile_k, n, n == left, h->stream))) return st;
       if (reref > 0 && h->steps % reref == 0 && (st = rereference(h))) return st;
       left -= n;
     }
@@ -2713,7 +2835,7 @@ int lbm_mix_step_noalloc(const lbm_mix_params* p, const float* d_in, float* d_ou
   a.seed = 0u;  // FP32 storage: no rounding to 16 bits
   a.wall_r = nullptr;  // FP32 storage: the wall prologue computes r and tau_q
   a.wall_omq = nullptr;
-  a.pdl_early = 0;  // a plain launch: the trigger would be a no-op
+  a.end_sd = nullptr;  // no room in the scratch: sums by row blocks
   dim3 blk(TX, TY), grd(nstrips, 1);
   lbm_step_kernel<float, true><<<grd, blk, 0, s>>>(L, a);
   CK(cudaGetLastError());
@@ -2723,55 +2845,35 @@ int lbm_mix_step_noalloc(const lbm_mix_params* p, const float* d_in, float* d_ou
 }  // extern "C"
 
 // ---------------------------------------------------------------- sweeps
-// A parametric study (Table 1) runs many independent channels.  Each
-// instance keeps its own handle and stream; K steps of an instance are
-// captured once as a CUDA graph (K fused step launches) and replayed, so the
-// host issues one graph launch per instance per convergence check and the
-// instances' kernels run concurrently, filling the GPU with channels that
-// are each too small to fill it alone.  The first blocks of
+// A parametric study (Table 1) runs many independent channels, each too small
+// to fill the GPU.  A sweep advances all of them by common launches on one
+// stream: the channels that fit tiles by lbm_tile_kernel, k steps a launch,
+// in tiles wide enough that the redundant halo work stays small; the others
+// by lbm_step_batch_kernel, one step a launch; then one launch each for the
+// records and for the residuals of a convergence check.  The launches carry
+// every channel's constants and pointers as kernel parameters, so each call
+// starts from the handles' state as it is.  The first blocks of
 // lbm_sweep_run_to_steady can serve as an autotuner of the node-to-CTA
-// schedule (rows per CTA): each candidate schedule runs one real block of
-// steps, the fastest is kept.  Schedules change only the order of the FP64
-// column reductions, not the time integration.
-// What a captured graph has baked into its launches besides the handle's
-// fixed buffers: the buffer parity it starts from, the schedule (rows per
-// CTA, row blocks and their partials), the reference-density table (swapped
-// by re-referencing) and the step phase that decides which captured steps
-// reduce diagnostics.  A graph is replayed only while all of them match.
-struct SweepCapKey {
-  int cur, rows, R;
-  const void* colpart;
-  const void* refrho;
-  long phase;
-  bool tiles;
-};
-
+// schedule: each candidate runs one real block of steps, the fastest is kept.
+// Schedules change only the order of the column sums, not the time
+// integration.
 struct lbm_sweep {
   int n = 0;
   lbm_mix** h = nullptr;
-  cudaGraphExec_t* exec = nullptr;
-  long* exec_K = nullptr;  // steps captured in exec[i]; 0 = none
-  SweepCapKey* key = nullptr;  // state each graph was captured from
-  int policy = -1;         // schedule in use (-1: the library default)
+  cudaStream_t stream = nullptr;
+  double* resid = nullptr;    // [n] residuals of a check
+  double* h_resid = nullptr;  // the same, pinned
+  int policy = -1;            // schedule in use (-1: the library default)
   double round_ms[LBM_SWEEP_NPOLICY] = {};
 };
 
 namespace {
 
-SweepCapKey cap_key(const lbm_mix* h) {
-  return SweepCapKey{h->cur, h->rows_per_block, h->R, h->colpart, h->refrho,
-                     h->steps % h->p.diag_every, uses_tiles(h)};
-}
-
-bool same_key(const SweepCapKey& a, const SweepCapKey& b) {
-  return a.cur == b.cur && a.rows == b.rows && a.R == b.R && a.colpart == b.colpart &&
-         a.refrho == b.refrho && a.phase == b.phase && a.tiles == b.tiles;
-}
-
-// Instance i has a graph of K steps that is valid for its current state.
-bool graph_valid(const lbm_sweep* s, int i, long K) {
-  return s->exec[i] && s->exec_K[i] == K && same_key(s->key[i], cap_key(s->h[i]));
-}
+// Channels of one launch (the parameters of a launch end at 32 764 bytes).
+constexpr int TILE_BATCH = 96, STEP_BATCH = 32;
+static_assert(sizeof(TileBatch<TILE_BATCH>) <= 32764 && sizeof(StepBatch<STEP_BATCH>) <= 32764 &&
+                  sizeof(RecBatch<TILE_BATCH>) <= 32764,
+              "kernel parameters");
 
 // Rows per CTA of instance h under schedule policy p.
 int policy_rows(const lbm_mix* h, int p) {
@@ -2792,54 +2894,145 @@ int policy_rows(const lbm_mix* h, int p) {
   }
 }
 
-void drop_graph(lbm_sweep* s, int i) {
-  if (s->exec[i]) cudaGraphExecDestroy(s->exec[i]);
-  s->exec[i] = nullptr;
-  s->exec_K[i] = 0;
-}
-
-// K (even) steps of instance i as one graph executable.  Capturing records
-// the launches without running them, so the host-side step count and buffer
-// parity are restored afterwards.
-int capture_steps(lbm_sweep* s, int i, long K) {
-  lbm_mix* h = s->h[i];
-  drop_graph(s, i);
-  const long steps0 = h->steps;
-  const int cur0 = h->cur;
-  const SweepCapKey key = cap_key(h);
-  CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-  int st = lbm_mix_step(h, K);
-  cudaGraph_t g = nullptr;
-  cudaError_t e = cudaStreamEndCapture(h->stream, &g);
-  h->steps = steps0;
-  h->cur = cur0;
-  if (st) {
-    if (g) cudaGraphDestroy(g);
-    return st;
+int apply_policy(lbm_sweep* s, int p) {
+  for (int i = 0; i < s->n; ++i) {
+    int st = set_rows_per_block(s->h[i], policy_rows(s->h[i], p));
+    if (st) return st;
+    s->h[i]->rows_set = p > 0;
   }
-  if (e != cudaSuccess)
-    return set_err(LBM_ECUDA, "stream capture failed: %s", cudaGetErrorString(e));
-  e = cudaGraphInstantiate(&s->exec[i], g, 0);
-  cudaGraphDestroy(g);
-  if (e != cudaSuccess) {
-    s->exec[i] = nullptr;
-    return set_err(LBM_ECUDA, "graph instantiation failed: %s", cudaGetErrorString(e));
-  }
-  s->exec_K[i] = K;
-  s->key[i] = key;
+  s->policy = p;
   return LBM_OK;
 }
 
-int apply_policy(lbm_sweep* s, int p) {
-  for (int i = 0; i < s->n; ++i) {
-    lbm_mix* h = s->h[i];
-    const SweepCapKey before = cap_key(h);
-    int st = set_rows_per_block(h, policy_rows(h, p));
-    if (st) return st;
-    h->rows_set = p > 0;
-    if (!same_key(before, cap_key(h))) drop_graph(s, i);
+// Estimated time (us) of one step of channels with that many nodes in all by
+// lbm_step_batch_kernel: 8 us of launch, start-up and tail, then 38 G nodes/s.
+double batch_step_cost(double nodes) { return 8.0 + nodes * 2.6e-5; }
+
+// Tile widths W[] and steps per launch of n channels of equal N advanced
+// together: for each k and each bound on a tile's nodes the estimate of
+// tile_cost with the channels' tiles sharing the waves, the least one kept.
+// Returns that estimate (us per step).
+double plan_batch(lbm_mix* const* hs, int n, int* W, int* k_out) {
+  const int sms = hs[0]->nsm > 0 ? hs[0]->nsm : 1, N = hs[0]->L.N, S = tile_stride(N);
+  int most = 0;  // columns of the largest tile
+  while (tile_smem(N, most + 1) <= (size_t)TILE_SMEM_MAX) ++most;
+  auto updated = [](const Lat& L) { return L.x_periodic ? L.Nx : L.Nx - 2; };
+  double best = INFINITY;
+  int best_w = 1;
+  *k_out = 1;
+  for (int k = 1; k <= TILE_KMAX && 2 * k < most; k += 2)
+    for (int w = most - 2 * k; w >= 1; w -= w > 8 ? w / 8 : 1) {
+      long tiles = 0;
+      for (int q = 0; q < n; ++q) tiles += (updated(hs[q]->L) + w - 1) / w;
+      const double us = (TILE_LAUNCH_US +
+                         (double)((tiles + sms - 1) / sms) *
+                             (TILE_LOAD_US + k * TILE_STEP_US +
+                              TILE_NODE_US * k * (w + k - 1) * (double)S)) / k;
+      if (us < best) {
+        best = us;
+        best_w = w;
+        *k_out = k;
+      }
+    }
+  for (int q = 0; q < n; ++q) {  // tiles of even width
+    const int nup = updated(hs[q]->L), tiles = (nup + best_w - 1) / best_w;
+    W[q] = (nup + tiles - 1) / tiles;
   }
-  s->policy = p;
+  return best;
+}
+
+// One step of the n <= STEP_BATCH channels hs; end: it ends the call.
+int launch_step_batch(lbm_mix* const* hs, int n, bool end, cudaStream_t st) {
+  StepBatch<STEP_BATCH> B;
+  // rows per CTA by the size of the whole launch (default_rows), but no fewer
+  // than a channel's own schedule has
+  long strip_rows = 0;
+  for (int q = 0; q < n; ++q) strip_rows += (long)hs[q]->L.N * hs[q]->nblocks;
+  const long most = (strip_rows / (WAVES * 3L * (hs[0]->nsm > 0 ? hs[0]->nsm : 1)) + TY - 1) / TY * TY;
+  int blocks = 0;
+  for (int q = 0; q < STEP_BATCH; ++q) {
+    B.block0[q] = blocks;
+    if (q >= n) continue;
+    lbm_mix* h = hs[q];
+    StepInst& I = B.inst[q];
+    I.L = h->L;
+    I.a = step_args<float>(h);
+    if (!h->rows_set) {
+      const long n8 = (h->L.N + TY - 1) / TY * TY, rows = most < 56 ? most : 56;
+      if (rows > I.a.rows_per_block) I.a.rows_per_block = (int)(rows < n8 ? rows : n8);
+    }
+    I.strips = h->nblocks;
+    I.blocks = (h->L.N + I.a.rows_per_block - 1) / I.a.rows_per_block;
+    I.diag = end || (h->steps + 1) % h->p.diag_every == 0;
+    blocks += I.strips * I.blocks;
+    h->cur = 1 - h->cur;
+    h->steps++;
+  }
+  B.block0[STEP_BATCH] = blocks;
+  return launch_batch(lbm_step_batch_kernel<STEP_BATCH>, B, dim3(blocks), dim3(TX, TY), 0, st);
+}
+
+// nsteps steps of the n channels hs of a sweep, on its stream.  Channels that
+// qualify for tiles take them, grouped by N, unless one step kernel over all
+// channels is estimated to be faster (many nodes in all, or tall channels);
+// the populations are the same bits either way.
+int batch_steps(lbm_sweep* s, lbm_mix* const* hs, int n, long nsteps) {
+  if (nsteps < 1) return LBM_OK;
+  lbm_mix** order = (lbm_mix**)malloc(2 * sizeof(lbm_mix*) * (size_t)n);
+  int* W = (int*)malloc(sizeof(int) * (size_t)n);
+  if (!order || !W) {
+    free(order), free(W);
+    return set_err(LBM_ENOMEM, "host allocation failed");
+  }
+  lbm_mix** rest = order + n;  // channels of the step kernel
+  int nt = 0, nr = 0, st = LBM_OK;
+  double nodes_t = 0.0, nodes_r = 0.0, us = 0.0;
+  for (int q = 0; q < n; ++q) {
+    const double nodes = (double)hs[q]->L.N * hs[q]->L.Nx;
+    (uses_tiles(hs[q]) ? nodes_t : nodes_r) += nodes;
+    if (uses_tiles(hs[q])) order[nt++] = hs[q];
+  }
+  std::sort(order, order + nt, [](const lbm_mix* a, const lbm_mix* b) { return a->L.N < b->L.N; });
+  auto group_end = [&](int q0) {
+    int q = q0;
+    while (q < nt && q - q0 < TILE_BATCH && order[q]->L.N == order[q0]->L.N) ++q;
+    return q;
+  };
+  int k = 1;
+  for (int q0 = 0, q1; q0 < nt; q0 = q1) us += plan_batch(order + q0, (q1 = group_end(q0)) - q0, W, &k);
+  const bool tiles = us + (nodes_r > 0 ? batch_step_cost(nodes_r) : 0.0) <= batch_step_cost(nodes_t + nodes_r);
+  for (int q0 = 0, q1; tiles && q0 < nt && !st; q0 = q1) {
+    const int m = (q1 = group_end(q0)) - q0;
+    plan_batch(order + q0, m, W, &k);
+    st = m <= 8 ? tile_steps<8>(order + q0, W, m, k, nsteps, true, s->stream)
+                : tile_steps<TILE_BATCH>(order + q0, W, m, k, nsteps, true, s->stream);
+  }
+  for (int q = 0; q < n; ++q)
+    if (!tiles || !uses_tiles(hs[q])) rest[nr++] = hs[q];
+  for (int q0 = 0; q0 < nr && !st; q0 += STEP_BATCH)
+    for (long t = 1; t <= nsteps && !st; ++t)
+      st = launch_step_batch(rest + q0, nr - q0 < STEP_BATCH ? nr - q0 : STEP_BATCH, t == nsteps,
+                             s->stream);
+  free(order), free(W);
+  return st;
+}
+
+// Residuals of the n channels hs of a sweep after k steps into s->h_resid, in
+// order; waits for them.
+int batch_residuals(lbm_sweep* s, lbm_mix* const* hs, int n, long k) {
+  for (int q0 = 0; q0 < n; q0 += TILE_BATCH) {
+    ResidBatch<TILE_BATCH> B;
+    const int m = n - q0 < TILE_BATCH ? n - q0 : TILE_BATCH;
+    for (int q = 0; q < m; ++q) {
+      lbm_mix* h = hs[q0 + q];
+      B.inst[q] = ResidInst{h->cs[h->cur], h->cs_snap, 4L * h->L.Nx, h->have_snap ? 1 : 0};
+      h->have_snap = true;
+    }
+    lbm_residual_kernel<TILE_BATCH><<<m, 1024, 0, s->stream>>>(B, (double)k, s->resid + q0);
+    CK(cudaGetLastError());
+  }
+  CK(cudaMemcpyAsync(s->h_resid, s->resid, sizeof(double) * n, cudaMemcpyDeviceToHost, s->stream));
+  CK(cudaStreamSynchronize(s->stream));
   return LBM_OK;
 }
 
@@ -2871,23 +3064,32 @@ int lbm_sweep_create(const lbm_mix_params* params, int n, lbm_sweep** out) {
   lbm_sweep* s = new (std::nothrow) lbm_sweep;
   if (!s) return set_err(LBM_ENOMEM, "host allocation failed");
   s->h = (lbm_mix**)calloc(n, sizeof(lbm_mix*));
-  s->exec = (cudaGraphExec_t*)calloc(n, sizeof(cudaGraphExec_t));
-  s->exec_K = (long*)calloc(n, sizeof(long));
-  s->key = (SweepCapKey*)calloc(n, sizeof(SweepCapKey));
-  if (!s->h || !s->exec || !s->exec_K || !s->key) {
+  if (!s->h) {
     lbm_sweep_destroy(s);
     return set_err(LBM_ENOMEM, "host allocation failed");
   }
   s->n = n;
+  cudaError_t e = cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaMalloc((void**)&s->resid, sizeof(double) * n);
+  if (e == cudaSuccess) e = cudaMallocHost((void**)&s->h_resid, sizeof(double) * n);
+  for (auto kern : {(const void*)lbm_tile_kernel<8>, (const void*)lbm_tile_kernel<TILE_BATCH>})
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, TILE_SMEM_MAX);
+  if (e != cudaSuccess) {
+    const int code = e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA;
+    set_err(code, "sweep: %s", cudaGetErrorString(e));
+    cudaGetLastError();
+    lbm_sweep_destroy(s);
+    return code;
+  }
   for (int i = 0; i < n; ++i) {
     lbm_mix_params p = params[i];
     p.reref_every = 0;
-    int st = lbm_mix_create(&p, nullptr, &s->h[i]);  // own stream per instance
+    int st = lbm_mix_create(&p, s->stream, &s->h[i]);  // all on the sweep's stream
     if (st) {
       lbm_sweep_destroy(s);
       return st;
     }
-    s->h[i]->pdl_early = true;
   }
   *out = s;
   return LBM_OK;
@@ -2895,14 +3097,13 @@ int lbm_sweep_create(const lbm_mix_params* params, int n, lbm_sweep** out) {
 
 void lbm_sweep_destroy(lbm_sweep* s) {
   if (!s) return;
-  for (int i = 0; i < s->n; ++i) {
-    if (s->exec) drop_graph(s, i);
+  if (s->stream) cudaStreamSynchronize(s->stream);
+  for (int i = 0; i < s->n; ++i)
     if (s->h) lbm_mix_destroy(s->h[i]);
-  }
   free(s->h);
-  free(s->exec);
-  free(s->exec_K);
-  free(s->key);
+  cudaFree(s->resid);
+  if (s->h_resid) cudaFreeHost(s->h_resid);
+  if (s->stream) cudaStreamDestroy(s->stream);
   delete s;
 }
 
@@ -2918,11 +3119,9 @@ int lbm_sweep_init(lbm_sweep* s) {
 int lbm_sweep_step(lbm_sweep* s, long nsteps) {
   if (!s) return set_err(LBM_EINVAL, "sweep is NULL");
   if (nsteps < 0) return set_err(LBM_EINVAL, "nsteps < 0");
-  for (int i = 0; i < s->n; ++i) {
-    int st = lbm_mix_step(s->h[i], nsteps);
-    if (st) return st;
-  }
-  for (int i = 0; i < s->n; ++i) CK(cudaStreamSynchronize(s->h[i]->stream));
+  int st = batch_steps(s, s->h, s->n, nsteps);
+  if (st) return st;
+  CK(cudaStreamSynchronize(s->stream));
   return LBM_OK;
 }
 
@@ -2937,15 +3136,16 @@ int lbm_sweep_run_to_steady(lbm_sweep* s, double tol, long max_steps, long check
   double* R = (double*)malloc(n * sizeof(double));
   int* status = (int*)malloc(n * sizeof(int));
   int* act = (int*)malloc(n * sizeof(int));
-  if (!taken || !R || !status || !act) {
-    free(taken), free(R), free(status), free(act);
+  lbm_mix** hs = (lbm_mix**)malloc(n * sizeof(lbm_mix*));
+  if (!taken || !R || !status || !act || !hs) {
+    free(taken), free(R), free(status), free(act), free(hs);
     return set_err(LBM_ENOMEM, "host allocation failed");
   }
   int na = 0;
   for (int i = 0; i < n; ++i) {
     R[i] = INFINITY;
     status[i] = LBM_ENOTCONVERGED;
-    // one diagnostic record per graph: the captured pattern repeats
+    // one diagnostic record per check block
     s->h[i]->p.diag_every = (int)check_every;
     if (max_steps > 0) act[na++] = i;
   }
@@ -2954,45 +3154,21 @@ int lbm_sweep_run_to_steady(lbm_sweep* s, double tol, long max_steps, long check
   if (!autotune && s->policy < 0) st = apply_policy(s, 0);
   while (na > 0 && st == LBM_OK) {
     if (trial >= 0 && (st = apply_policy(s, trial))) break;
-    // every active instance advances k steps: a replayed graph when k is
-    // the captured length, plain launches for a shorter last block
+    // every active instance advances k steps
     const long left = max_steps - taken[act[0]];
     const long k = check_every < left ? check_every : left;
-    // (re)capture where no graph exists or the state moved away from the one
-    // it was captured from (odd step counts, state uploads, schedule changes,
-    // re-referencing through the borrowed handle)
-    for (int a = 0; a < na && !st; ++a)
-      if (k == check_every && !graph_valid(s, act[a], k)) st = capture_steps(s, act[a], k);
-    if (st) break;
+    for (int a = 0; a < na; ++a) hs[a] = s->h[act[a]];
     const double t0 = now_ms();
-    for (int a = 0; a < na && !st; ++a) {
-      lbm_mix* h = s->h[act[a]];
-      if (k == check_every) {
-        cudaError_t e = cudaGraphLaunch(s->exec[act[a]], h->stream);
-        if (e != cudaSuccess) st = set_err(LBM_ECUDA, "graph launch: %s", cudaGetErrorString(e));
-        h->steps += k;
-      } else {
-        st = lbm_mix_step(h, k);
-      }
-      if (!st) st = launch_residual(h, k);
-    }
-    if (st) break;
+    if ((st = batch_steps(s, hs, na, k)) || (st = batch_residuals(s, hs, na, k))) break;
     int nb = 0;
     for (int a = 0; a < na; ++a) {
       const int i = act[a];
-      lbm_mix* h = s->h[i];
-      cudaError_t e = cudaStreamSynchronize(h->stream);
-      if (e != cudaSuccess) {
-        st = set_err(LBM_ECUDA, "instance %d: %s", i, cudaGetErrorString(e));
-        break;
-      }
       taken[i] += k;
-      R[i] = h->h_pinned[0];
+      R[i] = s->h_resid[a];
       if (isnan(R[i])) status[i] = LBM_ENONFINITE;
       else if (R[i] <= tol) status[i] = LBM_OK;
       else if (taken[i] < max_steps) act[nb++] = i;
     }
-    if (st) break;
     if (trial >= 0) {
       s->round_ms[trial] = now_ms() - t0;
       if (++trial == LBM_SWEEP_NPOLICY) {
@@ -3010,7 +3186,7 @@ int lbm_sweep_run_to_steady(lbm_sweep* s, double tol, long max_steps, long check
     if (residual_out) residual_out[i] = R[i];
     if (status_out) status_out[i] = status[i];
   }
-  free(taken), free(R), free(status), free(act);
+  free(taken), free(R), free(status), free(act), free(hs);
   return st;
 }
 

@@ -28,9 +28,9 @@
 // formed where the wall node's populations are still in registers.
 //
 // Sums over a column's rows (diagnostics, and the ends' density correction)
-// are taken by eight lanes in row order, compensated in FP32, then added as
-// error-free pairs, in an order that depends on N alone: neither the tile
-// width, nor k, nor the other channels of a batch change a bit of the result.
+// are taken by column_sum8, in an order that depends on N alone: neither the
+// tile width, nor k, nor the other channels of a batch change a bit of the
+// result.
 
 constexpr int TILE_TAUQ = 64;      // threads of the 1/tau_q role
 constexpr int TILE_WALL = 64;      // threads of the wall-row role
@@ -38,11 +38,10 @@ constexpr int TILE_INNER = 512;    // most threads of the inner-row role
 constexpr int TILE_THREADS = TILE_INNER + TILE_WALL + TILE_TAUQ;
 constexpr int TILE_KMAX = 15;      // most steps of one launch
 constexpr int TILE_SMEM_MAX = 227 * 1024 - 1024;
-constexpr int TILE_BATCH = 40;     // channels of one batched launch
 
 // One channel's share of a launch.
 struct TileInst {
-  Lat L;
+  LatCore L;
   const float* fin;      // deviations of the first step's input (strip layout)
   float* fout;           // deviations after step k
   const float* refrho;
@@ -72,44 +71,13 @@ __host__ __device__ inline size_t tile_smem(int N, int cols) {
          sizeof(float) * 20 + sizeof(float4) * PSI_SEGMENTS;
 }
 
-// Sum over the N values v[2 j] (one component of a pair column) by eight
-// neighbouring lanes (sub = lane & 7, every lane of the warp here): each
-// takes every eighth row in order, compensated, then three error-free
-// additions.  Every lane of the eight gets the same (sum, error) pair.
-__device__ __forceinline__ float2 column_sum8(const float* v, int N, int sub) {
-  KahanF a;
-  for (int j = sub; j < N; j += 8) a.add(v[2 * j]);
-  float hi = a.s, lo = -a.c;
-#pragma unroll
-  for (int o = 1; o < 8; o <<= 1) {
-    const float h2 = __shfl_xor_sync(0xffffffffu, hi, o);
-    const float l2 = __shfl_xor_sync(0xffffffffu, lo, o);
-    const float2 s = two_sum(hi, h2);
-    lo = __fadd_rn(__fadd_rn(lo, l2), s.y);
-    hi = s.x;
-  }
-  return make_float2(hi, lo);
-}
-__device__ __forceinline__ double pair_value(float2 v) { return (double)v.x + (double)v.y; }
-
-// N ref + (sum of deviations) as a float pair whose low part is cut at 2^-48
-// of the high one, so that its FP64 value splits into the same pair again: a
-// launch that starts from the stored FP64 sums continues bit for bit.
-__device__ __forceinline__ float2 column_total(int N, float ref, float2 dev) {
-  const float n = (float)N, p = __fmul_rn(n, ref), pl = fmaf(n, ref, -p);
-  float2 s = two_sum(p, dev.x);
-  s = quick_two_sum(s.x, __fadd_rn(s.y, __fadd_rn(pl, dev.y)));
-  const float grid = __fmul_rn(s.x, 0x1p-24f);
-  return make_float2(s.x, __fsub_rn(__fadd_rn(s.y, grid), grid));
-}
-
 // Pre-collision deviations of the tile node whose nine pairs start at f
 // (column x, S rows of pairs from one column to the next): the arithmetic of
 // pull_node.  E: kappa_in[2], kappa_out[2] and the ghost reference offsets of
 // load_ends; inl, outl: the neighbour column is the inlet, outlet ghost.
 // wall: -1 inner row, 0 bottom, 1 top (the same in all lanes of a warp but
 // for the mix of 0 and 1); r: the wall's.
-__device__ __forceinline__ void pull_tile(const float2* f, int S9, const Lat& L, const float* E,
+__device__ __forceinline__ void pull_tile(const float2* f, int S9, const LatCore& L, const float* E,
                                           float2 dl, float2 dr, bool inl, bool outl, int wall,
                                           float2 r, float2 g[9]) {
   // population i of the node at f + off, streamed from the column to its left
@@ -181,7 +149,7 @@ __device__ __forceinline__ void pull_tile(const float2* f, int S9, const Lat& L,
 // r of a wall node from its post-collision deviations g(0) .. g(8): the sums
 // of dbb_r.
 template <typename G>
-__device__ __forceinline__ float2 slip_tile(const Lat& L, float2 rb, float cm, G&& g) {
+__device__ __forceinline__ float2 slip_tile(const LatCore& L, float2 rb, float cm, G&& g) {
   float2 acc = f2(0.0f);
 #pragma unroll
   for (int i = 0; i < 9; ++i) acc = add2(acc, g(i));
@@ -198,7 +166,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 1)
   if (NI > 1)
     while ((int)blockIdx.x >= B.block0[ii + 1]) ++ii;
   const TileInst& I = B.inst[ii];
-  const Lat& L = I.L;
+  const LatCore& L = I.L;
   const int b = (int)blockIdx.x - B.block0[ii], k = B.k;
   const int N = L.N, Nx = L.Nx, S = tile_stride(N), S9 = 9 * S;
   const int T = (int)blockDim.x - TILE_WALL - TILE_TAUQ, tid = threadIdx.x;
@@ -378,7 +346,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 1)
         // still to be updated at the next step
         const int cf = x1 - xl;
         if (need && cf >= t + 1 && cf < C - t - 1) {  // warp-uniform
-          const float2 v = column_sum8((const float*)(sd + c * S) + sp, N, lane & 7);
+          const float2 v = column_sum8(N, lane & 7, [&](int r) { return sp ? sd[c * S + r].y : sd[c * S + r].x; });
           const float2 cs = column_total(N, sp ? RB[c].y : RB[c].x, v);
           const float2 cs2 = make_float2(__shfl_down_sync(0xffffffffu, cs.x, 16),
                                          __shfl_down_sync(0xffffffffu, cs.y, 16));
@@ -400,7 +368,8 @@ __global__ void __launch_bounds__(TILE_THREADS, 1)
       for (int it = tid; it < 32 * own; it += blockDim.x) {
         const int c = k + (it >> 5), q = (it >> 3) & 3;
         const float2* v = (q < 2 ? sd : mxs) + c * S;
-        const float2 s = column_sum8((const float*)v + (q & 1), N, it & 7);
+        const float2 s =
+            column_sum8(N, it & 7, [&](int r) { return (q & 1) ? v[r].y : v[r].x; });
         if ((it & 7) == 0) {
           const int x = xs + (it >> 5);
           if (diag) I.hist[((size_t)rec * 4 + q) * Nx + x] = s;
@@ -429,7 +398,9 @@ __global__ void __launch_bounds__(TILE_THREADS, 1)
 // flows and the total masses, the formulas and reductions of
 // column_epilogue.  The last block to finish advances the record counter.
 struct RecInst {
-  Lat L;
+  int N, Nx, x_periodic, light;
+  float s[2];
+  double C_in, C_out;
   const float2* hist;
   const float* refrho;
   double* diag;
@@ -448,8 +419,7 @@ __global__ void __launch_bounds__(256) lbm_records_kernel(const __grid_constant_
   __shared__ double wsum[8][6], wmin[8];
   __shared__ int wimin[8];
   pdl_wait();
-  const RecInst& I = B.inst[NI > 1 ? blockIdx.y : 0];
-  const Lat& L = I.L;
+  const RecInst &I = B.inst[NI > 1 ? blockIdx.y : 0], &L = I;
   const int r = blockIdx.x, nrec = I.nrec, tid = threadIdx.x, Nx = L.Nx;
   if (r >= nrec) return;
   const unsigned long long cnt0 = *(volatile unsigned long long*)I.diag_count;
@@ -457,7 +427,7 @@ __global__ void __launch_bounds__(256) lbm_records_kernel(const __grid_constant_
   double vmin = INFINITY, sm[6] = {0, 0, 0, 0, 0, 0};
   int imin = 0x7fffffff;
   for (int x = tid; x < Nx; x += 256) {
-    if (!interior(L, x)) {
+    if (!L.x_periodic && (x < 1 || x > Nx - 2)) {
       if (r == nrec - 1) I.clprof[x] = x == 0 ? L.C_in : L.C_out;
       continue;
     }

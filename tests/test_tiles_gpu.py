@@ -1,12 +1,12 @@
 """Several steps per launch (lbm_tile_kernel: tiles of whole columns with
 halos in shared memory), the default of small FP32 channels.
 
-Against the step kernel (a row count set by the caller) only the order of the
-column sums behind the ends' density correction differs, so the two agree to
-FP32 rounding noise: 1e-6 of the densities, 1e-5 of the largest velocity, the
-bounds the schedules of the step kernel are held to.  Against itself, split
-over calls in any way, a run is the same bit for bit: neither the steps per
-launch nor the launch boundaries enter the arithmetic."""
+Against the step kernel (a row count set by the caller) the densities are held
+to 1e-6 and the velocities to 1e-5 of their largest, the bounds the schedules
+of the step kernel are held to; and since every schedule adds the columns
+behind the ends' density correction in one order, the populations are the same
+bits under all of them, however a run is split over calls and whether a channel
+runs alone or in a sweep."""
 import numpy as np
 import pytest
 
@@ -123,3 +123,44 @@ def test_tuning_keeps_the_default_where_it_is_fastest():
     ref.step(50)
     assert np.array_equal(g.get_post_state_f64(), ref.get_post_state_f64())
     assert g.tune_rows([8, 16], steps=3) in (8, 16)
+
+
+# column counts around the strip edges of the end columns: N_x - 2 and N_x - 3
+# in one strip of 32 columns or in two (N_x = 98), both ends in one strip
+@pytest.mark.parametrize("N,Nx", [(20, 100), (33, 98), (9, 97), (64, 99), (130, 66), (12, 20)])
+@pytest.mark.parametrize("extra", [dict(), dict(wall=binding.LBM_WALL_BSR, C_l_out=0.4)])
+def test_populations_are_the_same_bits_under_every_schedule(N, Nx, extra):
+    p = workloads.preset("heli_argon_320x16", N=N, N_x=Nx, theta=1.3, Kn_out=0.3, **extra)
+    alpha = workloads.random_accommodation(Nx, seed=1, spread=0.2)
+    states = []
+    for rows, diag_every in ((0, 1), (0, 7), (8, 1), (8, 100), (24, 7), (64, 3)):
+        g = binding.LbmMix(diag_every=diag_every, **p)
+        g.set_rows_per_block(rows)
+        g.set_accommodation_field(alpha)
+        g.init()
+        g.step(30)
+        states.append(g.get_post_state_f64()[..., 1:-1])
+    for f in states[1:]:
+        assert np.array_equal(f, states[0])
+
+
+@pytest.mark.parametrize("count,N,Nx", [(3, 20, 700), (60, 20, 300), (24, 64, 1000),
+                                        (5, 130, 900)])
+def test_sweeps_take_the_steps_of_lone_channels(count, N, Nx):
+    """Few and many channels, small and tall ones: tiles or the batched step
+    kernel, the populations are those of each channel on its own."""
+    params = [workloads.preset("heli_argon_320x16", N=N, N_x=Nx + q % 3, theta=1.2 + 0.01 * q,
+                               Kn_out=0.3) for q in range(count)]
+    sw = binding.LbmSweep(params)
+    sw.init()
+    sw.step(7)
+    sw.run_to_steady(1e-14, 20, 10)
+    for q in (0, 1, count - 1):
+        g = binding.LbmMix(**params[q])
+        g.init()
+        g.step(27)
+        assert sw.instance(q).steps == 27
+        assert np.array_equal(sw.instance(q).get_post_state_f64()[..., 1:-1],
+                              g.get_post_state_f64()[..., 1:-1]), q
+        a, b = sw.instance(q).separation(), g.separation()
+        assert abs(a["CL"] - b["CL"]) < 1e-9 and a["x_min"] == b["x_min"]
