@@ -11,7 +11,8 @@ SRC = os.path.join(HERE, "csrc", "lbm_mix.cu")
 SRCS = [SRC, os.path.join(HERE, "csrc", "lbm_adjoint.cu")]
 HDR = os.path.join(ROOT, "include", "lbm_mix.h")
 INTERNAL_HDR = os.path.join(HERE, "csrc", "lbm_internal.h")
-DEVICE_HDRS = [os.path.join(HERE, "csrc", n) for n in ("lbm_tile.cuh", "lbm_node16.cuh", "lbm_psi_table.cuh")]
+DEVICE_HDRS = [os.path.join(HERE, "csrc", n) for n in (
+    "lbm_tile.cuh", "lbm_node16.cuh", "lbm_psi_table.cuh", "lbm_psi64_table.cuh")]
 LIB = os.path.join(HERE, "liblbm_mix.so")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-lineinfo",

@@ -47,6 +47,8 @@
 
 namespace {
 
+#include "lbm_psi64_table.cuh"
+
 // Programmatic dependent launch of the per-step kernel sequences: each
 // kernel lets the next one in its stream launch once all of its own CTAs
 // run (launch_dependents), and waits for the previous one's completion and
@@ -81,14 +83,17 @@ __device__ __forceinline__ double macc(double acc, double c, double x) {
 struct AL {
   int N, Nx, x_periodic, light;
   double s[2], mh[2], cw[2][3];  // rest weights w_i alpha_si: rest, axis, diagonal
-  double c_lam, c_xl[2], c_ts, c_td, om_e, om_eps, c_m0, H;
-  double inv_c_lam, inv_c_xl[2];  // reciprocals (multiplications replace FP64 divisions)
+  double c_lam, c_xl[2], c_ts, c_td, c_m0, H;
+  double we, wp;  // 1/(36 tau_e), 1/(36 tau_eps): relaxation over |M_k|^2
+  double be[2], bp[2];  // 2s - 4, 4 - 3s: constants of the equilibria of e, eps
+  // constants that replace divisions: 1/c_lam, s/c_xl, c_xl/s
+  double inv_c_lam, s_inv_c_xl[2], c_xl_s[2];
   double rho_in[2], rho_out[2], C_in, C_out, theta;
 };
 
 // ------------------------------------------------ special functions (FP64)
-// E_1 = E_i of Eq. psi in FP64, the FP64 pipe being the bound of the adjoint
-// kernels (six E_1 per node per step).  0 < x <= 1: the convergent series
+// E_1 = E_i of Eq. psi in FP64, for the arguments that the tables of psi
+// (below) leave out.  0 < x <= 1: the convergent series
 // (Abramowitz & Stegun 5.1.11) with a fixed number of terms (remainder
 // below 1e-20) by Horner's rule; 1 < x <= 32: R(x) = x e^x E_1(x), smooth
 // and between 0.59 and 0.97, as a Chebyshev series on [1,2], [2,4], [4,8],
@@ -279,10 +284,8 @@ __device__ double e1d(double x) {
 struct Psi3 {
   double v, d1, d2;
 };
-template <bool D2 = false>
-__device__ __forceinline__ Psi3 psid(double a) {
+__device__ __noinline__ Psi3 psid_general(double a) {
   Psi3 p;
-  p.d2 = 0.0;
   if (!(a > 0.0)) {
     p.v = 0.0;
     p.d1 = 2.0;
@@ -294,13 +297,44 @@ __device__ __forceinline__ Psi3 psid(double a) {
     const double R = e1_scaled(a);
     p.v = fma(ea, (a - 1.0) - a * R, 1.0);
     p.d1 = 2.0 * ea * (1.0 - R);
-    if (D2) p.d2 = -2.0 * ea * R / a;
+    p.d2 = -2.0 * ea * R / a;
     return p;
   }
   const double e1 = e1d(a);
   p.v = 1.0 + (a - 1.0) * ea - a * a * e1;
   p.d1 = 2.0 * ea - 2.0 * a * e1;
-  if (D2) p.d2 = -2.0 * e1;
+  p.d2 = -2.0 * e1;
+  return p;
+}
+// The same from the polynomials of lbm_psi64_table.cuh for 2^-10 <= a < 64: 8
+// FP64 operations a function where E_1 and exp took 80 together, on a pipe that
+// issues one warp instruction in 64 cycles per sub-partition (six psi a node
+// were over half of the forward step).  Relative error of psi below 2.1e-16,
+// absolute error of psi' 2.3e-16.  D1, D2: the derivatives wanted.
+template <bool D1 = true, bool D2 = false>
+__device__ __forceinline__ Psi3 psid(double a) {
+  const int hi = __double2hiint(a);
+  if (!(a >= 0x1p-10 && a < 64.0)) return psid_general(a);
+  const double2* q = reinterpret_cast<const double2*>(
+      kPsi64[(hi >> 15) - ((1023 + kPsi64Octave0) << 5)]);
+  const double u = a - __hiloint2double((hi & ~0x7fff) | 0x4000, 0);
+  double t[28];
+#pragma unroll
+  for (int k = 0; k < 14; ++k) {
+    const double2 w = __ldg(q + k);
+    t[2 * k] = w.x;
+    t[2 * k + 1] = w.y;
+  }
+  Psi3 p;
+  p.v = t[24];
+  p.d1 = t[25];
+  p.d2 = t[26];
+#pragma unroll
+  for (int k = 7; k >= 0; --k) {
+    p.v = fma(p.v, u, t[3 * k]);
+    if (D1) p.d1 = fma(p.d1, u, t[3 * k + 1]);
+    if (D2) p.d2 = fma(p.d2, u, t[3 * k + 2]);
+  }
   return p;
 }
 
@@ -334,13 +368,14 @@ __host__ __device__ inline size_t cols_width(int Nx) { return 18 * (size_t)Nx + 
 // Source value of population i of species sp at (xs, js): the stored state,
 // or the virtual ghost column at an end (Eq. rho1, all nine extrapolated and
 // scaled by Eq. rho2's kappa).
-__device__ double src(const AL& L, const double* f, const double* kap, int sp, int i, int js,
+__device__ __forceinline__ double src(const AL& L, const double* f, const double* kap, int sp, int i, int js,
                       int xs) {
   if (!L.x_periodic) {
-    if (xs == 0) return kap[sp] * (2.0 * f[fidx(L, sp, i, js, 1)] - f[fidx(L, sp, i, js, 2)]);
+    if (xs == 0)
+      return __dmul_rn(kap[sp], fma(2.0, f[fidx(L, sp, i, js, 1)], -f[fidx(L, sp, i, js, 2)]));
     if (xs == L.Nx - 1)
-      return kap[2 + sp] *
-             (2.0 * f[fidx(L, sp, i, js, L.Nx - 2)] - f[fidx(L, sp, i, js, L.Nx - 3)]);
+      return __dmul_rn(kap[2 + sp], fma(2.0, f[fidx(L, sp, i, js, L.Nx - 2)],
+                                        -f[fidx(L, sp, i, js, L.Nx - 3)]));
   }
   return f[fidx(L, sp, i, js, wrapx(L, xs))];
 }
@@ -348,9 +383,8 @@ __device__ double src(const AL& L, const double* f, const double* kap, int sp, i
 // f_i(x) = f'_i(x - c_i) with diffuse bounce-back at rows 0 and N-1: the
 // unknowns take (1 - r) of the opposite outgoing population plus r times the
 // wall equilibrium with zero normal species flux, 6 w_i (sum of outgoing).
-__device__ void pull(const AL& L, const double* f, const double* r2, const double* kap, int x,
-                     int j, double g[2][9]) {
-  const double rb = r2[x], rt = r2[L.Nx + x];
+__device__ __forceinline__ void pull(const AL& L, const double* f, double rb, double rt,
+                                     const double* kap, int x, int j, double g[2][9]) {
   #pragma unroll
   for (int sp = 0; sp < 2; ++sp) {
     double* q = g[sp];
@@ -361,9 +395,9 @@ __device__ void pull(const AL& L, const double* f, const double* r2, const doubl
       const double o4 = f[fidx(L, sp, 4, j, x)], o7 = f[fidx(L, sp, 7, j, x)],
                    o8 = f[fidx(L, sp, 8, j, x)];
       const double S = o4 + o7 + o8;
-      q[2] = (1.0 - rb) * o4 + rb * (2.0 / 3.0) * S;
-      q[5] = (1.0 - rb) * o7 + rb * S / 6.0;
-      q[6] = (1.0 - rb) * o8 + rb * S / 6.0;
+      q[2] = fma(rb, fma(2.0 / 3.0, S, -o4), o4);
+      q[5] = fma(rb, fma(1.0 / 6.0, S, -o7), o7);
+      q[6] = fma(rb, fma(1.0 / 6.0, S, -o8), o8);
     } else {
       q[2] = f[fidx(L, sp, 2, j - 1, x)];
       q[5] = src(L, f, kap, sp, 5, j - 1, x - 1);
@@ -373,9 +407,9 @@ __device__ void pull(const AL& L, const double* f, const double* r2, const doubl
       const double o2 = f[fidx(L, sp, 2, j, x)], o5 = f[fidx(L, sp, 5, j, x)],
                    o6 = f[fidx(L, sp, 6, j, x)];
       const double S = o2 + o5 + o6;
-      q[4] = (1.0 - rt) * o2 + rt * (2.0 / 3.0) * S;
-      q[7] = (1.0 - rt) * o5 + rt * S / 6.0;
-      q[8] = (1.0 - rt) * o6 + rt * S / 6.0;
+      q[4] = fma(rt, fma(2.0 / 3.0, S, -o2), o2);
+      q[7] = fma(rt, fma(1.0 / 6.0, S, -o5), o5);
+      q[8] = fma(rt, fma(1.0 / 6.0, S, -o6), o6);
     } else {
       q[4] = f[fidx(L, sp, 4, j + 1, x)];
       q[7] = src(L, f, kap, sp, 7, j + 1, x + 1);
@@ -387,11 +421,11 @@ __device__ void pull(const AL& L, const double* f, const double* r2, const doubl
 // ------------------------------------------------ node collision (FP64)
 // Forward intermediates of one node, kept for the reverse pass.
 struct NodeFwd {
-  double rho[2], jx[2], jy[2], rho_t, ux, uy, n, mx;
-  double inv_rho[2], inv_rt, inv_n, rs_mx, rs_xle[2];  // 1/rho_s, 1/rho, 1/n, m_x^-1/2, xle^-1/2
+  double m[2][9];                     // moments M g; rho_s, j_x, j_y are rows 0, 3, 5
+  double rho_t, ux, uy, n, mx;
+  double inv_rt, inv_n, rs_mx, rs_xle[2];  // 1/rho, 1/n, m_x^-1/2, xle^-1/2
   double lam, Pm, dPm, tsm, om_s;     // mixture mean free path, Psi, dPsi/dlam, tau_s - 1/2, 1/tau_s
-  double lams[2], Ps[2], dPs[2], xle[2], br, d, om_d;
-  double m[2][9], meq[2][9];
+  double Ps[2], dPs[2], xle[2], br, d, inv_d, om_d;  // inv_d = 1/(d/2 + c_td)
 };
 
 // 1 / |M_k|^2, the diagonal of (M M^T)^-1.
@@ -442,180 +476,216 @@ __device__ __forceinline__ void mrt_tr(const double d[9], double o[9]) {
   o[8] = Q + sm;
 }
 
-// Psi(y) = (psi(y/lambda) + psi((H-y)/lambda)) / 2 and dPsi/dlambda, from
+// Psi(y) = (psi(y/lambda) + psi((H-y)/lambda)) / 2 and (D1) dPsi/dlambda, from
 // 1/lambda.
+template <bool D1>
 __device__ __forceinline__ double half_psi(double y, double H, double inv_lam, double* dlam) {
-  const Psi3 a = psid(y * inv_lam), b = psid((H - y) * inv_lam);
-  *dlam = -0.5 * (a.d1 * y + b.d1 * (H - y)) * inv_lam * inv_lam;
+  const double y2 = H - y;
+  const Psi3 a = psid<D1>(__dmul_rn(y, inv_lam)),
+             b = psid<D1>(__dmul_rn(y2, inv_lam));
+  if (D1) *dlam = fma(a.d1, y, b.d1 * y2) * (-0.5 * inv_lam * inv_lam);
   return 0.5 * (a.v + b.v);
 }
 
-// f_out = Collide(g): moments, relaxation rates (1/tau_s of Eq. taos,
-// 1/tau_d of Eq. EQFrsp, 1/tau_q from the wall), MRT relaxation
-// f' = g - M^{-1} S (m - m^eq).
-// psi_in (nullable): the node's Psi and dPsi/dlambda of the mixture and of
-// both species as an earlier node_forward stored them through psi_out
-// (nullable), six values `plane` doubles apart; read instead of evaluated.
-__device__ void node_forward(const AL& L, const double g[2][9], double y, double omq,
-                             NodeFwd& F, double fo[2][9], const double* psi_in = nullptr,
-                             double* psi_out = nullptr, size_t plane = 0) {
-  #pragma unroll
-  for (int sp = 0; sp < 2; ++sp) {
-    mrt_fwd(g[sp], F.m[sp]);  // rho_s, j_x, j_y are rows 0, 3, 5
-    F.rho[sp] = F.m[sp][0];
-    F.jx[sp] = F.m[sp][3];
-    F.jy[sp] = F.m[sp][5];
-  }
-  F.rho_t = F.rho[0] + F.rho[1];
+// Moments of g, mixture quantities and relaxation rates (1/tau_s of Eq. taos,
+// 1/tau_d of Eq. EQFrsp).  KEEP: also dPsi/dlambda, all stored through psi;
+// READ: Psi and dPsi/dlambda of the mixture and of both species are read from
+// psi as an earlier call stored them (six values `plane` doubles apart).
+template <bool KEEP, bool READ, typename P>
+__device__ __forceinline__ void node_rates(const AL& L, const double g[2][9], double y, NodeFwd& F,
+                                           P* psi, size_t plane) {
+#pragma unroll
+  for (int sp = 0; sp < 2; ++sp) mrt_fwd(g[sp], F.m[sp]);
+  const double ra = F.m[0][0], rb = F.m[1][0];
+  F.rho_t = ra + rb;
   F.inv_rt = 1.0 / F.rho_t;
-  F.ux = (F.jx[0] + F.jx[1]) * F.inv_rt;
-  F.uy = (F.jy[0] + F.jy[1]) * F.inv_rt;
-  F.n = L.s[0] * F.rho[0] + L.s[1] * F.rho[1];
+  F.ux = (F.m[0][3] + F.m[1][3]) * F.inv_rt;
+  F.uy = (F.m[0][5] + F.m[1][5]) * F.inv_rt;
+  F.n = fma(L.s[0], ra, L.s[1] * rb);
   F.inv_n = 1.0 / F.n;
   F.mx = F.rho_t * F.inv_n;
   F.rs_mx = rsqrt(F.mx);
   F.lam = L.c_lam * F.inv_n * F.rs_mx;
-  if (psi_in) {
-    F.Pm = psi_in[0];
-    F.dPm = psi_in[plane];
+  if constexpr (READ) {
+    F.Pm = psi[0];
+    F.dPm = psi[plane];
   } else {
-    F.Pm = half_psi(y, L.H, F.n * F.mx * F.rs_mx * L.inv_c_lam, &F.dPm);
+    F.Pm = half_psi<KEEP>(y, L.H, F.n * F.mx * F.rs_mx * L.inv_c_lam, &F.dPm);
   }
-  F.tsm = F.lam * F.Pm * L.c_ts * F.rs_mx;
-  F.om_s = 1.0 / (0.5 + F.tsm);
+  const double h = F.lam * F.Pm * L.c_ts;
+  F.tsm = h * F.rs_mx;
+  F.om_s = 1.0 / fma(h, F.rs_mx, 0.5);
   F.br = 0.0;
-  #pragma unroll
+#pragma unroll
   for (int sp = 0; sp < 2; ++sp) {
-    F.inv_rho[sp] = 1.0 / F.rho[sp];
-    F.lams[sp] = L.c_xl[sp] / L.s[sp] * F.inv_rho[sp];
-    if (psi_in) {
-      F.Ps[sp] = psi_in[(2 + 2 * sp) * plane];
-      F.dPs[sp] = psi_in[(3 + 2 * sp) * plane];
+    if constexpr (READ) {
+      F.Ps[sp] = psi[(2 + 2 * sp) * plane];
+      F.dPs[sp] = psi[(3 + 2 * sp) * plane];
     } else {
-      F.Ps[sp] = half_psi(y, L.H, L.s[sp] * F.rho[sp] * L.inv_c_xl[sp], &F.dPs[sp]);
+      F.Ps[sp] = half_psi<KEEP>(y, L.H, F.m[sp][0] * L.s_inv_c_xl[sp], &F.dPs[sp]);
     }
     F.xle[sp] = L.c_xl[sp] * F.Ps[sp] * F.inv_n;
     F.rs_xle[sp] = rsqrt(F.xle[sp]);
     F.br += F.rs_xle[sp];
   }
-  if (psi_out) {
-    psi_out[0] = F.Pm;
-    psi_out[plane] = F.dPm;
+  if constexpr (KEEP) {
+    psi[0] = F.Pm;
+    psi[plane] = F.dPm;
 #pragma unroll
     for (int sp = 0; sp < 2; ++sp) {
-      psi_out[(2 + 2 * sp) * plane] = F.Ps[sp];
-      psi_out[(3 + 2 * sp) * plane] = F.dPs[sp];
+      psi[(2 + 2 * sp) * plane] = F.Ps[sp];
+      psi[(3 + 2 * sp) * plane] = F.dPs[sp];
     }
   }
   F.d = F.mx * F.br * F.br;
-  F.om_d = F.d / (0.5 * F.d + L.c_td);
-  const double u2 = F.ux * F.ux + F.uy * F.uy;
-  const double S[9] = {0.0, L.om_e, L.om_eps, F.om_d, omq, F.om_d, omq, F.om_s, F.om_s};
-  #pragma unroll
+  F.inv_d = 1.0 / fma(0.5, F.d, L.c_td);
+  F.om_d = F.d * F.inv_d;
+}
+
+// Products and sums from here on are written with explicit roundings where a
+// product feeds a sum: the kernels that inline them (with and without stored
+// Psi, with and without the gathered adjoint) then give the same bits, and the
+// gradient does not depend on the checkpoints.
+
+// What the equilibria share: 3u^2 (e, eps), ux^2 - uy^2 (p_xx), ux uy (p_xy).
+struct Equil {
+  double u3, uxx, uxy;
+};
+__device__ __forceinline__ Equil equil(const NodeFwd& F) {
+  const double uy2 = F.uy * F.uy;
+  return Equil{__dmul_rn(3.0, fma(F.ux, F.ux, uy2)), fma(F.ux, F.ux, -uy2), F.ux * F.uy};
+}
+
+// f_out = Collide(g): f' = g - M^T dl, dl_k = S_k (m_k - meq_k) / |M_k|^2, meq =
+// rho_s (1, -4 + 2s + 3u^2, 4 - 3s - 3u^2, ux, -ux, uy, -uy, ux^2 - uy^2, ux uy).
+template <bool KEEP>
+__device__ __forceinline__ void node_forward(const AL& L, const double g[2][9], double y,
+                                             double omq, double fo[2][9], double* psi,
+                                             size_t plane) {
+  NodeFwd F;
+  node_rates<KEEP, false>(L, g, y, F, psi, plane);
+  const Equil E = equil(F);
+  const double wd = F.om_d * inv_Mnorm(3), wq = omq * inv_Mnorm(4), ws = F.om_s * inv_Mnorm(7);
+#pragma unroll
   for (int sp = 0; sp < 2; ++sp) {
-    const double r = F.rho[sp], s = L.s[sp];
-    const double br[9] = {1.0, -4.0 + 2.0 * s + 3.0 * u2, 4.0 - 3.0 * s - 3.0 * u2, F.ux,
-                          -F.ux, F.uy, -F.uy, F.ux * F.ux - F.uy * F.uy, F.ux * F.uy};
-    double dl[9], c[9];
-    #pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      F.meq[sp][k] = r * br[k];
-      dl[k] = S[k] * (F.m[sp][k] - F.meq[sp][k]) * inv_Mnorm(k);
-    }
-    mrt_tr(dl, c);
-    #pragma unroll
-    for (int i = 0; i < 9; ++i) fo[sp][i] = g[sp][i] - c[i];
+    const double* m = F.m[sp];
+    const double r = m[0];
+    const double d1 = __dmul_rn(L.we, fma(-r, L.be[sp] + E.u3, m[1]));
+    const double d2 = __dmul_rn(L.wp, fma(-r, L.bp[sp] - E.u3, m[2]));
+    const double d3 = __dmul_rn(wd, fma(-r, F.ux, m[3])), d4 = __dmul_rn(wq, fma(r, F.ux, m[4]));
+    const double d5 = __dmul_rn(wd, fma(-r, F.uy, m[5])), d6 = __dmul_rn(wq, fma(r, F.uy, m[6]));
+    const double d7 = __dmul_rn(ws, fma(-r, E.uxx, m[7]));
+    const double d8 = __dmul_rn(ws, fma(-r, E.uxy, m[8]));
+    // g - M^T d, d_0 = 0 (see mrt_tr)
+    const double* v = g[sp];
+    double* o = fo[sp];
+    o[0] = fma(4.0, d1 - d2, v[0]);
+    const double B = fma(2.0, d2, d1), Bp = B - d7, Bm = B + d7;  // minus the axis class
+    const double xa = fma(-2.0, d4, d3), ya = fma(-2.0, d6, d5);
+    o[1] = v[1] + (Bp - xa);
+    o[3] = v[3] + (Bp + xa);
+    o[2] = v[2] + (Bm - ya);
+    o[4] = v[4] + (Bm + ya);
+    const double A = fma(2.0, d1, d2), P = A + d8, Q = A - d8;
+    const double X = d3 + d4, Y = d5 + d6, sp_ = X + Y, sm = X - Y;
+    o[5] = v[5] - (P + sp_);
+    o[7] = v[7] - (P - sp_);
+    o[6] = v[6] - (Q - sm);
+    o[8] = v[8] - (Q + sm);
   }
 }
 
 // Reverse of node_forward: from fbar (adjoint of f_out) to gbar (adjoint of
 // g), omq_bar (adjoint of 1/tau_q) and lnmu_bar (adjoint of ln mu, which
 // scales c_lam and c_xl).
-__device__ void node_reverse(const AL& L, const double g[2][9], double y, double omq,
-                             const double fbar[2][9], double gbar[2][9], double* omq_bar,
-                             double* lnmu_bar, const double* psi_in, size_t plane) {
+__device__ __forceinline__ void node_reverse(const AL& L, const double g[2][9], double y,
+                                             double omq, const double fbar[2][9],
+                                             double gbar[2][9], double* omq_bar,
+                                             double* lnmu_bar, const double* psi, size_t plane) {
   NodeFwd F;
-  double fo[2][9];
-  node_forward(L, g, y, omq, F, fo, psi_in, nullptr, plane);
-  const double S[9] = {0.0, L.om_e, L.om_eps, F.om_d, omq, F.om_d, omq, F.om_s, F.om_s};
-  double Sbar[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-  double rhob[2] = {0, 0};
+  node_rates<false, true>(L, g, y, F, psi, plane);
+  const Equil E = equil(F);
+  const double wd = F.om_d * inv_Mnorm(3), wq = omq * inv_Mnorm(4), ws = F.om_s * inv_Mnorm(7);
+  double wdb = 0, wqb = 0, wsb = 0;  // adjoints of wd, wq, ws (negative)
   double uxb = 0, uyb = 0;
-  const double u2 = F.ux * F.ux + F.uy * F.uy;
-  // adjoint of the moments m = M g; its rows 0, 3, 5 (rho_s, j_x, j_y) also
-  // collect the mixture terms below, and gbar = fbar + M^T mbar at the end
-  double mbar[2][9];
-  #pragma unroll
+  double rhob[2];
+  // q_k = S_k (M fbar)_k / |M_k|^2 is the adjoint of meq_k, and minus that of
+  // m_k; rows 0, 3, 5 of the latter also collect the mixture terms below, and
+  // gbar = fbar - M^T q at the end
+  double q[2][9];
+#pragma unroll
   for (int sp = 0; sp < 2; ++sp) {
-    const double r = F.rho[sp], s = L.s[sp];
-    // f_i = g_i - sum_k M_ki dl_k, dl_k = S_k (m_k - meq_k) / |M_k|^2
-    double Mf[9], meqbar[9];
+    const double* m = F.m[sp];
+    const double r = m[0];
+    double Mf[9];
     mrt_fwd(fbar[sp], Mf);
-    #pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      const double dlb = -Mf[k] * inv_Mnorm(k);
-      mbar[sp][k] = S[k] * dlb;
-      meqbar[k] = -S[k] * dlb;
-      Sbar[k] += (F.m[sp][k] - F.meq[sp][k]) * dlb;
-    }
-    // meq = rho_s (1, -4 + 2s + 3u^2, 4 - 3s - 3u^2, ux, -ux, uy, -uy, ux^2 - uy^2, ux uy)
-    const double br[9] = {1.0, -4.0 + 2.0 * s + 3.0 * u2, 4.0 - 3.0 * s - 3.0 * u2, F.ux,
-                          -F.ux, F.uy, -F.uy, F.ux * F.ux - F.uy * F.uy, F.ux * F.uy};
-    #pragma unroll
-    for (int k = 0; k < 9; ++k) rhob[sp] += meqbar[k] * br[k];
-    uxb += r * (6.0 * F.ux * (meqbar[1] - meqbar[2]) + meqbar[3] - meqbar[4] +
-                2.0 * F.ux * meqbar[7] + F.uy * meqbar[8]);
-    uyb += r * (6.0 * F.uy * (meqbar[1] - meqbar[2]) + meqbar[5] - meqbar[6] -
-                2.0 * F.uy * meqbar[7] + F.ux * meqbar[8]);
+    q[sp][1] = __dmul_rn(L.we, Mf[1]);
+    q[sp][2] = __dmul_rn(L.wp, Mf[2]);
+    q[sp][3] = __dmul_rn(wd, Mf[3]);
+    q[sp][4] = __dmul_rn(wq, Mf[4]);
+    q[sp][5] = __dmul_rn(wd, Mf[5]);
+    q[sp][6] = __dmul_rn(wq, Mf[6]);
+    q[sp][7] = __dmul_rn(ws, Mf[7]);
+    q[sp][8] = __dmul_rn(ws, Mf[8]);
+    wdb = fma(fma(-r, F.ux, m[3]), Mf[3], fma(fma(-r, F.uy, m[5]), Mf[5], wdb));
+    wqb = fma(fma(r, F.ux, m[4]), Mf[4], fma(fma(r, F.uy, m[6]), Mf[6], wqb));
+    wsb = fma(fma(-r, E.uxx, m[7]), Mf[7], fma(fma(-r, E.uxy, m[8]), Mf[8], wsb));
+    const double qa = q[sp][3] - q[sp][4], qb = q[sp][5] - q[sp][6];
+    double rb = q[sp][1] * (L.be[sp] + E.u3);
+    rb = fma(q[sp][2], L.bp[sp] - E.u3, rb);
+    rb = fma(qa, F.ux, rb);
+    rb = fma(qb, F.uy, rb);
+    rb = fma(q[sp][7], E.uxx, rb);
+    rhob[sp] = fma(q[sp][8], E.uxy, rb);
+    const double t = 6.0 * (q[sp][1] - q[sp][2]);
+    uxb = fma(r, fma(F.ux, fma(2.0, q[sp][7], t), fma(F.uy, q[sp][8], qa)), uxb);
+    uyb = fma(r, fma(F.uy, fma(-2.0, q[sp][7], t), fma(F.ux, q[sp][8], qb)), uyb);
   }
-  const double omdb = Sbar[3] + Sbar[5];
-  *omq_bar = Sbar[4] + Sbar[6];
-  const double omsb = Sbar[7] + Sbar[8];
-  double mxb = 0, nb = 0, lnmub = 0;
+  const double omdb = -wdb * inv_Mnorm(3);
+  *omq_bar = -wqb * inv_Mnorm(4);
+  const double omsb = -wsb * inv_Mnorm(7);
+  double nb = 0, lnmub = 0;
   // om_d = d / (d/2 + c_td); d = m_x br^2; br = sum_s xle_s^{-1/2}
-  const double den = 0.5 * F.d + L.c_td;
-  const double db = omdb * L.c_td / (den * den);
-  mxb += db * F.br * F.br;
-  const double brb = db * 2.0 * F.mx * F.br;
-  #pragma unroll
+  const double db = omdb * L.c_td * F.inv_d * F.inv_d;
+  double mxb = db * F.br * F.br;
+  const double brb = db * F.mx * F.br;  // half its adjoint
+#pragma unroll
   for (int sp = 0; sp < 2; ++sp) {
     const double rx = F.rs_xle[sp];
-    const double xleb = brb * (-0.5) * rx * rx * rx;
+    const double xleb = -brb * rx * rx * rx;
     // xle = c_xl Psi_s / n: proportional to mu through c_xl
-    const double Psb = xleb * L.c_xl[sp] * F.inv_n;
-    nb -= xleb * F.xle[sp] * F.inv_n;
-    lnmub += xleb * F.xle[sp];
-    const double lamsb = Psb * F.dPs[sp];
-    // lam_s = c_xl / (s rho_s)
-    rhob[sp] -= lamsb * F.lams[sp] * F.inv_rho[sp];
-    lnmub += lamsb * F.lams[sp];
+    const double t = __dmul_rn(xleb, F.xle[sp]);
+    nb = fma(-t, F.inv_n, nb);
+    lnmub += t;
+    // lam_s = c_xl / (s rho_s), times its adjoint
+    const double inv_rho = 1.0 / F.m[sp][0];
+    const double lamsb =
+        __dmul_rn(xleb * L.c_xl[sp] * F.inv_n * F.dPs[sp] * L.c_xl_s[sp], inv_rho);
+    rhob[sp] = fma(-lamsb, inv_rho, rhob[sp]);
+    lnmub += lamsb;
   }
   // om_s = 1 / (1/2 + tsm); tsm = lam Psi(lam) c_ts m_x^{-1/2}
   const double tsmb = -omsb * F.om_s * F.om_s;
-  const double rsm = L.c_ts * F.rs_mx;
-  const double inv_mx = F.n * F.inv_rt;
-  double lamb = tsmb * (F.Pm + F.lam * F.dPm) * rsm;
-  mxb += tsmb * F.tsm * (-0.5) * inv_mx;
-  // lam = c_lam n^{-1} m_x^{-1/2}
-  nb -= lamb * F.lam * F.inv_n;
-  mxb += lamb * F.lam * (-0.5) * inv_mx;
-  lnmub += lamb * F.lam;
+  const double half_inv_mx = 0.5 * F.n * F.inv_rt;
+  // lam = c_lam n^{-1} m_x^{-1/2}, times its adjoint
+  const double lamb =
+      __dmul_rn(tsmb * fma(F.lam, F.dPm, F.Pm) * (L.c_ts * F.rs_mx), F.lam);
+  nb = fma(-lamb, F.inv_n, nb);
+  mxb = fma(-fma(tsmb, F.tsm, lamb), half_inv_mx, mxb);
+  lnmub += lamb;
   // m_x = rho / n; n = sum s rho_s
-  double rhotb = mxb * F.inv_n;
-  nb -= mxb * F.rho_t * F.inv_n * F.inv_n;
+  nb = fma(-mxb * F.mx, F.inv_n, nb);
   // u = J / rho
-  rhotb -= (uxb * F.ux + uyb * F.uy) * F.inv_rt;
-  const double Jxb = uxb * F.inv_rt, Jyb = uyb * F.inv_rt;
-  #pragma unroll
+  const double rhotb = fma(mxb, F.inv_n, -fma(uxb, F.ux, uyb * F.uy) * F.inv_rt);
+#pragma unroll
   for (int sp = 0; sp < 2; ++sp) {
-    rhob[sp] += rhotb + nb * L.s[sp];
-    mbar[sp][0] += rhob[sp];
-    mbar[sp][3] += Jxb;
-    mbar[sp][5] += Jyb;
+    q[sp][0] = -(rhob[sp] + fma(nb, L.s[sp], rhotb));
+    q[sp][3] = fma(-uxb, F.inv_rt, q[sp][3]);
+    q[sp][5] = fma(-uyb, F.inv_rt, q[sp][5]);
     double c[9];
-    mrt_tr(mbar[sp], c);
-    #pragma unroll
-    for (int i = 0; i < 9; ++i) gbar[sp][i] = fbar[sp][i] + c[i];
+    mrt_tr(q[sp], c);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) gbar[sp][i] = fbar[sp][i] - c[i];
   }
   *lnmu_bar = lnmub;
 }
@@ -645,7 +715,7 @@ __device__ double tau_q_rho(const AL& L, double rho0, double rho1, double alpha,
   const double inv_lam = n * mx * rs * L.inv_c_lam;
   const double gg = L.c_ts * rs;
   const double a = L.H * inv_lam;
-  const Psi3 P = psid<true>(a);
+  const Psi3 P = psid<true, true>(a);
   const double tt = 0.5 * lam * P.v * gg;
   const double itt = 1.0 / tt;
   const double i16 = 0.0625 * itt;                   // 1 / (16 tt)
@@ -702,86 +772,75 @@ __device__ double dbb_r(const AL& L, const double* f, int x, int j, double alpha
 }
 
 // ------------------------------------------------------------ kernels
-// Sum of v over a block of 256 threads, in a fixed tree order (warp
-// shuffles, then the eight warp sums); every thread receives the total.
-__device__ double block_sum256(double v, double* sm /* [8] */) {
+// Sum over the warp by a butterfly: every lane gets the same value (each
+// stage adds the same two operands in every lane).
+__device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  __syncthreads();  // sm may still be read from a previous call
-  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double t = 0.0;
-#pragma unroll
-  for (int k = 0; k < 8; ++k) t += sm[k];
-  return t;
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
 }
 
-// kappa of both ends (Eq. rho2) from the column sums of columns 1, 2 and
-// N_x - 2, N_x - 3 of f; block e (of four) computes kappa[e], e = 2 end +
-// species.
-__global__ void __launch_bounds__(256) adj_kappa_kernel(AL L, const double* __restrict__ f,
-                                                        double* __restrict__ kap) {
+// The column data of a step: block (bx, w) of kColsWarps warps, columns [32
+// bx, 32 bx + 32) and wall w.  Warp 0, one thread per wall node: r and its
+// derivatives with respect to the node's species densities and the
+// accommodation coefficient (c.dr, for the reverse of the DBB rule).  Warp 1:
+// 1/tau_q of the wall's half and the derivatives of tau_q that the reverse
+// sweep multiplies by the adjoint of tau_q (c.dq); it depends on the wall
+// node's species densities alone, which the DBB rule conserves whatever r is,
+// so it pulls with r = 0 beside warp 0.  Where the block holds column 1 or N_x
+// - 2, whose pulls need kappa of that end (Eq. rho2), warps 2 and 3 sum it
+// first, one species each (both walls' blocks, the same bits; wall 0 stores
+// it).  The warps sit on the SM's four sub-partitions, whose FP64 pipes are
+// the bound of each chain; one launch instead of three.
+constexpr int kColsWarps = 4;
+__global__ void __launch_bounds__(32 * kColsWarps) adj_cols_kernel(
+    AL L, const double* __restrict__ f, const double* __restrict__ alpha, StepCols c) {
   pdl_enter();
-  __shared__ double sm[8];
-  const int t = threadIdx.x, e = blockIdx.x, sp = e & 1;
-  const int x1 = e < 2 ? 1 : L.Nx - 2, x2 = e < 2 ? 2 : L.Nx - 3;
-  double a1 = 0.0, a2 = 0.0;
-  if (!L.x_periodic) {
-    for (int j = t; j < L.N; j += blockDim.x)
+  __shared__ double kap[4];  // in_a, in_b, out_a, out_b
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int x0 = blockIdx.x * 32, x = x0 + lane, w = blockIdx.y, jw = w == 0 ? 0 : L.N - 1;
+  const bool node = x < L.Nx && interior(L, x);
+  const size_t k = (size_t)w * L.Nx + x, wn = 2 * (size_t)L.Nx;
+  const bool ends = (1 >= x0 && 1 < x0 + 32) || (L.Nx - 2 >= x0 && L.Nx - 2 < x0 + 32);
+  if (warp == 0) {
+    if (node) {
+      double drr[2], dra;
+      c.r[k] = dbb_r(L, f, x, jw, alpha[k], drr, &dra);
+      c.dr[k] = drr[0];
+      c.dr[wn + k] = drr[1];
+      c.dr[2 * wn + k] = dra;
+    } else if (x < L.Nx) {
+      c.r[k] = 0.0;
+      c.omq[k] = 1.0;
+    }
+  } else if (warp > 1) {
+    const int sp = warp - 2;
+    for (int end = 0; end < 2; ++end) {
+      const int x1 = end == 0 ? 1 : L.Nx - 2, x2 = end == 0 ? 2 : L.Nx - 3;
+      if (x1 < x0 || x1 >= x0 + 32) continue;  // warp-uniform
+      double a = 0.0;
+      for (int j = lane; j < L.N; j += 32)
 #pragma unroll
-      for (int i = 0; i < 9; ++i) {
-        a1 += f[fidx(L, sp, i, j, x1)];
-        a2 += f[fidx(L, sp, i, j, x2)];
+        for (int i = 0; i < 9; ++i)
+          a += fma(2.0, f[fidx(L, sp, i, j, x1)], -f[fidx(L, sp, i, j, x2)]);
+      const double D = warp_sum(a);
+      if (lane == 0) {
+        const double v = L.N * (end == 0 ? L.rho_in[sp] : L.rho_out[sp]) / D;
+        kap[2 * end + sp] = v;
+        if (w == 0) c.kappa[2 * end + sp] = v;
       }
+    }
   }
-  // column sums enter as 2 c(1) - c(2) (resp. N_x - 2, N_x - 3)
-  const double D = block_sum256(2.0 * a1 - a2, sm);
-  if (t == 0) {
-    const double target = e < 2 ? L.rho_in[sp] : L.rho_out[sp];
-    kap[e] = L.x_periodic ? 1.0 : L.N * target / D;
-  }
-}
-
-// r of wall w = blockIdx.y per column, and its derivatives with respect to
-// the wall node's species densities and the accommodation coefficient
-// (c.dr, for the reverse of the DBB rule).
-__global__ void adj_cols_kernel(AL L, const double* __restrict__ f, const double* __restrict__ alpha,
-                                StepCols c) {
-  pdl_enter();
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, w = blockIdx.y;
-  if (x >= L.Nx) return;
-  const size_t k = (size_t)w * L.Nx + x, wn = 2 * (size_t)L.Nx;
-  if (!interior(L, x)) {
-    c.r[k] = 0.0;
-    c.omq[k] = 1.0;
-    return;
-  }
-  double drr[2], dra;
-  c.r[k] = dbb_r(L, f, x, w == 0 ? 0 : L.N - 1, alpha[k], drr, &dra);
-  c.dr[k] = drr[0];
-  c.dr[wn + k] = drr[1];
-  c.dr[2 * wn + k] = dra;
-}
-// 1/tau_q of the half of wall w = blockIdx.y per column, and the
-// derivatives of tau_q the reverse sweep multiplies by the adjoint of tau_q
-// (c.dq).  One thread per (wall, column): the FP64 pipe takes a warp's 32
-// lanes at once, so a thread per wall node is the cheap layout.
-__global__ void adj_tauq_kernel(AL L, const double* __restrict__ f, const double* __restrict__ alpha,
-                                StepCols c) {
-  pdl_enter();
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, w = blockIdx.y;
-  if (x >= L.Nx || !interior(L, x)) return;
+  if (ends) __syncthreads();  // block-uniform
+  if (warp != 1 || !node) return;
   double g[2][9];
-  pull(L, f, c.r, c.kappa, x, w == 0 ? 0 : L.N - 1, g);
+  pull(L, f, 0.0, 0.0, kap, x, jw, g);
   double rho[2];
-  #pragma unroll
-  for (int sp = 0; sp < 2; ++sp) {
-    rho[sp] = 0;
-    #pragma unroll
-    for (int i = 0; i < 9; ++i) rho[sp] += g[sp][i];
-  }
+#pragma unroll
+  for (int sp = 0; sp < 2; ++sp)
+    rho[sp] = ((g[sp][0] + g[sp][1]) + (g[sp][2] + g[sp][3])) +
+              (((g[sp][4] + g[sp][5]) + (g[sp][6] + g[sp][7])) + g[sp][8]);
   TauqBar d;
-  const size_t k = (size_t)w * L.Nx + x, wn = 2 * (size_t)L.Nx;
   c.omq[k] = 1.0 / tau_q_rho(L, rho[0], rho[1], alpha[k], &d);
   c.dq[k] = d.rt;
   c.dq[wn + k] = d.n;
@@ -789,34 +848,32 @@ __global__ void adj_tauq_kernel(AL L, const double* __restrict__ f, const double
   c.dq[3 * wn + k] = d.lnmu;
 }
 
-// One FP64 step over all nodes: f_out = Collide(Pull(f_in)).  One warp per
-// block, block (bx, by) covers 32 columns x `rows` rows (see node_rows).
-// psi_out (nullable): [6][N][Nx] Psi values of this step for the reverse
-// sweep (see node_forward).  Registers are allocated per SM sub-partition
-// (four of 16384): at the 96 this bound leaves (a few values spill to L1)
-// each holds five warps, 20 per SM, so one row per block fits the 2560
-// warps of a 1280 x 64 channel in one wave on 152 SMs.
-__global__ void __launch_bounds__(32, 19) adj_step_kernel(AL L, const double* __restrict__ fin,
+// One FP64 step over all nodes: f_out = Collide(Pull(f_in)).  Block (bx, j):
+// one warp, 32 columns of row j.  KEEP: psi_out gets the [6][N][Nx] Psi values
+// of this step for the reverse sweep (see node_rates).  Bound by the FP64 pipe,
+// which issues a warp instruction in 64 cycles per SM sub-partition: 398 of
+// them per warp (about 920 before psi came from tables) are 52 us on a 1280 x
+// 64 channel if the 2560 warps spread evenly over 608 sub-partitions; it takes
+// 70 us (120 before), most sub-partitions getting 4 warps and some 5.  One row
+// per block leaves the spreading to the hardware; three or four warps resident
+// per sub-partition (without spills) run as fast as five.
+template <bool KEEP>
+__global__ void __launch_bounds__(32, 12) adj_step_kernel(AL L, const double* __restrict__ fin,
                                                       double* __restrict__ fout, StepCols c,
-                                                      double* __restrict__ psi_out, int rows) {
+                                                      double* __restrict__ psi_out) {
   pdl_enter();
-  const int x = blockIdx.x * 32 + threadIdx.x;
+  const int x = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y;
   if (x >= L.Nx || !interior(L, x)) return;
-  const int j0 = blockIdx.y * rows, j1 = min(L.N, j0 + rows);
   const int half = (L.N + 1) / 2;
   const size_t plane = (size_t)L.N * L.Nx;
-  for (int j = j0; j < j1; ++j) {
-    double g[2][9], fo[2][9];
-    pull(L, fin, c.r, c.kappa, x, j, g);
-    const double omq = c.omq[(j < half ? 0 : 1) * L.Nx + x];
-    NodeFwd F;
-    node_forward(L, g, j + 0.5, omq, F, fo, nullptr,
-                 psi_out ? psi_out + (size_t)j * L.Nx + x : nullptr, plane);
+  double g[2][9], fo[2][9];
+  pull(L, fin, c.r[x], c.r[L.Nx + x], c.kappa, x, j, g);
+  const double omq = c.omq[(j < half ? 0 : 1) * L.Nx + x];
+  node_forward<KEEP>(L, g, j + 0.5, omq, fo, psi_out + (KEEP ? (size_t)j * L.Nx + x : 0), plane);
+  #pragma unroll
+  for (int sp = 0; sp < 2; ++sp)
     #pragma unroll
-    for (int sp = 0; sp < 2; ++sp)
-      #pragma unroll
-      for (int i = 0; i < 9; ++i) fout[fidx(L, sp, i, j, x)] = fo[sp][i];
-  }
+    for (int i = 0; i < 9; ++i) fout[fidx(L, sp, i, j, x)] = fo[sp][i];
 }
 
 // Initial state (rest equilibrium of the linear pressure and composition
@@ -883,121 +940,21 @@ __global__ void adj_seed_kernel(AL L, int objective, int xs, double Sl, double S
     }
 }
 
-// Reverse of Collide for every node: gbar = (dCollide/dg)^T lam_t, and
-// per node the adjoints of 1/tau_q (of the node's half) and of ln mu,
-// stored per row for adj_rev_tauq_kernel to sum in row order:
-// part[j][0][x], part[j][1][x].  One warp per block, block (bx, by) covers
-// 32 columns x `rows` rows (see node_rows: every block fits on the GPU at
-// once, so the SMs share the work to within one block).
-// psi: [6][N][Nx] Psi values the forward run or the replay of this step
-// stored.  At its 200 registers an SM sub-partition holds two warps, 8 per
-// SM, so node_rows gives the 1280 x 64 channel three rows per block (0.72
-// waves).  Capped at 168 registers (three warps per sub-partition, two rows
-// per block, 40 bytes spilled to L1) it ran 4 % slower.
-__global__ void __launch_bounds__(32) adj_rev_node_kernel(
-    AL L, const double* __restrict__ fin, const double* __restrict__ lam, StepCols c,
-    const double* __restrict__ psi, int rows, double* __restrict__ gbar,
-    double* __restrict__ part) {
-  pdl_enter();
-  const int x = blockIdx.x * 32 + threadIdx.x;
-  if (x >= L.Nx || !interior(L, x)) return;
-  const int j0 = blockIdx.y * rows, j1 = min(L.N, j0 + rows);
-  const int half = (L.N + 1) / 2;
-  for (int j = j0; j < j1; ++j) {
-    double g[2][9], fb[2][9], gb[2][9];
-    pull(L, fin, c.r, c.kappa, x, j, g);
-#pragma unroll
-    for (int sp = 0; sp < 2; ++sp)
-#pragma unroll
-      for (int i = 0; i < 9; ++i) fb[sp][i] = lam[fidx(L, sp, i, j, x)];
-    const int h = j < half ? 0 : 1;
-    double oqb, lmb;
-    node_reverse(L, g, j + 0.5, c.omq[h * L.Nx + x], fb, gb, &oqb, &lmb,
-                 psi + (size_t)j * L.Nx + x, (size_t)L.N * L.Nx);
-#pragma unroll
-    for (int sp = 0; sp < 2; ++sp)
-#pragma unroll
-      for (int i = 0; i < 9; ++i) gbar[fidx(L, sp, i, j, x)] = gb[sp][i];
-    part[(size_t)(2 * j) * L.Nx + x] = oqb;
-    part[(size_t)(2 * j + 1) * L.Nx + x] = lmb;
-  }
-}
-
-// Sum over the warp by a butterfly: every lane gets the same value (each
-// stage adds the same two operands in every lane).
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// Reverse of tau_q per column and wall: one warp per (wall, column), item
-// = w N_x + x, kRevTauqWarps per block.  The lanes load the per-row partials
-// of adj_rev_node_kernel over the rows of wall w's half (lane-strided, so
-// the loads are in flight together) and sum them by a butterfly; then the
-// adjoint of tau_q times the derivatives the forward run stored (c.dq) goes
-// to the wall node's gbar (lanes 0..17, one population each), the
-// accommodation adjoint and ln mu (lnmu_col[w][x]).  The scalar work after
-// the sum is a dozen FP64 operations, so its repetition across the lanes
-// costs little.
-constexpr int kRevTauqWarps = 4;
-__global__ void __launch_bounds__(32 * kRevTauqWarps) adj_rev_tauq_kernel(
-    AL L, StepCols c, const double* __restrict__ part, double* __restrict__ gbar,
-    double* __restrict__ alphabar, double* __restrict__ lnmu_col) {
-  pdl_enter();
-  const int lane = threadIdx.x & 31;
-  const int item = blockIdx.x * kRevTauqWarps + (threadIdx.x >> 5);
-  if (item >= 2 * L.Nx) return;  // warp-uniform
-  const int w = item >= L.Nx ? 1 : 0, x = item - w * L.Nx;
-  if (!interior(L, x)) return;   // warp-uniform
-  const int half = (L.N + 1) / 2;
-  const int ja = w == 0 ? 0 : half, jb = w == 0 ? half : L.N;
-  double omqbar = 0.0, lm = 0.0;
-  for (int j = ja + lane; j < jb; j += 32) {
-    omqbar += part[(size_t)(2 * j) * L.Nx + x];
-    lm += part[(size_t)(2 * j + 1) * L.Nx + x];
-  }
-  omqbar = warp_sum(omqbar);
-  lm = warp_sum(lm);
-  const size_t k = (size_t)w * L.Nx + x, wn = 2 * (size_t)L.Nx;
-  const double omq = c.omq[k];
-  const double taub = -omqbar * omq * omq;  // omq = 1/tau_q
-  if (lane < 18) {
-    const int sp = lane >= 9 ? 1 : 0;
-    const int jw = w == 0 ? 0 : L.N - 1;
-    gbar[fidx(L, sp, lane - 9 * sp, jw, x)] += taub * (c.dq[k] + c.dq[wn + k] * L.s[sp]);
-  }
-  if (lane == 0) {
-    alphabar[k] += taub * c.dq[2 * wn + k];
-    lnmu_col[k] += lm;
-    lnmu_col[k] += taub * c.dq[3 * wn + k];
-  }
-}
-
-// Transpose of Pull: lam_prev(x, j) gathers the gbar of every node that
-// pulled population i of node (x, j) plainly, through the DBB rule of its
-// own wall row or through a ghost column, and the DBB rule's r adjoint is
-// carried into the wall node's densities and accommodation (with the
-// derivatives of r the forward run stored).  Every gather loads from an
-// address inside the array whether or not its source exists (the value is
-// then dropped), so the loads are independent of one another; the FP64
-// work is a few multiply-adds per node, the FP64 pipe being narrow.
-// gk: [4] the kappa terms of adj_rev_kappa_kernel, per (end, species).
-__global__ void __launch_bounds__(128) adj_rev_pull_kernel(
-    AL L, const double* __restrict__ fin, StepCols c, const double* __restrict__ gbar,
-    const double* __restrict__ gk, double* __restrict__ lamp, double* __restrict__ alphabar) {
-  pdl_enter();
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y;
-  if (x >= L.Nx) return;
-  if (!interior(L, x)) {
-    #pragma unroll
-    for (int sp = 0; sp < 2; ++sp)
-      #pragma unroll
-      for (int i = 0; i < 9; ++i) lamp[fidx(L, sp, i, j, x)] = 0.0;
-    return;
-  }
-  double lp[2][9];
+// Transpose of Pull at node (x, j): lp gathers the gbar of every node that
+// pulled population i of node (x, j) plainly, through the DBB rule of its own
+// wall row or through a ghost column, and the DBB rule's r adjoint is carried
+// into the wall node's densities and accommodation (with the derivatives of r
+// the forward run stored).  Every gather loads from an address inside the
+// array whether or not its source exists (the value is then dropped), so the
+// loads are independent of one another; the FP64 work is a few multiply-adds
+// per node, the FP64 pipe being narrow.  fin, c, gk: input, column data and
+// [4] kappa terms (adj_rev_cols_kernel, per end and species) of the step that
+// is transposed.
+__device__ __forceinline__ void pull_transpose(const AL& L, const double* __restrict__ fin,
+                                               const StepCols& c, const double* __restrict__ gbar,
+                                               const double* __restrict__ gk,
+                                               double* __restrict__ alphabar, int x, int j,
+                                               double lp[2][9]) {
   #pragma unroll
   for (int sp = 0; sp < 2; ++sp)
     #pragma unroll
@@ -1009,6 +966,7 @@ __global__ void __launch_bounds__(128) adj_rev_pull_kernel(
     }
   // diffuse bounce-back: the unknowns (2, 5, 6) at row 0 and (4, 7, 8) at
   // row N-1 are pulled from this node's own outgoing populations
+  #pragma unroll
   for (int w = 0; w < 2; ++w) {
     const int jw = w == 0 ? 0 : L.N - 1;
     if (j != jw) continue;
@@ -1023,25 +981,27 @@ __global__ void __launch_bounds__(128) adj_rev_pull_kernel(
       const double o0 = fin[fidx(L, sp, out[0], j, x)], o1 = fin[fidx(L, sp, out[1], j, x)],
                    o2 = fin[fidx(L, sp, out[2], j, x)];
       const double S = o0 + o1 + o2;
-      const double T = (2.0 / 3.0) * G0 + (G1 + G2) / 6.0;
-      lp[sp][out[0]] += (1.0 - r) * G0 + r * T;
-      lp[sp][out[1]] += (1.0 - r) * G1 + r * T;
-      lp[sp][out[2]] += (1.0 - r) * G2 + r * T;
-      rbar += G0 * (-o0 + (2.0 / 3.0) * S) + G1 * (-o1 + S / 6.0) + G2 * (-o2 + S / 6.0);
+      const double T = fma(2.0 / 3.0, G0, __dmul_rn(1.0 / 6.0, G1 + G2));
+      lp[sp][out[0]] += fma(r, T - G0, G0);
+      lp[sp][out[1]] += fma(r, T - G1, G1);
+      lp[sp][out[2]] += fma(r, T - G2, G2);
+      rbar = fma(G0, fma(2.0 / 3.0, S, -o0), rbar);
+      rbar = fma(G1, fma(1.0 / 6.0, S, -o1), rbar);
+      rbar = fma(G2, fma(1.0 / 6.0, S, -o2), rbar);
     }
     const size_t k = (size_t)w * L.Nx + x, wn = 2 * (size_t)L.Nx;
     #pragma unroll
     for (int sp = 0; sp < 2; ++sp) {
-      const double v = rbar * c.dr[sp * wn + k];
+      const double v = __dmul_rn(rbar, c.dr[sp * wn + k]);
       #pragma unroll
       for (int i = 0; i < 9; ++i) lp[sp][i] += v;
     }
-    alphabar[k] += rbar * c.dr[2 * wn + k];
+    alphabar[k] = fma(rbar, c.dr[2 * wn + k], alphabar[k]);
   }
   // the ends: node (x1, jd) pulled population i (c_ix pointing into the
   // channel) from the ghost column kappa (2 f(x1) - f(x2)), and kappa itself
-  // depends on the columns x1 = 1, x2 = 2 (N_x - 2, N_x - 3) through gk
-  // (adj_rev_kappa_kernel): their transposes land in those columns
+  // depends on the columns x1 = 1, x2 = 2 (N_x - 2, N_x - 3) through gk:
+  // their transposes land in those columns
   if (!L.x_periodic && (x <= 2 || x >= L.Nx - 3)) {
     #pragma unroll
     for (int end = 0; end < 2; ++end) {
@@ -1058,10 +1018,31 @@ __global__ void __launch_bounds__(128) adj_rev_pull_kernel(
           const int jd = j + cyd(i);
           const bool ok = cxd(i) == dir && jd >= 0 && jd < L.N;
           const double gv = gbar[fidx(L, sp, i, ok ? jd : j, x1)];
-          lp[sp][i] += wgt * ((ok ? kap * gv : 0.0) + gk[e]);
+          lp[sp][i] = fma(wgt, ok ? fma(kap, gv, gk[e]) : gk[e], lp[sp][i]);
         }
       }
     }
+  }
+}
+
+// lam_prev = Pull^T gbar for every node, the adjoint of a step's input.  Only
+// the first step of a checkpoint interval needs it as an array; inside an
+// interval adj_rev_node_kernel forms it where it is used.
+__global__ void __launch_bounds__(128) adj_rev_pull_kernel(
+    AL L, const double* __restrict__ fin, StepCols c, const double* __restrict__ gbar,
+    const double* __restrict__ gk, double* __restrict__ lamp, double* __restrict__ alphabar) {
+  pdl_enter();
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  const int j = blockIdx.y;
+  if (x >= L.Nx) return;
+  double lp[2][9];
+  if (interior(L, x)) {
+    pull_transpose(L, fin, c, gbar, gk, alphabar, x, j, lp);
+  } else {
+    #pragma unroll
+    for (int sp = 0; sp < 2; ++sp)
+      #pragma unroll
+      for (int i = 0; i < 9; ++i) lp[sp][i] = 0.0;
   }
   #pragma unroll
   for (int sp = 0; sp < 2; ++sp)
@@ -1069,39 +1050,141 @@ __global__ void __launch_bounds__(128) adj_rev_pull_kernel(
     for (int i = 0; i < 9; ++i) lamp[fidx(L, sp, i, j, x)] = lp[sp][i];
 }
 
-// The ends in reverse: the adjoint of kappa_e for (end, species) e = blockIdx.x
-// = 2 end + species, reduced over the end columns' rows in a fixed order,
-// gives gk[e] = -kappa_bar kappa / D, the weight of d kappa / d f at columns
-// x1, x2 (times 2 and -1) that adj_rev_pull_kernel adds, and the inlet's
-// theta adjoint (theta_acc[species]).  Threads take (row, population)
-// items.
-__global__ void __launch_bounds__(256) adj_rev_kappa_kernel(
-    AL L, const double* __restrict__ fin, StepCols c, const double* __restrict__ gbar,
+// What the reverse of a step reads of the step after it, to form the adjoint
+// of its own output by pull_transpose.
+struct RevNext {
+  const double* fin;
+  StepCols c;
+  const double* gbar;
+  const double* gk;
+  double* alphabar;
+};
+
+// Reverse of Collide for every node: gbar = (dCollide/dg)^T lam_t, and
+// per node the adjoints of 1/tau_q (of the node's half) and of ln mu,
+// stored per row for adj_rev_cols_kernel to sum in row order:
+// part[j][0][x], part[j][1][x].  lam_t is the array lam (GATHER = false: the
+// last step of an interval) or the transpose of the next step's pull, gathered
+// here (saves a launch and a state written and read per step).  Block (bx, j):
+// one warp, 32 columns of row j, 410 FP64 instructions.  psi: [6][N][Nx] Psi
+// values the forward run or the replay of this step stored.  Three rows per
+// block and two warps per sub-partition took 96 us per reversed step on 1280 x
+// 64, this shape 94 us; on 640 x 32 74 and 40 us.
+template <bool GATHER>
+__global__ void __launch_bounds__(32, 12) adj_rev_node_kernel(
+    AL L, const double* __restrict__ fin, const double* __restrict__ lam, RevNext nx, StepCols c,
+    const double* __restrict__ psi, double* __restrict__ gbar, double* __restrict__ part) {
+  pdl_enter();
+  const int x = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y;
+  if (x >= L.Nx || !interior(L, x)) return;
+  const int half = (L.N + 1) / 2;
+  double g[2][9], fb[2][9], gb[2][9];
+  pull(L, fin, c.r[x], c.r[L.Nx + x], c.kappa, x, j, g);
+  if constexpr (GATHER) {
+    pull_transpose(L, nx.fin, nx.c, nx.gbar, nx.gk, nx.alphabar, x, j, fb);
+  } else {
+#pragma unroll
+    for (int sp = 0; sp < 2; ++sp)
+#pragma unroll
+      for (int i = 0; i < 9; ++i) fb[sp][i] = lam[fidx(L, sp, i, j, x)];
+  }
+  const int h = j < half ? 0 : 1;
+  double oqb, lmb;
+  node_reverse(L, g, j + 0.5, c.omq[h * L.Nx + x], fb, gb, &oqb, &lmb,
+               psi + (size_t)j * L.Nx + x, (size_t)L.N * L.Nx);
+#pragma unroll
+  for (int sp = 0; sp < 2; ++sp)
+#pragma unroll
+    for (int i = 0; i < 9; ++i) gbar[fidx(L, sp, i, j, x)] = gb[sp][i];
+  part[(size_t)(2 * j) * L.Nx + x] = oqb;
+  part[(size_t)(2 * j + 1) * L.Nx + x] = lmb;
+}
+
+// Reverse of the column data, one launch.
+// Blocks from 4 on, one warp per (wall, column), item = w N_x + x: the lanes
+// load the per-row partials of adj_rev_node_kernel over the rows of wall w's
+// half (lane-strided, so the loads are in flight together) and sum them by a
+// butterfly; then the adjoint of tau_q times the derivatives the forward run
+// stored (c.dq) goes to the wall node's gbar (lanes 0..17, one population
+// each), the accommodation adjoint and ln mu (lnmu_col[w][x]).
+// Blocks 0 to 3, e = 2 end + species, take the items of the column x1 next to
+// that end (species e & 1; the first species' block the scalars), and then
+// the adjoint of kappa_e, reduced over the end columns' rows in a fixed order:
+// gk[e] = -kappa_bar kappa / D, the weight of d kappa / d f at columns x1, x2
+// (times 2 and -1) that pull_transpose adds, and the inlet's theta adjoint
+// (theta_acc[species]).
+constexpr int kRevWarps = 4;
+__global__ void __launch_bounds__(32 * kRevWarps) adj_rev_cols_kernel(
+    AL L, const double* __restrict__ fin, StepCols c, const double* __restrict__ part,
+    double* __restrict__ gbar, double* __restrict__ alphabar, double* __restrict__ lnmu_col,
     double* __restrict__ gk, double* __restrict__ theta_acc) {
   pdl_enter();
-  __shared__ double sm[8];
-  const int t = threadIdx.x, e = blockIdx.x;
-  if (L.x_periodic) return;
-  const int sp = e & 1, inlet = e < 2;
+  __shared__ double red[2][kRevWarps];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int half = (L.N + 1) / 2;
+  const size_t wn = 2 * (size_t)L.Nx;
+  // item (w, x) by one warp: species sp0 .. sp0 + nsp - 1
+  auto wall_item = [&](int w, int x, int sp0, int nsp, bool scalars) {
+    const int ja = w == 0 ? 0 : half, jb = w == 0 ? half : L.N;
+    double omqbar = 0.0, lm = 0.0;
+    for (int j = ja + lane; j < jb; j += 32) {
+      omqbar += part[(size_t)(2 * j) * L.Nx + x];
+      lm += part[(size_t)(2 * j + 1) * L.Nx + x];
+    }
+    omqbar = warp_sum(omqbar);
+    lm = warp_sum(lm);
+    const size_t k = (size_t)w * L.Nx + x;
+    const double omq = c.omq[k];
+    const double taub = -omqbar * omq * omq;  // omq = 1/tau_q
+    if (lane < 9 * nsp) {
+      const int sp = sp0 + (lane >= 9 ? 1 : 0), i = lane >= 9 ? lane - 9 : lane;
+      gbar[fidx(L, sp, i, w == 0 ? 0 : L.N - 1, x)] += taub * (c.dq[k] + c.dq[wn + k] * L.s[sp]);
+    }
+    if (lane == 0 && scalars) {
+      alphabar[k] += taub * c.dq[2 * wn + k];
+      lnmu_col[k] += lm;
+      lnmu_col[k] += taub * c.dq[3 * wn + k];
+    }
+  };
+  if (blockIdx.x >= 4) {
+    const int item = ((int)blockIdx.x - 4) * kRevWarps + warp;
+    if (item >= 2 * L.Nx) return;  // warp-uniform
+    const int w = item >= L.Nx ? 1 : 0, x = item - w * L.Nx;
+    if (!interior(L, x) || x == 1 || x == L.Nx - 2) return;  // warp-uniform
+    wall_item(w, x, 0, 2, true);
+    return;
+  }
+  const int e = blockIdx.x, sp = e & 1, inlet = e < 2;
   const int x1 = inlet ? 1 : L.Nx - 2, x2 = inlet ? 2 : L.Nx - 3, dir = inlet ? 1 : -1;
+  if (warp < 2) wall_item(warp, x1, sp, 1, sp == 0);
+  __syncthreads();
   const double kap = c.kappa[e];
   // node (x1, jd) pulled population i (c_ix = dir) from the ghost column:
   // kappa (2 f(x1, js) - f(x2, js)), js = jd - c_iy
-  double acc = 0.0, cs1 = 0.0, cs2 = 0.0;
-  for (int k = t; k < 9 * L.N; k += blockDim.x) {
+  double acc = 0.0, cs = 0.0;
+  for (int k = threadIdx.x; k < 9 * L.N; k += 32 * kRevWarps) {
     const int jd = k / 9, i = k - 9 * jd;
     const int js = jd - cyd(i);
     const bool ok = cxd(i) == dir && js >= 0 && js < L.N;
     const int jsc = ok ? js : jd;
     const double gb = gbar[fidx(L, sp, i, jd, x1)];
     const double a1 = fin[fidx(L, sp, i, jsc, x1)], a2 = fin[fidx(L, sp, i, jsc, x2)];
-    acc += ok ? gb * (2.0 * a1 - a2) : 0.0;
-    cs1 += fin[fidx(L, sp, i, jd, x1)];
-    cs2 += fin[fidx(L, sp, i, jd, x2)];
+    acc += ok ? gb * fma(2.0, a1, -a2) : 0.0;
+    cs += fma(2.0, fin[fidx(L, sp, i, jd, x1)], -fin[fidx(L, sp, i, jd, x2)]);
   }
-  const double kb = block_sum256(acc, sm);
-  const double D = block_sum256(2.0 * cs1 - cs2, sm);
-  if (t == 0) {
+  acc = warp_sum(acc);
+  cs = warp_sum(cs);
+  if (lane == 0) {
+    red[0][warp] = acc;
+    red[1][warp] = cs;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double kb = 0.0, D = 0.0;
+    for (int q = 0; q < kRevWarps; ++q) {
+      kb += red[0][q];
+      D += red[1][q];
+    }
     // kappa_in = N rho_in / D, rho_in,s = theta C_s m_s
     if (inlet) theta_acc[sp] += kb * kap / L.theta;
     // d kappa / d f(x, j) = -kappa / D * (2 at column x1, -1 at column x2)
@@ -1160,11 +1243,16 @@ AL derive_al(const lbm_mix_params* p, int Nx) {
   }
   L.c_lam = 3.0 * mu * sqrt(kPiD / 6.0);
   L.inv_c_lam = 1.0 / L.c_lam;
-  for (int sp = 0; sp < 2; ++sp) L.inv_c_xl[sp] = 1.0 / L.c_xl[sp];
+  for (int sp = 0; sp < 2; ++sp) {
+    L.s_inv_c_xl[sp] = L.s[sp] / L.c_xl[sp];
+    L.c_xl_s[sp] = L.c_xl[sp] / L.s[sp];
+    L.be[sp] = 2.0 * L.s[sp] - 4.0;
+    L.bp[sp] = 4.0 - 3.0 * L.s[sp];
+  }
   L.c_ts = sqrt(6.0 / kPiD);
   L.c_td = 1.5 * sqrt(3.0 * (L.mh[0] + L.mh[1]) * L.mh[0] * L.mh[1]);
-  L.om_e = 1.0 / p->tau_e;
-  L.om_eps = 1.0 / p->tau_eps;
+  L.we = 1.0 / (36.0 * p->tau_e);
+  L.wp = 1.0 / (36.0 * p->tau_eps);
   L.c_m0 = p->c_m0;
   L.H = p->N;
   return L;
@@ -1192,16 +1280,15 @@ struct lbm_adj {
   cudaStream_t rstream = nullptr;   // the replays of the backward sweep
   cudaEvent_t ev_start = nullptr, ev_rep[2] = {nullptr, nullptr}, ev_rev[2] = {nullptr, nullptr};
   double* work[2] = {nullptr, nullptr};
-  double* lam[2] = {nullptr, nullptr};
-  double* gbar = nullptr;
+  double* lam = nullptr;
+  double* gbar[2] = {nullptr, nullptr};
   double* dtheta0 = nullptr;  // d f^0 / d theta
   double* alpha = nullptr;    // [2][Nx]
   double* alphabar = nullptr;
   double* part_rev = nullptr;  // [N][2][Nx] per-row partials of adj_rev_node_kernel
-  int rows_step = 1, rows_rev = 1;  // rows per block of the two node kernels (node_rows)
   double* lnmu_col = nullptr; // [2][Nx] (per wall)
   double* theta_acc = nullptr;  // [2] (per species)
-  double* gk = nullptr;         // [4] kappa terms of the step being reversed
+  double* gk = nullptr;         // [2][4] kappa terms of the steps being reversed
   double* colsum = nullptr;   // [3][Nx]
   double* part = nullptr;     // [256]
   double* h_col = nullptr;    // host copy of colsum
@@ -1221,23 +1308,6 @@ StepCols cols_of(lbm_adj* a, double* base) {
   c.dq = base + 4 * a->L.Nx + 4;
   c.dr = base + 12 * a->L.Nx + 4;
   return c;
-}
-
-// Rows per block of a node kernel launched with one-warp blocks of 32
-// columns: the fewest rows for which every block is resident at once (the
-// occupancy calculator's blocks per SM times the SMs), so that the FP64
-// work is spread evenly, with no partial second wave.
-cudaError_t node_rows(const void* kernel, int Nx, int N, int* rows) {
-  int dev = 0, nsm = 0, occ = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, 32, 0);
-  if (e != cudaSuccess) return e;
-  const long slots = (long)nsm * (occ > 0 ? occ : 1), ncb = (Nx + 31) / 32;
-  int r = 1;
-  while (r < N && ncb * ((N + r - 1) / r) > slots) ++r;
-  *rows = r;
-  return cudaSuccess;
 }
 
 // Launches kern with programmatic stream serialisation (see pdl_enter).
@@ -1260,15 +1330,10 @@ cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, cudaStream
 int fwd_step(lbm_adj* a, const double* f, double* fo, StepCols c, cudaStream_t st,
              double* psi_out = nullptr) {
   const AL& L = a->L;
-  CKA(launch_pdl(adj_kappa_kernel, dim3(4), dim3(256), st, L, f, c.kappa));
-  // one thread per (column, wall): small blocks spread the FP64 work of
-  // the wall columns over many SMs
-  const dim3 wg((L.Nx + 31) / 32, 2);
-  CKA(launch_pdl(adj_cols_kernel, wg, dim3(32), st, L, f, (const double*)a->alpha, c));
-  CKA(launch_pdl(adj_tauq_kernel, wg, dim3(32), st, L, f, (const double*)a->alpha, c));
-  CKA(launch_pdl(adj_step_kernel,
-                 dim3((L.Nx + 31) / 32, (L.N + a->rows_step - 1) / a->rows_step), dim3(32), st,
-                 L, f, fo, c, psi_out, a->rows_step));
+  CKA(launch_pdl(adj_cols_kernel, dim3((L.Nx + 31) / 32, 2), dim3(32 * kColsWarps), st, L, f,
+                 (const double*)a->alpha, c));
+  CKA(launch_pdl(psi_out ? adj_step_kernel<true> : adj_step_kernel<false>,
+                 dim3((L.Nx + 31) / 32, L.N), dim3(32), st, L, f, fo, c, psi_out));
   return LBM_OK;
 }
 
@@ -1354,16 +1419,16 @@ int lbm_adj_create(const lbm_mix_params* p, long nsteps, int checkpoint_every, v
   }
   ALLOCA(a->work[0], sizeof(double) * a->S);
   ALLOCA(a->work[1], sizeof(double) * a->S);
-  ALLOCA(a->lam[0], sizeof(double) * a->S);
-  ALLOCA(a->lam[1], sizeof(double) * a->S);
-  ALLOCA(a->gbar, sizeof(double) * a->S);
+  ALLOCA(a->lam, sizeof(double) * a->S);
+  ALLOCA(a->gbar[0], sizeof(double) * a->S);
+  ALLOCA(a->gbar[1], sizeof(double) * a->S);
   ALLOCA(a->dtheta0, sizeof(double) * a->S);
   ALLOCA(a->alpha, sizeof(double) * 2 * Nx);
   ALLOCA(a->alphabar, sizeof(double) * 2 * Nx);
   ALLOCA(a->part_rev, sizeof(double) * 2 * Nx * (size_t)p->N);
   ALLOCA(a->lnmu_col, sizeof(double) * 2 * Nx);
   ALLOCA(a->theta_acc, sizeof(double) * 2);
-  ALLOCA(a->gk, sizeof(double) * 4);
+  ALLOCA(a->gk, sizeof(double) * 8);
   ALLOCA(a->colsum, sizeof(double) * 3 * Nx);
   ALLOCA(a->part, sizeof(double) * 256);
 #undef ALLOCA
@@ -1379,8 +1444,6 @@ int lbm_adj_create(const lbm_mix_params* p, long nsteps, int checkpoint_every, v
       free(al);
     }
   }
-  if (e == cudaSuccess) e = node_rows((const void*)adj_step_kernel, Nx, p->N, &a->rows_step);
-  if (e == cudaSuccess) e = node_rows((const void*)adj_rev_node_kernel, Nx, p->N, &a->rows_rev);
   if (e != cudaSuccess) {
     const int code = e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA;
     lbm_internal_error(code, "adjoint allocation failed: %s", cudaGetErrorString(e));
@@ -1408,9 +1471,9 @@ void lbm_adj_destroy(lbm_adj* a) {
   if (a->rstream) cudaStreamDestroy(a->rstream);
   for (int k = 0; k < 2; ++k) {
     cudaFree(a->work[k]);
-    cudaFree(a->lam[k]);
+    cudaFree(a->gbar[k]);
   }
-  cudaFree(a->gbar);
+  cudaFree(a->lam);
   cudaFree(a->dtheta0);
   cudaFree(a->alpha);
   cudaFree(a->alphabar);
@@ -1504,9 +1567,9 @@ int lbm_adj_gradient(lbm_adj* a, int objective, double* dtheta, double* dkn, dou
   CKA(cudaMemsetAsync(a->alphabar, 0, sizeof(double) * 2 * L.Nx, a->stream));
   CKA(cudaMemsetAsync(a->lnmu_col, 0, sizeof(double) * 2 * L.Nx, a->stream));
   CKA(cudaMemsetAsync(a->theta_acc, 0, sizeof(double) * 2, a->stream));
-  adj_seed_kernel<<<grd, 128, 0, a->stream>>>(L, objective, a->xstar, a->Sl, a->Sh, a->lam[0]);
+  adj_seed_kernel<<<grd, 128, 0, a->stream>>>(L, objective, a->xstar, a->Sl, a->Sh, a->lam);
   CKA(cudaGetLastError());
-  int cur = 0;  // lam[cur] is the adjoint of the state after the step being reversed
+  // lam: the adjoint of the state after the interval being reversed
   const long nseg = a->nseg;
   // the replay's last output of a segment is not needed (only its column
   // data are); it goes to the work buffer that does not hold f^T, so that
@@ -1553,29 +1616,31 @@ int lbm_adj_gradient(lbm_adj* a, int objective, double* dtheta, double* dkn, dou
     if (!(last_kept && sg == nseg - 1)) CKA(cudaStreamWaitEvent(a->stream, a->ev_rep[b], 0));
     const long t0 = sg * a->K;
     const long t1 = (t0 + a->K < a->T) ? t0 + a->K : a->T;
+    // gbar and gk alternate: a step's reverse reads those of the step after it
+    RevNext nx = {};
+    int gcur = 0;
     for (long t = t1; t > t0; --t) {
       const long k = t - t0 - 1;
       const double* fin = a->seg[b] + a->S * (size_t)k;
       StepCols c = cols_of(a, a->segcols[b] + cw * k);
-      CKA(launch_pdl(adj_rev_node_kernel,
-                     dim3((L.Nx + 31) / 32, (L.N + a->rows_rev - 1) / a->rows_rev), dim3(32),
-                     a->stream, L, fin, (const double*)a->lam[cur], c,
-                     (const double*)(a->segpsi[b] + psi_step * (size_t)k), a->rows_rev, a->gbar,
-                     a->part_rev));
-      CKA(launch_pdl(adj_rev_tauq_kernel, dim3((2 * L.Nx + kRevTauqWarps - 1) / kRevTauqWarps),
-                     dim3(32 * kRevTauqWarps), a->stream, L, c, (const double*)a->part_rev,
-                     a->gbar, a->alphabar, a->lnmu_col));
-      // one block per (end, species); the pull adds its kappa terms
-      CKA(launch_pdl(adj_rev_kappa_kernel, dim3(4), dim3(256), a->stream, L, fin, c,
-                     (const double*)a->gbar, a->gk, a->theta_acc));
-      CKA(launch_pdl(adj_rev_pull_kernel, grd, dim3(128), a->stream, L, fin, c,
-                     (const double*)a->gbar, (const double*)a->gk, a->lam[1 - cur], a->alphabar));
-      cur = 1 - cur;
+      double* gbar = a->gbar[gcur];
+      double* gk = a->gk + 4 * gcur;
+      const dim3 ng((L.Nx + 31) / 32, L.N);
+      CKA(launch_pdl(t < t1 ? adj_rev_node_kernel<true> : adj_rev_node_kernel<false>, ng, dim3(32),
+                     a->stream, L, fin, (const double*)a->lam, nx, c,
+                     (const double*)(a->segpsi[b] + psi_step * (size_t)k), gbar, a->part_rev));
+      CKA(launch_pdl(adj_rev_cols_kernel, dim3(4 + (2 * L.Nx + kRevWarps - 1) / kRevWarps),
+                     dim3(32 * kRevWarps), a->stream, L, fin, c, (const double*)a->part_rev, gbar,
+                     a->alphabar, a->lnmu_col, gk, a->theta_acc));
+      nx = RevNext{fin, c, gbar, gk, a->alphabar};
+      gcur = 1 - gcur;
     }
+    CKA(launch_pdl(adj_rev_pull_kernel, grd, dim3(128), a->stream, L, nx.fin, nx.c, nx.gbar, nx.gk,
+                   a->lam, a->alphabar));
     CKA(cudaEventRecord(a->ev_rev[b], a->stream));
   }
   // theta through the initial state: lam^0 . d f^0 / d theta
-  adj_dot_kernel<<<256, 256, 0, a->stream>>>(a->lam[cur], a->dtheta0, a->S, a->part);
+  adj_dot_kernel<<<256, 256, 0, a->stream>>>(a->lam, a->dtheta0, a->S, a->part);
   CKA(cudaGetLastError());
   double* h = a->h_col;  // staging: [2][Nx] ln mu, [2] theta, [256] parts
   CKA(cudaMemcpyAsync(h, a->lnmu_col, sizeof(double) * 2 * L.Nx, cudaMemcpyDeviceToHost,
