@@ -1533,26 +1533,65 @@ __global__ void lbm_convert_kernel(Lat L, ST* __restrict__ f, const float* __res
   }
 }
 
-// Volume flow through column x: sum over the rows of the mixture velocity
-// u_x = (rho_a u_a,x + rho_b u_b,x) / (rho_a + rho_b) of a moments array
-// [6][N][Nx] (rho_a, rho_b, u_a (x, y), u_b (x, y)); one block, fixed order.
-__global__ void lbm_volume_flow_kernel(const double* __restrict__ mom, int N, int Nx, int x,
-                                       double* __restrict__ out) {
-  __shared__ double red[256];
-  const size_t plane = (size_t)N * Nx;
+// Volume flow through column x: sum over the rows of the mixture velocity u_x
+// = (j_a,x + j_b,x) / (rho_a + rho_b), to which the species velocities of Eq.
+// rhou add up, of the state obtained by streaming fin (direct = 0) or of fin
+// itself (direct = 1); one block, fixed order, straight to host memory.
+template <typename ST>
+__global__ void __launch_bounds__(256)
+    lbm_volume_flow_kernel(Lat L, const ST* __restrict__ fin, const float* __restrict__ refrho,
+                           const double* __restrict__ cs_in, const float* __restrict__ alpha,
+                           int direct, int x, double* __restrict__ out) {
+  __shared__ double red[8];
+  const ColRef C = col_ref(L, refrho, x);
+  const Ends E = load_ends(L, cs_in, refrho, x, 1);
   double v = 0.0;
-  for (int j = threadIdx.x; j < N; j += blockDim.x) {
-    const size_t o = (size_t)j * Nx + x;
-    const double ra = mom[o], rb = mom[plane + o];
-    v += (ra * mom[2 * plane + o] + rb * mom[4 * plane + o]) / (ra + rb);
+  for (int j = threadIdx.x; j < L.N; j += 256) {
+    float fs[2][9];
+    if (direct) {
+#pragma unroll
+      for (int sp = 0; sp < 2; ++sp)
+#pragma unroll
+        for (int i = 0; i < 9; ++i) fs[sp][i] = ld(fin, L, sp, i, j, x);
+    } else {
+      float2 r = make_float2(0.0f, 0.0f);
+      if (j == 0 || j == L.N - 1)
+        r = dbb_r(L, C, fin, x, j, alpha[(j == 0 ? 0 : L.Nx) + x]);
+      pull_node(fin, L, E, C, x, j, r, r, fs);
+    }
+    float2 g[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) g[i] = make_float2(fs[0][i], fs[1][i]);
+    Flow2 w;
+    flow2(g, 0.0f, w);
+    const float2 sd = density_sum(g);
+    const double rho = ((double)C.rb[0] + sd.x) + ((double)C.rb[1] + sd.y);
+    v += ((double)w.jx.x + (double)w.jx.y) / rho;
   }
-  red[threadIdx.x] = v;
+  v = warp_sum(v);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
   if (threadIdx.x == 0) {
     double s = 0.0;
-    for (int k = 0; k < (int)blockDim.x; ++k) s += red[k];
+    for (int k = 0; k < 8; ++k) s += red[k];
     *out = s;
   }
+}
+
+// The number of records, the latest one and (profile != 0) C_l(x), straight to
+// host memory: out[0], out[1 .. NREC], out[16 ...].  One launch and one wait
+// where the count, the record and the profile took a copy and a wait each.
+__global__ void __launch_bounds__(256)
+    lbm_latest_kernel(const double* __restrict__ diag,
+                      const unsigned long long* __restrict__ diag_count,
+                      const double* __restrict__ clprof, int Nx, int profile,
+                      double* __restrict__ out) {
+  const unsigned long long cnt = *diag_count;
+  const int t = threadIdx.x;
+  if (t == 0) out[0] = (double)cnt;
+  if (t < NREC) out[1 + t] = cnt == 0 ? 0.0 : diag[(size_t)((cnt - 1) % DIAG_CAP) * NREC + t];
+  if (profile)
+    for (int x = t; x < Nx; x += 256) out[16 + x] = clprof[x];
 }
 
 // Steady-state residual over the column sums: R = |c - c_old| / (K |c|),
@@ -1644,9 +1683,8 @@ struct lbm_mix {
   unsigned* strip_cnt; // [nblocks]
   int R, rows_per_block;
   int R_alloc;        // row blocks colpart has room for
-  double* resid;
   double* mom;
-  double* h_pinned;  // small pinned staging area
+  double* h_pinned;  // [16 + Nx] pinned: what the getters' kernels write
   // Several steps per launch (lbm_tile_kernel): own columns per tile and
   // most steps of a launch; tile_W = 0: the channel does not qualify.  A
   // schedule the caller set (rows_set) takes the step kernel instead.
@@ -1867,14 +1905,14 @@ int rereference(lbm_mix* h) {
 }
 
 // Steady-state residual of the last k steps (Sec. 4 convergence check, over
-// the column sums of the latest DIAG step) into h->h_pinned[0], async.
+// the column sums of the latest DIAG step) into h->h_pinned[0], async, by the
+// kernel itself.
 int launch_residual(lbm_mix* h, long k) {
   ResidBatch<1> B;
   B.inst[0] = ResidInst{h->cs[h->cur], h->cs_snap, 4L * h->L.Nx, h->have_snap ? 1 : 0};
-  lbm_residual_kernel<1><<<1, 1024, 0, h->stream>>>(B, (double)k, h->resid);
+  lbm_residual_kernel<1><<<1, 1024, 0, h->stream>>>(B, (double)k, h->h_pinned);
   CK(cudaGetLastError());
   h->have_snap = true;
-  CK(cudaMemcpyAsync(h->h_pinned, h->resid, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   return LBM_OK;
 }
 
@@ -2175,17 +2213,19 @@ int check_handle(const lbm_mix* h) {
   return LBM_OK;
 }
 
-// Latest diagnostic record (host copy). Returns LBM_ENONFINITE on NaN/Inf.
-int latest_record(lbm_mix* h, double rec[NREC]) {
-  unsigned long long cnt = 0;
-  CK(cudaMemcpyAsync(&cnt, h->diag_count, sizeof cnt, cudaMemcpyDeviceToHost, h->stream));
+// Latest diagnostic record (host copy) and, where wanted, C_l(x). Returns
+// LBM_ENONFINITE on NaN/Inf.
+int latest_record(lbm_mix* h, double rec[NREC], double* profile) {
+  lbm_latest_kernel<<<1, 256, 0, h->stream>>>(h->diag, h->diag_count, h->clprof, h->L.Nx,
+                                              profile ? 1 : 0, h->h_pinned);
+  CK(cudaGetLastError());
   CK(cudaStreamSynchronize(h->stream));
+  const unsigned long long cnt = (unsigned long long)h->h_pinned[0];
   if (cnt == 0) return set_err(LBM_EINVAL, "no step taken yet");
-  CK(cudaMemcpyAsync(rec, h->diag + ((cnt - 1) % DIAG_CAP) * NREC, sizeof(double) * NREC,
-                     cudaMemcpyDeviceToHost, h->stream));
-  CK(cudaStreamSynchronize(h->stream));
+  memcpy(rec, h->h_pinned + 1, sizeof(double) * NREC);
   for (int k = 1; k < NREC; ++k)
     if (!isfinite(rec[k])) return set_err(LBM_ENONFINITE, "non-finite diagnostic at step %llu", cnt);
+  if (profile) memcpy(profile, h->h_pinned + 16, sizeof(double) * (size_t)h->L.Nx);
   return LBM_OK;
 }
 
@@ -2411,7 +2451,6 @@ int lbm_mix_create(const lbm_mix_params* p, void* stream, lbm_mix** out) {
     if (p->storage == LBM_FP32 && !p->x_periodic)
       carve(base, sizeof(float2) * 4 * (size_t)h->L.N, &h->end_sd);
     carve(base, sizeof(double) * 4 * (size_t)Nx * (size_t)h->R, &h->colpart0);
-    carve(base, sizeof(double), &h->resid);
     if (h->tile_W > 0) carve(base, sizeof(float2) * 4 * (size_t)Nx * h->hist_rows, &h->hist);
   };
   layout(nullptr);
@@ -2420,7 +2459,7 @@ int lbm_mix_create(const lbm_mix_params* p, void* stream, lbm_mix** out) {
     layout((char*)h->arena);
     h->colpart = h->colpart0;
   }
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&h->h_pinned, sizeof(double) * 64);
+  if (e == cudaSuccess) e = cudaMallocHost((void**)&h->h_pinned, sizeof(double) * (16 + (size_t)Nx));
   if (e != cudaSuccess) {
     int code = (e == cudaErrorMemoryAllocation) ? LBM_ENOMEM : LBM_ECUDA;
     set_err(code, "allocation failed: %s", cudaGetErrorString(e));
@@ -2641,12 +2680,17 @@ int lbm_mix_volume_flow(lbm_mix* h, int x, double* Qv) {
   if (x < 0) x = h->L.x_periodic ? 0 : h->L.Nx - 2;
   if (x >= h->L.Nx || (!h->L.x_periodic && (x < 1 || x > h->L.Nx - 2)))
     return set_err(LBM_EINVAL, "column %d is not an updated column", x);
-  const size_t plane = (size_t)h->L.N * h->L.Nx;
-  if (!h->mom) CK(cudaMalloc((void**)&h->mom, sizeof(double) * 6 * plane));
-  if ((st = launch_moments(h, h->mom))) return st;
-  lbm_volume_flow_kernel<<<1, 256, 0, h->stream>>>(h->mom, h->L.N, h->L.Nx, x, h->resid);
-  CK(cudaGetLastError());
-  CK(cudaMemcpyAsync(h->h_pinned, h->resid, sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  // the state of step n is the stream of buffer P_{n-1} (launch_moments)
+  const int direct = h->steps == 0 ? 1 : 0, b = direct ? h->cur : 1 - h->cur;
+  st = with_storage(h, [&](auto tag) -> int {
+    using ST = decltype(tag);
+    lbm_volume_flow_kernel<ST><<<1, 256, 0, h->stream>>>(h->L, (const ST*)h->buf[b], h->refrho,
+                                                         h->cs[b], h->alpha, direct, x,
+                                                         h->h_pinned);
+    CK(cudaGetLastError());
+    return LBM_OK;
+  });
+  if (st) return st;
   CK(cudaStreamSynchronize(h->stream));
   *Qv = h->h_pinned[0];
   if (!isfinite(*Qv)) return set_err(LBM_ENONFINITE, "non-finite volume flow");
@@ -2658,17 +2702,12 @@ int lbm_mix_separation(lbm_mix* h, double* CL, double* Cl_tilde, double* mdot_a,
   int st = check_handle(h);
   if (st) return st;
   double rec[NREC];
-  if ((st = latest_record(h, rec))) return st;
+  if ((st = latest_record(h, rec, Cl_profile))) return st;
   if (CL) *CL = rec[1];
   if (Cl_tilde) *Cl_tilde = rec[2];
   if (mdot_a) *mdot_a = rec[3];
   if (mdot_b) *mdot_b = rec[4];
   if (x_min) *x_min = (int)rec[5];
-  if (Cl_profile) {
-    CK(cudaMemcpyAsync(Cl_profile, h->clprof, sizeof(double) * h->L.Nx, cudaMemcpyDeviceToHost,
-                       h->stream));
-    CK(cudaStreamSynchronize(h->stream));
-  }
   return LBM_OK;
 }
 
@@ -2861,8 +2900,7 @@ struct lbm_sweep {
   int n = 0;
   lbm_mix** h = nullptr;
   cudaStream_t stream = nullptr;
-  double* resid = nullptr;    // [n] residuals of a check
-  double* h_resid = nullptr;  // the same, pinned
+  double* h_resid = nullptr;  // [n] residuals of a check, pinned
   int policy = -1;            // schedule in use (-1: the library default)
   double round_ms[LBM_SWEEP_NPOLICY] = {};
 };
@@ -3028,10 +3066,9 @@ int batch_residuals(lbm_sweep* s, lbm_mix* const* hs, int n, long k) {
       B.inst[q] = ResidInst{h->cs[h->cur], h->cs_snap, 4L * h->L.Nx, h->have_snap ? 1 : 0};
       h->have_snap = true;
     }
-    lbm_residual_kernel<TILE_BATCH><<<m, 1024, 0, s->stream>>>(B, (double)k, s->resid + q0);
+    lbm_residual_kernel<TILE_BATCH><<<m, 1024, 0, s->stream>>>(B, (double)k, s->h_resid + q0);
     CK(cudaGetLastError());
   }
-  CK(cudaMemcpyAsync(s->h_resid, s->resid, sizeof(double) * n, cudaMemcpyDeviceToHost, s->stream));
   CK(cudaStreamSynchronize(s->stream));
   return LBM_OK;
 }
@@ -3070,7 +3107,6 @@ int lbm_sweep_create(const lbm_mix_params* params, int n, lbm_sweep** out) {
   }
   s->n = n;
   cudaError_t e = cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&s->resid, sizeof(double) * n);
   if (e == cudaSuccess) e = cudaMallocHost((void**)&s->h_resid, sizeof(double) * n);
   for (auto kern : {(const void*)lbm_tile_kernel<8>, (const void*)lbm_tile_kernel<TILE_BATCH>})
     if (e == cudaSuccess)
@@ -3101,7 +3137,6 @@ void lbm_sweep_destroy(lbm_sweep* s) {
   for (int i = 0; i < s->n; ++i)
     if (s->h) lbm_mix_destroy(s->h[i]);
   free(s->h);
-  cudaFree(s->resid);
   if (s->h_resid) cudaFreeHost(s->h_resid);
   if (s->stream) cudaStreamDestroy(s->stream);
   delete s;
