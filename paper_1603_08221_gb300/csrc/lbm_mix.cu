@@ -848,21 +848,23 @@ __device__ __forceinline__ void wall_prologue(const Lat& L, const ST* __restrict
 // One thread per column and task (blockIdx.y: 0, 1 = r of the bottom, top
 // wall; 2, 3 = 1/tau_q of the bottom, top half): r_out [2][Nx] (species
 // pair), omq_out [2][Nx].
+constexpr int WALL_COLS = 128;  // columns of a block
 template <typename ST>
-__global__ void __launch_bounds__(128) lbm_walls_kernel(Lat L, const ST* __restrict__ fin,
-                                                        const float* __restrict__ refrho,
-                                                        const double* __restrict__ cs_in,
-                                                        const float* __restrict__ alpha,
-                                                        float2* __restrict__ r_out,
-                                                        float* __restrict__ omq_out) {
+__device__ __forceinline__ void walls_cta(const Lat& L, int block, int task,
+                                          const ST* __restrict__ fin,
+                                          const float* __restrict__ refrho,
+                                          const double* __restrict__ cs_in,
+                                          const float* __restrict__ alpha,
+                                          float2* __restrict__ r_out,
+                                          float* __restrict__ omq_out) {
   pdl_launch_dependents();
   pdl_wait();
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  const int x = block * WALL_COLS + threadIdx.x;
   if (x >= L.Nx) return;
-  const int wall = blockIdx.y & 1;
-  const bool tq = blockIdx.y >= 2;
+  const int wall = task & 1;
+  const bool tq = task >= 2;
   const ColRef C = col_ref(L, refrho, x);
-  const Ends E = ends_of<ST>(L, cs_in, refrho, blockIdx.x * blockDim.x, blockDim.x);
+  const Ends E = ends_of<ST>(L, cs_in, refrho, block * WALL_COLS, WALL_COLS);
   float2 rv;
   float v;
   wall_task(L, fin, alpha, E, C, x, wall, tq, rv, v);
@@ -870,6 +872,13 @@ __global__ void __launch_bounds__(128) lbm_walls_kernel(Lat L, const ST* __restr
     omq_out[wall * L.Nx + x] = v;
   else
     r_out[wall * L.Nx + x] = rv;
+}
+template <typename ST>
+__global__ void __launch_bounds__(WALL_COLS)
+    lbm_walls_kernel(Lat L, const ST* __restrict__ fin, const float* __restrict__ refrho,
+                     const double* __restrict__ cs_in, const float* __restrict__ alpha,
+                     float2* __restrict__ r_out, float* __restrict__ omq_out) {
+  walls_cta(L, blockIdx.x, blockIdx.y, fin, refrho, cs_in, alpha, r_out, omq_out);
 }
 
 // Compensated FP32 running sum (Kahan): a thread's partial over its rows of
@@ -1336,21 +1345,24 @@ __global__ void __launch_bounds__(TX* TY, 3) lbm_step_kernel(Lat L, StepArgs<ST>
   step_cta<ST, WK>(L, a, gp, DIAG);
 }
 
-// One step of several channels (FP32 storage, wall prologue) as one launch:
-// the CTAs of channel q are [block0[q], block0[q + 1]), strips fastest, as in
-// the channel's own grid.  A sweep of 52 channels of 700 x 20 spent 147 us per
-// step on 52 launches from as many graphs, 2.8 us each.
+// One step of several channels (FP32 storage) as one launch: the CTAs of
+// channel q are [block0[q], block0[q + 1]), strips fastest, as in the channel's
+// own grid.  A sweep of 52 channels of 700 x 20 spent 147 us per step on 52
+// launches from as many graphs, 2.8 us each.  WK: r and 1/tau_q come from
+// lbm_walls_batch_kernel ahead of it, blocks of it first channel first too.
 struct StepInst {
   Lat L;
   StepArgs<float> a;
+  float2* wall_r;
+  float* wall_omq;
   int strips, blocks, diag;
 };
 template <int NI>
 struct StepBatch {
-  int block0[NI + 1];
+  int block0[NI + 1], wall0[NI + 1];
   StepInst inst[NI];
 };
-template <int NI>
+template <int NI, bool WK>
 __global__ void __launch_bounds__(TX* TY, 3)
     lbm_step_batch_kernel(const __grid_constant__ StepBatch<NI> B) {
   int q = 0;
@@ -1358,9 +1370,17 @@ __global__ void __launch_bounds__(TX* TY, 3)
   const StepInst& I = B.inst[q];
   const int b = (int)blockIdx.x - B.block0[q];
   const GridPos gp{b % I.strips, b / I.strips, I.strips, I.blocks};
-  step_cta<float, false>(I.L, I.a, gp, I.diag != 0);
+  step_cta<float, WK>(I.L, I.a, gp, I.diag != 0);
 }
-
+template <int NI>
+__global__ void __launch_bounds__(WALL_COLS)
+    lbm_walls_batch_kernel(const __grid_constant__ StepBatch<NI> B) {
+  int q = 0;
+  while ((int)blockIdx.x >= B.wall0[q + 1]) ++q;
+  const StepInst& I = B.inst[q];
+  walls_cta(I.L, (int)blockIdx.x - B.wall0[q], blockIdx.y, I.a.fin, I.a.refrho, I.a.cs_in,
+            I.a.alpha, I.wall_r, I.wall_omq);
+}
 
 #include "lbm_tile.cuh"
 
@@ -2001,8 +2021,8 @@ int launch_step(lbm_mix* h, bool diag) {
     cfg.numAttrs = 1;
     const bool wk = sizeof(ST) < 4 || uses_wall_kernel(h);
     if (wk) {
-      cfg.gridDim = dim3((h->L.Nx + 127) / 128, 4);
-      cfg.blockDim = dim3(128);
+      cfg.gridDim = dim3((h->L.Nx + WALL_COLS - 1) / WALL_COLS, 4);
+      cfg.blockDim = dim3(WALL_COLS);
       CK(cudaLaunchKernelEx(&cfg, lbm_walls_kernel<ST>, h->L, a.fin, (const float*)h->refrho,
                             (const double*)a.cs_in, (const float*)h->alpha, h->wall_r,
                             h->wall_omq));
@@ -2987,9 +3007,10 @@ int launch_step_batch(lbm_mix* const* hs, int n, bool end, cudaStream_t st) {
   long strip_rows = 0;
   for (int q = 0; q < n; ++q) strip_rows += (long)hs[q]->L.N * hs[q]->nblocks;
   const long most = (strip_rows / (WAVES * 3L * (hs[0]->nsm > 0 ? hs[0]->nsm : 1)) + TY - 1) / TY * TY;
-  int blocks = 0;
+  int blocks = 0, walls = 0;
   for (int q = 0; q < STEP_BATCH; ++q) {
     B.block0[q] = blocks;
+    B.wall0[q] = walls;
     if (q >= n) continue;
     lbm_mix* h = hs[q];
     StepInst& I = B.inst[q];
@@ -3003,11 +3024,23 @@ int launch_step_batch(lbm_mix* const* hs, int n, bool end, cudaStream_t st) {
     I.blocks = (h->L.N + I.a.rows_per_block - 1) / I.a.rows_per_block;
     I.diag = end || (h->steps + 1) % h->p.diag_every == 0;
     blocks += I.strips * I.blocks;
+    walls += (h->L.Nx + WALL_COLS - 1) / WALL_COLS;
+    I.wall_r = h->wall_r;
+    I.wall_omq = h->wall_omq;
     h->cur = 1 - h->cur;
     h->steps++;
   }
   B.block0[STEP_BATCH] = blocks;
-  return launch_batch(lbm_step_batch_kernel<STEP_BATCH>, B, dim3(blocks), dim3(TX, TY), 0, st);
+  B.wall0[STEP_BATCH] = walls;
+  // the wall kernel by the rule of a lone channel's step (uses_wall_kernel)
+  if (blocks < WALL_KERNEL_WAVES * 3L * (hs[0]->nsm > 0 ? hs[0]->nsm : 1))
+    return launch_batch(lbm_step_batch_kernel<STEP_BATCH, false>, B, dim3(blocks), dim3(TX, TY), 0,
+                        st);
+  int s = launch_batch(lbm_walls_batch_kernel<STEP_BATCH>, B, dim3(walls, 4), dim3(WALL_COLS), 0,
+                       st);
+  if (s) return s;
+  return launch_batch(lbm_step_batch_kernel<STEP_BATCH, true>, B, dim3(blocks), dim3(TX, TY), 0,
+                      st);
 }
 
 // nsteps steps of the n channels hs of a sweep, on its stream.  Channels that
