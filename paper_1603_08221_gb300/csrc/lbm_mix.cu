@@ -1345,6 +1345,20 @@ __global__ void __launch_bounds__(TX* TY, 3) lbm_step_kernel(Lat L, StepArgs<ST>
   step_cta<ST, WK>(L, a, gp, DIAG);
 }
 
+// The channel whose CTAs [block0[q], block0[q + 1]) hold b, by bisection.
+template <int NI>
+__device__ __forceinline__ int channel_of(const int* block0, int b) {
+  int lo = 0, hi = NI;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (b >= block0[mid])
+      lo = mid;
+    else
+      hi = mid;
+  }
+  return lo;
+}
+
 // One step of several channels (FP32 storage) as one launch: the CTAs of
 // channel q are [block0[q], block0[q + 1]), strips fastest, as in the channel's
 // own grid.  A sweep of 52 channels of 700 x 20 spent 147 us per step on 52
@@ -1365,8 +1379,7 @@ struct StepBatch {
 template <int NI, bool WK>
 __global__ void __launch_bounds__(TX* TY, 3)
     lbm_step_batch_kernel(const __grid_constant__ StepBatch<NI> B) {
-  int q = 0;
-  while ((int)blockIdx.x >= B.block0[q + 1]) ++q;
+  const int q = channel_of<NI>(B.block0, blockIdx.x);
   const StepInst& I = B.inst[q];
   const int b = (int)blockIdx.x - B.block0[q];
   const GridPos gp{b % I.strips, b / I.strips, I.strips, I.blocks};
@@ -1375,8 +1388,7 @@ __global__ void __launch_bounds__(TX* TY, 3)
 template <int NI>
 __global__ void __launch_bounds__(WALL_COLS)
     lbm_walls_batch_kernel(const __grid_constant__ StepBatch<NI> B) {
-  int q = 0;
-  while ((int)blockIdx.x >= B.wall0[q + 1]) ++q;
+  const int q = channel_of<NI>(B.wall0, blockIdx.x);
   const StepInst& I = B.inst[q];
   walls_cta(I.L, (int)blockIdx.x - B.wall0[q], blockIdx.y, I.a.fin, I.a.refrho, I.a.cs_in,
             I.a.alpha, I.wall_r, I.wall_omq);

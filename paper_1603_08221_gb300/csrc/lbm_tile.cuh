@@ -162,9 +162,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 1)
     lbm_tile_kernel(const __grid_constant__ TileBatch<NI> B) {
   extern __shared__ float2 tile_mem[];
   pdl_launch_dependents();
-  int ii = 0;
-  if (NI > 1)
-    while ((int)blockIdx.x >= B.block0[ii + 1]) ++ii;
+  const int ii = channel_of<NI>(B.block0, blockIdx.x);
   const TileInst& I = B.inst[ii];
   const LatCore& L = I.L;
   const int b = (int)blockIdx.x - B.block0[ii], k = B.k;
