@@ -456,6 +456,32 @@ __device__ __forceinline__ void pull_fast(const ST* __restrict__ p, const ST* __
   g[8] = fma2(L.cw5_2, dl, Stor<ST>::ld2(pl + 8 * PS + RS));
 }
 
+// pull_fast for a strip that holds column 1 or N_x - 2: their neighbours
+// outside are the virtual ghost columns (src), everything else is as above.
+template <typename ST>
+__device__ __forceinline__ void pull_edge(const ST* __restrict__ f, const ST* __restrict__ p,
+                                          const ST* __restrict__ pl, const ST* __restrict__ pr,
+                                          const Lat& L, const Ends& E, const ColRef& C, int x,
+                                          int j, float2 g[9]) {
+  pull_fast(p, pl, pr, L, C, g);
+  if (x == 1) {
+    auto ghost = [&](int sp, int i, int js, float cw) {
+      return fmaf(cw, C.dl[sp], src(f, L, E, cw, sp, i, js, 0));
+    };
+    g[1] = make_float2(ghost(0, 1, j, L.cw1[0]), ghost(1, 1, j, L.cw1[1]));
+    g[5] = make_float2(ghost(0, 5, j - 1, L.cw5[0]), ghost(1, 5, j - 1, L.cw5[1]));
+    g[8] = make_float2(ghost(0, 8, j + 1, L.cw5[0]), ghost(1, 8, j + 1, L.cw5[1]));
+  }
+  if (x == L.Nx - 2) {
+    auto ghost = [&](int sp, int i, int js, float cw) {
+      return fmaf(cw, C.dr[sp], src(f, L, E, cw, sp, i, js, L.Nx - 1));
+    };
+    g[3] = make_float2(ghost(0, 3, j, L.cw1[0]), ghost(1, 3, j, L.cw1[1]));
+    g[6] = make_float2(ghost(0, 6, j - 1, L.cw5[0]), ghost(1, 6, j - 1, L.cw5[1]));
+    g[7] = make_float2(ghost(0, 7, j + 1, L.cw5[0]), ghost(1, 7, j + 1, L.cw5[1]));
+  }
+}
+
 // ---------------------------------------------------------------- moments
 // The node arithmetic is written with explicit fma, mul and add wherever a
 // product feeds a sum, so that every kernel that inlines it rounds alike:
@@ -1029,6 +1055,18 @@ struct GridPos {
   int strip, block;     // strip and row block of this CTA
   int strips, blocks;   // of the channel
 };
+// The place of CTA b of a channel: the row blocks of the two end strips first,
+// then the other strips, row block by row block (the shorter last ones fill
+// the tail of the launch).  The end strips also reduce their column sums at
+// every step, a chain of some microseconds; last in the grid, it and their
+// rows were a tail of 14 us of a 107 us step (BF16 16384 x 256) and of 9 us of
+// 27 us (FP16 5001 x 130).
+__device__ __forceinline__ GridPos grid_pos(const LatCore& L, int b, int strips, int blocks) {
+  if (L.x_periodic || strips < 3) return GridPos{b % strips, b / strips, strips, blocks};
+  const int inner = strips - 2, r = b - 2 * blocks;
+  if (r < 0) return GridPos{(b & 1) ? strips - 1 : 0, b >> 1, strips, blocks};
+  return GridPos{1 + r % inner, r / inner, strips, blocks};
+}
 template <bool DIAG, typename ST>
 __device__ __forceinline__ void column_epilogue(const Lat& L, const StepArgs<ST>& a,
                                                 const GridPos& gp, int x, const double acc[4],
@@ -1279,6 +1317,8 @@ __device__ __forceinline__ void step_cta(const Lat& L, const StepArgs<ST>& a, co
       if (tx == 0 && j + TY < j_end) prefetch_row_l2(p + TY * RS);
       if (!edge_strip && j != 0 && j != L.N - 1) {
         pull_fast(p, p + offl, p + offr, L, C, g);
+      } else if (j != 0 && j != L.N - 1) {
+        pull_edge(a.fin, p, p + offl, p + offr, L, E, C, x, j, g);
       } else {
         float fs[2][9];
         pull_node(a.fin, L, E, C, x, j, wall_r(0), wall_r(1), fs);
@@ -1341,7 +1381,8 @@ __device__ __forceinline__ void step_cta(const Lat& L, const StepArgs<ST>& a, co
 
 template <typename ST, bool DIAG, bool WK = (sizeof(ST) < 4)>
 __global__ void __launch_bounds__(TX* TY, 3) lbm_step_kernel(Lat L, StepArgs<ST> a) {
-  const GridPos gp{(int)blockIdx.x, (int)blockIdx.y, (int)gridDim.x, (int)gridDim.y};
+  const GridPos gp =
+      grid_pos(L, blockIdx.y * gridDim.x + blockIdx.x, (int)gridDim.x, (int)gridDim.y);
   step_cta<ST, WK>(L, a, gp, DIAG);
 }
 
@@ -1382,7 +1423,7 @@ __global__ void __launch_bounds__(TX* TY, 3)
   const int q = channel_of<NI>(B.block0, blockIdx.x);
   const StepInst& I = B.inst[q];
   const int b = (int)blockIdx.x - B.block0[q];
-  const GridPos gp{b % I.strips, b / I.strips, I.strips, I.blocks};
+  const GridPos gp = grid_pos(I.L, b, I.strips, I.blocks);
   step_cta<float, WK>(I.L, I.a, gp, I.diag != 0);
 }
 template <int NI>
