@@ -140,7 +140,7 @@ int lbm_mix_init(lbm_mix* h);
  * halos, see lbm_mix_set_rows_per_block); a call gives the same bits however
  * its steps are split over calls.  All others take one fused collide-stream
  * pass per step: with 16-bit storage, and with FP32 storage when the step's
- * grid holds two or more waves of CTAs on the device, a small kernel computes
+ * grid holds several waves of CTAs on the device, a small kernel computes
  * r (Eq. R) and tau_q (Eq. taoq) of every column ahead of each pass.  All
  * are launched with programmatic dependent launch.  Every
  * diag_every-th step (counted from init) and the last step of the call
@@ -255,8 +255,8 @@ int lbm_mix_dims(const lbm_mix* h, int* N, int* N_x, long* steps);
 
 /* Kernel launches of an lbm_mix_step call of one step under h's current
  * schedule (lbm_mix_set_rows_per_block): 2 when the wall kernel runs ahead of
- * the step kernel (16-bit storage; FP32 grids of two or more waves of CTAs)
- * and for channels that take several steps per launch (the steps and their
+ * the step kernel (16-bit storage; FP32 grids of five or more waves of CTAs,
+ * two or more under a schedule set by the caller) and for channels that take several steps per launch (the steps and their
  * records; longer calls need fewer per step), else 1; re-referencing adds its
  * own.  Returns the count, or LBM_EINVAL
  * for a NULL handle. */
@@ -321,7 +321,7 @@ int lbm_mix_step_noalloc(const lbm_mix_params* p, const float* d_in, float* d_ou
 
 /* Node-to-CTA schedule of h: rows of one strip handled by one CTA of the
  * step kernel, a multiple of 8 (capped at N rounded up to 8); 0 restores the
- * library default (16 to 80 rows by the channel's size; several steps per
+ * library default (16 to 96 rows by the channel's size; several steps per
  * launch where the channel qualifies, see lbm_mix_step, which a row count
  * turns off).  Changes only
  * the order of the FP64 column reductions.  May allocate; not during stream capture.

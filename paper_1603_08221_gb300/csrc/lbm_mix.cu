@@ -1912,17 +1912,18 @@ unsigned host_hash32(unsigned x) {
 }
 
 // Rows of one strip per CTA of the step kernel unless the caller sets a
-// schedule: as many as leave WAVES waves of resident CTAs (3 per SM), a
-// multiple of TY within [16, 56] (FP32) or [16, 80] (16-bit).  A warp takes
+// schedule: as many as leave `waves` waves of resident CTAs (3 per SM), a
+// multiple of TY within [16, 56] (FP32) or [16, 96] (16-bit).  A warp takes
 // its CTA's rows one after another, every TY-th, so on a channel of few strips
 // fewer rows per CTA shorten the step until the CTAs' own start-up counts.
-// Measured on GB300, us per step at 96 rows (the rule before) and at this
-// rule's count: FP32 5001 x 130 54.5 -> 34.6 (16 rows), 8000 x 128 67.7 ->
-// 43.9 (16), 16384 x 256 131 -> 117 (40), 32768 x 512 396.6 -> 384.6 (56);
-// BF16 67.8 -> 35.5, 72.6 -> 43.9, 131 -> 105, 313 -> 312 (80).
-constexpr int WAVES = 8;
+// Measured on GB300, us per step at 96 rows and at this rule's count: FP32
+// 5001 x 130 37.8 -> 26.0 (16 rows), 8000 x 128 42.8 -> 32.6 (24), 20000 x 64
+// 39.5 (32), 16384 x 256 104 -> 102 (56), 32768 x 512 367 -> 367 (56); BF16
+// 39.9 -> 27.9 (16), 42.2 -> 34.4 (24), 16384 x 256 102 (96), 32768 x 512 345
+// (96).
+constexpr int WAVES = 3;
 int default_rows(int N, int strips, int nsm, bool fp32) {
-  const int n8 = (N + TY - 1) / TY * TY, most = fp32 ? 56 : 80;
+  const int n8 = (N + TY - 1) / TY * TY, most = fp32 ? 56 : 96;
   const long ctas = (long)WAVES * 3 * (nsm > 0 ? nsm : 1);
   long rows = ((long)N * strips / ctas + TY - 1) / TY * TY;
   rows = rows < 16 ? 16 : rows < most ? rows : most;
@@ -2019,14 +2020,18 @@ int reset_diag(lbm_mix* h) {
 
 // FP32 storage takes r and tau_q from lbm_walls_kernel when the step's grid
 // holds at least WALL_KERNEL_WAVES waves of resident CTAs (3 per SM): there
-// the CTA prologue's barrier costs more than a launch of its own (0.400
-// against 0.406 ms on the 32768 x 512 channel).  A grid of a wave or less,
-// like the channels of a parametric sweep, keeps the prologue, which costs
-// less than the extra launch.  16-bit storage always uses the wall kernel.
-constexpr long WALL_KERNEL_WAVES = 2;
+// the prologue's barrier in every CTA costs more than a launch and its 7 us
+// (32768 x 512, 22 waves: 369.5 against 367 us; 15000 x 300, 6.2 waves: 109.0
+// against 108.2; the other way 5001 x 130, 3.1 waves: 25.9 against 31.8, and
+// 20000 x 64, 4.1 waves: 37.6 against 42.5).  A schedule that the caller
+// set, often of few rows per CTA, and the launches of a sweep take it from two
+// waves on (64 x 6000 at 8 rows: 23.5 against 20.5 us; 24 mixed channels 98.6
+// against 101.4).  16-bit storage always uses the wall kernel.
+constexpr long WALL_KERNEL_WAVES = 5, WALL_KERNEL_WAVES_SET = 2;
 bool uses_wall_kernel(const lbm_mix* h) {
   const long ctas = (long)h->nblocks * (long)h->R;
-  return ctas >= WALL_KERNEL_WAVES * 3L * (long)(h->nsm > 0 ? h->nsm : 1);
+  const long waves = h->rows_set ? WALL_KERNEL_WAVES_SET : WALL_KERNEL_WAVES;
+  return ctas >= waves * 3L * (long)(h->nsm > 0 ? h->nsm : 1);
 }
 
 // Arguments of h's next step.
@@ -2117,12 +2122,11 @@ double tile_cost(int N, int nup, int W, int k, int sms) {
   const double nodes = (double)k * (W + k - 1) * tile_stride(N);
   return (TILE_LAUNCH_US + waves * (TILE_LOAD_US + k * TILE_STEP_US + TILE_NODE_US * nodes)) / k;
 }
-// The same for the step kernel under its default schedule (measured from
-// 96 x 1600, 20.7 us, to 128 x 8000, 43.9 us): below about 600 000 nodes of
-// at most 64 rows the tiles win (64 x 6000: 17.0 against 23.6 us), with 128
-// rows only up to 1300 columns (13.2 against 18.3 us; 2560: 25.1 against
-// 23.9).
-double step_kernel_cost(int N, int Nx) { return 14.0 + 2.9e-5 * (double)N * Nx; }
+// The same for the step kernel under its default schedule (measured from 64 x
+// 3000, 18.3 us, to 128 x 8000, 32.6 us): below some 400 000 nodes of at most 64
+// rows the tiles win (64 x 6000: 17.0 against 19.1 us), with 128 rows only up
+// to 1300 columns (13.2 against 18 us).
+double step_kernel_cost(int N, int Nx) { return 15.0 + 1.75e-5 * (double)N * Nx; }
 
 // Tile width and steps per launch (odd, so that launches alternate the two
 // buffers as single steps do) of least estimated cost on `sms` SMs; W = 0
@@ -3059,7 +3063,7 @@ int launch_step_batch(lbm_mix* const* hs, int n, bool end, cudaStream_t st) {
   // than a channel's own schedule has
   long strip_rows = 0;
   for (int q = 0; q < n; ++q) strip_rows += (long)hs[q]->L.N * hs[q]->nblocks;
-  const long most = (strip_rows / (WAVES * 3L * (hs[0]->nsm > 0 ? hs[0]->nsm : 1)) + TY - 1) / TY * TY;
+  const long most = (strip_rows / (8 * 3L * (hs[0]->nsm > 0 ? hs[0]->nsm : 1)) + TY - 1) / TY * TY;
   int blocks = 0, walls = 0;
   for (int q = 0; q < STEP_BATCH; ++q) {
     B.block0[q] = blocks;
@@ -3085,8 +3089,7 @@ int launch_step_batch(lbm_mix* const* hs, int n, bool end, cudaStream_t st) {
   }
   B.block0[STEP_BATCH] = blocks;
   B.wall0[STEP_BATCH] = walls;
-  // the wall kernel by the rule of a lone channel's step (uses_wall_kernel)
-  if (blocks < WALL_KERNEL_WAVES * 3L * (hs[0]->nsm > 0 ? hs[0]->nsm : 1))
+  if (blocks < WALL_KERNEL_WAVES_SET * 3L * (hs[0]->nsm > 0 ? hs[0]->nsm : 1))
     return launch_batch(lbm_step_batch_kernel<STEP_BATCH, false>, B, dim3(blocks), dim3(TX, TY), 0,
                         st);
   int s = launch_batch(lbm_walls_batch_kernel<STEP_BATCH>, B, dim3(walls, 4), dim3(WALL_COLS), 0,
