@@ -907,10 +907,7 @@ __global__ void __launch_bounds__(WALL_COLS)
   walls_cta(L, blockIdx.x, blockIdx.y, fin, refrho, cs_in, alpha, r_out, omq_out);
 }
 
-// Compensated FP32 running sum (Kahan): a thread's partial over its rows of
-// one column, accurate to ~1 FP32 ulp of the sum, handed to the FP64 column
-// reduction at the end of the sweep (FP64 arithmetic is a slow pipe on this
-// part).
+// Compensated FP32 running sum (Kahan), accurate to ~1 FP32 ulp of the sum.
 struct KahanF {
   float s = 0.0f, c = 0.0f;
   __device__ __forceinline__ void add(float v) {
@@ -919,8 +916,26 @@ struct KahanF {
     c = (t - s) - y;
     s = t;
   }
-  __device__ __forceinline__ double value() const { return (double)s - (double)c; }
 };
+
+// Running sums of two quantities with the rounding error of every addition
+// kept (Knuth's two-sum, packed): a thread's partials over its rows of one
+// column, handed to column_epilogue.  Seven packed instructions where two
+// KahanF take eight, and no bits lost where the sum's sign changes.
+struct Sum2 {
+  float2 s = {0.0f, 0.0f}, e = {0.0f, 0.0f};
+  __device__ __forceinline__ void add(float2 v) {
+    const float2 t = add2(s, v), b = sub2(t, s);
+    e = add2(e, add2(sub2(s, sub2(t, b)), sub2(v, b)));
+    s = t;
+  }
+};
+
+// Sum of two (sum, error) pairs of floats, to about 2^-46 of its larger terms.
+__device__ __forceinline__ float2 pair_add(float2 a, float2 b) {
+  const float2 s = two_sum(a.x, b.x);
+  return quick_two_sum(s.x, __fadd_rn(s.y, __fadd_rn(a.y, b.y)));
+}
 
 // Sum of v(0) .. v(N - 1), the rows of a column, by eight neighbouring lanes
 // (sub = lane & 7, every lane of the warp here): each
@@ -999,12 +1014,12 @@ struct StepArgs {
   const double* __restrict__ cs_in;  // [4][Nx] column sums of the state in fin
   double* __restrict__ cs_out;       // [4][Nx] column sums of the state of step t
   const float* __restrict__ alpha;   // [2][Nx]
-  double* __restrict__ partials;     // [gridDim.x][NPART]
+  double* __restrict__ partials;     // [NPART][strips]
   unsigned* __restrict__ counter;
   double* __restrict__ diag;         // [DIAG_CAP][NREC]
   unsigned long long* __restrict__ diag_count;
   double* __restrict__ clprof;       // [Nx]
-  double* __restrict__ colpart;      // [R][4][Nx] per-row-block column sums (R > 1)
+  float2* __restrict__ colpart;      // [R][4][Nx] per-row-block column sums (R > 1)
   unsigned* __restrict__ strip_cnt;  // [strips] row blocks finished this step
   int rows_per_block;                // rows of one row block (multiple of TY)
   unsigned seed;                     // 16-bit storage: per-step seed of the
@@ -1020,10 +1035,9 @@ struct StepArgs {
 };
 
 struct RedSmem {
-  double col[4][TY][TX];
-  double wsum[TY][6];
-  double wmin[TY];
-  int wimin[TY];
+  float2 col[4][TY][TX];
+  double total[4][TX];
+  double sum[NPART];
   int last;
   int last_strip;
 };
@@ -1046,10 +1060,6 @@ __device__ __forceinline__ void warp_min(double& v, int& idx) {
   }
 }
 
-// Column sums -> next step's density correction, C_l(x), per-CTA partials;
-// the last CTA to finish reduces the partials in CTA order into one record.
-// DIAG = false: only the column sums (the next step's Eq. rho2 input) are
-// produced; DIAG = true: also C_l(x), the per-strip partials and the record.
 // g: the CTA's place in its channel's grid.
 struct GridPos {
   int strip, block;     // strip and row block of this CTA
@@ -1067,34 +1077,42 @@ __device__ __forceinline__ GridPos grid_pos(const LatCore& L, int b, int strips,
   if (r < 0) return GridPos{(b & 1) ? strips - 1 : 0, b >> 1, strips, blocks};
   return GridPos{1 + r % inner, r / inner, strips, blocks};
 }
+// Column sums -> next step's density correction, C_l(x), per-strip partials;
+// the last CTA to finish reduces the partials in strip order into one record.
+// DIAG = false: only the column sums (the next step's Eq. rho2 input) are
+// produced; DIAG = true: also C_l(x), the per-strip partials and the record.
+// Every CTA of a DIAG step comes here, and an FP64 instruction holds its SM
+// sub-partition for some 64 cycles; the sums of a CTA are therefore pairs of
+// floats, by one warp per quantity, and FP64 begins at the strip's totals.
+// Sums in FP64 throughout, most of them in one warp, cost a DIAG step of
+// 32768 x 512 80 us beyond the others (45 now, mostly the fence and the ticket
+// of each CTA), one of 5001 x 130 29 us (14), and the end strips' chain of
+// every step 4 us of 27.5 there (FP32).
 template <bool DIAG, typename ST>
 __device__ __forceinline__ void column_epilogue(const Lat& L, const StepArgs<ST>& a,
-                                                const GridPos& gp, int x, const double acc[4],
+                                                const GridPos& gp, int x, const Sum2 acc[2],
                                                 RedSmem& rs) {
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int tid = ty * TX + tx;
   const int R = gp.blocks;  // row blocks per strip
+  const bool in = interior(L, x);
 #pragma unroll
-  for (int k = 0; k < 4; ++k) rs.col[k][ty][tx] = acc[k];
+  for (int k = 0; k < 2; ++k) {
+    rs.col[2 * k][ty][tx] = make_float2(acc[k].s.x, acc[k].e.x);
+    rs.col[2 * k + 1][ty][tx] = make_float2(acc[k].s.y, acc[k].e.y);
+  }
   __syncthreads();
-  double c[4];
-  if (ty == 0) {
+  float2 c = make_float2(0.0f, 0.0f);  // quantity ty of column x, in warps 0 .. 3
+  if (ty < 4) {
+    c = rs.col[ty][0][tx];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      double v = 0.0;
-      for (int t = 0; t < TY; ++t) v += rs.col[k][t][tx];
-      c[k] = v;
-    }
+    for (int t = 1; t < TY; ++t) c = pair_add(c, rs.col[ty][t][tx]);
   }
   if (R > 1) {
     // Row-block partials of this strip; the last of its R CTAs to finish
     // adds them in row-block order (independent of arrival order).
-    if (ty == 0) {
-      if (x < L.Nx) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          a.colpart[((size_t)gp.block * 4 + k) * L.Nx + x] = c[k];
-      }
+    if (ty < 4) {
+      if (x < L.Nx) a.colpart[((size_t)gp.block * 4 + ty) * L.Nx + x] = c;
       __threadfence();  // the writers publish before the ticket is taken
     }
     __syncthreads();
@@ -1104,53 +1122,53 @@ __device__ __forceinline__ void column_epilogue(const Lat& L, const StepArgs<ST>
     }
     __syncthreads();
     if (!rs.last_strip) return;
-    if (ty == 0) {
-      __threadfence();
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        double v = 0.0;
-        if (x < L.Nx)
-          for (int r = 0; r < R; ++r) v += __ldcg(a.colpart + ((size_t)r * 4 + k) * L.Nx + x);
-        c[k] = v;
-      }
-      if (tx == 0) a.strip_cnt[gp.strip] = 0u;
+    __threadfence();
+    if (ty < 4 && x < L.Nx) {
+      const float2* cp = a.colpart + (size_t)ty * L.Nx + x;
+      c = __ldcg(cp);
+#pragma unroll 4
+      for (int r = 1; r < R; ++r) c = pair_add(c, __ldcg(cp + (size_t)r * 4 * L.Nx));
     }
+    if (tid == 0) a.strip_cnt[gp.strip] = 0u;
   }
-  if (sizeof(ST) == 4 && a.end_sd && ty == 0) {
+  if (ty < 4) {
+    // column sum of rho_s = N rhobar_s + sum of deviations
+    double v = pair_value(c);
+    if (ty < 2 && in) v += (double)L.N * (double)a.refrho[ty * L.Nx + x];
+    rs.total[ty][tx] = v;
+  }
+  if (sizeof(ST) == 4 && a.end_sd) {
     // The columns behind the next step's density correction, in the order of
     // column_sum8 over all rows: the populations of a run are then the same
-    // bits under every schedule, this kernel's and lbm_tile_kernel's.
-    const int x0 = x - tx;
-    for (int e = 0; e < 4; ++e) {
-      const int xe = e == 0 ? 1 : e == 1 ? 2 : e == 2 ? L.Nx - 2 : L.Nx - 3;
-      if (xe < x0 || xe >= x0 + TX) continue;  // warp-uniform
-#pragma unroll
-      for (int sp = 0; sp < 2; ++sp) {
-        const float2 v = column_sum8(L.N, tx & 7, [&](int r) {
-          const float2 d = __ldcg(a.end_sd + (size_t)e * L.N + r);
-          return sp ? d.y : d.x;
-        });
-        const double t = pair_value(column_total(L.N, a.refrho[sp * L.Nx + xe], v));
-        if (x == xe) c[sp] = t;
-      }
+    // bits under every schedule, this kernel's and lbm_tile_kernel's.  One
+    // warp for each of the four columns and two species.
+    __syncthreads();
+    const int e = ty >> 1, sp = ty & 1, x0 = x - tx;
+    const int xe = e == 0 ? 1 : e == 1 ? 2 : e == 2 ? L.Nx - 2 : L.Nx - 3;
+    if (xe >= x0 && xe < x0 + TX) {  // warp-uniform
+      const float2 v = column_sum8(L.N, tx & 7, [&](int r) {
+        const float2 d = __ldcg(a.end_sd + (size_t)e * L.N + r);
+        return sp ? d.y : d.x;
+      });
+      const double t = pair_value(column_total(L.N, a.refrho[sp * L.Nx + xe], v));
+      if (x == xe) rs.total[sp][tx] = t;
     }
+    __syncthreads();
   }
-  if (!DIAG) {
-    if (ty == 0 && x < L.Nx) {
-#pragma unroll
-      for (int k = 0; k < 4; ++k) a.cs_out[(size_t)k * L.Nx + x] = c[k];
-    }
-    return;
-  }
-  if (ty == 0) {
-    const bool in = interior(L, x);
-    if (x < L.Nx) {
-#pragma unroll
-      for (int k = 0; k < 4; ++k) a.cs_out[(size_t)k * L.Nx + x] = c[k];
-    }
+  // (a warp writes back the totals that it formed itself, or all have met)
+  if (ty < 4 && x < L.Nx) a.cs_out[(size_t)ty * L.Nx + x] = rs.total[ty][tx];
+  if (!DIAG) return;
+  __syncthreads();
+  // The strip's partials: a quantity's sum over the columns in each of four
+  // warps, C_l in a fifth.
+  double* p = a.partials + gp.strip;
+  if (ty < 4) {
+    const double v = warp_sum(in ? rs.total[ty][tx] : 0.0);
+    if (tx == 0) p[(size_t)(ty < 2 ? 5 + ty : 1 + ty) * gp.strips] = v;
+  } else if (ty == 4) {
     double Cl = 0.0;
     if (in) {
-      double na = c[0] * L.s[0], nb = c[1] * L.s[1];
+      double na = rs.total[0][tx] * L.s[0], nb = rs.total[1][tx] * L.s[1];
       Cl = (L.light == 0 ? na : nb) / (na + nb);
       a.clprof[x] = Cl;
     } else if (x < L.Nx) {
@@ -1159,25 +1177,16 @@ __device__ __forceinline__ void column_epilogue(const Lat& L, const StepArgs<ST>
     double vmin = in ? Cl : INFINITY;
     int imin = in ? x : 0x7fffffff;
     warp_min(vmin, imin);
-    double p_dev = warp_sum(in ? Cl - L.C_in : 0.0);
-    double p_ma = warp_sum(in ? c[2] : 0.0);
-    double p_mb = warp_sum(in ? c[3] : 0.0);
-    double p_ra = warp_sum(in ? c[0] : 0.0);
-    double p_rb = warp_sum(in ? c[1] : 0.0);
-    double p_n = warp_sum(in ? 1.0 : 0.0);
+    const double dev = warp_sum(in ? Cl - L.C_in : 0.0);
+    const int cols = __popc(__ballot_sync(0xffffffffu, in));
     if (tx == 0) {
-      double* p = a.partials + (size_t)gp.strip * NPART;
       p[0] = vmin;
-      p[1] = (double)imin;
-      p[2] = p_dev;
-      p[3] = p_ma;
-      p[4] = p_mb;
-      p[5] = p_ra;
-      p[6] = p_rb;
-      p[7] = p_n;
-      __threadfence();
+      p[(size_t)1 * gp.strips] = (double)imin;
+      p[(size_t)2 * gp.strips] = dev;
+      p[(size_t)7 * gp.strips] = (double)cols;
     }
   }
+  __threadfence();
   __syncthreads();
   if (tid == 0) {
     unsigned ticket = atomicAdd(a.counter, 1u);
@@ -1186,60 +1195,56 @@ __device__ __forceinline__ void column_epilogue(const Lat& L, const StepArgs<ST>
   __syncthreads();
   if (!rs.last) return;
   __threadfence();
-  // Last CTA: every thread folds a fixed subset of the partials in CTA order,
-  // then a fixed shuffle tree per warp and warp order in thread 0, so the
-  // result does not depend on which CTA finished last.
-  const int nt = TX * TY;
-  double vmin = INFINITY, sm[6] = {0, 0, 0, 0, 0, 0};
-  int imin = 0x7fffffff;
-  for (int b = tid; b < gp.strips; b += nt) {
-    const double* p = a.partials + (size_t)b * NPART;
-    double v = __ldcg(p + 0);
-    int i = (int)__ldcg(p + 1);
-    if (v < vmin || (v == vmin && i < imin)) {
-      vmin = v;
-      imin = i;
-    }
-#pragma unroll
-    for (int k = 0; k < 6; ++k) sm[k] += __ldcg(p + 2 + k);
-  }
-  warp_min(vmin, imin);
-#pragma unroll
-  for (int k = 0; k < 6; ++k) sm[k] = warp_sum(sm[k]);
-  const int lane = tid & 31, wid = tid >> 5;
-  if (lane == 0) {
-    rs.wmin[wid] = vmin;
-    rs.wimin[wid] = imin;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) rs.wsum[wid][k] = sm[k];
-  }
-  __syncthreads();
-  if (tid == 0) {
-    double tot[6] = {0, 0, 0, 0, 0, 0};
-    double mn = INFINITY;
-    int im = 0x7fffffff;
-    for (int w = 0; w < nt / 32; ++w) {
-      for (int k = 0; k < 6; ++k) tot[k] += rs.wsum[w][k];
-      if (rs.wmin[w] < mn || (rs.wmin[w] == mn && rs.wimin[w] < im)) {
-        mn = rs.wmin[w];
-        im = rs.wimin[w];
+  // Last CTA: each warp folds one partial over the strips, every lane a fixed
+  // subset in strip order, then a fixed shuffle tree, so the result does not
+  // depend on which CTA finished last.
+  static_assert(TY == NPART, "a warp per partial");
+  if (ty == 0) {
+    double vmin = INFINITY;
+    int imin = 0x7fffffff;
+    for (int b = tx; b < gp.strips; b += TX) {
+      const double v = __ldcg(a.partials + b);
+      const int i = (int)__ldcg(a.partials + gp.strips + b);
+      if (v < vmin || (v == vmin && i < imin)) {
+        vmin = v;
+        imin = i;
       }
     }
-    double dev = tot[0];
+    warp_min(vmin, imin);
+    if (tx == 0) {
+      rs.sum[0] = vmin;
+      rs.sum[1] = (double)imin;
+    }
+  } else if (ty != 1) {
+    double v = 0.0;
+    for (int b = tx; b < gp.strips; b += TX) v += __ldcg(a.partials + (size_t)ty * gp.strips + b);
+    v = warp_sum(v);
+    if (tx == 0) rs.sum[ty] = v;
+  }
+  __syncthreads();
+  if (tid < NREC) {
+    const unsigned long long cnt = *a.diag_count + 1ull;
+    double dev = rs.sum[2];
     if (!L.x_periodic) dev += (L.C_out - L.C_in);  // the outlet boundary column
-    const double ncol = tot[5];
-    unsigned long long cnt = *a.diag_count + 1ull;
-    double* rec = a.diag + (size_t)((cnt - 1ull) % DIAG_CAP) * NREC;
-    rec[0] = (double)cnt;
-    rec[1] = (L.C_in - mn) / L.C_in;
-    rec[2] = dev / ((double)L.Nx * L.C_in);
-    rec[3] = tot[1] / ncol;
-    rec[4] = tot[2] / ncol;
-    rec[5] = (double)im;
-    rec[6] = tot[3];
-    rec[7] = tot[4];
-    *a.diag_count = cnt;
-    *a.counter = 0u;
+    const double ncol = rs.sum[7];
+    // one division for all eight entries
+    double num = 0.0, den = 1.0;
+    switch (tid) {
+      case 0: num = (double)cnt; break;
+      case 1: num = L.C_in - rs.sum[0], den = L.C_in; break;
+      case 2: num = dev, den = (double)L.Nx * L.C_in; break;
+      case 3: num = rs.sum[3], den = ncol; break;
+      case 4: num = rs.sum[4], den = ncol; break;
+      case 5: num = rs.sum[1]; break;
+      case 6: num = rs.sum[5]; break;
+      case 7: num = rs.sum[6]; break;
+    }
+    a.diag[(size_t)((cnt - 1ull) % DIAG_CAP) * NREC + tid] = num / den;
+    __syncwarp((1u << NREC) - 1u);
+    if (tid == 0) {
+      *a.diag_count = cnt;
+      *a.counter = 0u;
+    }
     __threadfence();
   }
 }
@@ -1296,7 +1301,7 @@ __device__ __forceinline__ void step_cta(const Lat& L, const StepArgs<ST>& a, co
   const unsigned base = gp.strip * L.SS + 2 * tx;  // row 0, i = 0, species a of column x
   const int offl = (int)(idx(L, 0, 0, 0, xm) - base), offr = (int)(idx(L, 0, 0, 0, xp) - base);
   const int half = (L.N + 1) / 2;  // rows j < half (1-based 2J <= N+1) use the bottom tau_q
-  KahanF acc[4];
+  Sum2 acc[2];  // species densities, species x momenta
   const bool reduce = diag || edge_strip;
   unsigned rng = 0u;  // generator of the stochastic rounding
   // one run over the rows, with 16-bit storage one per sequence of random bits
@@ -1348,10 +1353,8 @@ __device__ __forceinline__ void step_cta(const Lat& L, const StepArgs<ST>& a, co
         if (end_r >= 0) a.end_sd[end_r * L.N + j] = sd;
       }
       if (reduce) {
-        acc[0].add(sd.x);
-        acc[1].add(sd.y);
-        acc[2].add(mxs.x);
-        acc[3].add(mxs.y);
+        acc[0].add(sd);
+        acc[1].add(mxs);
       }
       ST* o = a.fout + base + j * RS;
       if (sizeof(ST) < 4 && a.seed != 0u) {
@@ -1364,19 +1367,10 @@ __device__ __forceinline__ void step_cta(const Lat& L, const StepArgs<ST>& a, co
     }
   }
   if (!reduce) return;  // CTA-uniform
-  // column sum of rho_s = N rhobar_s + sum of deviations; the reference part
-  // is added once per column (by the ty = 0 thread of the first row block)
-  const bool adds_ref = in && ty == 0 && gp.block == 0;
-  double accd[4];
-#pragma unroll
-  for (int sp = 0; sp < 2; ++sp)
-    accd[sp] = (adds_ref ? (double)L.N * (double)C.rb[sp] : 0.0) + acc[sp].value();
-  accd[2] = acc[2].value();
-  accd[3] = acc[3].value();
   if (diag)
-    column_epilogue<true>(L, a, gp, x, accd, rsm);
+    column_epilogue<true>(L, a, gp, x, acc, rsm);
   else
-    column_epilogue<false>(L, a, gp, x, accd, rsm);
+    column_epilogue<false>(L, a, gp, x, acc, rsm);
 }
 
 template <typename ST, bool DIAG, bool WK = (sizeof(ST) < 4)>
@@ -1750,8 +1744,8 @@ struct lbm_mix {
   float2* wall_r;      // [2][Nx] r per wall and column (lbm_walls_kernel)
   float* wall_omq;     // [2][Nx] 1/tau_q per half and column (lbm_walls_kernel)
   float2* end_sd;      // [4][N] (FP32 storage with pressure ends, else null)
-  double* colpart;     // [R][4][Nx]
-  double* colpart0;    // its place in the arena
+  float2* colpart;     // [R][4][Nx]
+  float2* colpart0;    // its place in the arena
   void* arena;         // holds the arrays above and below but scratch and mom
   unsigned* strip_cnt; // [nblocks]
   int R, rows_per_block;
@@ -1999,7 +1993,7 @@ int set_rows_per_block(lbm_mix* h, int rows) {
   if (rows > nmax) rows = nmax;
   const int R = (h->L.N + rows - 1) / rows;
   if (R > h->R_alloc) {
-    double* cp = nullptr;
+    float2* cp = nullptr;
     CK(cudaStreamSynchronize(h->stream));
     CK(cudaMalloc((void**)&cp, sizeof(double) * 4 * (size_t)h->L.Nx * (size_t)R));
     if (h->colpart != h->colpart0) cudaFree(h->colpart);
@@ -2527,7 +2521,7 @@ int lbm_mix_create(const lbm_mix_params* p, void* stream, lbm_mix** out) {
     carve(base, sizeof(float) * 2 * (size_t)Nx, &h->wall_omq);
     if (p->storage == LBM_FP32 && !p->x_periodic)
       carve(base, sizeof(float2) * 4 * (size_t)h->L.N, &h->end_sd);
-    carve(base, sizeof(double) * 4 * (size_t)Nx * (size_t)h->R, &h->colpart0);
+    carve(base, sizeof(float2) * 4 * (size_t)Nx * (size_t)h->R, &h->colpart0);
     if (h->tile_W > 0) carve(base, sizeof(float2) * 4 * (size_t)Nx * h->hist_rows, &h->hist);
   };
   layout(nullptr);

@@ -1,0 +1,47 @@
+"""The records' sums over columns, row blocks and strips against FP64 sums of the
+populations, over row blocks of every kind (one, several, a short last one),
+widths around the strips, and storage types.
+
+Tolerances, derived.  Between schedules the terms are the same and only their
+order differs: every partial sum is a pair of floats, exact to 2^-44 of the
+largest partial sum, of which there are fewer than 2^10 in a row, so 2^-34 of the
+sums of the terms' magnitudes.  Against the populations: a node's density and
+momentum are formed from nine FP32 deviations and the collision conserves them to
+rounding, fewer than 64 roundings of 2^-24 of the magnitudes, with 16-bit storage
+one more, stochastic, of 2^-7 (BF16) or 2^-10 (FP16) of each stored deviation;
+deviations and reference add up to at most twice the populations' magnitudes."""
+import numpy as np
+import pytest
+
+from paper_1603_08221_gb300 import binding, workloads
+
+pytestmark = pytest.mark.gpu
+
+STORED = {binding.LBM_FP32: 0.0, binding.LBM_BF16: 2.0 ** -7, binding.LBM_FP16: 2.0 ** -10}
+
+
+@pytest.mark.parametrize("storage", list(STORED))
+@pytest.mark.parametrize("N,Nx,periodic", [(3, 6, 0), (17, 33, 0), (64, 98, 0), (131, 257, 0),
+                                           (40, 64, 1)])
+def test_record_sums(storage, N, Nx, periodic):
+    p = workloads.preset("heli_argon_320x16", N=N, N_x=Nx, theta=1.2, Kn_out=0.3, storage=storage,
+                         x_periodic=periodic, wall=periodic, diag_every=1)
+    f0 = workloads.random_post_state(N, Nx, seed=4, lo=0.099, hi=0.101).astype(np.float32)
+    cols = slice(0, Nx) if periodic else slice(1, Nx - 1)
+    first = None
+    for rows in (8, 16, 64, 512):
+        g = binding.LbmMix(**p)
+        g.set_post_state(f0)
+        g.set_rows_per_block(rows)
+        g.step(1)
+        rec = g.history(1)[0]
+        f = np.asarray(g.get_post_state_f64(), dtype=np.float64).reshape(2, 9, N, Nx)[..., cols]
+        total = f.sum(axis=(1, 2, 3))
+        tol = 2 * (64 * 2.0 ** -24 + STORED[storage]) * np.abs(f).sum(axis=(1, 2, 3))
+        assert np.all(np.abs(rec[6:8] - total) <= tol), rows
+        n = f.shape[-1]
+        if first is None:
+            first = rec
+        assert np.all(np.abs(rec[6:8] - first[6:8]) <= 2.0 ** -34 * total)
+        assert np.all(np.abs(rec[3:5] - first[3:5]) <= 2.0 ** -34 * total / n)
+        assert abs(rec[1] - first[1]) <= 2.0 ** -30 and abs(rec[2] - first[2]) <= 2.0 ** -30
