@@ -192,7 +192,7 @@ def parity_against_oracle(o, stream):
 def run_sweep(args, rank, world, barrier):
     """The seeded 96-channel parametric study, every instance run to a
     steady-state residual of 1e-8 (or the step cap, or divergence), as one
-    graph-replayed concurrent sweep with the schedule autotuner.  The
+    sweep of common launches with the schedule autotuner.  The
     sequential baseline (lone handles, plain launches, the same convergence
     test) is timed on every fourth instance and scaled to the whole study by
     node updates (each lone run takes exactly its instance's steps in the

@@ -135,8 +135,8 @@ void lbm_mix_destroy(lbm_mix* h);
 int lbm_mix_init(lbm_mix* h);
 
 /* Advances nsteps >= 0 time steps (Eq. MRT) on the handle's stream,
- * asynchronously.  FP32 channels of up to 200 000 nodes whose columns fit in
- * shared memory take several steps per launch (tiles of whole columns with
+ * asynchronously.  Small FP32 channels (up to some 400 000 nodes of at most
+ * 64 rows, 170 000 of 128) take several steps per launch (tiles of whole columns with
  * halos, see lbm_mix_set_rows_per_block); a call gives the same bits however
  * its steps are split over calls.  All others take one fused collide-stream
  * pass per step: with 16-bit storage, and with FP32 storage when the step's
@@ -256,10 +256,10 @@ int lbm_mix_dims(const lbm_mix* h, int* N, int* N_x, long* steps);
 /* Kernel launches of an lbm_mix_step call of one step under h's current
  * schedule (lbm_mix_set_rows_per_block): 2 when the wall kernel runs ahead of
  * the step kernel (16-bit storage; FP32 grids of five or more waves of CTAs,
- * two or more under a schedule set by the caller) and for channels that take several steps per launch (the steps and their
- * records; longer calls need fewer per step), else 1; re-referencing adds its
- * own.  Returns the count, or LBM_EINVAL
- * for a NULL handle. */
+ * two or more under a schedule set by the caller) and for channels that take
+ * several steps per launch (the steps and their records; longer calls need
+ * fewer per step), else 1; re-referencing adds its own.  Returns the count, or
+ * LBM_EINVAL for a NULL handle. */
 int lbm_mix_launches_per_step(const lbm_mix* h);
 
 /* Waits for all work enqueued on the handle's stream. */
@@ -348,16 +348,19 @@ int lbm_mix_tune_rows(lbm_mix* h, const int* candidates, int n, long steps, int*
  * Parametric sweeps (the study of Table 1 and Sec. 4: many independent
  * channels).  No counterpart in the paper's method: a batching device.
  *
- * A sweep owns n handles, each on its own CUDA stream.  K steps of an
- * instance are captured once as a CUDA graph and replayed, so each
- * convergence check costs the host one graph launch per instance and the
- * instances' step kernels run concurrently on the GPU.  FP32 storage only;
- * every instance's diag_every is set to the check interval.
+ * A sweep owns n handles on one CUDA stream of its own and takes their steps
+ * by common launches: the instances whose channels take several steps per
+ * launch (lbm_mix_step) together, the others by one step per launch over all
+ * of their CTAs.  The populations are bit for bit those of a lone handle
+ * driven through the same calls; the records' sums differ in rounding at
+ * most.  FP32 storage only; every instance's diag_every is set to the check
+ * interval by lbm_sweep_run_to_steady.
  * ------------------------------------------------------------------- */
 typedef struct lbm_sweep lbm_sweep;
 
-/* Node-to-CTA schedules the autotuner tries: 0 library default, 1: 64, 2: 32, 3: 16 rows, 4: enough rows per CTA to give each
- * instance about two CTAs per SM. */
+/* Node-to-CTA schedules the autotuner tries: 0 library default, 1: 64, 2: 32,
+ * 3: 16 rows, 4: enough rows per CTA to give each instance about two CTAs per
+ * SM. */
 #define LBM_SWEEP_NPOLICY 5
 
 /* Creates n instances from params[0..n-1] (validated like lbm_mix_create)
@@ -371,8 +374,7 @@ void lbm_sweep_destroy(lbm_sweep* s);
 /* lbm_mix_init on every instance. */
 int lbm_sweep_init(lbm_sweep* s);
 
-/* nsteps plain steps on every instance (each on its stream), then waits
- * for all of them. */
+/* nsteps plain steps on every instance, then waits for them. */
 int lbm_sweep_step(lbm_sweep* s, long nsteps);
 
 /* Every instance steps in blocks of check_every (even, >= 2) with the
@@ -380,11 +382,9 @@ int lbm_sweep_step(lbm_sweep* s, long nsteps);
  * boundaries, so the same step counts as a lone run) until its residual
  * drops to tol (status LBM_OK), it has taken max_steps (LBM_ENOTCONVERGED)
  * or turns non-finite (LBM_ENONFINITE); converged instances stop stepping.
- * A graph is replayed only while the instance's buffer parity, schedule,
- * reference-density table and step phase are those it was captured from;
- * calls on a borrowed handle that change them (odd step counts, state
- * uploads, lbm_mix_set_rows_per_block, lbm_mix_rereference) lead to a new
- * capture.
+ * Calls on a borrowed handle between runs (odd step counts, state uploads,
+ * lbm_mix_set_rows_per_block, lbm_mix_rereference) take effect as on a lone
+ * handle.
  * autotune != 0: the first LBM_SWEEP_NPOLICY blocks run under each
  * node-to-CTA schedule in turn (real steps, timed on the host around the
  * whole block), the rest under the fastest.  steps_out, residual_out,

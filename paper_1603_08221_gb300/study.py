@@ -1,6 +1,6 @@
 """The paper's parametric study (Table 1, Sec. 4) on the GPU: every run of
 Table 1 on the 20 x 700 lattice is advanced to a steady residual as one
-graph-replayed sweep, then CL, C~_l (Eq. CL, Eq. Clline), the volume flow
+sweep of common launches, then CL, C~_l (Eq. CL, Eq. Clline), the volume flow
 Q_v at the outlet, the species mass flows and the separation rate V_s of
 the CL(t) history are reported per run, one JSON line each.
 
