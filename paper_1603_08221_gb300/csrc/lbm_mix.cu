@@ -1927,6 +1927,21 @@ int default_rows(const lbm_mix* h) {
   return default_rows(h->L.N, h->nblocks, h->nsm, h->p.storage == LBM_FP32);
 }
 
+// Rows of one strip per CTA of a recorded step under the default schedule.
+// Every CTA of such a step ends in column_epilogue (a fence, a ticket), so
+// twice the rows pay there: at least 56, at most 96 (FP32) or 128 (16-bit).
+// us per recorded step at the rows of the others and at these: FP32 5001 x 130
+// 38.4 -> 30.9 (16, 56 rows), 12000 x 200 82.4 -> 73.5 (56, 96), 15000 x 300
+// 128.2 -> 126.0, 32768 x 512 407.9 -> 392.3; BF16 40.3 -> 38.4 (16, 56), 32768
+// x 512 389.4 -> 381.5 (96, 128).
+int recorded_rows(const lbm_mix* h) {
+  const int rows = h->rows_per_block, n8 = (h->L.N + TY - 1) / TY * TY;
+  const int most = h->p.storage == LBM_FP32 ? 96 : 128;
+  int r = 2 * rows < 56 ? 56 : 2 * rows < most ? 2 * rows : most;
+  if (r > n8) r = n8;
+  return h->rows_set || r < rows ? rows : r;
+}
+
 // Calls f(type tag) with the storage element type of the handle.
 template <typename F>
 int with_storage(const lbm_mix* h, F&& f) {
@@ -2060,7 +2075,8 @@ StepArgs<ST> step_args(const lbm_mix* h) {
 int launch_step(lbm_mix* h, bool diag) {
   int st = with_storage(h, [&](auto tag) -> int {
     using ST = decltype(tag);
-    const StepArgs<ST> a = step_args<ST>(h);
+    StepArgs<ST> a = step_args<ST>(h);
+    if (diag) a.rows_per_block = recorded_rows(h);  // no fewer than R was sized for
     // Both kernels are launched with programmatic stream serialisation, so
     // that each one's launch and CTA ramp overlap the end of the kernel
     // before it (see pdl_wait).
@@ -2079,7 +2095,7 @@ int launch_step(lbm_mix* h, bool diag) {
                             (const double*)a.cs_in, (const float*)h->alpha, h->wall_r,
                             h->wall_omq));
     }
-    cfg.gridDim = dim3(h->nblocks, h->R);
+    cfg.gridDim = dim3(h->nblocks, (h->L.N + a.rows_per_block - 1) / a.rows_per_block);
     cfg.blockDim = dim3(TX, TY);
     if (sizeof(ST) < 4 || !wk) {
       if (diag)
