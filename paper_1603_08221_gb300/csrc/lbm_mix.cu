@@ -496,6 +496,13 @@ __device__ __forceinline__ float number_density(const LatCore& L, float rho_a, f
   return fmaf(rho_a, L.s[0], __fmul_rn(rho_b, L.s[1]));  // Eq. P
 }
 
+// m_x = rho / n.  NaN where n < 0: with both species negative the ratio is that
+// of a gas, and psi's table, which takes no note of its argument's sign, would
+// go on from there with finite rates.
+__device__ __forceinline__ float mixture_mass(float rho, float n, float inv_n) {
+  return n < 0.0f ? NAN : __fmul_rn(rho, inv_n);
+}
+
 __device__ __forceinline__ void macro(const Lat& L, const ColRef& C, const float fs[2][9],
                                       Macro& m) {
 #pragma unroll
@@ -507,7 +514,7 @@ __device__ __forceinline__ void macro(const Lat& L, const ColRef& C, const float
   }
   m.n = number_density(L, m.rho[0], m.rho[1]);
   m.inv_n = rcp_fast(m.n);
-  m.mx = __fmul_rn(__fadd_rn(m.rho[0], m.rho[1]), m.inv_n);  // m_x = rho / n
+  m.mx = mixture_mass(__fadd_rn(m.rho[0], m.rho[1]), m.n, m.inv_n);
 }
 
 // ------------------------------------------- packed per-node arithmetic
@@ -533,7 +540,7 @@ __device__ __forceinline__ void macro2(const LatCore& L, float2 rb, const float2
   m.inv_rho = rcp_fast(rho);
   m.n = number_density(L, m.rho.x, m.rho.y);
   m.inv_n = rcp_fast(m.n);
-  m.mx = __fmul_rn(rho, m.inv_n);  // m_x = rho / n
+  m.mx = mixture_mass(rho, m.n, m.inv_n);
 }
 
 // Sums and differences of opposite populations, from which the momenta, the

@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(TILE_THREADS, 1)
                   open && x == Nx - 2, w, r, g);
         const float2 rho = add2(rb, density_sum(g));
         const float n = number_density(L, rho.x, rho.y), inv_n = rcp_fast(n);
-        const float mx = __fmul_rn(__fadd_rn(rho.x, rho.y), inv_n);
+        const float mx = mixture_mass(__fadd_rn(rho.x, rho.y), n, inv_n);
         OMQ[w * C + c] = inv_tau_q(L, PT, kDpsiTab, n, inv_n, mx, A12[w * C + c]);
       }
       __syncwarp();
