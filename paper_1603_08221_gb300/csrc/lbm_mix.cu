@@ -1639,8 +1639,9 @@ __global__ void __launch_bounds__(256)
     Flow2 w;
     flow2(g, 0.0f, w);
     const float2 sd = density_sum(g);
-    const double rho = ((double)C.rb[0] + sd.x) + ((double)C.rb[1] + sd.y);
-    v += ((double)w.jx.x + (double)w.jx.y) / rho;
+    const double ra = (double)C.rb[0] + sd.x, rb = (double)C.rb[1] + sd.y;
+    // without a positive density of both species Eq. rhou has no velocities
+    v += ra > 0.0 && rb > 0.0 ? ((double)w.jx.x + (double)w.jx.y) / (ra + rb) : (double)NAN;
   }
   v = warp_sum(v);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;

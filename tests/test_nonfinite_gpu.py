@@ -38,3 +38,22 @@ def test_negative_densities_are_reported(species, factor, storage, rows, lam):
     m = g.moments()
     assert not any(np.isfinite(m[k][8, 33]) for k in ("ua_x", "ua_y", "ub_x", "ub_y"))
     assert not np.isfinite(g.get_post_state_f64()[:, 1:, 8, 33]).any()
+
+
+@pytest.mark.parametrize("species", list(SPECIES))
+@pytest.mark.parametrize("factor", [-1.0, 0.0])
+@pytest.mark.parametrize("steps", [0, 1])
+@pytest.mark.parametrize("storage", [binding.LBM_FP32, binding.LBM_FP16])
+def test_volume_flow_through_a_node_without_gas_is_refused(species, factor, steps, storage):
+    """As the fields are: Eq. rhou divides by each species' density."""
+    p = workloads.preset("heli_argon_320x16", N=16, N_x=64, storage=storage)
+    g = binding.LbmMix(**p)
+    g.init()
+    g.step(3)
+    g.set_post_state(_state(g, species, factor))
+    g.step(steps)
+    assert np.isnan(g.moments()["ua_x"][8, 33] + g.moments()["ub_x"][8, 33])
+    with pytest.raises(binding.LbmError) as e:
+        g.volume_flow(33)
+    assert e.value.status == binding.LBM_ENONFINITE
+    assert np.isfinite(g.volume_flow(50))
