@@ -914,21 +914,21 @@ __global__ void __launch_bounds__(WALL_COLS)
   walls_cta(L, blockIdx.x, blockIdx.y, fin, refrho, cs_in, alpha, r_out, omq_out);
 }
 
-// Compensated FP32 running sum (Kahan), accurate to ~1 FP32 ulp of the sum.
-struct KahanF {
-  float s = 0.0f, c = 0.0f;
+// Running sum with the rounding error of every addition kept (Knuth's two-sum).
+// (Kahan's form, one operation less, loses the bits of the running sum below a
+// larger term's last: 1e-8 of a column's deviations.  Its four operations are
+// also one chain, of these six only the sum's own is.)
+struct Sum1 {
+  float s = 0.0f, e = 0.0f;
   __device__ __forceinline__ void add(float v) {
-    float y = v - c;
-    float t = s + y;
-    c = (t - s) - y;
-    s = t;
+    const float2 t = two_sum(s, v);
+    e = __fadd_rn(e, t.y);
+    s = t.x;
   }
 };
 
-// Running sums of two quantities with the rounding error of every addition
-// kept (Knuth's two-sum, packed): a thread's partials over its rows of one
-// column, handed to column_epilogue.  Seven packed instructions where two
-// KahanF take eight, and no bits lost where the sum's sign changes.
+// Two of them, packed, in seven instructions: a thread's partials over its rows
+// of one column, handed to column_epilogue.
 struct Sum2 {
   float2 s = {0.0f, 0.0f}, e = {0.0f, 0.0f};
   __device__ __forceinline__ void add(float2 v) {
@@ -945,14 +945,14 @@ __device__ __forceinline__ float2 pair_add(float2 a, float2 b) {
 }
 
 // Sum of v(0) .. v(N - 1), the rows of a column, by eight neighbouring lanes
-// (sub = lane & 7, every lane of the warp here): each
-// takes every eighth row in order, compensated, then three error-free
-// additions.  Every lane of the eight gets the same (sum, error) pair.
+// (sub = lane & 7, every lane of the warp here): each takes every eighth row in
+// order, then three additions, all error-free but for the errors' own sum.
+// Every lane of the eight gets the same (sum, error) pair.
 template <typename V>
 __device__ __forceinline__ float2 column_sum8(int N, int sub, V&& v) {
-  KahanF a;
+  Sum1 a;
   for (int j = sub; j < N; j += 8) a.add(v(j));
-  float hi = a.s, lo = -a.c;
+  float hi = a.s, lo = a.e;
 #pragma unroll
   for (int o = 1; o < 8; o <<= 1) {
     const float h2 = __shfl_xor_sync(0xffffffffu, hi, o);

@@ -10,6 +10,8 @@ momentum are formed from nine FP32 deviations and the collision conserves them t
 rounding, fewer than 64 roundings of 2^-24 of the magnitudes, with 16-bit storage
 one more, stochastic, of 2^-7 (BF16) or 2^-10 (FP16) of each stored deviation;
 deviations and reference add up to at most twice the populations' magnitudes."""
+import math
+
 import numpy as np
 import pytest
 
@@ -71,3 +73,27 @@ def test_default_schedule_of_recorded_steps(storage, N, Nx):
     # the largest shapes, under every schedule alike)
     assert np.array_equal(fa, fb, equal_nan=True)
     np.testing.assert_allclose(ra[:, 6:8], rb[:, 6:8], rtol=2.0 ** -34, atol=0.0, equal_nan=True)
+
+
+# The stored sums of a column's densities against exact sums of the densities
+# of the same state (the moment fields hold reference plus deviation, exact to
+# 2^-53): the nodes' deviations are added as pairs of floats, exact but for the
+# sum of the errors (2^-48 of the terms), and the total is cut at 2^-48, so 2^-44
+# of it covers either, and N additions of the fields' last bits.
+@pytest.mark.parametrize("N,Nx", [(9, 40), (20, 700), (37, 1001), (64, 500), (130, 300)])
+@pytest.mark.parametrize("rows", [0, 8, 64])
+def test_column_sums_are_exact_sums(N, Nx, rows):
+    torch = pytest.importorskip("torch")
+    p = workloads.preset("heli_argon_320x16", N=N, N_x=Nx, theta=1.3, Kn_out=0.3)
+    g = binding.LbmMix(**p)
+    g.set_rows_per_block(rows)
+    # deviations as large as the densities, of either sign within a column
+    g.set_post_state(workloads.random_post_state(N, Nx, seed=N).astype(np.float32))
+    g.step(1)
+    g.sync()
+    cs = torch.as_tensor(g.device_views()["colsum"], device="cuda").cpu().numpy()
+    m = g.moments()
+    for x in range(1, Nx - 1):
+        for sp, name in enumerate(("rho_a", "rho_b")):
+            exact = math.fsum(m[name][:, x])
+            assert abs(cs[sp, x] - exact) <= 2.0 ** -44 * exact, (x, name)
