@@ -1084,17 +1084,26 @@ __device__ __forceinline__ GridPos grid_pos(const LatCore& L, int b, int strips,
   if (r < 0) return GridPos{(b & 1) ? strips - 1 : 0, b >> 1, strips, blocks};
   return GridPos{1 + r % inner, r / inner, strips, blocks};
 }
+// Most rows whose end columns column_sum8 adds up, eight lanes a column, as in
+// lbm_tile_kernel (whose tiles hold at most 424 rows); beyond, all threads of
+// the CTA take a column after the other, 256 rows at a time.
+constexpr int END_ROWS = 512;
 // Column sums -> next step's density correction, C_l(x), per-strip partials;
 // the last CTA to finish reduces the partials in strip order into one record.
-// DIAG = false: only the column sums (the next step's Eq. rho2 input) are
-// produced; DIAG = true: also C_l(x), the per-strip partials and the record.
+// DIAG = false (end strips only): the sums that the next step's Eq. rho2 needs,
+// with FP32 storage those of the four end columns alone; DIAG = true: those of
+// every column, C_l(x), the per-strip partials and the record.
 // Every CTA of a DIAG step comes here, and an FP64 instruction holds its SM
 // sub-partition for some 64 cycles; the sums of a CTA are therefore pairs of
 // floats, by one warp per quantity, and FP64 begins at the strip's totals.
 // Sums in FP64 throughout, most of them in one warp, cost a DIAG step of
 // 32768 x 512 80 us beyond the others (45 now, mostly the fence and the ticket
-// of each CTA), one of 5001 x 130 29 us (14), and the end strips' chain of
-// every step 4 us of 27.5 there (FP32).
+// of each CTA), one of 5001 x 130 29 us (14).
+// A channel of many rows has long chains here, in one CTA a strip: the row
+// blocks' sums (a hundred cycles a block) and the end columns' rows.  All rows
+// by eight lanes a column and the row blocks at every step took 188 us per step
+// of 64 x 16384, 606 of 64 x 65536 (one row block of 512: 17.2); whole CTAs for
+// the end columns and row blocks at DIAG steps alone 60, 188 (13.5).
 template <bool DIAG, typename ST>
 __device__ __forceinline__ void column_epilogue(const Lat& L, const StepArgs<ST>& a,
                                                 const GridPos& gp, int x, const Sum2 acc[2],
@@ -1103,34 +1112,42 @@ __device__ __forceinline__ void column_epilogue(const Lat& L, const StepArgs<ST>
   const int tid = ty * TX + tx;
   const int R = gp.blocks;  // row blocks per strip
   const bool in = interior(L, x);
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    rs.col[2 * k][ty][tx] = make_float2(acc[k].s.x, acc[k].e.x);
-    rs.col[2 * k + 1][ty][tx] = make_float2(acc[k].s.y, acc[k].e.y);
-  }
-  __syncthreads();
+  // sums of all of the strip's columns; otherwise of the end columns alone,
+  // whose rows are in end_sd (FP32 storage: the strips are then end strips)
+  constexpr bool SUMS = DIAG || sizeof(ST) < 4;
   float2 c = make_float2(0.0f, 0.0f);  // quantity ty of column x, in warps 0 .. 3
-  if (ty < 4) {
-    c = rs.col[ty][0][tx];
+  if constexpr (SUMS) {
 #pragma unroll
-    for (int t = 1; t < TY; ++t) c = pair_add(c, rs.col[ty][t][tx]);
+    for (int k = 0; k < 2; ++k) {
+      rs.col[2 * k][ty][tx] = make_float2(acc[k].s.x, acc[k].e.x);
+      rs.col[2 * k + 1][ty][tx] = make_float2(acc[k].s.y, acc[k].e.y);
+    }
+    __syncthreads();
+    if (ty < 4) {
+      c = rs.col[ty][0][tx];
+#pragma unroll
+      for (int t = 1; t < TY; ++t) c = pair_add(c, rs.col[ty][t][tx]);
+    }
   }
   if (R > 1) {
     // Row-block partials of this strip; the last of its R CTAs to finish
-    // adds them in row-block order (independent of arrival order).
-    if (ty < 4) {
+    // adds them in row-block order (independent of arrival order).  A fence
+    // after a barrier, by the thread that takes the ticket too, publishes what
+    // the CTA's threads wrote before that barrier (the rows of end_sd).
+    if (SUMS && ty < 4) {
       if (x < L.Nx) a.colpart[((size_t)gp.block * 4 + ty) * L.Nx + x] = c;
-      __threadfence();  // the writers publish before the ticket is taken
+      __threadfence();
     }
     __syncthreads();
     if (tid == 0) {
+      if (!SUMS) __threadfence();
       unsigned ticket = atomicAdd(a.strip_cnt + gp.strip, 1u);
       rs.last_strip = (ticket == (unsigned)R - 1u);
     }
     __syncthreads();
     if (!rs.last_strip) return;
     __threadfence();
-    if (ty < 4 && x < L.Nx) {
+    if (SUMS && ty < 4 && x < L.Nx) {
       const float2* cp = a.colpart + (size_t)ty * L.Nx + x;
       c = __ldcg(cp);
 #pragma unroll 4
@@ -1138,32 +1155,73 @@ __device__ __forceinline__ void column_epilogue(const Lat& L, const StepArgs<ST>
     }
     if (tid == 0) a.strip_cnt[gp.strip] = 0u;
   }
-  if (ty < 4) {
+  if (SUMS && ty < 4) {
     // column sum of rho_s = N rhobar_s + sum of deviations
     double v = pair_value(c);
     if (ty < 2 && in) v += (double)L.N * (double)a.refrho[ty * L.Nx + x];
     rs.total[ty][tx] = v;
   }
   if (sizeof(ST) == 4 && a.end_sd) {
-    // The columns behind the next step's density correction, in the order of
-    // column_sum8 over all rows: the populations of a run are then the same
-    // bits under every schedule, this kernel's and lbm_tile_kernel's.  One
-    // warp for each of the four columns and two species.
+    // The columns behind the next step's density correction, in an order that
+    // depends on N alone: the populations of a run are then the same bits under
+    // every schedule, this kernel's and lbm_tile_kernel's.  e: which column.
+    auto end_column = [&](int e) {
+      return e == 0 ? 1 : e == 1 ? 2 : e == 2 ? L.Nx - 2 : L.Nx - 3;
+    };
+    const int x0 = x - tx;
+    // the sum over end column x of species sp, from that of its deviations
+    auto put = [&](int sp, float2 v) {
+      const double t = pair_value(column_total(L.N, a.refrho[sp * L.Nx + x], v));
+      if constexpr (SUMS)
+        rs.total[sp][tx] = t;
+      else
+        a.cs_out[(size_t)sp * L.Nx + x] = t;
+    };
     __syncthreads();
-    const int e = ty >> 1, sp = ty & 1, x0 = x - tx;
-    const int xe = e == 0 ? 1 : e == 1 ? 2 : e == 2 ? L.Nx - 2 : L.Nx - 3;
-    if (xe >= x0 && xe < x0 + TX) {  // warp-uniform
-      const float2 v = column_sum8(L.N, tx & 7, [&](int r) {
-        const float2 d = __ldcg(a.end_sd + (size_t)e * L.N + r);
-        return sp ? d.y : d.x;
-      });
-      const double t = pair_value(column_total(L.N, a.refrho[sp * L.Nx + xe], v));
-      if (x == xe) rs.total[sp][tx] = t;
+    if (L.N <= END_ROWS) {
+      // as lbm_tile_kernel does; one warp for each column and species
+      const int e = ty >> 1, sp = ty & 1, xe = end_column(e);
+      if (xe >= x0 && xe < x0 + TX) {  // warp-uniform
+        const float2 v = column_sum8(L.N, tx & 7, [&](int r) {
+          const float2 d = __ldcg(a.end_sd + (size_t)e * L.N + r);
+          return sp ? d.y : d.x;
+        });
+        if (x == xe) put(sp, v);
+      }
+    } else {
+      // the whole CTA, one column after another
+      for (int e = 0; e < 4; ++e) {
+        const int xe = end_column(e);
+        if (xe < x0 || xe >= x0 + TX) continue;  // CTA-uniform
+        const float2* d = a.end_sd + (size_t)e * L.N;
+        Sum2 v;
+#pragma unroll 8
+        for (int r = tid; r < L.N; r += TX * TY) v.add(__ldcg(d + r));
+        float2 pa = make_float2(v.s.x, v.e.x), pb = make_float2(v.s.y, v.e.y);
+#pragma unroll
+        for (int o = 1; o < TX; o <<= 1) {
+          pa = pair_add(pa, make_float2(__shfl_xor_sync(0xffffffffu, pa.x, o),
+                                        __shfl_xor_sync(0xffffffffu, pa.y, o)));
+          pb = pair_add(pb, make_float2(__shfl_xor_sync(0xffffffffu, pb.x, o),
+                                        __shfl_xor_sync(0xffffffffu, pb.y, o)));
+        }
+        if (tx == 0) {
+          rs.col[0][ty][0] = pa;
+          rs.col[1][ty][0] = pb;
+        }
+        __syncthreads();
+        if (ty < 2 && x == xe) {
+          float2 t = rs.col[ty][0][0];
+          for (int w = 1; w < TY; ++w) t = pair_add(t, rs.col[ty][w][0]);
+          put(ty, t);
+        }
+        __syncthreads();
+      }
     }
     __syncthreads();
   }
   // (a warp writes back the totals that it formed itself, or all have met)
-  if (ty < 4 && x < L.Nx) a.cs_out[(size_t)ty * L.Nx + x] = rs.total[ty][tx];
+  if (SUMS && ty < 4 && x < L.Nx) a.cs_out[(size_t)ty * L.Nx + x] = rs.total[ty][tx];
   if (!DIAG) return;
   __syncthreads();
   // The strip's partials: a quantity's sum over the columns in each of four
@@ -1359,7 +1417,7 @@ __device__ __forceinline__ void step_cta(const Lat& L, const StepArgs<ST>& a, co
         if (end_l >= 0) a.end_sd[end_l * L.N + j] = sd;
         if (end_r >= 0) a.end_sd[end_r * L.N + j] = sd;
       }
-      if (reduce) {
+      if (FP32 ? diag : reduce) {
         acc[0].add(sd);
         acc[1].add(mxs);
       }
