@@ -1825,6 +1825,8 @@ struct lbm_mix {
   bool rows_set;
   float2* hist;      // [hist_rows][4][Nx] column sums awaiting lbm_records_kernel
   int hist_rows;
+  double* rec_part;  // [hist_rows][NPART][record_blocks]: see lbm_records_kernel
+  unsigned* rec_cnt; // [hist_rows]
   int cur;           // buffer holding the latest post-collision state
   long steps;
   bool have_snap;
@@ -2304,18 +2306,19 @@ int launch_tiles(lbm_mix* const* hs, const int* W, int n, int k, bool last, int*
 template <int NI>
 int launch_records(lbm_mix* const* hs, int n, int* rows, cudaStream_t st) {
   RecBatch<NI> B;
-  int most = 0;
+  int most = 0, blocks = 1;
   for (int q = 0; q < n; ++q) {
     lbm_mix* h = hs[q];
     const Lat& L = h->L;
     B.inst[q] = RecInst{L.N,     L.Nx,    L.x_periodic, L.light, {L.s[0], L.s[1]}, L.C_in,
                         L.C_out, h->hist, h->refrho,    h->diag, h->diag_count,    h->counter,
-                        h->clprof, rows[q]};
+                        h->clprof, h->rec_part, h->rec_cnt, rows[q], record_blocks(L.Nx)};
     most = rows[q] > most ? rows[q] : most;
+    blocks = B.inst[q].blocks > blocks ? B.inst[q].blocks : blocks;
     rows[q] = 0;
   }
   if (most == 0) return LBM_OK;
-  return launch_batch(lbm_records_kernel<NI>, B, dim3(most, n), dim3(256), 0, st);
+  return launch_batch(lbm_records_kernel<NI>, B, dim3(blocks, most, n), dim3(256), 0, st);
 }
 
 // nsteps steps of the n <= NI channels hs on stream st: launches of kmax
@@ -2591,6 +2594,7 @@ int lbm_mix_create(const lbm_mix_params* p, void* stream, lbm_mix** out) {
     carve(base, cbytes, &h->cs[1]);
     carve(base, sizeof(unsigned long long), &h->diag_count);
     carve(base, sizeof(double) * DIAG_CAP * NREC, &h->diag);
+    if (h->tile_W > 0) carve(base, sizeof(unsigned) * h->hist_rows, &h->rec_cnt);
     zeroed = total;
     carve(base, sizeof(float) * 2 * (size_t)Nx, &h->refrho);
     carve(base, sizeof(float) * 2 * (size_t)Nx, &h->refrho_alt);
@@ -2604,7 +2608,10 @@ int lbm_mix_create(const lbm_mix_params* p, void* stream, lbm_mix** out) {
     if (p->storage == LBM_FP32 && !p->x_periodic)
       carve(base, sizeof(float2) * 4 * (size_t)h->L.N, &h->end_sd);
     carve(base, sizeof(float2) * 4 * (size_t)Nx * (size_t)h->R, &h->colpart0);
-    if (h->tile_W > 0) carve(base, sizeof(float2) * 4 * (size_t)Nx * h->hist_rows, &h->hist);
+    if (h->tile_W > 0) {
+      carve(base, sizeof(float2) * 4 * (size_t)Nx * h->hist_rows, &h->hist);
+      carve(base, sizeof(double) * NPART * record_blocks(Nx) * (size_t)h->hist_rows, &h->rec_part);
+    }
   };
   layout(nullptr);
   if (e == cudaSuccess) e = cudaMalloc((void**)&h->arena, total);

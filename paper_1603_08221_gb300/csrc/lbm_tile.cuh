@@ -392,9 +392,16 @@ __global__ void __launch_bounds__(TILE_THREADS, 1)
 }
 
 // The diagnostic records of a call's steps from the column sums the tile
-// kernel left in hist, one block per record: C_l(x), CL, C~_l, the mean mass
-// flows and the total masses, the formulas and reductions of
-// column_epilogue.  The last block to finish advances the record counter.
+// kernel left in hist: C_l(x), CL, C~_l, the mean mass flows and the total
+// masses, the formulas and reductions of column_epilogue.  Grid: blocks of
+// columns x records x channels.  The FP64 work of 256 columns holds an SM for
+// some 2.5 us, so a record has a block per 256 columns up to REC_BLOCKS, the
+// last of which folds their partials in block order.  With one block per record
+// a call of a single step took 82 us on 5000 x 64 and 441 on 40000 x 8 (54 and
+// 79 now), a step with a record of its own, many to a launch, 27 and 121 (18
+// and 32); 320 x 16 the same either way.
+// The last record to finish advances the record counter.
+constexpr int REC_BLOCKS = 128;
 struct RecInst {
   int N, Nx, x_periodic, light;
   float s[2];
@@ -405,28 +412,37 @@ struct RecInst {
   unsigned long long* diag_count;
   unsigned* counter;
   double* clprof;
-  int nrec;
+  double* part;      // [records][NPART][blocks]
+  unsigned* rec_cnt; // [records] blocks finished
+  int nrec, blocks;
 };
 template <int NI>
 struct RecBatch {
   RecInst inst[NI];
 };
+inline int record_blocks(int Nx) {
+  const int b = (Nx + 255) / 256;
+  return b < REC_BLOCKS ? b : REC_BLOCKS;
+}
 
 template <int NI>
 __global__ void __launch_bounds__(256) lbm_records_kernel(const __grid_constant__ RecBatch<NI> B) {
-  __shared__ double wsum[8][6], wmin[8];
-  __shared__ int wimin[8];
+  // partials by warp, then of the block, then of the record: min C_l, its
+  // column, sums of C_l - C_in, the momenta, the masses and the columns
+  __shared__ double wpart[NPART][8], tot[NPART];
+  __shared__ int last;
   pdl_wait();
-  const RecInst &I = B.inst[NI > 1 ? blockIdx.y : 0], &L = I;
-  const int r = blockIdx.x, nrec = I.nrec, tid = threadIdx.x, Nx = L.Nx;
-  if (r >= nrec) return;
+  const RecInst &I = B.inst[NI > 1 ? blockIdx.z : 0], &L = I;
+  const int r = blockIdx.y, b = blockIdx.x, nb = I.blocks, tid = threadIdx.x, Nx = L.Nx;
+  if (r >= I.nrec || b >= nb) return;
   const unsigned long long cnt0 = *(volatile unsigned long long*)I.diag_count;
   const float2* h = I.hist + (size_t)r * 4 * Nx;
+  const bool profile = r == I.nrec - 1;
   double vmin = INFINITY, sm[6] = {0, 0, 0, 0, 0, 0};
   int imin = 0x7fffffff;
-  for (int x = tid; x < Nx; x += 256) {
+  for (int x = 256 * b + tid; x < Nx; x += 256 * nb) {
     if (!L.x_periodic && (x < 1 || x > Nx - 2)) {
-      if (r == nrec - 1) I.clprof[x] = x == 0 ? L.C_in : L.C_out;
+      if (profile) I.clprof[x] = x == 0 ? L.C_in : L.C_out;
       continue;
     }
     double c[4];
@@ -434,9 +450,9 @@ __global__ void __launch_bounds__(256) lbm_records_kernel(const __grid_constant_
     for (int q = 0; q < 4; ++q) c[q] = pair_value(h[(size_t)q * Nx + x]);
     c[0] += (double)L.N * (double)I.refrho[x];
     c[1] += (double)L.N * (double)I.refrho[Nx + x];
-    const double na = c[0] * L.s[0], nb = c[1] * L.s[1];
-    const double Cl = (L.light == 0 ? na : nb) / (na + nb);
-    if (r == nrec - 1) I.clprof[x] = Cl;
+    const double na = c[0] * L.s[0], nb_ = c[1] * L.s[1];
+    const double Cl = (L.light == 0 ? na : nb_) / (na + nb_);
+    if (profile) I.clprof[x] = Cl;
     if (Cl < vmin) {
       vmin = Cl;
       imin = x;
@@ -453,37 +469,77 @@ __global__ void __launch_bounds__(256) lbm_records_kernel(const __grid_constant_
   for (int q = 0; q < 6; ++q) sm[q] = warp_sum(sm[q]);
   const int lane = tid & 31, wid = tid >> 5;
   if (lane == 0) {
-    wmin[wid] = vmin;
-    wimin[wid] = imin;
+    wpart[0][wid] = vmin;
+    wpart[1][wid] = (double)imin;
 #pragma unroll
-    for (int q = 0; q < 6; ++q) wsum[wid][q] = sm[q];
+    for (int q = 0; q < 6; ++q) wpart[2 + q][wid] = sm[q];
   }
   __syncthreads();
-  if (tid != 0) return;
-  double tot[6] = {0, 0, 0, 0, 0, 0}, mn = INFINITY;
-  int im = 0x7fffffff;
-  for (int w = 0; w < 8; ++w) {
-    for (int q = 0; q < 6; ++q) tot[q] += wsum[w][q];
-    if (wmin[w] < mn || (wmin[w] == mn && wimin[w] < im)) {
-      mn = wmin[w];
-      im = wimin[w];
+  // n partials get(q, k) of each quantity q folded by warp q, warp 0 the minimum
+  // and its column; the result in tot
+  static_assert(NPART == 8, "a warp per partial");
+  auto fold = [&](int n, auto&& get) {
+    if (wid == 0) {
+      double v = INFINITY;
+      int i = 0x7fffffff;
+      for (int k = lane; k < n; k += 32) {
+        const double w = get(0, k);
+        const int iw = (int)get(1, k);
+        if (w < v || (w == v && iw < i)) {
+          v = w;
+          i = iw;
+        }
+      }
+      warp_min(v, i);
+      if (lane == 0) {
+        tot[0] = v;
+        tot[1] = (double)i;
+      }
+    } else if (wid != 1) {
+      double v = 0.0;
+      for (int k = lane; k < n; k += 32) v += get(wid, k);
+      v = warp_sum(v);
+      if (lane == 0) tot[wid] = v;
     }
+    __syncthreads();
+  };
+  fold(8, [&](int q, int k) { return wpart[q][k]; });
+  if (nb > 1) {
+    double* p = I.part + (size_t)r * NPART * nb;
+    if (tid < NPART) {
+      p[(size_t)tid * nb + b] = tot[tid];
+      __threadfence();
+    }
+    __syncthreads();
+    if (tid == 0) last = atomicAdd(I.rec_cnt + r, 1u) == (unsigned)nb - 1u;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (tid == 0) I.rec_cnt[r] = 0u;
+    fold(nb, [&](int q, int k) { return __ldcg(p + (size_t)q * nb + k); });
   }
-  double dev = tot[0];
+  if (tid >= NREC) return;
+  double dev = tot[2];
   if (!L.x_periodic) dev += (L.C_out - L.C_in);  // the outlet boundary column
   const unsigned long long cnt = cnt0 + (unsigned long long)r + 1ull;
-  double* rec = I.diag + (size_t)((cnt - 1ull) % DIAG_CAP) * NREC;
-  rec[0] = (double)cnt;
-  rec[1] = (L.C_in - mn) / L.C_in;
-  rec[2] = dev / ((double)Nx * L.C_in);
-  rec[3] = tot[1] / tot[5];
-  rec[4] = tot[2] / tot[5];
-  rec[5] = (double)im;
-  rec[6] = tot[3];
-  rec[7] = tot[4];
+  // one division for all eight entries
+  double num = 0.0, den = 1.0;
+  switch (tid) {
+    case 0: num = (double)cnt; break;
+    case 1: num = L.C_in - tot[0], den = L.C_in; break;
+    case 2: num = dev, den = (double)Nx * L.C_in; break;
+    case 3: num = tot[3], den = tot[7]; break;
+    case 4: num = tot[4], den = tot[7]; break;
+    case 5: num = tot[1]; break;
+    case 6: num = tot[5]; break;
+    case 7: num = tot[6]; break;
+  }
+  I.diag[(size_t)((cnt - 1ull) % DIAG_CAP) * NREC + tid] = num / den;
+  __syncwarp((1u << NREC) - 1u);
+  if (tid != 0) return;
   __threadfence();
-  if (atomicAdd(I.counter, 1u) == (unsigned)nrec - 1u) {
-    *I.diag_count = cnt0 + (unsigned long long)nrec;
+  if (atomicAdd(I.counter, 1u) == (unsigned)I.nrec - 1u) {
+    *I.diag_count = cnt0 + (unsigned long long)I.nrec;
     *I.counter = 0u;
   }
 }
