@@ -137,8 +137,9 @@ int lbm_mix_init(lbm_mix* h);
 /* Advances nsteps >= 0 time steps (Eq. MRT) on the handle's stream,
  * asynchronously.  Small FP32 channels (up to some 400 000 nodes of at most
  * 64 rows, 170 000 of 128) take several steps per launch (tiles of whole columns with
- * halos, see lbm_mix_set_rows_per_block); a call gives the same bits however
- * its steps are split over calls.  All others take one fused collide-stream
+ * halos, see lbm_mix_set_rows_per_block), wide ones a call's last step or two
+ * as below; the populations are the same bits however the steps are split over
+ * calls, the records' sums to rounding.  All others take one fused collide-stream
  * pass per step: with 16-bit storage, and with FP32 storage when the step's
  * grid holds several waves of CTAs on the device, a small kernel computes
  * r (Eq. R) and tau_q (Eq. taoq) of every column ahead of each pass.  All
@@ -256,8 +257,8 @@ int lbm_mix_dims(const lbm_mix* h, int* N, int* N_x, long* steps);
 /* Kernel launches of an lbm_mix_step call of one step under h's current
  * schedule (lbm_mix_set_rows_per_block): 2 when the wall kernel runs ahead of
  * the step kernel (16-bit storage; FP32 grids of five or more waves of CTAs,
- * two or more under a schedule set by the caller) and for channels that take
- * several steps per launch (the steps and their records; longer calls need
+ * two or more under a schedule set by the caller) and for channels of up to 2048
+ * columns that take several steps per launch (the steps and their records; longer calls need
  * fewer per step), else 1; re-referencing adds its own.  Returns the count, or
  * LBM_EINVAL for a NULL handle. */
 int lbm_mix_launches_per_step(const lbm_mix* h);

@@ -2321,6 +2321,14 @@ int launch_records(lbm_mix* const* hs, int n, int* rows, cudaStream_t st) {
   return launch_batch(lbm_records_kernel<NI>, B, dim3(blocks, most, n), dim3(256), 0, st);
 }
 
+// Columns beyond which a lone channel takes single steps by lbm_step_kernel: a
+// launch of lbm_tile_kernel for one step fills, sums and empties its tiles for
+// it, and its record is a launch of its own.  us per call of one step, by tiles
+// and record and by the step kernel: 700 x 20 17.7 and 15, 2000 x 16 19 and 15,
+// 4000 x 16 32 and 17, 8000 x 16 41 and 18, 40000 x 8 78 and 39 (as many calls
+// in a row as the host issues; up to 2000 it bounds either).
+constexpr int SINGLE_STEP_COLUMNS = 2048;
+
 // nsteps steps of the n <= NI channels hs on stream st: launches of kmax
 // steps or fewer, the last one of a single step, so that the two buffers end
 // up holding the states of the last two steps.  end: the last step ends the
@@ -2334,6 +2342,12 @@ int tile_steps(lbm_mix* const* hs, const int* W, int n, int kmax, long nsteps, b
     int k = left - 1 < kmax ? (int)(left - 1) : kmax;
     k -= 1 - (k & 1);  // odd
     if (k < 1) k = 1;
+    if (NI == 1 && k == 1 && hs[0]->L.Nx > SINGLE_STEP_COLUMNS) {
+      const bool diag = (end && left == 1) || (hs[0]->steps + 1) % hs[0]->p.diag_every == 0;
+      if ((s = launch_records<NI>(hs, n, rows, st)) || (s = launch_step(hs[0], diag))) return s;
+      --left;
+      continue;
+    }
     bool full = false;
     for (int q = 0; q < n; ++q) full |= rows[q] + k + 1 > hs[q]->hist_rows;
     if (full && (s = launch_records<NI>(hs, n, rows, st))) return s;
@@ -2955,7 +2969,8 @@ int lbm_mix_dims(const lbm_mix* h, int* N, int* N_x, long* steps) {
 int lbm_mix_launches_per_step(const lbm_mix* h) {
   int st = check_handle(h);
   if (st) return st;
-  return (h->elem < 4 || uses_tiles(h) || uses_wall_kernel(h)) ? 2 : 1;
+  const bool tiles = uses_tiles(h) && h->L.Nx <= SINGLE_STEP_COLUMNS;
+  return (h->elem < 4 || tiles || uses_wall_kernel(h)) ? 2 : 1;
 }
 
 int lbm_mix_sync(lbm_mix* h) {
@@ -3184,8 +3199,11 @@ int launch_step_batch(lbm_mix* const* hs, int n, bool end, cudaStream_t st) {
 
 // nsteps steps of the n channels hs of a sweep, on its stream.  Channels that
 // qualify for tiles take them, grouped by N, unless one step kernel over all
-// channels is estimated to be faster (many nodes in all, or tall channels);
-// the populations are the same bits either way.
+// channels is estimated to be faster (many nodes in all, or tall channels) or
+// the call has one or two steps of more than SINGLE_STEP_COLUMNS columns, each of
+// which would be a launch of tiles (us per step of calls of two: 8 channels of
+// 400 x 32 30.8 by tiles, 18.2 by the step kernel, 3 of 700 x 20 22.0 and 20.6;
+// one of 320 x 16 17.1 and 19.5); the populations are the same bits either way.
 int batch_steps(lbm_sweep* s, lbm_mix* const* hs, int n, long nsteps) {
   if (nsteps < 1) return LBM_OK;
   lbm_mix** order = (lbm_mix**)malloc(2 * sizeof(lbm_mix*) * (size_t)n);
@@ -3197,7 +3215,9 @@ int batch_steps(lbm_sweep* s, lbm_mix* const* hs, int n, long nsteps) {
   lbm_mix** rest = order + n;  // channels of the step kernel
   int nt = 0, nr = 0, st = LBM_OK;
   double nodes_t = 0.0, nodes_r = 0.0, us = 0.0;
+  long columns = 0;
   for (int q = 0; q < n; ++q) {
+    columns += hs[q]->L.Nx;
     const double nodes = (double)hs[q]->L.N * hs[q]->L.Nx;
     (uses_tiles(hs[q]) ? nodes_t : nodes_r) += nodes;
     if (uses_tiles(hs[q])) order[nt++] = hs[q];
@@ -3210,7 +3230,9 @@ int batch_steps(lbm_sweep* s, lbm_mix* const* hs, int n, long nsteps) {
   };
   int k = 1;
   for (int q0 = 0, q1; q0 < nt; q0 = q1) us += plan_batch(order + q0, (q1 = group_end(q0)) - q0, W, &k);
-  const bool tiles = us + (nodes_r > 0 ? batch_step_cost(nodes_r) : 0.0) <= batch_step_cost(nodes_t + nodes_r);
+  const bool tiles = (nsteps > 2 || columns <= SINGLE_STEP_COLUMNS) &&
+                     us + (nodes_r > 0 ? batch_step_cost(nodes_r) : 0.0) <=
+                         batch_step_cost(nodes_t + nodes_r);
   for (int q0 = 0, q1; tiles && q0 < nt && !st; q0 = q1) {
     const int m = (q1 = group_end(q0)) - q0;
     plan_batch(order + q0, m, W, &k);

@@ -72,3 +72,68 @@ def test_a_record_does_not_dominate_a_call_of_one_step(N, Nx):
     take some twice as long, but not a multiple that grows with the columns."""
     p = workloads.preset("heli_argon_320x16", N=N, N_x=Nx, theta=1.2, Kn_out=0.3)
     assert us_per_call(p, 0) < 3.0 * us_per_call(p, 8 * ((N + 7) // 8)) + 5.0
+
+
+# calls of one, two and three steps, of channels on both sides of the line
+# between single steps by tiles and by the step kernel, and of sweeps
+@pytest.mark.parametrize("N,Nx", [(16, 2048), (16, 2049), (8, 8263), (8, 40000), (2, 100000)])
+def test_short_calls_take_no_longer_than_the_step_kernel(N, Nx):
+    """Narrow channels take two launches where the step kernel takes one, a wide
+    one nothing beyond it (its timing's spread: a third and 5 us)."""
+    p = workloads.preset("heli_argon_320x16", N=N, N_x=Nx, theta=1.2, Kn_out=0.3)
+    slack = 2.0 if Nx <= 2048 else 4.0 / 3.0
+    assert us_per_call(p, 0) < slack * us_per_call(p, 8 * ((N + 7) // 8)) + 5.0
+
+
+@pytest.mark.parametrize("N,Nx", [(8, 2049), (16, 4000), (64, 3000)])
+def test_wide_channels_split_over_calls_in_any_way(N, Nx):
+    """The same populations whichever kernel takes a step, and the records to the
+    rounding of their sums."""
+    p = workloads.preset("heli_argon_320x16", N=N, N_x=Nx, diag_every=4, theta=1.2, Kn_out=0.3)
+    total, runs = 40, []
+    for rows, split in ((0, [40]), (0, [1] * 40), (0, [2, 3, 4, 5, 6, 7, 13]), (8, [40])):
+        g = binding.LbmMix(**p)
+        g.set_rows_per_block(rows)
+        g.init()
+        for n in split:
+            g.step(n)
+        assert g.steps == total
+        runs.append(g)
+    ref = runs[0]
+    h = ref.history()
+    assert len(h) == 10
+    for g in runs[1:]:
+        assert np.array_equal(g.get_post_state_f64()[..., 1:-1],
+                              ref.get_post_state_f64()[..., 1:-1])
+        m, mr = g.moments(), ref.moments()
+        assert all(np.array_equal(m[k], mr[k]) for k in m)
+        assert np.abs(g.history(1)[0, 6:8] / h[-1, 6:8] - 1).max() <= 2.0 ** -34
+    assert np.array_equal(runs[3].history()[:, 0], h[:, 0])
+
+
+@pytest.mark.parametrize("count,N,Nx,extra", [(8, 32, 400, dict(x_periodic=1)), (3, 20, 700, {}),
+                                              (52, 20, 700, {})])
+@pytest.mark.parametrize("split", [[1] * 12, [2] * 6, [3, 1, 2, 6]])
+def test_sweeps_by_short_calls(count, N, Nx, extra, split):
+    params = [workloads.preset("heli_argon_320x16", N=N, N_x=Nx + q % 2, theta=1.2 + 0.01 * q,
+                               Kn_out=0.3, **extra) for q in range(count)]
+    f0 = workloads.random_post_state(N, Nx, seed=4, lo=0.099, hi=0.101)
+    f0[:, 0] *= 4.0
+    sw, lone = binding.LbmSweep(params), {}
+    sw.init()
+    for q in (0, count - 1):
+        lone[q] = g = binding.LbmMix(**params[q])
+        g.init()
+    if extra:
+        for g in [sw.instance(0), lone[0]]:
+            g.set_post_state(f0.astype(np.float32))
+    for n in split:
+        sw.step(n)
+        for g in lone.values():
+            g.step(n)
+    for q, g in lone.items():
+        a, b = sw.instance(q), g
+        assert a.steps == b.steps == 12
+        cols = slice(None) if extra else slice(1, -1)
+        assert np.array_equal(a.get_post_state_f64()[..., cols], b.get_post_state_f64()[..., cols])
+        assert np.abs(a.history(1)[0, 6:8] / b.history(1)[0, 6:8] - 1).max() <= 2.0 ** -34
