@@ -534,7 +534,8 @@ def run_ours(args):
                    "rows_per_block": rows,
                    "schedule": ("given (--rows)" if args.rows > 0 else
                                 f"rows per CTA tuned over {TUNE_STEPS} steps per candidate "
-                                "(lbm_mix_tune_rows) before init; not timed"),
+                                "(lbm_mix_tune_rows; 0: the library's default schedule) before "
+                                "init; not timed"),
                    "l2": (f"state (2 x {state_gb:.2f} GB {args.storage.upper()}) larger "
                           "than L2; no flush" if state_gb > 0.129 else
                           f"state (2 x {state_gb:.3f} GB) fits in L2: not a DRAM figure"),

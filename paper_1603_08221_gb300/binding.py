@@ -355,7 +355,8 @@ def lbm_mix_set_rows_per_block(h, rows: int) -> None:
 
 def lbm_mix_tune_rows(h, candidates=None, steps: int = 20) -> int:
     """Times `steps` real steps under each candidate rows-per-CTA (None: the
-    library's list) and keeps the fastest; returns it.  Advances the state."""
+    library's default schedule and its list) and keeps the fastest; returns it,
+    0 for the default schedule.  Advances the state."""
     best = _I()
     if candidates is None:
         arr, n = None, 0

@@ -2791,15 +2791,12 @@ int lbm_mix_tune_rows(lbm_mix* h, const int* candidates, int n, long steps, int*
     if (e0) cudaEventDestroy(e0);
     return set_err(LBM_ECUDA, "cudaEventCreate failed");
   }
-  int best = h->rows_per_block;
-  bool best_set = h->rows_set;
+  int best = h->rows_set ? h->rows_per_block : 0;  // 0: the default schedule
   float best_ms = INFINITY;
-  // the library's own list starts with its default where that is not a row
-  // count of the step kernel but lbm_tile_kernel
-  const int first = own_list && h->tile_W > 0 ? -1 : 0;
-  for (int k = first; k < n && st == LBM_OK; ++k) {
-    if ((st = set_rows_per_block(h, k < 0 ? 0 : candidates[k]))) break;
-    h->rows_set = k >= 0;
+  // the library's own list is of counts beyond its default's, which it tries first
+  for (int k = own_list ? -1 : 0; k < n && st == LBM_OK; ++k) {
+    const int rows = k < 0 ? 0 : candidates[k];
+    if ((st = lbm_mix_set_rows_per_block(h, rows))) break;
     // two untimed steps settle the new schedule (first-touch of its buffers)
     if ((st = lbm_mix_step(h, 2))) break;
     if (cudaEventRecord(e0, h->stream) != cudaSuccess ||
@@ -2812,15 +2809,13 @@ int lbm_mix_tune_rows(lbm_mix* h, const int* candidates, int n, long steps, int*
     cudaEventElapsedTime(&ms, e0, e1);
     if (ms < best_ms) {
       best_ms = ms;
-      best = h->rows_per_block;
-      best_set = h->rows_set;
+      best = rows == 0 ? 0 : h->rows_per_block;
     }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (st) return st;
-  if ((st = set_rows_per_block(h, best))) return st;
-  h->rows_set = best_set;
+  if ((st = lbm_mix_set_rows_per_block(h, best))) return st;
   if (best_rows) *best_rows = best;
   return LBM_OK;
 }
