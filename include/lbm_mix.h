@@ -350,8 +350,9 @@ int lbm_mix_tune_rows(lbm_mix* h, const int* candidates, int n, long steps, int*
  * Parametric sweeps (the study of Table 1 and Sec. 4: many independent
  * channels).  No counterpart in the paper's method: a batching device.
  *
- * A sweep owns n handles on one CUDA stream of its own and takes their steps
- * by common launches: the instances whose channels take several steps per
+ * A sweep owns n handles, each on its own CUDA stream, and takes their steps by
+ * common launches on one more, after what calls on borrowed handles have left
+ * on theirs: the instances whose channels take several steps per
  * launch (lbm_mix_step) together, the others by one step per launch over all
  * of their CTAs.  The populations are bit for bit those of a lone handle
  * driven through the same calls; the records' sums differ in rounding at

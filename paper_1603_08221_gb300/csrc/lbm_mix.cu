@@ -1796,6 +1796,7 @@ struct lbm_mix {
   int nsm;            // streaming multiprocessors of the device
   cudaStream_t stream;
   bool own_stream;
+  bool pending;      // a call may have left work on the stream (see join_handles)
   int nblocks;
   void* buf[2];       // post-collision deviations, A/B (element type per storage)
   size_t elem;        // bytes per stored population
@@ -2071,6 +2072,13 @@ int launch_residual(lbm_mix* h, long k) {
   return LBM_OK;
 }
 
+// Waits for the handle's stream.
+cudaError_t wait_stream(lbm_mix* h) {
+  const cudaError_t e = cudaStreamSynchronize(h->stream);
+  if (e == cudaSuccess) h->pending = false;
+  return e;
+}
+
 // Node-to-CTA schedule: rows per CTA (a multiple of TY); the per-row-block
 // partials grow when a schedule needs more row blocks than allocated.
 int set_rows_per_block(lbm_mix* h, int rows) {
@@ -2081,7 +2089,7 @@ int set_rows_per_block(lbm_mix* h, int rows) {
   const int R = (h->L.N + rows - 1) / rows;
   if (R > h->R_alloc) {
     float2* cp = nullptr;
-    CK(cudaStreamSynchronize(h->stream));
+    CK(wait_stream(h));
     CK(cudaMalloc((void**)&cp, sizeof(double) * 4 * (size_t)h->L.Nx * (size_t)R));
     if (h->colpart != h->colpart0) cudaFree(h->colpart);
     h->colpart = cp;
@@ -2382,8 +2390,14 @@ int launch_moments(lbm_mix* h, double* d_out) {
   return LBM_OK;
 }
 
+// On entry to a call; one that may enqueue work has a handle that is not const.
 int check_handle(const lbm_mix* h) {
   if (!h) return set_err(LBM_EINVAL, "handle is NULL");
+  return LBM_OK;
+}
+int check_handle(lbm_mix* h) {
+  if (!h) return set_err(LBM_EINVAL, "handle is NULL");
+  h->pending = true;
   return LBM_OK;
 }
 
@@ -2395,7 +2409,7 @@ int latest_record(lbm_mix* h, double rec[NREC], double* profile) {
   lbm_latest_kernel<<<1, 256, 0, h->stream>>>(h->diag, h->diag_count, h->clprof, h->L.Nx,
                                               profile && !wide ? 1 : 0, h->h_pinned);
   CK(cudaGetLastError());
-  CK(cudaStreamSynchronize(h->stream));
+  CK(wait_stream(h));
   const unsigned long long cnt = (unsigned long long)h->h_pinned[0];
   if (cnt == 0) return set_err(LBM_EINVAL, "no step taken yet");
   memcpy(rec, h->h_pinned + 1, sizeof(double) * NREC);
@@ -2404,7 +2418,7 @@ int latest_record(lbm_mix* h, double rec[NREC], double* profile) {
   if (profile && wide) {
     CK(cudaMemcpyAsync(profile, h->clprof, sizeof(double) * (size_t)h->L.Nx,
                        cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaStreamSynchronize(h->stream));
+    CK(wait_stream(h));
   } else if (profile) {
     memcpy(profile, h->h_pinned + 16, sizeof(double) * (size_t)h->L.Nx);
   }
@@ -2493,7 +2507,7 @@ int get_post_state_t(lbm_mix* h, T* f, long n) {
        })))
     return st;
   CK(cudaMemcpyAsync(f, h->scratch, bytes, cudaMemcpyDeviceToHost, h->stream));
-  CK(cudaStreamSynchronize(h->stream));
+  CK(wait_stream(h));
   return LBM_OK;
 }
 
@@ -2747,7 +2761,7 @@ int lbm_mix_run_to_steady(lbm_mix* h, double tol, long max_steps, long check_eve
     if ((st = lbm_mix_step(h, k))) return st;
     taken += k;
     if ((st = launch_residual(h, k))) return st;
-    CK(cudaStreamSynchronize(h->stream));
+    CK(wait_stream(h));
     R = h->h_pinned[0];
     if (isnan(R)) {
       result = set_err(LBM_ENONFINITE, "non-finite residual after %ld steps", taken);
@@ -2839,7 +2853,7 @@ int lbm_mix_moments(lbm_mix* h, double* rho_a, double* rho_b, double* ua_x, doub
     if (outs[k])
       CK(cudaMemcpyAsync(outs[k], h->mom + k * plane, sizeof(double) * plane,
                          cudaMemcpyDeviceToHost, h->stream));
-  CK(cudaStreamSynchronize(h->stream));
+  CK(wait_stream(h));
   return LBM_OK;
 }
 
@@ -2873,7 +2887,7 @@ int lbm_mix_volume_flow(lbm_mix* h, int x, double* Qv) {
     return LBM_OK;
   });
   if (st) return st;
-  CK(cudaStreamSynchronize(h->stream));
+  CK(wait_stream(h));
   *Qv = h->h_pinned[0];
   if (!isfinite(*Qv)) return set_err(LBM_ENONFINITE, "non-finite volume flow");
   return LBM_OK;
@@ -2899,7 +2913,7 @@ int lbm_mix_history(lbm_mix* h, double* rec, long max_records, long* count) {
   if (!rec || max_records < 0 || !count) return set_err(LBM_EINVAL, "bad history arguments");
   unsigned long long cnt = 0;
   CK(cudaMemcpyAsync(&cnt, h->diag_count, sizeof cnt, cudaMemcpyDeviceToHost, h->stream));
-  CK(cudaStreamSynchronize(h->stream));
+  CK(wait_stream(h));
   long have = (long)(cnt < (unsigned long long)DIAG_CAP ? cnt : DIAG_CAP);
   long take = have < max_records ? have : max_records;
   for (long k = 0; k < take; ++k) {
@@ -2907,7 +2921,7 @@ int lbm_mix_history(lbm_mix* h, double* rec, long max_records, long* count) {
     CK(cudaMemcpyAsync(rec + k * NREC, h->diag + idx * NREC, sizeof(double) * NREC,
                        cudaMemcpyDeviceToHost, h->stream));
   }
-  CK(cudaStreamSynchronize(h->stream));
+  CK(wait_stream(h));
   *count = take;
   return LBM_OK;
 }
@@ -2955,7 +2969,7 @@ int lbm_mix_set_post_state(lbm_mix* h, const float* f, long n) {
   }
   if ((st = launch_colsum(h, 0))) return st;
   if ((st = reset_diag(h))) return st;
-  CK(cudaStreamSynchronize(h->stream));
+  CK(wait_stream(h));
   return LBM_OK;
 }
 
@@ -2984,7 +2998,7 @@ int lbm_mix_launches_per_step(const lbm_mix* h) {
 int lbm_mix_sync(lbm_mix* h) {
   int st = check_handle(h);
   if (st) return st;
-  CK(cudaStreamSynchronize(h->stream));
+  CK(wait_stream(h));
   return LBM_OK;
 }
 
@@ -3068,8 +3082,8 @@ int lbm_mix_step_noalloc(const lbm_mix_params* p, const float* d_in, float* d_ou
 
 // ---------------------------------------------------------------- sweeps
 // A parametric study (Table 1) runs many independent channels, each too small
-// to fill the GPU.  A sweep advances all of them by common launches on one
-// stream: the channels that fit tiles by lbm_tile_kernel, k steps a launch,
+// to fill the GPU.  A sweep advances all of them by common launches on a
+// stream of its own, its handles keep theirs for calls of their own: the channels that fit tiles by lbm_tile_kernel, k steps a launch,
 // in tiles wide enough that the redundant halo work stays small; the others
 // by lbm_step_batch_kernel, one step a launch; then one launch each for the
 // records and for the residuals of a convergence check.  The launches carry
@@ -3083,6 +3097,7 @@ struct lbm_sweep {
   int n = 0;
   lbm_mix** h = nullptr;
   cudaStream_t stream = nullptr;
+  cudaEvent_t joined = nullptr;  // see join_handles
   double* h_resid = nullptr;  // [n] residuals of a check, pinned
   int policy = -1;            // schedule in use (-1: the library default)
   double round_ms[LBM_SWEEP_NPOLICY] = {};
@@ -3205,6 +3220,19 @@ int launch_step_batch(lbm_mix* const* hs, int n, bool end, cudaStream_t st) {
                       st);
 }
 
+// Lets the sweep's stream wait for what calls on its handles left on theirs.
+// (The other way round every call of a sweep ends with a wait of the host.)
+int join_handles(lbm_sweep* s) {
+  for (int i = 0; i < s->n; ++i) {
+    lbm_mix* h = s->h[i];
+    if (!h->pending) continue;
+    CK(cudaEventRecord(s->joined, h->stream));
+    CK(cudaStreamWaitEvent(s->stream, s->joined, 0));
+    h->pending = false;
+  }
+  return LBM_OK;
+}
+
 // nsteps steps of the n channels hs of a sweep, on its stream.  Channels that
 // qualify for tiles take them, grouped by N, unless one step kernel over all
 // channels is estimated to be faster (many nodes in all, or tall channels) or
@@ -3309,6 +3337,7 @@ int lbm_sweep_create(const lbm_mix_params* params, int n, lbm_sweep** out) {
   }
   s->n = n;
   cudaError_t e = cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s->joined, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaMallocHost((void**)&s->h_resid, sizeof(double) * n);
   for (auto kern : {(const void*)lbm_tile_kernel<8>, (const void*)lbm_tile_kernel<TILE_BATCH>})
     if (e == cudaSuccess)
@@ -3323,7 +3352,7 @@ int lbm_sweep_create(const lbm_mix_params* params, int n, lbm_sweep** out) {
   for (int i = 0; i < n; ++i) {
     lbm_mix_params p = params[i];
     p.reref_every = 0;
-    int st = lbm_mix_create(&p, s->stream, &s->h[i]);  // all on the sweep's stream
+    int st = lbm_mix_create(&p, nullptr, &s->h[i]);  // a stream of its own
     if (st) {
       lbm_sweep_destroy(s);
       return st;
@@ -3340,6 +3369,7 @@ void lbm_sweep_destroy(lbm_sweep* s) {
     if (s->h) lbm_mix_destroy(s->h[i]);
   free(s->h);
   if (s->h_resid) cudaFreeHost(s->h_resid);
+  if (s->joined) cudaEventDestroy(s->joined);
   if (s->stream) cudaStreamDestroy(s->stream);
   delete s;
 }
@@ -3356,9 +3386,11 @@ int lbm_sweep_init(lbm_sweep* s) {
 int lbm_sweep_step(lbm_sweep* s, long nsteps) {
   if (!s) return set_err(LBM_EINVAL, "sweep is NULL");
   if (nsteps < 0) return set_err(LBM_EINVAL, "nsteps < 0");
-  int st = batch_steps(s, s->h, s->n, nsteps);
+  int st = join_handles(s);
+  if (!st) st = batch_steps(s, s->h, s->n, nsteps);
+  const cudaError_t e = cudaStreamSynchronize(s->stream);  // also after an error
   if (st) return st;
-  CK(cudaStreamSynchronize(s->stream));
+  CK(e);
   return LBM_OK;
 }
 
@@ -3386,9 +3418,9 @@ int lbm_sweep_run_to_steady(lbm_sweep* s, double tol, long max_steps, long check
     s->h[i]->p.diag_every = (int)check_every;
     if (max_steps > 0) act[na++] = i;
   }
-  int st = LBM_OK;
+  int st = join_handles(s);
   int trial = autotune ? 0 : -1;  // next schedule to try
-  if (!autotune && s->policy < 0) st = apply_policy(s, 0);
+  if (st == LBM_OK && !autotune && s->policy < 0) st = apply_policy(s, 0);
   while (na > 0 && st == LBM_OK) {
     if (trial >= 0 && (st = apply_policy(s, trial))) break;
     // every active instance advances k steps
@@ -3418,6 +3450,7 @@ int lbm_sweep_run_to_steady(lbm_sweep* s, double tol, long max_steps, long check
     }
     na = nb;
   }
+  if (st) cudaStreamSynchronize(s->stream);
   for (int i = 0; i < n; ++i) {
     if (steps_out) steps_out[i] = taken[i];
     if (residual_out) residual_out[i] = R[i];
