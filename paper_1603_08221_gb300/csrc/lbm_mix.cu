@@ -3205,19 +3205,25 @@ int launch_step_batch(lbm_mix* const* hs, int n, bool end, cudaStream_t st) {
     walls += (h->L.Nx + WALL_COLS - 1) / WALL_COLS;
     I.wall_r = h->wall_r;
     I.wall_omq = h->wall_omq;
-    h->cur = 1 - h->cur;
-    h->steps++;
   }
   B.block0[STEP_BATCH] = blocks;
   B.wall0[STEP_BATCH] = walls;
-  if (blocks < WALL_KERNEL_WAVES_SET * 3L * (hs[0]->nsm > 0 ? hs[0]->nsm : 1))
-    return launch_batch(lbm_step_batch_kernel<STEP_BATCH, false>, B, dim3(blocks), dim3(TX, TY), 0,
-                        st);
-  int s = launch_batch(lbm_walls_batch_kernel<STEP_BATCH>, B, dim3(walls, 4), dim3(WALL_COLS), 0,
+  int s = LBM_OK;
+  if (blocks < WALL_KERNEL_WAVES_SET * 3L * (hs[0]->nsm > 0 ? hs[0]->nsm : 1)) {
+    s = launch_batch(lbm_step_batch_kernel<STEP_BATCH, false>, B, dim3(blocks), dim3(TX, TY), 0,
+                     st);
+  } else {
+    s = launch_batch(lbm_walls_batch_kernel<STEP_BATCH>, B, dim3(walls, 4), dim3(WALL_COLS), 0, st);
+    if (!s)
+      s = launch_batch(lbm_step_batch_kernel<STEP_BATCH, true>, B, dim3(blocks), dim3(TX, TY), 0,
                        st);
+  }
   if (s) return s;
-  return launch_batch(lbm_step_batch_kernel<STEP_BATCH, true>, B, dim3(blocks), dim3(TX, TY), 0,
-                      st);
+  for (int q = 0; q < n; ++q) {
+    hs[q]->cur = 1 - hs[q]->cur;
+    hs[q]->steps++;
+  }
+  return LBM_OK;
 }
 
 // Lets the sweep's stream wait for what calls on its handles left on theirs.

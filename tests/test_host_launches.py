@@ -1,0 +1,107 @@
+"""The library's host code against a stand-in for the CUDA runtime (no GPU):
+what calls launch, within which grids, and what they leave behind when a launch
+fails."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import pytest
+
+from paper_1603_08221_gb300 import binding, build, workloads
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    if shutil.which("nvcc") is None and not os.path.exists("/usr/local/cuda/bin/nvcc"):
+        pytest.skip("no nvcc")
+    out = tmp_path_factory.mktemp("fake") / "liblbm_fake.so"
+    # PTX only and unoptimised: the device code is never run
+    subprocess.run([build.nvcc(), "-gencode", "arch=compute_103a,code=compute_103a", "-Xcicc", "-O0",
+                    "-std=c++17", "-Xcompiler", "-fPIC", "-cudart", "none",
+                    "-shared", build.SRC, os.path.join(HERE, "fake_cudart.c"), "-o", str(out)],
+                   check=True)
+    lib = ctypes.CDLL(str(out))
+    for name, (res, args) in binding._SIGS.items():
+        if not name.startswith("lbm_adj"):
+            fn = getattr(lib, name)
+            fn.restype, fn.argtypes = res, args
+    lib.fake_launch.restype = ctypes.c_char_p
+    return lib
+
+
+def _params(lib, **kw):
+    p = binding.lbm_mix_params()
+    lib.lbm_mix_default_params(ctypes.byref(p))
+    for k, v in workloads.preset("heli_argon_320x16", **kw).items():
+        setattr(p, k, v)
+    return p
+
+
+def _launches(lib):
+    grid = (ctypes.c_uint * 3)()
+    out = []
+    for k in range(lib.fake_launches()):
+        name = lib.fake_launch(k, grid).decode()
+        out.append((name, tuple(grid)))
+    return out
+
+
+class Handle:
+    def __init__(self, lib, **kw):
+        self.lib, p = lib, _params(lib, **kw)
+        h = ctypes.c_void_p()
+        assert lib.lbm_mix_create(ctypes.byref(p), None, ctypes.byref(h)) == 0
+        self.h = h
+        assert lib.lbm_mix_init(h) == 0
+
+    def __enter__(self):
+        return self.h
+
+    def __exit__(self, *exc):
+        self.lib.lbm_mix_destroy(self.h)
+
+
+def _steps(lib, h):
+    n, nx, steps = ctypes.c_int(), ctypes.c_int(), ctypes.c_long()
+    assert lib.lbm_mix_dims(h, ctypes.byref(n), ctypes.byref(nx), ctypes.byref(steps)) == 0
+    return steps.value
+
+
+# channels whose sweep takes batched step kernels with and without the wall
+# kernel ahead of them, and tiles with their records
+@pytest.mark.parametrize("count,N,Nx", [(1, 600, 100), (40, 600, 100), (12, 600, 3000), (3, 20, 600)])
+def test_a_failed_launch_of_a_sweep_leaves_no_step_behind(fake, count, N, Nx):
+    """Steps are counted, and the buffers change places, where their launch was
+    accepted: after a failure at the k-th launch of a call every handle has taken
+    the steps of the launches before it."""
+    lib = fake
+    ps = (binding.lbm_mix_params * count)(*[_params(lib, N=N, N_x=Nx) for _ in range(count)])
+    for fail in (0, 1):
+        s = ctypes.c_void_p()
+        assert lib.lbm_sweep_create(ps, count, ctypes.byref(s)) == 0
+        assert lib.lbm_sweep_init(s) == 0
+        lib.fake_reset()
+        lib.fake_fail(fail)
+        status = lib.lbm_sweep_step(s, 1)
+        log = _launches(lib)
+        lib.fake_reset()
+        if fail >= len(log):
+            assert status == 0
+            lib.lbm_sweep_destroy(s)
+            continue
+        assert status == binding.LBM_ECUDA
+        accepted = [n for n, _ in log[:fail]]
+        h = ctypes.c_void_p()
+        taken = 0
+        for k in range(count):
+            assert lib.lbm_sweep_instance(s, k, ctypes.byref(h)) == 0
+            taken += _steps(lib, h)
+        # a launch of steps holds 32 channels of the step kernel at most, all of
+        # these tiles
+        most = sum(min(32, count) if "step_batch" in n else count if "tile" in n else 0
+                   for n in accepted)
+        assert taken == most, (fail, log)
+        lib.lbm_sweep_destroy(s)
