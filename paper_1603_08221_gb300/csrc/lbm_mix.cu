@@ -1994,6 +1994,8 @@ int default_rows(int N, int strips, int nsm, bool fp32) {
   const long ctas = (long)WAVES * 3 * (nsm > 0 ? nsm : 1);
   long rows = ((long)N * strips / ctas + TY - 1) / TY * TY;
   rows = rows < 16 ? 16 : rows < most ? rows : most;
+  const long fit = (N + 65534L) / 65535;  // a grid has 65535 row blocks at most
+  if (rows < fit) rows = (fit + TY - 1) / TY * TY;
   return (int)(rows < n8 ? rows : n8);
 }
 int default_rows(const lbm_mix* h) {

@@ -105,3 +105,17 @@ def test_a_failed_launch_of_a_sweep_leaves_no_step_behind(fake, count, N, Nx):
                    for n in accepted)
         assert taken == most, (fail, log)
         lib.lbm_sweep_destroy(s)
+
+
+# the tallest channels that validate takes (18 N pitch below 2^31), and one row
+# either side of 65535 blocks of the 56 rows that FP32 row blocks have at most
+@pytest.mark.parametrize("N", [56 * 65535, 56 * 65535 + 1, 3728000])
+@pytest.mark.parametrize("storage", [binding.LBM_FP32, binding.LBM_BF16])
+def test_grids_of_the_tallest_channels(fake, N, storage):
+    """A grid has 65535 blocks in y at most."""
+    lib = fake
+    with Handle(lib, N=N, N_x=8, storage=storage, diag_every=2) as h:
+        lib.fake_reset()
+        assert lib.lbm_mix_step(h, 3) == 0
+        rows = [g[1] for n, g in _launches(lib) if "lbm_step_kernel" in n]
+        assert len(rows) == 3 and max(rows) <= 65535
