@@ -414,24 +414,18 @@ def run_ours(args):
     barrier()
     ev0 = torch.cuda.Event(enable_timing=True)
     ev1 = torch.cuda.Event(enable_timing=True)
+    launches = binding.lbm_mix_launches(sim.h)
     with ClockSampler(local) as clk:
         ev0.record(stream)
         binding.lbm_mix_step(sim.h, args.steps)
         ev1.record(stream)
         ev1.synchronize()
+    launches = binding.lbm_mix_launches(sim.h) - launches  # in the timed region
     barrier()
     elapsed = ev0.elapsed_time(ev1) / 1e3
     sep = sim.separation()  # raises on a non-finite state
-    # kernels in the timed region: the step kernel, and the wall kernel ahead
-    # of it where the library runs one (16-bit storage; FP32 grids of two or
-    # more waves), per step; 16-bit storage adds, every 256 steps (counted
-    # from the handle's first step), the two kernels of a re-reference
-    per_step = binding.lbm_mix_launches_per_step(sim.h)
     # bytes of one population buffer (strips of 32 columns, 18 values per node)
     state_gb = 18 * sim.N * 32 * ((sim.N_x + 31) // 32) * (4 if args.storage == "fp32" else 2) / 1e9
-    launches = args.steps * per_step
-    if args.storage != "fp32":
-        launches += 2 * ((args.warmup + args.steps) // 256 - args.warmup // 256)
 
     # ---------------- end to end through the C ABI with host buffers
     f_host = torch.empty((2, 9, sim.N, sim.N_x), dtype=torch.float32, pin_memory=True)

@@ -263,6 +263,12 @@ int lbm_mix_dims(const lbm_mix* h, int* N, int* N_x, long* steps);
  * LBM_EINVAL for a NULL handle. */
 int lbm_mix_launches_per_step(const lbm_mix* h);
 
+/* Kernels that the calls advancing h by itself (lbm_mix_step, and those made of
+ * it) have launched so far: steps, the wall kernels and records beside them,
+ * re-referencing.  The common launches of a sweep and replays of captured steps
+ * are not counted.  Returns the count, or LBM_EINVAL for a NULL handle. */
+long lbm_mix_launches(const lbm_mix* h);
+
 /* Waits for all work enqueued on the handle's stream. */
 int lbm_mix_sync(lbm_mix* h);
 

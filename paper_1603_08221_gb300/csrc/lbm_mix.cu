@@ -1796,6 +1796,7 @@ struct lbm_mix {
   int nsm;            // streaming multiprocessors of the device
   cudaStream_t stream;
   bool own_stream;
+  long launches;     // kernels launched by its own steps so far
   bool pending;      // a call may have left work on the stream (see join_handles)
   int nblocks;
   void* buf[2];       // post-collision deviations, A/B (element type per storage)
@@ -2056,6 +2057,7 @@ int rereference(lbm_mix* h) {
     return LBM_OK;
   });
   if (st) return st;
+  h->launches += 2;
   float* t = h->refrho;
   h->refrho = h->refrho_alt;
   h->refrho_alt = t;
@@ -2176,6 +2178,7 @@ int launch_step(lbm_mix* h, bool diag) {
       CK(cudaLaunchKernelEx(&cfg, lbm_walls_kernel<ST>, h->L, a.fin, (const float*)h->refrho,
                             (const double*)a.cs_in, (const float*)h->alpha, h->wall_r,
                             h->wall_omq));
+      h->launches++;
     }
     cfg.gridDim = dim3(h->nblocks, (h->L.N + a.rows_per_block - 1) / a.rows_per_block);
     cfg.blockDim = dim3(TX, TY);
@@ -2193,6 +2196,7 @@ int launch_step(lbm_mix* h, bool diag) {
     return LBM_OK;
   });
   if (st) return st;
+  h->launches++;
   h->cur = 1 - h->cur;
   h->steps++;
   return LBM_OK;
@@ -2309,6 +2313,7 @@ int launch_tiles(lbm_mix* const* hs, const int* W, int n, int k, bool last, int*
   int s = launch_batch(lbm_tile_kernel<NI>, B, dim3(blocks),
                        dim3(threads + TILE_WALL + TILE_TAUQ), smem, st);
   if (s) return s;
+  if (NI == 1) hs[0]->launches++;
   for (int q = 0; q < n; ++q) {
     hs[q]->cur = 1 - hs[q]->cur;
     hs[q]->steps += k;
@@ -2332,6 +2337,7 @@ int launch_records(lbm_mix* const* hs, int n, int* rows, cudaStream_t st) {
     rows[q] = 0;
   }
   if (most == 0) return LBM_OK;
+  if (NI == 1) hs[0]->launches++;
   return launch_batch(lbm_records_kernel<NI>, B, dim3(blocks, most, n), dim3(256), 0, st);
 }
 
@@ -2995,6 +3001,11 @@ int lbm_mix_launches_per_step(const lbm_mix* h) {
   if (st) return st;
   const bool tiles = uses_tiles(h) && h->L.Nx <= SINGLE_STEP_COLUMNS;
   return (h->elem < 4 || tiles || uses_wall_kernel(h)) ? 2 : 1;
+}
+
+long lbm_mix_launches(const lbm_mix* h) {
+  int st = check_handle(h);
+  return st ? st : h->launches;
 }
 
 int lbm_mix_sync(lbm_mix* h) {

@@ -119,3 +119,22 @@ def test_grids_of_the_tallest_channels(fake, N, storage):
         assert lib.lbm_mix_step(h, 3) == 0
         rows = [g[1] for n, g in _launches(lib) if "lbm_step_kernel" in n]
         assert len(rows) == 3 and max(rows) <= 65535
+
+
+# tiles with records of their own and in common, single steps of wide channels,
+# the step kernel with and without the wall kernel, 16-bit storage,
+# re-referencing in between
+@pytest.mark.parametrize("kw", [dict(N=16, N_x=320), dict(N=16, N_x=320, diag_every=1),
+                                dict(N=16, N_x=320, reref_every=7), dict(N=16, N_x=8000, diag_every=4),
+                                dict(N=600, N_x=100), dict(N=512, N_x=32768),
+                                dict(N=130, N_x=5001, storage=binding.LBM_BF16, reref_every=5)])
+def test_launches_are_counted(fake, kw):
+    lib = fake
+    with Handle(lib, **kw) as h:
+        lib.fake_reset()
+        base = lib.lbm_mix_launches(h)
+        for n in (1, 2, 3, 16, 400):
+            assert lib.lbm_mix_step(h, n) == 0
+            assert lib.lbm_mix_launches(h) - base == lib.fake_launches(), n
+        if kw == dict(N=16, N_x=320):
+            assert lib.fake_launches() < 422 / 4  # several steps a launch
