@@ -538,7 +538,7 @@ def run_ours(args):
                      "frac": achieved / peak, "traffic": traffic,
                      "peak_source": peak_kind, "kernel": KERNEL,
                      "timed": ("whole step: the step kernel and the wall kernel ahead of it"
-                               if per_step == 2 else "whole step: the step kernel"),
+                               if launches >= 2 * args.steps else "whole step"),
                      "nominal_peak": NOMINAL_HBM_GBS,
                      "frac_of_nominal": achieved / NOMINAL_HBM_GBS},
         "cpu_baseline": cpu,

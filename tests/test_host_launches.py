@@ -18,11 +18,12 @@ def fake(tmp_path_factory):
     if shutil.which("nvcc") is None and not os.path.exists("/usr/local/cuda/bin/nvcc"):
         pytest.skip("no nvcc")
     out = tmp_path_factory.mktemp("fake") / "liblbm_fake.so"
-    # PTX only and unoptimised: the device code is never run
-    subprocess.run([build.nvcc(), "-gencode", "arch=compute_103a,code=compute_103a", "-Xcicc", "-O0",
-                    "-std=c++17", "-Xcompiler", "-fPIC", "-cudart", "none",
-                    "-shared", build.SRC, os.path.join(HERE, "fake_cudart.c"), "-o", str(out)],
-                   check=True)
+    # PTX only and unoptimised: the device code is never run; its own runtime, not
+    # one that the process has loaded
+    subprocess.run([build.nvcc(), "-gencode", "arch=compute_103a,code=compute_103a",
+                    "-Xcicc", "-O0", "-std=c++17", "-Xcompiler", "-fPIC", "-cudart", "none",
+                    "-Xlinker", "-Bsymbolic", "-shared", build.SRC,
+                    os.path.join(HERE, "fake_cudart.c"), "-o", str(out)], check=True)
     lib = ctypes.CDLL(str(out))
     for name, (res, args) in binding._SIGS.items():
         if not name.startswith("lbm_adj"):
@@ -72,7 +73,8 @@ def _steps(lib, h):
 
 # channels whose sweep takes batched step kernels with and without the wall
 # kernel ahead of them, and tiles with their records
-@pytest.mark.parametrize("count,N,Nx", [(1, 600, 100), (40, 600, 100), (12, 600, 3000), (3, 20, 600)])
+@pytest.mark.parametrize("count,N,Nx", [(1, 600, 100), (40, 600, 100), (12, 600, 3000),
+                                        (3, 20, 600)])
 def test_a_failed_launch_of_a_sweep_leaves_no_step_behind(fake, count, N, Nx):
     """Steps are counted, and the buffers change places, where their launch was
     accepted: after a failure at the k-th launch of a call every handle has taken
@@ -125,7 +127,8 @@ def test_grids_of_the_tallest_channels(fake, N, storage):
 # the step kernel with and without the wall kernel, 16-bit storage,
 # re-referencing in between
 @pytest.mark.parametrize("kw", [dict(N=16, N_x=320), dict(N=16, N_x=320, diag_every=1),
-                                dict(N=16, N_x=320, reref_every=7), dict(N=16, N_x=8000, diag_every=4),
+                                dict(N=16, N_x=320, reref_every=7),
+                                dict(N=16, N_x=8000, diag_every=4),
                                 dict(N=600, N_x=100), dict(N=512, N_x=32768),
                                 dict(N=130, N_x=5001, storage=binding.LBM_BF16, reref_every=5)])
 def test_launches_are_counted(fake, kw):
