@@ -8,6 +8,11 @@ its values at the nine Chebyshev nodes in 40-digit arithmetic: the remainder is
 below 1e-18 of psi.  A row holds the 27
 coefficients as (psi_k, psi'_k, psi''_k), k = 0 .. 8, and one pad.
 
+From 16 on, where the derivatives fall by e within a segment or two of an octave
+(relative remainder 9e-14 on [16, 32], 4e-11 on [32, 64]), psi' and psi'' have a
+table of their own with segments of a quarter, 64 and 128 in the two octaves, rows
+(psi'_k, psi''_k): remainder 8e-17 of either.
+
     python paper_1603_08221_gb300/csrc/gen_psi64_table.py > \
         paper_1603_08221_gb300/csrc/lbm_psi64_table.cuh
 """
@@ -17,6 +22,7 @@ import mpmath as mp
 
 mp.mp.dps = 40
 OCTAVE0, OCTAVES, SEGS, DEG = -10, 16, 32, 8
+FAR, WIDTH = 16, mp.mpf(1) / 4
 
 
 def functions(a):
@@ -38,21 +44,32 @@ def newton(us, fs):
     return c
 
 
+def segment(c, h):
+    """Polynomials in u = a - c of psi, psi' and psi'' on [c - h / 2, c + h / 2]."""
+    us = [h / 2 * mp.cos(mp.pi * (2 * k + 1) / (2 * (DEG + 1))) for k in range(DEG + 1)]
+    vals = [functions(c + u) for u in us]
+    return [newton(us, [v[f] for v in vals]) for f in range(3)]
+
+
 def main():
-    rows = []
+    rows, far = [], []
     for o in range(OCTAVE0, OCTAVE0 + OCTAVES):
         for s in range(SEGS):
-            h = mp.mpf(2) ** o / SEGS
-            c = mp.mpf(2) ** o * (1 + (mp.mpf(s) + mp.mpf(1) / 2) / SEGS)
-            us = [h / 2 * mp.cos(mp.pi * (2 * k + 1) / (2 * (DEG + 1))) for k in range(DEG + 1)]
-            vals = [functions(c + u) for u in us]
-            polys = [newton(us, [v[f] for v in vals]) for f in range(3)]
+            polys = segment(mp.mpf(2) ** o * (1 + (mp.mpf(s) + mp.mpf(1) / 2) / SEGS),
+                            mp.mpf(2) ** o / SEGS)
             rows.append([polys[f][k] for k in range(DEG + 1) for f in range(3)] + [mp.mpf(0)])
+    for s in range(int((64 - FAR) / WIDTH)):
+        polys = segment(FAR + (s + mp.mpf(1) / 2) * WIDTH, WIDTH)
+        far.append([polys[f][k] for k in range(DEG + 1) for f in (1, 2)])
     print("// lbm_psi64_table.cuh - generated by gen_psi64_table.py (segments and forms there).")
     print(f"constexpr int kPsi64Octave0 = {OCTAVE0}, kPsi64Octaves = {OCTAVES}, kPsi64Row = "
           f"{3 * (DEG + 1) + 1};")
     print(f"__device__ __align__(16) const double kPsi64[{OCTAVES * SEGS}][kPsi64Row] = {{")
     for r in rows:
+        print("    {" + ", ".join(mp.nstr(v, 18) for v in r) + "},")
+    print("};")
+    print(f"__device__ __align__(16) const double kPsi64Far[{len(far)}][{2 * (DEG + 1)}] = {{")
+    for r in far:
         print("    {" + ", ".join(mp.nstr(v, 18) for v in r) + "},")
     print("};")
 

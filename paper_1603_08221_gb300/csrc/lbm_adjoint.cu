@@ -309,31 +309,35 @@ __device__ __noinline__ Psi3 psid_general(double a) {
 // The same from the polynomials of lbm_psi64_table.cuh for 2^-10 <= a < 64: 8
 // FP64 operations a function where E_1 and exp took 80 together, on a pipe that
 // issues one warp instruction in 64 cycles per sub-partition (six psi a node
-// were over half of the forward step).  Relative error of psi below 2.1e-16,
-// absolute error of psi' 2.3e-16.  D1, D2: the derivatives wanted.
+// were over half of the forward step).  Relative errors: psi 2.1e-16; psi' and
+// psi'' 2e-16 up to 8, 3.5e-16 and 5e-16 up to 16 (general form: 1.3e-15 and
+// 3e-16), 3.4e-16 beyond (3.8e-15, 3.6e-16), where they come from a table of their
+// own.  D1, D2: the derivatives wanted.
 template <bool D1 = true, bool D2 = false>
 __device__ __forceinline__ Psi3 psid(double a) {
   const int hi = __double2hiint(a);
   if (!(a >= 0x1p-10 && a < 64.0)) return psid_general(a);
-  const double2* q = reinterpret_cast<const double2*>(
-      kPsi64[(hi >> 15) - ((1023 + kPsi64Octave0) << 5)]);
+  const double* q = kPsi64[(hi >> 15) - ((1023 + kPsi64Octave0) << 5)];
   const double u = a - __hiloint2double((hi & ~0x7fff) | 0x4000, 0);
-  double t[28];
-#pragma unroll
-  for (int k = 0; k < 14; ++k) {
-    const double2 w = __ldg(q + k);
-    t[2 * k] = w.x;
-    t[2 * k + 1] = w.y;
-  }
   Psi3 p;
-  p.v = t[24];
-  p.d1 = t[25];
-  p.d2 = t[26];
+  p.v = __ldg(q + 24);
 #pragma unroll
-  for (int k = 7; k >= 0; --k) {
-    p.v = fma(p.v, u, t[3 * k]);
-    if (D1) p.d1 = fma(p.d1, u, t[3 * k + 1]);
-    if (D2) p.d2 = fma(p.d2, u, t[3 * k + 2]);
+  for (int k = 7; k >= 0; --k) p.v = fma(p.v, u, __ldg(q + 3 * k));
+  if (D1) {
+    // psi', psi'' side by side, `step` doubles from one power to the next; from
+    // 16 on segments of a quarter: the top 6 mantissa bits below 32, 7 above
+    const bool far = hi >= 0x40300000;
+    const int above = hi >= 0x40400000 ? 1 : 0, shift = 14 - above, step = far ? 2 : 3;
+    const double* d = far ? kPsi64Far[((hi & 0xfffff) >> shift) + 64 * above] : q + 1;
+    const double w =
+        far ? a - __hiloint2double((hi & -(1 << shift)) | (1 << (shift - 1)), 0) : u;
+    p.d1 = __ldg(d + 8 * step);
+    if (D2) p.d2 = __ldg(d + 8 * step + 1);
+#pragma unroll
+    for (int k = 7; k >= 0; --k) {
+      p.d1 = fma(p.d1, w, __ldg(d + k * step));
+      if (D2) p.d2 = fma(p.d2, w, __ldg(d + k * step + 1));
+    }
   }
   return p;
 }
