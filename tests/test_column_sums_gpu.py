@@ -97,3 +97,37 @@ def test_column_sums_are_exact_sums(N, Nx, rows):
         for sp, name in enumerate(("rho_a", "rho_b")):
             exact = math.fsum(m[name][:, x])
             assert abs(cs[sp, x] - exact) <= 2.0 ** -44 * exact, (x, name)
+
+
+def _disturbed(g, amplitude, seed):
+    """The initial equilibrium, every population changed by its own factor."""
+    g.init()
+    f = np.asarray(g.get_post_state(), dtype=np.float64)
+    rng = np.random.default_rng(seed)
+    return (f * (1.0 + amplitude * rng.uniform(-1.0, 1.0, f.shape))).astype(np.float32)
+
+
+# The shapes of the test above, from a state that stays finite, so that every
+# record counts, and the mass flows beside the totals: 2^-34 of the sums of the
+# magnitudes (see the top), which for the momenta are at most the masses.
+@pytest.mark.parametrize("storage,N,Nx", [(binding.LBM_FP32, 130, 5001), (binding.LBM_FP32, 57, 9000),
+                                          (binding.LBM_BF16, 8, 64), (binding.LBM_BF16, 57, 98),
+                                          (binding.LBM_FP16, 131, 257)])
+def test_recorded_steps_of_a_finite_state(storage, N, Nx):
+    p = workloads.preset("heli_argon_320x16", N=N, N_x=Nx, theta=1.2, Kn_out=0.3, storage=storage,
+                         diag_every=2)
+    out = []
+    for rows in (0, 16):
+        g = binding.LbmMix(**p)
+        g.set_post_state(_disturbed(g, 0.01, seed=N))
+        g.set_rows_per_block(rows)
+        g.step(5)
+        out.append((np.asarray(g.get_post_state_f64())[..., 1:-1], g.history()))
+    (fa, ra), (fb, rb) = out
+    assert len(ra) == len(rb) == 3
+    assert all(np.isfinite(v).all() for v in (fa, fb, ra, rb))
+    assert np.array_equal(fa, fb)
+    total = rb[:, 6:8]
+    assert np.all(np.abs(ra[:, 6:8] - total) <= 2.0 ** -34 * total)
+    assert np.all(np.abs(ra[:, 3:5] - rb[:, 3:5]) <= 2.0 ** -34 * total / (Nx - 2))
+    assert np.all(np.abs(ra[:, 1:3] - rb[:, 1:3]) <= 2.0 ** -30)

@@ -164,3 +164,25 @@ def test_sweeps_take_the_steps_of_lone_channels(count, N, Nx):
                               g.get_post_state_f64()[..., 1:-1]), q
         a, b = sw.instance(q).separation(), g.separation()
         assert abs(a["CL"] - b["CL"]) < 1e-9 and a["x_min"] == b["x_min"]
+
+
+@pytest.mark.parametrize("steps", [[9], [1, 8], [5, 2, 2]])
+def test_sweeps_of_tiled_and_other_channels(steps):
+    """Channels that qualify for tiles, of three row counts, among more others
+    than one launch of the step kernel holds (32): each as on its own."""
+    small = [dict(N=n, N_x=300 + 40 * q) for q, n in enumerate([16, 20, 20, 24, 16, 20])]
+    tall = [dict(N=440 + 8 * (q % 3), N_x=60 + 7 * (q % 5)) for q in range(38)]
+    params = [workloads.preset("heli_argon_320x16", theta=1.2 + 0.005 * q, Kn_out=0.3, **d)
+              for q, d in enumerate(tall[:20] + small + tall[20:])]
+    sw = binding.LbmSweep(params)
+    sw.init()
+    for n in steps:
+        sw.step(n)
+    for q in (0, 19, 20, 22, 25, 26, 40, len(params) - 1):
+        g = binding.LbmMix(**params[q])
+        g.init()
+        for n in steps:
+            g.step(n)
+        assert sw.instance(q).steps == sum(steps)
+        assert np.array_equal(sw.instance(q).get_post_state_f64()[..., 1:-1],
+                              g.get_post_state_f64()[..., 1:-1]), q
