@@ -49,12 +49,11 @@ namespace {
 
 #include "lbm_psi64_table.cuh"
 
-// Programmatic dependent launch of the per-step kernel sequences: each
-// kernel lets the next one in its stream launch once all of its own CTAs
-// run (launch_dependents), and waits for the previous one's completion and
-// memory (wait) before its first global memory access, so that launches
-// and CTA ramps overlap the end of the kernel before.  Both return at once
-// for a kernel launched without the attribute.
+// The kernels of the per-step sequences are launched with programmatic stream
+// serialisation and wait here for the one before them, its completion and its
+// memory, before their first global memory access.  None lets its successor
+// launch early: that made the gradient slower, the successor's CTAs then sitting
+// unevenly on the SMs that the running kernel leaves free.
 __device__ __forceinline__ void pdl_enter() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 constexpr double kPiD = 3.14159265358979323846;
@@ -1279,7 +1278,7 @@ struct lbm_adj {
   // inputs, column data and Psi values: the backward sweep replays into
   // them; the forward run fills set (nseg - 1) & 1 with the last interval.
   double* seg[2] = {nullptr, nullptr};      // [K][S] inputs of one segment's steps
-  double* segcols[2] = {nullptr, nullptr};  // [K][4 Nx + 4] column data of those steps
+  double* segcols[2] = {nullptr, nullptr};  // [K][18 Nx + 4] column data of those steps
   double* segpsi[2] = {nullptr, nullptr};   // [K][6][N][Nx] Psi values of those steps
   cudaStream_t rstream = nullptr;   // the replays of the backward sweep
   cudaEvent_t ev_start = nullptr, ev_rep[2] = {nullptr, nullptr}, ev_rev[2] = {nullptr, nullptr};

@@ -2,7 +2,7 @@
 //
 // One time step of the two-species D2Q9 MRT lattice Boltzmann model of
 // Wang, Xu & Guo (arXiv:1603.08221, Sec. 3) is ONE fused kernel launch
-// (lbm_step_kernel; on grids of two or more waves and with 16-bit storage,
+// (lbm_step_kernel; on grids of several waves and with 16-bit storage,
 // lbm_walls_kernel computes the wall parameters r and tau_q of every column
 // ahead of it), and small FP32 channels take several steps per launch
 // (lbm_tile_kernel, lbm_tile.cuh): pull-streaming from the previous post-collision buffer
@@ -10,9 +10,10 @@
 // extrapolation-correction ends (Eqs. rho1, rho2) folded into the loads,
 // moments (Eq. rhou), effective relaxation times (Eqs. EQFrb, EQFrsp, psi,
 // taos, taoq, A12), the MRT collision (Eqs. MR, m, S, feq) for both species,
-// the store of the new post-collision buffer, and FP64 per-column reductions
-// that feed the next step's density correction and the separation
-// diagnostics (Eqs. C, CL, Clline).
+// the store of the new post-collision buffer, and per-column reductions (pairs
+// of floats, 2^-44 of the sum and better, FP64 over the columns) that feed the
+// next step's density correction and the separation diagnostics (Eqs. C, CL,
+// Clline).
 //
 // Data layout in HBM (per buffer): the channel is cut into strips of 32
 // columns; strip s holds, row after row, the nine populations of its 32
@@ -110,10 +111,7 @@ struct Lat : LatCore {
   int light;             // index of the light species
   float cw0[2];          // rest-equilibrium weights w_i alpha_si: rest (9 - 5s)/9,
   float cw1[2], cw5[2];  // axis s/9, diagonal s/36
-  float ke[2][3], kp[2][3];  // the coefficients behind ce2, cp2, unscaled
-  float2 ke2[3], kp2[3];     // the same in pairs
-  float c_xl[2];         // 3 mu_s sqrt(pi/(6 m_s)): x_s lambda_s = c_xl / n
-  float inv_c_xl[2];
+  float2 ke2[3], kp2[3]; // the coefficients behind ce2, cp2, unscaled
   float om_e, om_eps;    // 1/tau_e, 1/tau_eps
   double mh[2];          // m_sigma / m_min
   double rho_in[2], rho_out[2];
@@ -1407,8 +1405,7 @@ __device__ __forceinline__ void step_cta(const Lat& L, const StepArgs<ST>& a, co
       } else {
         n16::Macro2 m;
         n16::macro2(L, C, g, m);
-        // bound by instruction issue: skipping the unused form of psi pays
-        n16::rates2<true>(L, m, (float)j + 0.5f, om_s, om_d);
+        n16::rates2(L, m, (float)j + 0.5f, om_s, om_d);
         const float om_q = wall_omq(j < half ? 0 : 1);
         mxs = n16::collide2(g, L, m.rho, m.ux, m.uy, L.om_e, L.om_eps, om_d, om_q, om_s);
         sd = m.sd;
@@ -1920,13 +1917,6 @@ Lat derive(const lbm_mix_params* p, int Nx) {
     L.cw0[sp] = (float)((9.0 - 5.0 * (double)L.s[sp]) / 9.0);
     L.cw1[sp] = (float)((double)L.s[sp] / 9.0);
     L.cw5[sp] = (float)((double)L.s[sp] / 36.0);
-    const float sf = L.s[sp];
-    L.ke[sp][0] = -2.0f * sf;
-    L.ke[sp][1] = 3.0f - 2.0f * sf;
-    L.ke[sp][2] = 6.0f - 2.0f * sf;
-    L.kp[sp][0] = 3.0f * sf;
-    L.kp[sp][1] = 3.0f * sf - 6.0f;
-    L.kp[sp][2] = 3.0f * sf - 3.0f;
   }
   for (int sp = 0; sp < 2; ++sp) {
     float* s2 = &L.s2.x;
@@ -1935,9 +1925,12 @@ Lat derive(const lbm_mix_params* p, int Nx) {
     (&L.cw5_2.x)[sp] = L.cw5[sp];
     const double we = 1.0 / (36.0 * p->tau_e), wp = 1.0 / (36.0 * p->tau_eps);
     const double sd = (double)L.s[sp];
+    const float sf = L.s[sp];
+    const float ke[3] = {-2.0f * sf, 3.0f - 2.0f * sf, 6.0f - 2.0f * sf};
+    const float kp[3] = {3.0f * sf, 3.0f * sf - 6.0f, 3.0f * sf - 3.0f};
     for (int k = 0; k < 3; ++k) {
-      (&L.ke2[k].x)[sp] = L.ke[sp][k];
-      (&L.kp2[k].x)[sp] = L.kp[sp][k];
+      (&L.ke2[k].x)[sp] = ke[k];
+      (&L.kp2[k].x)[sp] = kp[k];
       (&L.ce2[k].x)[sp] = (float)(we * (3.0 * k - 2.0 * sd));
       (&L.cp2[k].x)[sp] = (float)(wp * (3.0 * sd - (k == 0 ? 0.0 : k == 1 ? 6.0 : 3.0)));
     }
@@ -1946,10 +1939,8 @@ Lat derive(const lbm_mix_params* p, int Nx) {
     L.mh[sp] = mh[sp];
     L.rsqrt_mh[sp] = (float)(1.0 / sqrt(mh[sp]));
     double cxl = 3.0 * mu_s[sp] * sqrt(PI / (6.0 * mh[sp]));
-    L.c_xl[sp] = (float)cxl;
-    L.inv_c_xl[sp] = (float)(1.0 / cxl);
-    (&L.c_xl2.x)[sp] = L.c_xl[sp];
-    (&L.inv_c_xl2.x)[sp] = L.inv_c_xl[sp];
+    (&L.c_xl2.x)[sp] = (float)cxl;
+    (&L.inv_c_xl2.x)[sp] = (float)(1.0 / cxl);
     L.rho_in[sp] = p->theta * Ci[sp] * mh[sp];
     L.rho_out[sp] = Co[sp] * mh[sp];
     for (int end = 0; end < 2; ++end) {
@@ -2218,10 +2209,12 @@ double tile_cost(int N, int nup, int W, int k, int sms) {
   const double nodes = (double)k * (W + k - 1) * tile_stride(N);
   return (TILE_LAUNCH_US + waves * (TILE_LOAD_US + k * TILE_STEP_US + TILE_NODE_US * nodes)) / k;
 }
-// The same for the step kernel under its default schedule (measured from 64 x
-// 3000, 18.3 us, to 128 x 8000, 32.6 us): below some 400 000 nodes of at most 64
-// rows the tiles win (64 x 6000: 17.0 against 19.1 us), with 128 rows only up
-// to 1300 columns (13.2 against 18 us).
+// The same for the step kernel under its default schedule as the tiles were
+// fitted against it (64 x 3000 18.3 us, 128 x 8000 32.6).  With the end strips first
+// it has since become faster, 10 us up to some 100 000 nodes and 14 at 250 000, so
+// near the line tiles are no longer the better choice: columns x rows 4000 x 64
+// 12.8 us by tiles and 13.4, 14000 x 32 18.9 and 14.1, 2000 x 128 21.1 and 13.2
+// (either was 50 and more before tiles).
 double step_kernel_cost(int N, int Nx) { return 15.0 + 1.75e-5 * (double)N * Nx; }
 
 // Tile width and steps per launch (odd, so that launches alternate the two
@@ -3193,8 +3186,10 @@ double plan_batch(lbm_mix* const* hs, int n, int* W, int* k_out) {
 // One step of the n <= STEP_BATCH channels hs; end: it ends the call.
 int launch_step_batch(lbm_mix* const* hs, int n, bool end, cudaStream_t st) {
   StepBatch<STEP_BATCH> B;
-  // rows per CTA by the size of the whole launch (default_rows), but no fewer
-  // than a channel's own schedule has
+  // rows per CTA for some eight waves of the whole launch's CTAs, but no fewer
+  // than a channel's own schedule has: with 2 to 8 waves 24 mixed channels, 33 of
+  // 500 x 256, 12 of 3000 x 600 and 96 of 1000 x 64 are within 2 % of each other,
+  // with 16 3 to 6 % slower (two of 5001 x 130: 39.7 us at 3, 42.5 at 8)
   long strip_rows = 0;
   for (int q = 0; q < n; ++q) strip_rows += (long)hs[q]->L.N * hs[q]->nblocks;
   const long most = (strip_rows / (8 * 3L * (hs[0]->nsm > 0 ? hs[0]->nsm : 1)) + TY - 1) / TY * TY;

@@ -9,15 +9,16 @@
 // series and a rational form in packed FP32x2, and the moments, rates and
 // collision formed population by population.  FP32 storage uses the shorter
 // forms of lbm_mix.cu (psi from a table, sums shared by moments and
-// collision); here they would save another 12 % of the step (BF16 16384 x
-// 256: 113 against 127 us at 40 rows per CTA).  What does not change a bit is
+// collision); here they would save a fifth of the instructions (445 against 566
+// a node) and took 113 against 127 us of a BF16 16384 x 256 step when last
+// measured (before the end strips came first: 102).  What does not change a bit is
 // taken: the reciprocals and reciprocal square roots of the special-function
 // unit without the scaling for subnormal arguments (5 %).
 
 namespace n16 {
 
-// a / b as the approximate division forms it for arguments far from the ends
-// of the FP32 range.
+// a / b as the PTX ISA defines div.approx.f32, a times the approximate reciprocal
+// of b, for arguments far from the ends of the FP32 range.
 __device__ __forceinline__ float quotient(float a, float b) { return __fmul_rn(a, rcp_fast(b)); }
 
 // psi(a) = 1 + (a - 1) e^{-a} - a^2 E_1(a)  (Eq. psi).
@@ -65,22 +66,15 @@ __device__ __forceinline__ float dpsi_dev(float a) {
 
 // psi at two positive arguments at once.  The lanes of a warp sweep one row
 // (the same y) of 32 neighbouring columns, whose mean free paths differ
-// little, so with SKIP the two formulas of psi_dev are taken as warp-uniform
-// branches: the entire-part series when some lane has an argument <= 1, the
-// rational form when some lane has one in (1, 16).  Without SKIP both are
-// evaluated and selected (straight-line code that the compiler can
-// interleave with the loads of a memory-bound sweep).  At a >= 16,
-// 1 - psi(a) < 2 e^{-a}/a < 2^{-25} rounds away and psi = 1.
-template <bool SKIP>
+// little, so the two formulas of psi_dev are warp-uniform branches: the
+// entire-part series when some lane has an argument <= 1, the rational form when
+// some lane has one in (1, 16) (the kernel is bound by instruction issue).  At a
+// >= 16, 1 - psi(a) < 2 e^{-a}/a < 2^{-25} rounds away and psi = 1.
 __device__ __forceinline__ float2 psi2(float2 a) {
   const bool small = (a.x <= 1.0f) || (a.y <= 1.0f);
   const bool mid = (a.x > 1.0f && a.x < 16.0f) || (a.y > 1.0f && a.y < 16.0f);
-  bool do_small = true, do_mid = true;
-  if (SKIP) {
-    const unsigned lanes = __activemask();
-    do_small = __any_sync(lanes, small);
-    do_mid = __any_sync(lanes, mid);
-  }
+  const unsigned lanes = __activemask();
+  const bool do_small = __any_sync(lanes, small), do_mid = __any_sync(lanes, mid);
   float2 ps = f2(0.0f), pl = f2(1.0f);
   if (do_small) {
     const float2 as = make_float2(fminf(a.x, 1.0f), fminf(a.y, 1.0f));
@@ -120,9 +114,8 @@ __device__ __forceinline__ float2 psi2(float2 a) {
 }
 
 struct Macro {
-  float sd[2];           // sum of deviations: rho_s - rhobar_s
-  float rho[2], jx[2], jy[2];
-  float ux, uy;
+  float sd[2];  // sum of deviations: rho_s - rhobar_s
+  float rho[2];
   float n, inv_n, mx;
 };
 
@@ -133,21 +126,16 @@ __device__ __forceinline__ void macro(const Lat& L, const ColRef& C, const float
     const float* g = fs[sp];
     m.sd[sp] = ((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8];
     m.rho[sp] = C.rb[sp] + m.sd[sp];
-    m.jx[sp] = (g[1] - g[3]) + (g[5] - g[6]) + (g[8] - g[7]);
-    m.jy[sp] = (g[2] - g[4]) + (g[5] - g[7]) + (g[6] - g[8]);
   }
-  float rho = m.rho[0] + m.rho[1];
-  float inv_rho = __fdividef(1.0f, rho);
-  m.ux = (m.jx[0] + m.jx[1]) * inv_rho;
-  m.uy = (m.jy[0] + m.jy[1]) * inv_rho;
   m.n = fmaf(m.rho[0], L.s[0], m.rho[1] * L.s[1]);  // number density (Eq. P)
   m.inv_n = __fdividef(1.0f, m.n);
-  m.mx = rho * m.inv_n;  // m_x = rho / n
+  m.mx = (m.rho[0] + m.rho[1]) * m.inv_n;  // m_x = rho / n
 }
 
 // ------------------------------------------- packed per-node arithmetic
-// The node update of the step and moments kernels works on g[i] =
-// (species a, species b) pairs of the pre-collision deviations.
+// The node update of the step kernel works on g[i] = (species a, species b)
+// pairs of the pre-collision deviations.  (The moment fields of 16-bit states
+// are read with the FP32 forms.)
 struct Macro2 {
   float2 sd;   // sum of deviations: rho_s - rhobar_s
   float2 rho;  // species densities
@@ -177,7 +165,6 @@ __device__ __forceinline__ void macro2(const Lat& L, const ColRef& C, const floa
 // with the wall-confinement factor Psi(y) = (psi(y/lambda) + psi((H-y)/lambda))/2
 // of the effective mean free path; the six psi values come from three packed
 // evaluations.
-template <bool SKIP>
 __device__ __forceinline__ void rates2(const Lat& L, const Macro2& m, float y, float& om_s,
                                        float& om_d) {
   const float rs_mx = rsqrt_fast(m.mx);
@@ -188,9 +175,9 @@ __device__ __forceinline__ void rates2(const Lat& L, const Macro2& m, float y, f
   // mixture pressure
   const float2 ns = mul2(m.rho, L.s2);
   const float2 inv_ls = mul2(L.lam_mix ? f2(m.n) : ns, L.inv_c_xl2);
-  const float2 pm = psi2<SKIP>(mul2(yy, f2(inv_lam)));
-  const float2 pa = psi2<SKIP>(mul2(yy, f2(inv_ls.x)));
-  const float2 pb = psi2<SKIP>(mul2(yy, f2(inv_ls.y)));
+  const float2 pm = psi2(mul2(yy, f2(inv_lam)));
+  const float2 pa = psi2(mul2(yy, f2(inv_ls.x)));
+  const float2 pb = psi2(mul2(yy, f2(inv_ls.y)));
   const float ts = lam * (0.5f * (pm.x + pm.y)) * L.c_ts * rs_mx;  // tau_s - 1/2
   om_s = rcp_fast(0.5f + ts);
   // x_s lambda_se = c_xl / n * Psi(y; lambda_s) (partial pressure), times

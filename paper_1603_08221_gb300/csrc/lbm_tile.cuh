@@ -4,10 +4,11 @@
 //
 // What bounds a small channel is not memory or arithmetic but the length of
 // one step: a launch per step, the CTA's wall prologue, and rows that a warp
-// takes one after another.  lbm_step_kernel needs 14.5 us per step on a 320 x
-// 16 channel, 18 us on 700 x 20 and 33 us on 1280 x 64, whose state is 6 MB;
-// this kernel needs 1.9, 2.1 and 4.3 us.  lbm_tile_kernel cuts
-// the channel into tiles of W whole columns, one CTA each, loads a tile with
+// takes one after another.  lbm_step_kernel needs 9.0 us per step on a 320 x 16
+// channel, 9.7 us on 700 x 20 and on 1280 x 64, whose state is 6 MB (14.5, 18 and
+// 33 before it took rows and end strips by the channel's size); this kernel needs
+// 2.2, 2.3 and 4.6 us in calls of 100 steps.  lbm_tile_kernel cuts the channel
+// into tiles of W whole columns, one CTA each, loads a tile with
 // a halo of k columns on both sides into shared memory and takes k steps
 // there, the updated range shrinking by one column per side and step.  What a
 // column needs besides its neighbours (r and tau_q of its walls) is inside
@@ -48,7 +49,7 @@ struct TileInst {
   const float* alpha;
   const double* cs_in;   // [4][Nx]; the columns next to the ends are read
   double* cs_out;        // [4][Nx] column sums after step k
-  float2* hist;          // [records][4][Nx] column sums (error-free pairs) of
+  float2* hist;          // [records][4][Nx] column sums (pairs, column_sum8) of
                          // the launch's diagnostic steps, without N rhobar
   int W;                 // own columns per tile
   int diag_every, diag_phase;  // steps taken since the last multiple of diag_every
