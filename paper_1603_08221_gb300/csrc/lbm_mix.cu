@@ -2213,8 +2213,7 @@ double tile_cost(int N, int nup, int W, int k, int sms) {
 // fitted against it (64 x 3000 18.3 us, 128 x 8000 32.6).  With the end strips first
 // it has since become faster, 10 us up to some 100 000 nodes and 14 at 250 000, so
 // near the line tiles are no longer the better choice: columns x rows 4000 x 64
-// 12.8 us by tiles and 13.4, 14000 x 32 18.9 and 14.1, 2000 x 128 21.1 and 13.2
-// (either was 50 and more before tiles).
+// 12.8 us by tiles and 13.4, 14000 x 32 18.9 and 14.1, 2000 x 128 21.1 and 13.2.
 double step_kernel_cost(int N, int Nx) { return 15.0 + 1.75e-5 * (double)N * Nx; }
 
 // Tile width and steps per launch (odd, so that launches alternate the two

@@ -9,9 +9,9 @@
 // series and a rational form in packed FP32x2, and the moments, rates and
 // collision formed population by population.  FP32 storage uses the shorter
 // forms of lbm_mix.cu (psi from a table, sums shared by moments and
-// collision); here they would save a fifth of the instructions (445 against 566
-// a node) and took 113 against 127 us of a BF16 16384 x 256 step when last
-// measured (before the end strips came first: 102).  What does not change a bit is
+// collision); here they would save a fifth of the instructions (445 against 566 a
+// node) and, when last measured, 12 % of the step (BF16 16384 x 256 at 40 rows per
+// CTA: 113 against 127 us).  What does not change a bit is
 // taken: the reciprocals and reciprocal square roots of the special-function
 // unit without the scaling for subnormal arguments (5 %).
 
