@@ -145,7 +145,8 @@ int lbm_mix_init(lbm_mix* h);
  * r (Eq. R) and tau_q (Eq. taoq) of every column ahead of each pass.  All
  * are launched with programmatic dependent launch.  Every
  * diag_every-th step (counted from init) and the last step of the call
- * also reduce the separation diagnostics of the new state in FP64 (one
+ * also reduce the separation diagnostics of the new state (sums over a column
+ * as pairs of floats, 2^-44 of the sum, over the columns in FP64; one
  * history record each), so lbm_mix_separation after lbm_mix_step always
  * describes the current state.  After every reref_every-th step (counted
  * from init) the stored deviations are re-referenced (lbm_mix_rereference). */
@@ -331,7 +332,7 @@ int lbm_mix_step_noalloc(const lbm_mix_params* p, const float* d_in, float* d_ou
  * library default (16 to 96 rows by the channel's size; several steps per
  * launch where the channel qualifies, see lbm_mix_step, which a row count
  * turns off).  Changes only
- * the order of the FP64 column reductions.  May allocate; not during stream capture.
+ * the order of the column reductions.  May allocate; not during stream capture.
  * Errors: LBM_EINVAL (bad handle, rows not a multiple of 8), LBM_ENOMEM,
  * LBM_ECUDA. */
 int lbm_mix_set_rows_per_block(lbm_mix* h, int rows);
